@@ -20,7 +20,7 @@
 namespace pimd {
 size_t step_smem_bytes(int A, int P);
 size_t close_smem_bytes(int A, int P);
-size_t est_smem_bytes(int A, int P);
+int est_rows(int N, int A);
 cudaError_t launch_step(const StepArgs &a, int threads, cudaStream_t s);
 cudaError_t launch_close(const StepArgs &a, int threads, cudaStream_t s);
 cudaError_t launch_advance(int64_t *step, int n, cudaStream_t s);
@@ -182,10 +182,10 @@ struct pimd_handle {
   double *cref = nullptr, *ccur = nullptr, *blkmax = nullptr;
   int *nbr = nullptr, *nbr_off = nullptr;
   int nbr_groups = 1;
-  double *est_part = nullptr, *est_out = nullptr;
+  double *est_part = nullptr, *est_tot = nullptr, *est_out = nullptr;
   int nblk_est = 0;
   int64_t *d_step = nullptr;
-  unsigned *d_err = nullptr;
+  unsigned *d_err = nullptr;   // [0] error bits, [1] the estimators' finished-block counter
   // pinned host mirrors
   double *h_est = nullptr;
   unsigned *h_err = nullptr;
@@ -302,6 +302,13 @@ static int tile_atoms(int N, int P) {
 static int tile_threads(int A, int P) {
   int t = ((3 * A * P + 31) / 32) * 32;
   return std::min(256, std::max(32, t));
+}
+
+// Estimator tiles: up to 256 (atom, mode) tasks per block, fewer where the
+// system is small, so that its FP64 work spreads over the SMs (64 molecules x
+// 32 beads: one atom per block 192 blocks, not 8 per block on 24).
+static int est_tile_atoms(int N, int P) {
+  return std::min(std::max(1, 256 / P), std::max(1, (N + 303) / 304));
 }
 
 static int est_threads(int A, int P) {
@@ -765,8 +772,9 @@ static void carve(pimd_handle *h, Carver &c) {
     h->nbr_groups = water_lane_groups(P);
     h->nbr_off = c.take<int>((size_t)h->nmol * (kLJWarps * h->nbr_groups + 1));
   }
-  h->nblk_est = (N + h->A_est - 1) / h->A_est;
-  h->est_part = c.take<double>((size_t)h->nblk_est * (2 * P + 4));
+  h->nblk_est = est_rows(N, h->A_est);
+  h->est_part = c.take<double>((size_t)h->nblk_est * est_columns(P));
+  h->est_tot = c.take<double>(est_columns(P));
   h->est_out = c.take<double>(3 * P + 12);
   h->d_step = c.take<int64_t>(1);
   h->d_err = c.take<unsigned>(4);
@@ -1000,7 +1008,7 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
   h->A_step = tile_atoms(N, P);
   h->threads_step = tile_threads(h->A_step, P);
   h->split_warp = prm.precision == PIMD_PREC_SPLIT && split_warp_class(P);
-  h->A_est = std::max(1, 256 / P);
+  h->A_est = est_tile_atoms(N, P);
   h->threads_est = est_threads(h->A_est, P);
   const char *ng = getenv("PIMD_NO_GRAPH");
   h->use_graph = !(ng && ng[0] == '1');
@@ -1195,6 +1203,9 @@ extern "C" pimd_status pimd_estimators(pimd_handle *h, pimd_estimates *out) {
   a.v = h->v;
   a.F = h->F;
   a.wn2 = h->wn * h->wn;
+  a.nblk_force = h->nblk_force;
+  a.Upart = h->Upart;
+  a.Wpart = h->Wpart;
   a.part = h->est_part;
   pimd_status st0 = enqueue(h, PIMD_KIND_EST, 1, [&] { return launch_est(a, h->threads_est, h->stream); });
   if (st0 != PIMD_OK) return st0;
@@ -1202,10 +1213,9 @@ extern "C" pimd_status pimd_estimators(pimd_handle *h, pimd_estimates *out) {
   f.N = h->N;
   f.P = P;
   f.nblk_est = h->nblk_est;
-  f.nblk_force = h->nblk_force;
   f.part = h->est_part;
-  f.Upart = h->Upart;
-  f.Wpart = h->Wpart;
+  f.tot = h->est_tot;
+  f.count = h->d_err + 1;
   f.kT = kBoltzmann * h->T;
   f.kB = kBoltzmann;
   f.volume = (h->potential == PIMD_POT_WATERLIKE) ? h->box[0] * h->box[1] * h->box[2] : 0.0;

@@ -318,6 +318,10 @@ struct SplitForceArgs {
   int nbr_groups;
 };
 
+// Columns of an estimator row: K, S, U and Tr Xi per mode or bead, then
+// sum r.F, sum (r - r_c).F and m^(0) |v~_0|^2.
+__host__ __device__ constexpr int est_columns(int P) { return 4 * P + 3; }
+
 struct EstArgs {
   int N, P, A;
   int method;                  // 0 nmpimd, 1 pimd (Cartesian: v holds bead velocities)
@@ -325,13 +329,16 @@ struct EstArgs {
   const double *mass_mm;       // [N] m mvv2e
   const double *x, *v, *F;
   double wn2;                  // omega_n^2
-  double *part;                // [nblk][2P + 4]
+  int nblk_force;
+  const double *Upart, *Wpart; // [nblk_force][P]
+  double *part;                // [rows][est_columns(P)]
 };
 
 struct EstFinalArgs {
-  int N, P, nblk_est, nblk_force;
-  const double *part;          // [nblk_est][2P + 4]
-  const double *Upart, *Wpart; // [nblk_force][P]
+  int N, P, nblk_est;
+  const double *part;          // [nblk_est][est_columns(P)]
+  double *tot;                 // [est_columns(P)] column sums
+  unsigned *count;             // finished blocks, zero between calls
   double kT, volume, kB;
   const double *dbox;          // device box edges (barostat): volume = L0 L1 L2, or null
   double *out;                 // [3P + 12]
