@@ -29,6 +29,7 @@ cudaError_t launch_thermal_v(double *v, const double *sigv, const double *imu, u
                              cudaStream_t s);
 cudaError_t launch_fixcom(const FixcomArgs &a, cudaStream_t s);
 cudaError_t launch_baro_kick(const BaroArgs &a, cudaStream_t s);
+size_t sums_part_doubles(int N, int P, int method);
 cudaError_t launch_pna_to_nap(const double *src, double *dst, int N, int P, cudaStream_t s);
 cudaError_t launch_nap_to_pna(const double *src, double *dst, int N, int P, cudaStream_t s);
 cudaError_t launch_force_harmonic(const ForceArgs &a, cudaStream_t s);
@@ -142,6 +143,10 @@ struct pimd_handle {
   int N = 0, P = 0, potential = 0, nmol = 0, integrator = 0, thermostat = 0, precision = 0;
   int method = 0, fixcom = 0, barostat = 0;
   int baro_axes = 0;          // anisotropic barostat: mask of edges with their own v_W (0: isotropic)
+  // fixcom and barostat: partial sums, the mean velocity that the next kernel
+  // subtracts ([P][3]), the total mass (m mvv2e)
+  double *sums_part = nullptr, *fix_u = nullptr;
+  double msum = 0;
   double *W3part = nullptr;   // anisotropic barostat: [nmol][P][3] diagonal virial rows
   double T = 0, dt = 0, tau = 0, scale = 0, sp = 0, fmass = 1.0, pext = 0, taup = 0;
   double *baro = nullptr;     // device barostat state (kBaroWords), or null
@@ -185,7 +190,7 @@ struct pimd_handle {
   double *est_part = nullptr, *est_tot = nullptr, *est_out = nullptr;
   int nblk_est = 0;
   int64_t *d_step = nullptr;
-  unsigned *d_err = nullptr;   // [0] error bits, [1] the estimators' finished-block counter
+  unsigned *d_err = nullptr;   // [0] error bits, [1], [2] finished-block counters (estimators; sums over atoms)
   // pinned host mirrors
   double *h_est = nullptr;
   unsigned *h_err = nullptr;
@@ -547,8 +552,12 @@ static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, bool advanc
 
 // B_W of the barostat over [t0, t0 + tB] of the kick the next kernel
 // applies (App. E); with step_follows also that step's O_W and box.
-static pimd_status enqueue_baro(pimd_handle *h, double t0, double tB, bool step_follows) {
+// fix_pending: the previous step's fixcom is still to be subtracted from v.
+static pimd_status enqueue_baro(pimd_handle *h, double t0, double tB, bool step_follows, bool fix_pending) {
   BaroArgs b{};
+  b.fix_u = fix_pending ? h->fix_u : nullptr;
+  b.part = h->sums_part;
+  b.count = h->d_err + 2;
   b.obabo = h->integrator == PIMD_OBABO;
   b.N = h->N;
   b.P = h->P;
@@ -604,6 +613,8 @@ static pimd_status enqueue_step(pimd_handle *h, bool first) {
   StepArgs a = step_args(h);
   a.first = first ? 1 : 0;
   a.kick = first ? 0.5 * h->dt : h->dt;
+  const bool fix_pending = h->fixcom && !first;
+  a.fix_u = fix_pending ? h->fix_u : nullptr;
   pimd_status st;
   if (h->baro && h->integrator == PIMD_OBABO) {
     // OBABO: the opening B_W needs the velocities after both O(h/2), so the
@@ -611,15 +622,17 @@ static pimd_status enqueue_step(pimd_handle *h, bool first) {
     StepArgs a1 = a, a2 = a;
     a1.phase = 1;
     a2.phase = 2;
+    a2.fix_u = nullptr;   // phase 1 stored the velocities
     st = enqueue(h, PIMD_KIND_STEP, 1, [&] { return launch_step(a1, h->threads_step, h->stream); });
     if (st != PIMD_OK) return st;
-    if ((st = enqueue_baro(h, 0.0, 0.5 * h->dt, true)) != PIMD_OK) return st;
+    if ((st = enqueue_baro(h, 0.0, 0.5 * h->dt, true, false)) != PIMD_OK) return st;
     st = enqueue(h, PIMD_KIND_STEP, 1, [&] { return launch_step(a2, h->threads_step, h->stream); });
     if (st != PIMD_OK) return st;
   } else {
     // the B_W beside this step's opening B(h/2), which follows the previous
     // step's closing B(h/2) inside a merged kick
-    if (h->baro && (st = enqueue_baro(h, first ? 0.0 : 0.5 * h->dt, 0.5 * h->dt, true)) != PIMD_OK)
+    if (h->baro &&
+        (st = enqueue_baro(h, first ? 0.0 : 0.5 * h->dt, 0.5 * h->dt, true, fix_pending)) != PIMD_OK)
       return st;
     st = enqueue(h, PIMD_KIND_STEP, 1, [&] { return launch_step(a, h->threads_step, h->stream); });
     if (st != PIMD_OK) return st;
@@ -627,10 +640,10 @@ static pimd_status enqueue_step(pimd_handle *h, bool first) {
   st = enqueue_forces(h, false, true);
   if (st != PIMD_OK) return st;
   // the B_W beside this step's closing B(h/2) (applied by the next kernel)
-  if (h->baro && (st = enqueue_baro(h, 0.0, 0.5 * h->dt, false)) != PIMD_OK) return st;
+  if (h->baro && (st = enqueue_baro(h, 0.0, 0.5 * h->dt, false, false)) != PIMD_OK) return st;
   if (!h->fixcom) return st;
   // fixcom at the end of this step: the next kernel (step or close) applies
-  // this step's closing B(h/2) (and O(h/2)); remove the momentum it will leave
+  // this step's closing B(h/2) (and O(h/2)) and removes the momentum it would leave
   FixcomArgs f{};
   f.N = h->N;
   f.P = h->P;
@@ -639,6 +652,10 @@ static pimd_status enqueue_step(pimd_handle *h, bool first) {
   f.x = h->x;
   f.F = h->F;
   f.v = h->v;
+  f.u = h->fix_u;
+  f.msum = h->msum;
+  f.part = h->sums_part;
+  f.count = h->d_err + 2;
   f.half = 0.5 * h->dt;
   f.imu0 = 1.0 / h->fmass;   // mu_0 = fmass in both methods
   f.wn2 = h->wn * h->wn;
@@ -659,6 +676,7 @@ static pimd_status enqueue_close(pimd_handle *h) {
   }
   StepArgs a = step_args(h);
   a.step_off = -1;
+  a.fix_u = h->fixcom ? h->fix_u : nullptr;
   return enqueue(h, PIMD_KIND_CLOSE, 1, [&] { return launch_close(a, h->threads_step, h->stream); });
 }
 
@@ -779,6 +797,10 @@ static void carve(pimd_handle *h, Carver &c) {
   h->d_step = c.take<int64_t>(1);
   h->d_err = c.take<unsigned>(4);
   if (h->barostat) h->baro = c.take<double>(kBaroWords);
+  if (h->barostat || h->fixcom) {
+    h->sums_part = c.take<double>(sums_part_doubles(N, P, h->method));
+    h->fix_u = c.take<double>((size_t)3 * P);
+  }
   if (h->baro_axes) h->W3part = c.take<double>((size_t)h->nmol * P * 3);
   if (h->precision == PIMD_PREC_SPLIT) {
     h->xc = c.take<double>((size_t)N * 3);
@@ -1043,6 +1065,7 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
     inv_mm[i] = 1.0 / mm;
     sigv[i] = std::sqrt(P * kBoltzmann * T / mm);
     ksp[i] = mm * sys->ff[0] * sys->ff[0];
+    h->msum += mm;
   }
   pimd_status st = PIMD_OK;
   auto up = [&](double *dst, const std::vector<double> &src) -> pimd_status {

@@ -186,6 +186,7 @@ struct StepArgs {
   // step's closing B O and this step's O (velocities only), phase 2 = B(h/2)
   // A(h) and the new positions; phase 0 = the whole step in one launch
   int phase;
+  const double *fix_u;         // fixcom of the previous step, still to be subtracted from v: [k][3], or null
   int noise_pre;               // 1: PILE_L deviates drawn once per (atom, mode) into shared memory
 };
 
@@ -214,17 +215,23 @@ struct BaroArgs {
   const int64_t *step;
   double Lmin;                 // smallest allowed box edge (2 rc)
   unsigned *err;
+  const double *fix_u;         // fixcom still to be subtracted from v (centroid mode), or null
+  double *part;                // partial sums (sums_part_doubles)
+  unsigned *count;             // finished blocks, zero between launches
 };
 
-// fixcom: remove the centre-of-mass velocity of the centroid mode (normal
-// modes) or of every bead (Cartesian) as it will stand after the closing
-// B(h/2) that the next kernel applies (the removal belongs at the end of the
-// step; subtracting its predicted value first is the same linear operation).
+// fixcom: the centre-of-mass velocity of the centroid mode (normal modes) or
+// of every bead (Cartesian) as it will stand after the closing B(h/2) that the
+// next kernel applies (the removal belongs at the end of the step; subtracting
+// its predicted value first is the same linear operation).
 struct FixcomArgs {
   int N, P, method;
   const double *mass_mm;       // [N] m mvv2e
-  const double *x, *F;         // [N][3][P]
-  double *v;                   // [N][3][P]
+  double msum;                 // their sum
+  const double *x, *F, *v;     // [N][3][P]
+  double *u;                   // out: [nb][3], subtracted by the next kernel
+  double *part;                // partial sums (sums_part_doubles)
+  unsigned *count;             // finished blocks, zero between launches
   double half;                 // h/2
   double imu0;                 // 1 / mu_0 (normal modes) or 1 / fmass (Cartesian)
   double wn2;                  // omega_n^2 (Cartesian springs)

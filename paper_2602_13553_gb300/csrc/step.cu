@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(256) k_step_f64(StepArgs a) {
     const double f = fa + fb;
     double q = qa + qb;
     double v = sV[task];
+    if (a.fix_u && k == 0) v -= a.fix_u[r % 3];   // the previous step's fixcom
     const double im = __ldg(a.inv_mm + i) * __ldg(a.mt.imu + k);   // 1 / (m^(k) mvv2e)
     const double cA = __ldg(a.mt.cA + k), sA = __ldg(a.mt.sA + k), wsA = __ldg(a.mt.wsA + k);
     const double c1 = __ldg(a.mt.c1 + k), c2s = __ldg(a.mt.c2 + k) * __ldg(a.sigv + i);
@@ -307,7 +308,9 @@ __global__ void __launch_bounds__(256) k_close_f64(StepArgs a) {
       fb = fma(__ldg(Mt + (j + 1) * P + k), fx[j + 1], fb);
     }
     if (j < P) fa = fma(__ldg(Mt + j * P + k), fx[j], fa);
-    double v = fma(a.half * (__ldg(a.inv_mm + i) * __ldg(a.mt.imu + k)), fa + fb, a.v[base + task]);
+    double v = a.v[base + task];
+    if (a.fix_u && k == 0) v -= a.fix_u[d];   // the last step's fixcom
+    v = fma(a.half * (__ldg(a.inv_mm + i) * __ldg(a.mt.imu + k)), fa + fb, v);
     if (a.integrator == 1 && a.thermo) {
       const double c1 = __ldg(a.mt.c1 + k), c2s = __ldg(a.mt.c2 + k) * __ldg(a.sigv + i);
       v = fma(c1, v, c2s * gauss1(a.seed, (uint32_t)i, (uint32_t)k, kStreamO2, step, d));
@@ -366,6 +369,7 @@ __global__ void __launch_bounds__(256) k_step_cart_f64(StepArgs a) {
     const double im = __ldg(a.inv_mm + i) * a.ifmass;
     const double c2s = c2 * __ldg(a.sigv + i);
     double v = a.v[base + task];
+    if (a.fix_u) v -= a.fix_u[3 * k + r % 3];   // the previous step's fixcom
     double x = sX[task];
     if (a.integrator == 0) {
       v = fma(a.kick * im, f, v);
@@ -442,183 +446,12 @@ __global__ void __launch_bounds__(256) k_close_cart_f64(StepArgs a) {
     const int d = (int)(r % 3);
     const int i = (int)(r / 3);
     const double f = a.F[t] + spring_force(a.x + r * P, k, P, __ldg(a.mass_mm + i) * a.wn2);
-    double v = fma(a.half * (__ldg(a.inv_mm + i) * a.ifmass), f, a.v[t]);
+    double v = a.v[t];
+    if (a.fix_u) v -= a.fix_u[3 * k + d];   // the last step's fixcom
+    v = fma(a.half * (__ldg(a.inv_mm + i) * a.ifmass), f, v);
     if (a.integrator == 1 && a.thermo)
       v = fma(c1, v, c2 * __ldg(a.sigv + i) * gauss1(a.seed, (uint32_t)i, (uint32_t)k, kStreamO2, step, d));
     a.v[t] = v;
-  }
-}
-
-// fixcom: one block; deterministic sums (fixed per-thread strides, then a
-// fixed tree) of m v, F and (Cartesian) m x per (bead or centroid mode,
-// component), then v -= u on every atom.
-__device__ double block_sum(double v, double *red) {
-  red[threadIdx.x] = v;
-  __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-    __syncthreads();
-  }
-  const double r = red[0];
-  __syncthreads();
-  return r;
-}
-
-__global__ void __launch_bounds__(256) k_fixcom_f64(FixcomArgs a) {
-  __shared__ double red[256];
-  __shared__ double sp[3 * kMaxBeads], sf[3 * kMaxBeads], sx[3 * kMaxBeads], u[3 * kMaxBeads];
-  const int P = a.P, N = a.N;
-  const int nb = a.method == 0 ? 1 : P;
-  double m = 0.0;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) m += a.mass_mm[i];
-  const double msum = block_sum(m, red);
-  for (int kc = 0; kc < 3 * nb; ++kc) {
-    const int k = kc / 3, c = kc % 3;
-    double pv = 0.0, pf = 0.0, px = 0.0, pn = 0.0;
-    const uint64_t s = (uint64_t)(*a.step - 1);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const size_t row = ((size_t)i * 3 + c) * P;
-      const double mm = a.mass_mm[i];
-      pv = fma(mm, a.v[row + k], pv);
-      if (a.obabo_thermo)
-        pn = fma(mm * a.sigv[i], gauss1(a.seed, (uint32_t)i, (uint32_t)k, kStreamO2, s, c), pn);
-      if (a.method == 0) {
-        double fs = 0.0;   // sqrt(P) F~_0 = sum over beads
-        for (int j = 0; j < P; ++j) fs += a.F[row + j];
-        pf += fs;
-      } else {
-        pf += a.F[row + k];
-        px = fma(mm, a.x[row + k], px);
-      }
-    }
-    pv = block_sum(pv, red);
-    pf = block_sum(pf, red);
-    px = block_sum(px, red);
-    pn = block_sum(pn, red);
-    if (threadIdx.x == 0) {
-      // the closing O(h/2) scales by c1 and adds c2 sigv eta: remove its mean too
-      sp[kc] = a.obabo_thermo ? pv + a.c2[k] * pn / a.c1[k] : pv;
-      sf[kc] = a.method == 0 ? pf / sqrt((double)P) : pf;
-      sx[kc] = px;
-    }
-  }
-  __syncthreads();
-  for (int kc = threadIdx.x; kc < 3 * nb; kc += blockDim.x) {
-    const int k = kc / 3, c = kc % 3;
-    double f = sf[kc];
-    if (a.method == 1) {
-      const int km = k == 0 ? P - 1 : k - 1, kp = k == P - 1 ? 0 : k + 1;
-      f -= a.wn2 * (2.0 * sx[kc] - sx[3 * km + c] - sx[3 * kp + c]);
-    }
-    u[kc] = fma(a.half * a.imu0, f, sp[kc]) / msum;
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < N * 3 * nb; t += blockDim.x) {
-    const int k = t % nb;
-    const int ic = t / nb;
-    a.v[(size_t)ic * P + k] -= u[3 * k + ic % 3];
-  }
-}
-
-// B_W of the BZP barostat (App. E) over [t0, t0 + tB] of the kick that the
-// next kernel applies to the current velocities, with n = P.  Isotropic:
-//   v_W += (3 tB / W)[n V P_CV - n V P_ext + n kB T] + (tB^2 / W) sum F~0.v~0
-//          + (tB^3 / 3W) sum |F~0|^2 / m~0,
-//   3 n V P_CV = sum m~0 |v~0|^2 - sum (r - r_c).F + sum_k Tr Xi^(k);
-// anisotropic, for each edge a in the mask, the same with the a components
-// alone, W the per-edge mass and 3 n V P_CV -> n V P_CV^aa (the Xi_aa rows).
-// Then, if a step follows, its v_W at the first A, after O_W (PILE_L: each
-// edge its own deviate) and the box after both A sub-steps.  One block;
-// fixed-order sums.
-__global__ void __launch_bounds__(256) k_baro_kick(BaroArgs a) {
-  __shared__ double red[256];
-  const int P = a.P;
-  double mv2[3] = {0.0, 0.0, 0.0}, fv[3] = {0.0, 0.0, 0.0}, f2m[3] = {0.0, 0.0, 0.0};
-  double rcf[3] = {0.0, 0.0, 0.0}, vir[3] = {0.0, 0.0, 0.0};
-  for (int i = threadIdx.x; i < a.N; i += blockDim.x) {
-    const double mm = a.mass_mm[i] * a.mu0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const size_t row = ((size_t)i * 3 + c) * P;
-      double f0 = 0.0, xm = 0.0;
-      for (int j = 0; j < P; ++j) {
-        f0 = fma(a.Mt[j * P], a.F[row + j], f0);   // F~0 = (M F)_0
-        xm += a.x[row + j];
-      }
-      xm /= P;
-      for (int j = 0; j < P; ++j) rcf[c] = fma(a.x[row + j] - xm, a.F[row + j], rcf[c]);
-      const double v0 = fma(a.t0, f0 / mm, a.v[row]);   // at t0 into the kick
-      mv2[c] = fma(mm * v0, v0, mv2[c]);
-      fv[c] = fma(f0, v0, fv[c]);
-      f2m[c] += f0 * f0 / mm;
-    }
-  }
-  if (a.axes) {
-    for (int t = threadIdx.x; t < a.nmol * P; t += blockDim.x)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) vir[c] += a.W3part[(size_t)t * 3 + c];
-  } else {
-    for (int t = threadIdx.x; t < a.nmol * P; t += blockDim.x) vir[0] += a.Wpart[t];
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    mv2[c] = block_sum(mv2[c], red);
-    fv[c] = block_sum(fv[c], red);
-    f2m[c] = block_sum(f2m[c], red);
-    rcf[c] = block_sum(rcf[c], red);
-    vir[c] = block_sum(vir[c], red);
-  }
-  if (threadIdx.x != 0) return;
-  double *b = a.baro;
-  const double V = b[kBaroL] * b[kBaroL + 1] * b[kBaroL + 2];
-  const double tB = a.tB;
-  // O_W: v_W <- c1 v_W + sigW eta, eta from Philox atom 0xffffffff, stream 3,
-  // the given mode; each edge its own deviate, the isotropic v_W the first
-  auto langevin = [&](double *w, uint32_t mode, uint64_t st) {
-    double e[3];
-    gauss3(a.seed, 0xffffffffu, mode, 3u, st, e[0], e[1], e[2]);
-    if (a.axes) {
-      for (int c = 0; c < 3; ++c)
-        if (a.axes >> c & 1) w[c] = a.c1W * w[c] + a.sigW * e[c];
-    } else {
-      w[0] = w[1] = w[2] = a.c1W * w[0] + a.sigW * e[0];
-    }
-  };
-  const uint64_t step = (uint64_t)*a.step;
-  double vW[3] = {b[kBaroV], b[kBaroV + 1], b[kBaroV + 2]};
-  if (a.obabo && a.step_follows && a.thermo) langevin(vW, 0u, step);   // this step's first O(h/2)
-  if (a.axes) {
-    for (int c = 0; c < 3; ++c)
-      vW[c] = (a.axes >> c & 1)
-                  ? vW[c] + tB / a.W * (mv2[c] - rcf[c] + vir[c] - V * a.npext + a.nkT) +
-                        tB * tB / a.W * fv[c] + tB * tB * tB / (3.0 * a.W) * f2m[c]
-                  : 0.0;
-  } else {
-    const double smv2 = mv2[0] + mv2[1] + mv2[2], srcf = rcf[0] + rcf[1] + rcf[2];
-    const double sfv = fv[0] + fv[1] + fv[2], sf2m = f2m[0] + f2m[1] + f2m[2];
-    const double w = vW[0] + 3.0 * tB / a.W * ((smv2 - srcf + vir[0]) / 3.0 - V * a.npext + a.nkT) +
-                     tB * tB / a.W * sfv + tB * tB * tB / (3.0 * a.W) * sf2m;
-    vW[0] = vW[1] = vW[2] = w;
-  }
-  if (!a.step_follows) {
-    // OBABO: the closing O(h/2) of the step just completed (the counter has
-    // already been advanced past it)
-    if (a.obabo && a.thermo) langevin(vW, 1u, step - 1);
-    for (int c = 0; c < 3; ++c) b[kBaroV + c] = vW[c];
-    return;
-  }
-  double vO[3] = {vW[0], vW[1], vW[2]};
-  if (a.thermo && !a.obabo) langevin(vO, 0u, step);
-  for (int c = 0; c < 3; ++c) {
-    b[kBaroVA1 + c] = vW[c];
-    b[kBaroVA2 + c] = vO[c];
-    b[kBaroV + c] = vO[c];
-    // BAOAB: A(h/2) at v_W, O_W, A(h/2) at v_O; OBABO: one A(h) at v_W
-    const double L = a.obabo ? b[kBaroL + c] * exp(a.tA * vW[c])
-                             : b[kBaroL + c] * exp(a.tA * vW[c]) * exp(a.tA * vO[c]);
-    b[kBaroL + c] = L;
-    b[kBaroInvL + c] = 1.0 / L;
-    if (!(L > a.Lmin)) atomicOr(a.err, kErrBoxSmall);
   }
 }
 
@@ -698,16 +531,6 @@ cudaError_t launch_close(const StepArgs &a, int threads, cudaStream_t s) {
   }
   const int grid = (a.N + a.A - 1) / a.A;
   k_close_f64<<<grid, threads, close_smem_bytes(a.A, a.P), s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_baro_kick(const BaroArgs &a, cudaStream_t s) {
-  k_baro_kick<<<1, 256, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fixcom(const FixcomArgs &a, cudaStream_t s) {
-  k_fixcom_f64<<<1, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
