@@ -14,12 +14,13 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fixed.cuh"
 #include "pimd.h"
 #include "runtime.h"
 
 namespace pimd {
-size_t step_smem_bytes(int A, int P);
-size_t close_smem_bytes(int A, int P);
+int step_tile_atoms(int N, int P);
+int step_threads(int A, int P);
 int est_rows(int N, int A);
 cudaError_t launch_step(const StepArgs &a, int threads, cudaStream_t s);
 cudaError_t launch_close(const StepArgs &a, int threads, cudaStream_t s);
@@ -182,6 +183,11 @@ struct pimd_handle {
   double *M = nullptr, *Mt = nullptr, *cA = nullptr, *sA = nullptr, *wsA = nullptr;
   double *c1 = nullptr, *c2 = nullptr, *lam = nullptr, *mu = nullptr, *imu = nullptr;
   double *Tf = nullptr, *Ti = nullptr;   // folded transforms, [P/2 + 1][P]
+  // FP64 normal-mode step: folded transforms in fixed point, A O A as one map
+  // per mode, [2][N] B(h/2) and B(h) durations over m mvv2e
+  int4 *fTf = nullptr, *fTi = nullptr;
+  int fem = 0, mu_one = 0;
+  double *map6 = nullptr, *kmm = nullptr;
   double *Upart = nullptr, *Wpart = nullptr;
   int nblk_force = 0;
   double *cref = nullptr, *ccur = nullptr, *blkmax = nullptr;
@@ -326,8 +332,11 @@ static StepArgs step_args(pimd_handle *h) {
   a.N = h->N;
   a.P = h->P;
   a.A = h->A_step;
-  a.mt = ModeTables{h->M, h->Mt, h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf, h->Ti};
+  a.mt = ModeTables{h->M, h->Mt, h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf, h->Ti,
+                    h->fTf, h->fTi, h->fem, h->map6, 1.0 / std::sqrt((double)h->P)};
   a.inv_mm = h->inv_mm;
+  a.mu_one = h->mu_one;
+  a.kmm = h->kmm;   // B(h/2)
   a.sigv = h->sigv;
   a.x = h->x;
   a.v = h->v;
@@ -572,17 +581,19 @@ static pimd_status enqueue_baro(pimd_handle *h, double t0, double tB, bool step_
   b.axes = h->baro_axes;
   b.baro = h->baro;
   b.t0 = t0;
-  b.tB = tB;
   b.tA = b.obabo ? h->dt : 0.5 * h->dt;
   b.step_follows = step_follows ? 1 : 0;
   const double kT = kBoltzmann * h->T;
-  b.W = (h->baro_axes ? 1.0 : 3.0) * h->P * h->N * kT * h->taup * h->taup;
+  const double W = (h->baro_axes ? 1.0 : 3.0) * h->P * h->N * kT * h->taup * h->taup;
+  b.k1 = (h->baro_axes ? 1.0 : 3.0) * tB / W;
+  b.k2 = tB * tB / W;
+  b.k3 = tB * tB * tB / (3.0 * W);
   b.nkT = h->P * kT;
   b.npext = h->P * h->pext;
   b.mu0 = h->fmass;
   b.thermo = h->thermostat == PIMD_THERMO_PILE_L;
   b.c1W = std::exp(-(b.obabo ? 0.5 * h->dt : h->dt) / h->tau);   // the O_W's own duration
-  b.sigW = std::sqrt(1.0 - b.c1W * b.c1W) * std::sqrt(b.nkT / b.W);
+  b.sigW = std::sqrt(1.0 - b.c1W * b.c1W) * std::sqrt(b.nkT / W);
   b.seed = h->seed;
   b.step = h->d_step;
   b.Lmin = 2.0 * h->ff[6];
@@ -613,6 +624,8 @@ static pimd_status enqueue_step(pimd_handle *h, bool first) {
   StepArgs a = step_args(h);
   a.first = first ? 1 : 0;
   a.kick = first ? 0.5 * h->dt : h->dt;
+  // BAOAB merges the closing B(h/2) of the previous step into its kick
+  if (!first && h->integrator == PIMD_BAOAB) a.kmm = h->kmm + h->N;
   const bool fix_pending = h->fixcom && !first;
   a.fix_u = fix_pending ? h->fix_u : nullptr;
   pimd_status st;
@@ -778,6 +791,10 @@ static void carve(pimd_handle *h, Carver &c) {
   h->imu = c.take<double>(P);
   h->Tf = c.take<double>((size_t)(P / 2 + 1) * P);
   h->Ti = c.take<double>((size_t)(P / 2 + 1) * P);
+  h->fTf = c.take<int4>((size_t)fix_pairs(P) * P);
+  h->fTi = c.take<int4>((size_t)fix_pairs(P) * P);
+  h->map6 = c.take<double>((size_t)6 * P);
+  h->kmm = c.take<double>((size_t)2 * N);
   // rows of per-bead U / Tr Xi sums: one per molecule (water) or per block
   h->nblk_force = h->potential == PIMD_POT_WATERLIKE ? h->nmol : force_blocks(h->N, P);
   h->Upart = c.take<double>((size_t)h->nblk_force * P);
@@ -982,6 +999,48 @@ void build_tables(int P, double T, double dt, const pimd_params &prm, HostTables
 }
 }  // namespace pimd
 
+// A folded transform table [P/2 + 1][P] in the fixed point of fixed.cuh:
+// entries over 2^em, the power of two at or above the largest, as 55-bit
+// integers in two signed 28-bit limbs, two terms to an int4.  Returns em.
+static int fixed_table(int P, const std::vector<double> &T, std::vector<int4> &out) {
+  double mx = 0.0;
+  for (double t : T) mx = std::max(mx, std::fabs(t));
+  int em = 0;
+  const double fr = std::frexp(mx, &em);   // mx = fr 2^em, fr in [1/2, 1)
+  if (fr == 0.5) --em;
+  const int np = fix_pairs(P), H = P / 2;
+  out.assign((size_t)np * P, int4{0, 0, 0, 0});
+  for (int j = 0; j <= H; ++j)
+    for (int k = 0; k < P; ++k) {
+      const long long m = std::llrint(std::ldexp(T[(size_t)j * P + k], kFixBits - em));
+      const long long r = m + 0x8000000;
+      const int hi = (int)(r >> 28), lo = (int)(r & 0xfffffff) - 0x8000000;
+      int4 &o = out[(size_t)(j / 2) * P + k];
+      if (j & 1) {
+        o.z = hi;
+        o.w = lo;
+      } else {
+        o.x = hi;
+        o.y = lo;
+      }
+    }
+  return em;
+}
+
+// A(h/2) O(h) A(h/2) of every mode as one linear map of (q, v, n), n the
+// unit-mode noise sqrt(P kB T / (m mvv2e)) eta (ModeTables::map6).
+static void aoa_map(int P, const HostTables &t, bool thermo, std::vector<double> &m) {
+  m.assign((size_t)6 * P, 0.0);
+  for (int k = 0; k < P; ++k) {
+    const long double c = t.cA[k], s = t.sA[k], w = t.wsA[k];
+    const long double c1 = thermo ? t.c1[k] : 1.0, c2 = thermo ? t.c2[k] : 0.0;
+    // q1 = c q + s v, v1 = c v - w q; v2 = c1 v1 + c2 n; q' = c q1 + s v2, v' = c v2 - w q1
+    const long double row[6] = {c * c - s * c1 * w, c * s + s * c1 * c, s * c2,
+                                -(c * c1 * w) - w * c, c * c1 * c - w * s, c * c2};
+    for (int r = 0; r < 6; ++r) m[(size_t)r * P + k] = (double)row[r];
+  }
+}
+
 extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, double dt,
                                    double gamma0, const pimd_params *params, void *stream,
                                    pimd_handle **out) {
@@ -1027,8 +1086,13 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
     }
     h->own_stream = true;
   }
-  h->A_step = tile_atoms(N, P);
-  h->threads_step = tile_threads(h->A_step, P);
+  if (prm.precision == PIMD_PREC_FP64 && prm.method == PIMD_METHOD_NMPIMD) {
+    h->A_step = step_tile_atoms(N, P);
+    h->threads_step = step_threads(h->A_step, P);
+  } else {
+    h->A_step = tile_atoms(N, P);
+    h->threads_step = tile_threads(h->A_step, P);
+  }
   h->split_warp = prm.precision == PIMD_PREC_SPLIT && split_warp_class(P);
   h->A_est = est_tile_atoms(N, P);
   h->threads_est = est_threads(h->A_est, P);
@@ -1080,6 +1144,30 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
       (st = up(h->mass_mm, mass_mm)) || (st = up(h->kspring, ksp))) {
     release(h);
     return st;
+  }
+  {
+    std::vector<int4> fTf, fTi;
+    h->fem = fixed_table(P, tb.Tf, fTf);
+    const int fi = fixed_table(P, tb.Ti, fTi);
+    if (fi != h->fem) {   // the entries of both are those of M
+      release(h);
+      return fail(PIMD_EINVAL, "internal: transform scales %d and %d differ", h->fem, fi);
+    }
+    std::vector<double> map6, kmm(2 * (size_t)N);
+    aoa_map(P, tb, h->thermostat == PIMD_THERMO_PILE_L, map6);
+    for (int i = 0; i < N; ++i) {
+      kmm[i] = 0.5 * dt * inv_mm[i];
+      kmm[N + i] = dt * inv_mm[i];
+    }
+    h->mu_one = std::all_of(tb.imu.begin(), tb.imu.end(), [](double m) { return m == 1.0; });
+    auto upi = [&](int4 *dst, const std::vector<int4> &src) -> pimd_status {
+      CK(cudaMemcpy(dst, src.data(), src.size() * sizeof(int4), cudaMemcpyHostToDevice));
+      return PIMD_OK;
+    };
+    if ((st = up(h->map6, map6)) || (st = up(h->kmm, kmm)) || (st = upi(h->fTf, fTf)) || (st = upi(h->fTi, fTi))) {
+      release(h);
+      return st;
+    }
   }
   if (h->precision == PIMD_PREC_SPLIT) {
     auto upf = [&](float *dst, const std::vector<double> &src) -> pimd_status {
@@ -1220,7 +1308,8 @@ extern "C" pimd_status pimd_estimators(pimd_handle *h, pimd_estimates *out) {
   a.P = P;
   a.A = h->A_est;
   a.method = h->method;
-  a.mt = ModeTables{h->M, h->Mt, h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf, h->Ti};
+  a.mt = ModeTables{h->M, h->Mt, h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf, h->Ti,
+                    h->fTf, h->fTi, h->fem, h->map6, 1.0 / std::sqrt((double)P)};
   a.mass_mm = h->mass_mm;
   a.x = h->x;
   a.v = h->v;

@@ -34,7 +34,11 @@ enum : unsigned { kErrNbrOverflow = 1u, kErrNonFinite = 2u, kErrBoxSmall = 4u };
 //   [0..2] v_W after the last completed sub-step
 //   [3..5] v_W of this step's first A (after its B_W), [6..8] after its O
 //   [9..11] box edges L, [12..14] 1 / L (the layout of ForceArgs::dbox)
-enum { kBaroV = 0, kBaroVA1 = 3, kBaroVA2 = 6, kBaroL = 9, kBaroInvL = 12, kBaroWords = 16 };
+//   [16..24], [25..33] factors of the centroid mode's A at those two v_W, for
+//   each edge e^a, e^-a and (e^a - e^-a) / (2 v_W), a = tA v_W
+enum {
+  kBaroV = 0, kBaroVA1 = 3, kBaroVA2 = 6, kBaroL = 9, kBaroInvL = 12, kBaroA1 = 16, kBaroA2 = 25, kBaroWords = 36
+};
 
 // ---------------------------------------------------------------------------
 // Philox-4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of
@@ -59,42 +63,46 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 // Noise streams of the counter's second word (bits 16..31).
 enum : uint32_t { kStreamO1 = 0u, kStreamO2 = 1u, kStreamInit = 2u };
 
-// Three standard normal deviates for (atom, normal mode, stream, step):
-// counter = (atom, mode | stream << 16, step lo, step hi), key = seed;
-// u = (w + 1/2) 2^-32; Box-Muller: (eta_x, eta_y) = r0 (cos, sin)(2 pi u1),
-// eta_z = r1 cos(2 pi u3), r = sqrt(-2 ln u).
+// The four words of (atom, normal mode, stream, step): counter = (atom,
+// mode | stream << 16, step lo, step hi), key = seed.
+__device__ __forceinline__ uint4 noise_words(uint64_t seed, uint32_t atom, uint32_t mode, uint32_t stream,
+                                             uint64_t step) {
+  return philox4x32_10(make_uint4(atom, (mode & 0xffffu) | (stream << 16), (uint32_t)step, (uint32_t)(step >> 32)),
+                       make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+}
+
+// Box-Muller on u = (w + 1/2) 2^-32: radius sqrt(-2 ln u), and sine and cosine
+// of the angle 2 pi u.
+__device__ __forceinline__ double bm_radius64(uint32_t w) {
+  return sqrt(-2.0 * log(((double)w + 0.5) * 2.3283064365386962890625e-10));
+}
+
+__device__ __forceinline__ void bm_angle64(uint32_t w, double &sn, double &cs) {
+  sincospi(2.0 * (((double)w + 0.5) * 2.3283064365386962890625e-10), &sn, &cs);
+}
+
+// Three standard normal deviates of (atom, mode, stream, step): (eta_x, eta_y)
+// = r0 (cos, sin)(2 pi u1), eta_z = r1 cos(2 pi u3).
 __device__ __forceinline__ void gauss3(uint64_t seed, uint32_t atom, uint32_t mode, uint32_t stream,
                                        uint64_t step, double &e0, double &e1, double &e2) {
-  const uint4 w = philox4x32_10(
-      make_uint4(atom, (mode & 0xffffu) | (stream << 16), (uint32_t)step, (uint32_t)(step >> 32)),
-      make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
-  const double s = 2.3283064365386962890625e-10;  // 2^-32
-  const double u0 = ((double)w.x + 0.5) * s;
-  const double u1 = ((double)w.y + 0.5) * s;
-  const double u2 = ((double)w.z + 0.5) * s;
-  const double u3 = ((double)w.w + 0.5) * s;
-  const double r0 = sqrt(-2.0 * log(u0));
-  const double r1 = sqrt(-2.0 * log(u2));
-  double sn, cs;
-  sincospi(2.0 * u1, &sn, &cs);
+  const uint4 w = noise_words(seed, atom, mode, stream, step);
+  const double r0 = bm_radius64(w.x), r1 = bm_radius64(w.z);
+  double sn, cs, s3, c3;
+  bm_angle64(w.y, sn, cs);
+  bm_angle64(w.w, s3, c3);
   e0 = r0 * cs;
   e1 = r0 * sn;
-  e2 = r1 * cospi(2.0 * u3);
+  e2 = r1 * c3;
 }
 
 // One standard normal deviate of the triple above (component d = 0, 1, 2),
 // computed on its own so that one thread per component needs no exchange.
 __device__ __forceinline__ double gauss1(uint64_t seed, uint32_t atom, uint32_t mode, uint32_t stream,
                                          uint64_t step, int d) {
-  const uint4 w = philox4x32_10(
-      make_uint4(atom, (mode & 0xffffu) | (stream << 16), (uint32_t)step, (uint32_t)(step >> 32)),
-      make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
-  const double s = 2.3283064365386962890625e-10;  // 2^-32
-  const uint32_t wa = d < 2 ? w.x : w.z;
-  const uint32_t wb = d < 2 ? w.y : w.w;
-  const double r = sqrt(-2.0 * log(((double)wa + 0.5) * s));
-  const double ang = 2.0 * (((double)wb + 0.5) * s);
-  return r * (d == 1 ? sinpi(ang) : cospi(ang));
+  const uint4 w = noise_words(seed, atom, mode, stream, step);
+  double sn, cs;
+  bm_angle64(d < 2 ? w.y : w.w, sn, cs);
+  return bm_radius64(d < 2 ? w.x : w.z) * (d == 1 ? sn : cs);
 }
 
 // Compensated running sum: (s, c) holds s + c, every addition keeping its
@@ -150,12 +158,22 @@ struct ModeTables {
   //   Ti[i][j]: j <= H: M[i][j]; j > H: M[H + 1 + i][P - j] (0 past the modes)
   const double *Tf;
   const double *Ti;
+  // the folded transforms in fixed point (fixed.cuh): [fix_pairs(P)][P], limbs
+  // (h, l) of terms 2p and 2p + 1, scaled by 2^(55 - fem)
+  const int4 *fTf, *fTi;
+  int fem;
+  // A(h/2) O(h) A(h/2) of BAOAB per mode, [6][P]: q' = m0 q + m1 v + m2 n,
+  // v' = m3 q + m4 v + m5 n with n = sqrt(P kB T / (m mvv2e)) eta
+  const double *map6;
+  double rsp;          // 1 / sqrt(P)
 };
 
 struct StepArgs {
   int N, P, A;                 // atoms, beads, atoms per tile
   ModeTables mt;
   const double *inv_mm;        // [N] 1 / (m mvv2e)
+  const double *kmm;           // [N] duration of this step's kick / (m mvv2e)
+  int mu_one;                  // every imu_k is 1
   const double *sigv;          // [N] sqrt(P kB T / (m mvv2e))
   double *x;                   // [N][3][P] Cartesian positions
   double *v;                   // [N][3][P] normal-mode velocities
@@ -187,7 +205,7 @@ struct StepArgs {
   // A(h) and the new positions; phase 0 = the whole step in one launch
   int phase;
   const double *fix_u;         // fixcom of the previous step, still to be subtracted from v: [k][3], or null
-  int noise_pre;               // 1: PILE_L deviates drawn once per (atom, mode) into shared memory
+  int noise_pre;               // Cartesian: 1: PILE_L deviates drawn once per (atom, bead) into shared memory
 };
 
 // B_W of the barostat (App. E) over a kick of length tB that starts from the
@@ -202,13 +220,16 @@ struct BaroArgs {
   const double *W3part;        // [nmol][P][3] diagonal Xi_aa rows (anisotropic), or null
   int axes;                    // 0: isotropic; else the mask of edges with their own v_W
   double *baro;
-  double t0, tB, tA;            // the B_W covers [t0, t0 + tB] of the kick that the next kernel applies
+  double t0, tA;               // the B_W covers [t0, t0 + tB] of the kick that the next kernel applies
   int step_follows;
   // OBABO: the start-of-step call first applies the opening O_W (mode 0) and
   // scales the box once by exp(tA v_W), tA = h; the end-of-step call applies
   // the closing O_W (mode 1, keyed on the step just completed) after its B_W
   int obabo;
-  double W, nkT, npext, mu0;   // W (3 n N kB T taup^2, or n N kB T taup^2 per edge); n kB T; n P_ext; mu_0
+  double nkT, npext, mu0;      // n kB T; n P_ext; mu_0
+  // weights of B_W's three terms: 3 tB / W (per edge tB / W), tB^2 / W and
+  // tB^3 / 3W, W = 3 n N kB T taup^2 (n N kB T taup^2 per edge)
+  double k1, k2, k3;
   int thermo;
   double c1W, sigW;            // exp(-h / tau_0); c2 sqrt(n kB T / W)
   uint64_t seed;

@@ -2,20 +2,21 @@
 // (Sec. IV.A; App. B normal modes; App. D PILE_L), FP64.
 //
 // One thread block owns a tile of A atoms with all P beads of every one of
-// them staged in shared memory, so the three normal-mode transforms of a step
-// (forces, positions forward; positions back) never leave the SM: the
-// inter-bead communication of the paper's MPI design becomes shared-memory
-// traffic.  Per step and atom tile the kernel reads x, v~, F once and writes
-// x, v~ once, coalesced (every atom's P beads are contiguous per component).
+// them on chip, so the three normal-mode transforms of a step (forces,
+// positions forward; positions back) never leave the SM: the inter-bead
+// communication of the paper's MPI design becomes shared-memory traffic.  Per
+// step and atom tile the kernel reads x, v~, F once and writes x, v~ once,
+// coalesced (every atom's P beads are contiguous per component).
 //
-// Tasks: thread (mode k, component d, atom a) forms
+// Thread (component c, atom a, mode k) forms
 //   F~_k = sum_j M[k][j] F_j and q~_k = sum_j M[k][j] x_j        (Eq. A1)
 // applies B / A / O / A (BAOAB) or the pending B O of the previous step then
 // O B A (OBABO) in registers, and stores v~; after a barrier, thread
-// (bead j, component d, atom a) forms x_j = sum_k M[k][j] q~_k (Eq. A3).
+// (c, a, bead j) forms x_j = sum_k M[k][j] q~_k (Eq. A3).
 // For water-like systems the same kernel also measures, per oxygen, the
 // centroid drift since the last neighbour-list build and the bead spread.
 #include "common.cuh"
+#include "fixed.cuh"
 
 #include <algorithm>
 
@@ -32,12 +33,10 @@ __device__ __forceinline__ void rotate(double &q, double &v, double c, double s_
 
 // Centroid mode under the barostat for time tA at v_W (App. E):
 //   q~0 <- e^a q~0 + (e^a - e^-a) / (2 v_W) v~0,  v~0 <- e^-a v~0,  a = tA v_W
-__device__ __forceinline__ void baro_drift(double &q, double &v, double vW, double tA) {
-  const double a = tA * vW;
-  const double ea = exp(a), ema = exp(-a);
-  const double sh = fabs(a) < 1e-8 ? tA * (1.0 + a * a / 6.0) : (ea - ema) / (2.0 * vW);
-  q = ea * q + sh * v;
-  v = ema * v;
+// with the three factors as the barostat's kick left them.
+__device__ __forceinline__ void baro_drift(double &q, double &v, const double *f) {
+  q = f[0] * q + f[2] * v;
+  v = f[1] * v;
 }
 
 __device__ __forceinline__ double warp_max(double v) {
@@ -46,276 +45,257 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
-// Thread task t = (al * 3 + d) * P + k: atom al of the tile, component d,
-// mode k (forward) or bead j = k (inverse).  This is also the offset of the
-// element in the tile, so loads, stores and shared memory share one index.
-// The transforms use the parity of the rows of M (Eq. A1) under j -> P - j:
-// modes k <= H = floor(P/2) (constant, cosine and alternating rows) are even,
-// the sine rows k > H odd.  Staging each row folded -- u_j = x_j + x_{P-j}
-// and u_{P-j} = x_j - x_{P-j} for 0 < j < P - j, x_0 and x_{P/2} kept --
-// makes every forward output a sum over one half of the row (Tf), and every
-// inverse pair x_j, x_{P-j} = C_j +- S_j of an even-mode sum C_j and an
-// odd-mode sum S_j (Ti): about P/2 FMAs per output instead of P.
-__global__ void __launch_bounds__(256) k_step_f64(StepArgs a) {
-  extern __shared__ double sm[];
-  const int P = a.P;
-  const int tileLen = a.A * 3 * P;
-  double *sX = sm;
-  double *sV = sX + tileLen;
-  double *sF = sV + tileLen;
-  double *sQ = sF + tileLen;
-  double *sE = sQ + tileLen;     // PILE_L deviates of this step, stream O1, per element
-  double *sE2 = sE + tileLen;    // OBABO: stream O2 of the previous step
-  __shared__ float sred[2][8];
-  const int tile0 = blockIdx.x * a.A;
-  const int na = min(a.A, a.N - tile0);
-  const int len = na * 3 * P;
-  const size_t base = (size_t)tile0 * 3 * P;
-  const int H = P >> 1;
-  // stage the tile's x, F and v~ once each (16-byte loads where the tile
-  // starts on an even element: it is contiguous in [N][3][P])
-  if ((base & 1) == 0) {
-    const double2 *__restrict__ x2 = reinterpret_cast<const double2 *>(a.x + base);
-    const double2 *__restrict__ f2 = reinterpret_cast<const double2 *>(a.F + base);
-    const double2 *__restrict__ v2 = reinterpret_cast<const double2 *>(a.v + base);
-    for (int t = threadIdx.x; t < (len >> 1); t += blockDim.x) {
-      const double2 xv = x2[t], fv = f2[t], vv = v2[t];
-      sX[2 * t] = xv.x;
-      sX[2 * t + 1] = xv.y;
-      sF[2 * t] = fv.x;
-      sF[2 * t + 1] = fv.y;
-      sV[2 * t] = vv.x;
-      sV[2 * t + 1] = vv.y;
+// The fused step.  What bounds it is the FP64 pipe (one warp instruction in 64
+// clocks per SM partition), so everything that can be is taken off it:
+//  * the transforms run in 64-bit fixed point on the integer pipe (fixed.cuh),
+//    folded by the parity of the rows of M (Eq. A1) under j -> P - j: modes
+//    k <= H = floor(P/2) (constant, cosine and alternating rows) are even, the
+//    sine rows k > H odd, so u_j = x_j + x_{P-j} and u_{P-j} = x_{P-j} - x_j
+//    leave each output a sum over one half of the row (tables fTf, fTi), and the
+//    inverse pair x_j, x_{P-j} = C_j +- S_j an even-mode and an odd-mode sum;
+//  * A O A is one linear map of (q~, v~, eta) per mode (table map6);
+//  * one Philox draw's Box-Muller work is dealt to the three threads of an
+//    (atom, mode): the radius of the x, y pair, its angle, and all of z;
+//  * scalings are exponent additions; the skin test and the FP32 copy of x
+//    come from the integers.
+// Threads are component-major (c = threadIdx.x / S, S whole warps), so a warp
+// has one component and its Box-Muller share does not diverge.
+//
+// kPhase 0: the whole step.  1, 2: a step in two launches around the barostat's
+// OBABO kick (velocities only; then B(h/2), A(h) and the positions).  3: the
+// closing B(h/2) (OBABO: and O(h/2)) of a call's last step.
+//
+// Measured (GB300, per launch): see k_step_f64's rows in the design table.
+template <int kPhase, bool kObabo>
+__global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
+  constexpr bool kX = kPhase == 0 || kPhase == 2;   // positions move
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int P = a.P, H = P >> 1, A = a.A, AP = A * P, np = fix_pairs(P), rs = 4 * np;
+  const int S = blockDim.x / 3;
+  const int c = threadIdx.x / S, u = threadIdx.x - c * S;
+  const int al = u / P, k = u - al * P;
+  const int tile0 = blockIdx.x * A;
+  const int na = min(A, a.N - tile0);
+  const bool on = u < na * P;
+  const int i = tile0 + al, row = c * A + min(al, A - 1);   // padding threads stay inside the rows
+  const size_t g = ((size_t)i * 3 + c) * P + k;
+  int4 *uX = reinterpret_cast<int4 *>(smraw);                 // folded limbs, rs / 2 per row
+  int4 *uF = uX + 3 * A * (rs >> 1);
+  long long *rX = reinterpret_cast<long long *>(uF + 3 * A * (rs >> 1));   // [3][AP]
+  long long *rF = rX + 3 * AP;
+  long long *sC = rF + 3 * AP;                                // [3A] centroids, fixed point
+  double *sR = reinterpret_cast<double *>(sC + 3 * A);        // [2][AP] Box-Muller radius of x, y
+  double *sCs = sR + 2 * AP;                                  // [2][AP] cosine of their angle
+  int *sE = reinterpret_cast<int *>(sCs + 2 * AP);            // [3][3A] largest exponents of x, F, q~
+  float *sD = reinterpret_cast<float *>(sE + 9 * A);          // [3][AP] bead deviations
+  __shared__ float sred[2][12];
+  const bool needF = kPhase != 1 || !a.first;
+  double x = 0.0, f = 0.0, v = 0.0;
+  if (on) {
+    if (kX) x = a.x[g];
+    if (needF) f = a.F[g];
+    v = a.v[g];
+  }
+  for (int t = threadIdx.x; t < 9 * A; t += blockDim.x) sE[t] = kFixMinE;
+  const uint64_t step = (uint64_t)*a.step;
+  // the noise does not wait for the loads above: stream O1 of this step, O2 of
+  // the previous one
+  const bool d1 = a.thermo && (kPhase == 0 || kPhase == 1);
+  const bool d2 = kObabo && a.thermo && kPhase != 2 && (kPhase == 3 || !a.first);
+  double eta[2] = {0.0, 0.0};
+  auto draw = [&](int d, uint32_t stream, uint64_t st) {
+    const uint4 w = noise_words(a.seed, (uint32_t)i, (uint32_t)k, stream, st);
+    if (c == 0) {
+      sR[d * AP + u] = eta[d] = bm_radius64(w.x);
+    } else if (c == 1) {
+      double cs;
+      bm_angle64(w.y, eta[d], cs);
+      sCs[d * AP + u] = cs;
+    } else {
+      double sn, cs;
+      bm_angle64(w.w, sn, cs);
+      eta[d] = bm_radius64(w.z) * cs;
     }
-    if ((len & 1) && threadIdx.x == 0) {
-      sX[len - 1] = a.x[base + len - 1];
-      sF[len - 1] = a.F[base + len - 1];
-      sV[len - 1] = a.v[base + len - 1];
+  };
+  if (on && d1) draw(0, kStreamO1, step);
+  if (on && d2) draw(1, kStreamO2, step - 1);
+  __syncthreads();
+  if (on) {
+    if (kX) atomicMax(sE + row, exp_field(x));
+    if (needF) atomicMax(sE + 3 * A + row, exp_field(f));
+  }
+  if (c == 0) {   // e_x = r cos, e_y = r sin
+    if (on && d1) eta[0] *= sCs[u];
+    if (on && d2) eta[1] *= sCs[AP + u];
+  } else if (c == 1) {
+    if (on && d1) eta[0] *= sR[u];
+    if (on && d2) eta[1] *= sR[AP + u];
+  }
+  __syncthreads();
+  const int Ex = sE[row], Ef = sE[3 * A + row];
+  const int pj = k == 0 ? 0 : P - k;
+  const bool even = k <= H;
+  const int fold = row * rs + (even ? k : 2 * np + k - H - 1);   // this element's folded place
+  const int half_row = row * (rs >> 1) + (even ? 0 : np);        // the terms of mode (bead) k
+  long long X = 0, F = 0;
+  if (on) {
+    if (kX) rX[c * AP + u] = X = to_fixed(x, Ex);
+    if (needF) rF[c * AP + u] = F = to_fixed(f, Ef);
+  }
+  __syncthreads();
+  if (on) {
+    if (kX) {
+      const long long o = pj != k ? rX[c * AP + u - k + pj] : 0;
+      reinterpret_cast<int2 *>(uX)[fold] = fix_limbs(even ? X + o : o - X);
     }
-  } else {
-    for (int t = threadIdx.x; t < len; t += blockDim.x) {
-      sX[t] = a.x[base + t];
-      sF[t] = a.F[base + t];
-      sV[t] = a.v[base + t];
+    if (needF) {
+      const long long o = pj != k ? rF[c * AP + u - k + pj] : 0;
+      reinterpret_cast<int2 *>(uF)[fold] = fix_limbs(even ? F + o : o - F);
     }
   }
   __syncthreads();
-  // fold each staged row in place: (x_j, x_{P-j}) -> (x_j + x_{P-j}, x_j - x_{P-j})
-  // for 0 < j < P - j, one thread per pair
-  {
-    const int hp = (P - 1) >> 1;   // pairs per row
-    for (int t = threadIdx.x; t < na * 3 * hp; t += blockDim.x) {
-      const int r = t / hp, j = t - r * hp + 1;
-      double *xr = sX + r * P, *fr = sF + r * P;
-      const double xa = xr[j], xb = xr[P - j], fa = fr[j], fb = fr[P - j];
-      xr[j] = xa + xb;
-      xr[P - j] = xa - xb;
-      fr[j] = fa + fb;
-      fr[P - j] = fa - fb;
+  const int em = a.mt.fem;
+  const int4 *__restrict__ tf = a.mt.fTf + k;
+  double q = 0.0;
+  if (on) {
+    FixSum sx, sf;
+    if (kX && needF) {
+#pragma unroll 3
+      for (int p = 0; p < np; ++p) {
+        const int4 m = __ldg(tf + p * P);
+        sx.add2(uX[half_row + p], m);
+        sf.add2(uF[half_row + p], m);
+      }
+      q = from_fixed(sx.value(), Ex, em);
+    } else if (needF) {
+#pragma unroll 3
+      for (int p = 0; p < np; ++p) sf.add2(uF[half_row + p], __ldg(tf + p * P));
     }
-  }
-  const uint64_t step = (uint64_t)(*a.step + a.step_off);
-  // Large grids: one Philox draw and Box-Muller per (atom, mode) serve the
-  // three components (throughput).  Small grids (noise_pre = 0): each element
-  // draws its own component inline, in parallel with the others (latency).
-  if (a.thermo && a.noise_pre && a.phase != 2) {
-    const bool o2 = a.integrator == 1 && !a.first;
-    for (int t = threadIdx.x; t < na * P; t += blockDim.x) {
-      const int al = t / P, k = t - al * P;
-      const int e = al * 3 * P + k;
-      gauss3(a.seed, (uint32_t)(tile0 + al), (uint32_t)k, kStreamO1, step, sE[e], sE[e + P], sE[e + 2 * P]);
-      if (o2)
-        gauss3(a.seed, (uint32_t)(tile0 + al), (uint32_t)k, kStreamO2, step - 1, sE2[e], sE2[e + P],
-               sE2[e + 2 * P]);
-    }
-  }
-  __syncthreads();
-  const double *__restrict__ Tf = a.mt.Tf;
-  for (int task = threadIdx.x; task < len; task += blockDim.x) {
-    const int k = task % P;
-    const int r = task / P;
-    const int i = tile0 + r / 3;
-    auto noise = [&](uint32_t stream, uint64_t st, const double *pre) {
-      return a.noise_pre ? pre[task] : gauss1(a.seed, (uint32_t)i, (uint32_t)k, stream, st, r % 3);
-    };
-    // F~_k = (M F)_k and q~_k = (M x)_k over the even (k <= H) or odd half
-    // of the folded row, two independent chains each
-    const bool even = k <= H;
-    const int n = even ? H + 1 : P - H - 1;
-    const double *fx = sF + r * P + (even ? 0 : H + 1);
-    const double *xx = sX + r * P + (even ? 0 : H + 1);
-    const double *tf = Tf + k;
-    double fa = 0.0, fb = 0.0, qa = 0.0, qb = 0.0;
-    int j = 0;
-    for (; j + 1 < n; j += 2) {
-      const double m0 = __ldg(tf + j * P), m1 = __ldg(tf + (j + 1) * P);
-      fa = fma(m0, fx[j], fa);
-      fb = fma(m1, fx[j + 1], fb);
-      qa = fma(m0, xx[j], qa);
-      qb = fma(m1, xx[j + 1], qb);
-    }
-    if (j < n) {
-      const double m0 = __ldg(tf + j * P);
-      fa = fma(m0, fx[j], fa);
-      qa = fma(m0, xx[j], qa);
-    }
-    const double f = fa + fb;
-    double q = qa + qb;
-    double v = sV[task];
-    if (a.fix_u && k == 0) v -= a.fix_u[r % 3];   // the previous step's fixcom
-    const double im = __ldg(a.inv_mm + i) * __ldg(a.mt.imu + k);   // 1 / (m^(k) mvv2e)
-    const double cA = __ldg(a.mt.cA + k), sA = __ldg(a.mt.sA + k), wsA = __ldg(a.mt.wsA + k);
-    const double c1 = __ldg(a.mt.c1 + k), c2s = __ldg(a.mt.c2 + k) * __ldg(a.sigv + i);
-    if (a.integrator == 0) {
+    f = needF ? from_fixed(sf.value(), Ef, em) : 0.0;
+    if (!a.mu_one) f *= __ldg(a.mt.imu + k);   // 1 / m^(k) = imu_k / (m mvv2e)
+    if (k == 0 && a.fix_u) v -= a.fix_u[c];    // the previous step's fixcom
+    const double km = __ldg(a.kmm + i);        // this kick's time / (m mvv2e)
+    const double sg = __ldg(a.sigv + i);
+    if (!kObabo) {
       // B(h/2) of this step, merged with the final B(h/2) of the previous one
-      v = fma(a.kick * im, f, v);
-      if (k == 0 && a.baro) {   // the centroid rides on the barostat
-        baro_drift(q, v, a.baro[kBaroVA1 + r % 3], a.half);
-        if (a.thermo) v = fma(c1, v, c2s * noise(kStreamO1, step, sE));
-        baro_drift(q, v, a.baro[kBaroVA2 + r % 3], a.half);
-      } else {
-        rotate(q, v, cA, sA, wsA);
-        if (a.thermo) v = fma(c1, v, c2s * noise(kStreamO1, step, sE));
-        rotate(q, v, cA, sA, wsA);
+      v = fma(km, f, v);
+      if (kPhase != 3) {
+        const double n = sg * eta[0];
+        if (k == 0 && a.baro) {   // the centroid rides on the barostat
+          baro_drift(q, v, a.baro + kBaroA1 + 3 * c);
+          if (a.thermo) v = fma(__ldg(a.mt.c1), v, __ldg(a.mt.c2) * n);
+          baro_drift(q, v, a.baro + kBaroA2 + 3 * c);
+        } else {
+          // A(h/2) O(h) A(h/2): (q~, v~) <- linear map of (q~, v~, sigma eta)
+          const double *__restrict__ m6 = a.mt.map6 + k;
+          const double qn = fma(__ldg(m6 + 2 * P), n, fma(__ldg(m6 + P), v, __ldg(m6) * q));
+          v = fma(__ldg(m6 + 5 * P), n, fma(__ldg(m6 + 4 * P), v, __ldg(m6 + 3 * P) * q));
+          q = qn;
+        }
       }
     } else {
-      const double kb = a.half * im;
-      if (a.phase != 2) {
-        if (!a.first) {
+      const double c1 = __ldg(a.mt.c1 + k), c2s = __ldg(a.mt.c2 + k) * sg;
+      if (kPhase != 2) {
+        if (kPhase == 3 || !a.first) {
           // the previous step's closing B(h/2) O(h/2)
-          v = fma(kb, f, v);
-          if (a.thermo) v = fma(c1, v, c2s * noise(kStreamO2, step - 1, sE2));
+          v = fma(km, f, v);
+          if (a.thermo) v = fma(c1, v, c2s * eta[1]);
         }
-        if (a.thermo) v = fma(c1, v, c2s * noise(kStreamO1, step, sE));
+        if (kPhase != 3 && a.thermo) v = fma(c1, v, c2s * eta[0]);
       }
-      if (a.phase != 1) {
-        v = fma(kb, f, v);
+      if (kX) {
+        v = fma(km, f, v);
         if (k == 0 && a.baro)   // A(h) of the centroid under the barostat
-          baro_drift(q, v, a.baro[kBaroVA1 + r % 3], 2.0 * a.half);
+          baro_drift(q, v, a.baro + kBaroA1 + 3 * c);
         else
-          rotate(q, v, cA, sA, wsA);
+          rotate(q, v, __ldg(a.mt.cA + k), __ldg(a.mt.sA + k), __ldg(a.mt.wsA + k));
       }
     }
-    sQ[task] = q;
-    a.v[base + task] = v;
+    a.v[g] = v;
+    if (kX) atomicMax(sE + 6 * A + row, exp_field(q));
   }
-  if (a.phase == 1) return;   // velocities only: the barostat's B_W reads them next
+  if (!kX) return;
+  __syncthreads();
+  const int Eq = sE[6 * A + row];
+  const int sh = Eq - 1022 + em - kFixBits;   // x_j = S_j 2^sh below
+  const bool oxy = a.blkmax && on && i % 3 == 0;
+  double cen = 0.0;
+  if (on) {
+    reinterpret_cast<int2 *>(uX)[fold] = fix_limbs(to_fixed(q, Eq));
+    if (oxy && k == 0) {   // centroid c = q~_0 / sqrt(P), also in units of 2^sh
+      cen = q * a.mt.rsp;
+      sC[row] = Eq > kFixMaxE ? 0
+                              : __double2ll_rn(__hiloint2double(__double2hiint(cen) - (sh << 20), __double2loint(cen)));
+      if (cen == 0.0) sC[row] = 0;
+    }
+  }
   __syncthreads();
   // inverse, first half: C_j (bead j <= H, even modes) or S_{P-j} (bead
-  // j > H, odd modes) into sF, which the forward pass no longer needs
-  const double *__restrict__ Ti = a.mt.Ti;
-  for (int task = threadIdx.x; task < len; task += blockDim.x) {
-    const int j = task % P;
-    const bool even = j <= H;
-    const int n = even ? H + 1 : P - H - 1;
-    const double *qq = sQ + (task - j) + (even ? 0 : H + 1);
-    const double *ti = Ti + j;
-    double xa = 0.0, xb = 0.0;
-    int k = 0;
-    for (; k + 1 < n; k += 2) {
-      xa = fma(__ldg(ti + k * P), qq[k], xa);
-      xb = fma(__ldg(ti + (k + 1) * P), qq[k + 1], xb);
-    }
-    if (k < n) xa = fma(__ldg(ti + k * P), qq[k], xa);
-    sF[task] = xa + xb;
+  // j > H, odd modes)
+  if (on) {
+    const int4 *__restrict__ ti = a.mt.fTi + k;
+    FixSum s;
+#pragma unroll 3
+    for (int p = 0; p < np; ++p) s.add2(uX[half_row + p], __ldg(ti + p * P));
+    rX[c * AP + u] = X = s.value();
   }
   __syncthreads();
   // second half: x_j = C_j + S_j (j <= H), x_{P-j} = C_j - S_j
-  for (int task = threadIdx.x; task < len; task += blockDim.x) {
-    const int j = task % P, pj = j == 0 ? 0 : P - j;
-    const int row0 = task - j;
-    const double xn = j <= H ? sF[task] + (pj > H ? sF[row0 + pj] : 0.0) : sF[row0 + pj] - sF[task];
-    a.x[base + task] = xn;
-    if (a.x32) a.x32[base + task] = (float)xn;
-    sX[task] = xn;
+  float dev = 0.f;
+  if (on) {
+    const long long o = rX[c * AP + u - k + pj];
+    const long long Sj = even ? (pj > H ? X + o : X) : o - X;
+    const double xn = from_fixed(Sj, Eq, em);
+    a.x[g] = xn;
+    const float sc = sh < -126 ? 0.f : (sh > 127 ? __int_as_float(0x7f800000) : __int_as_float((sh + 127) << 23));
+    if (a.x32) a.x32[g] = Eq > kFixMaxE ? __int_as_float(0x7fc00000) : (float)Sj * sc;
+    if (oxy) {
+      dev = Eq > kFixMaxE ? __int_as_float(0x7f800000) : (float)(Sj - sC[row]) * sc;
+      sD[c * AP + u] = dev;
+    }
   }
   if (!a.blkmax) return;
-  // Neighbour-list skin check for the oxygens of this tile: centroid
-  // c = q~_0 / sqrt(P), its drift since the last build and the bead spread.
-  // Tiles without an oxygen report zero at once.  The differences are taken
-  // in FP64, their squares and the maxima in FP32 (the FP64 pipe is the
-  // scarce unit; a relative margin keeps the reported bound conservative).
+  // Neighbour-list skin check for the oxygens of this tile: the centroid's
+  // drift since the last build and the bead spread, squared and reduced in
+  // FP32 (a relative margin keeps the reported bound conservative).  Tiles
+  // without an oxygen report zero at once.
   if ((tile0 + 2) / 3 * 3 >= tile0 + na) {
     if (threadIdx.x < 2) a.blkmax[2 * blockIdx.x + threadIdx.x] = 0.0;
     return;
   }
+  float *sG = reinterpret_cast<float *>(sE);   // [3][A] squared drifts (the exponents are done with)
+  if (oxy && k == 0) {
+    const int m = i / 3;
+    const float d = (float)(cen - a.cref[3 * m + c]);
+    a.ccur[3 * m + c] = cen;
+    sG[row] = d * d;
+  }
   __syncthreads();
   float vdisp = 0.f, vdev = 0.f;
-  const double rsp = rsqrt((double)P);
-  for (int t = threadIdx.x; t < na * P; t += blockDim.x) {
-    const int al = t / P, k = t % P;
-    const int i = tile0 + al;
-    if (i % 3) continue;
-    const double *xq = sQ + al * 3 * P;
-    const double c0 = xq[0] * rsp, c1 = xq[P] * rsp, c2 = xq[2 * P] * rsp;
-    const double *xs = sX + al * 3 * P;
-    const float e0 = (float)(xs[k] - c0), e1 = (float)(xs[P + k] - c1), e2 = (float)(xs[2 * P + k] - c2);
-    vdev = fmaxf(vdev, e0 * e0 + e1 * e1 + e2 * e2);
-    if (k == 0) {
-      const int m = i / 3;
-      const float g0 = (float)(c0 - a.cref[3 * m]), g1 = (float)(c1 - a.cref[3 * m + 1]);
-      const float g2 = (float)(c2 - a.cref[3 * m + 2]);
-      vdisp = fmaxf(vdisp, g0 * g0 + g1 * g1 + g2 * g2);
-      a.ccur[3 * m] = c0;
-      a.ccur[3 * m + 1] = c1;
-      a.ccur[3 * m + 2] = c2;
-    }
+  if (c == 0 && oxy) {
+    const float e1 = sD[AP + u], e2 = sD[2 * AP + u];
+    vdev = dev * dev + e1 * e1 + e2 * e2;
+    if (k == 0) vdisp = sG[al] + sG[A + al] + sG[2 * A + al];
+    // NaN positions force a rebuild (and fail later at a synchronising call)
+    if (vdisp != vdisp) vdisp = __int_as_float(0x7f800000);
+    if (vdev != vdev) vdev = __int_as_float(0x7f800000);
   }
-  // NaN positions force a rebuild (and fail later at a synchronising call)
-  if (vdisp != vdisp) vdisp = __int_as_float(0x7f800000);
-  if (vdev != vdev) vdev = __int_as_float(0x7f800000);
+  if (c == 0) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    vdisp = fmaxf(vdisp, __shfl_down_sync(0xffffffffu, vdisp, o));
-    vdev = fmaxf(vdev, __shfl_down_sync(0xffffffffu, vdev, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sred[0][threadIdx.x >> 5] = vdisp;
-    sred[1][threadIdx.x >> 5] = vdev;
+    for (int o = 16; o > 0; o >>= 1) {
+      vdisp = fmaxf(vdisp, __shfl_down_sync(0xffffffffu, vdisp, o));
+      vdev = fmaxf(vdev, __shfl_down_sync(0xffffffffu, vdev, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+      sred[0][threadIdx.x >> 5] = vdisp;
+      sred[1][threadIdx.x >> 5] = vdev;
+    }
   }
   __syncthreads();
   if (threadIdx.x < 2) {
     float mx = 0.f;
-    for (int w = 0; w < (int)((blockDim.x + 31) / 32); ++w) mx = fmaxf(mx, sred[threadIdx.x][w]);
+    for (int w = 0; w < (S >> 5); ++w) mx = fmaxf(mx, sred[threadIdx.x][w]);
     a.blkmax[2 * blockIdx.x + threadIdx.x] = mx <= 3.0e38f ? sqrt((double)mx) * (1.0 + 1e-6) : 1e300;
-  }
-}
-
-// Closing kick of the last step of a call: B(h/2) (and, for OBABO, the final
-// O(h/2) of that step), leaving v~ at integer time.
-__global__ void __launch_bounds__(256) k_close_f64(StepArgs a) {
-  extern __shared__ double sm[];
-  const int P = a.P;
-  double *sF = sm;
-  const int tile0 = blockIdx.x * a.A;
-  const int na = min(a.A, a.N - tile0);
-  const int len = na * 3 * P;
-  const size_t base = (size_t)tile0 * 3 * P;
-  for (int t = threadIdx.x; t < len; t += blockDim.x) sF[t] = a.F[base + t];
-  __syncthreads();
-  const uint64_t step = (uint64_t)(*a.step + a.step_off);
-  const double *__restrict__ Mt = a.mt.Mt;
-  for (int task = threadIdx.x; task < len; task += blockDim.x) {
-    const int k = task % P;
-    const int r = task / P;
-    const int d = r % 3;
-    const int i = tile0 + r / 3;
-    const double *fx = sF + r * P;
-    double fa = 0.0, fb = 0.0;
-    int j = 0;
-    for (; j + 1 < P; j += 2) {
-      fa = fma(__ldg(Mt + j * P + k), fx[j], fa);
-      fb = fma(__ldg(Mt + (j + 1) * P + k), fx[j + 1], fb);
-    }
-    if (j < P) fa = fma(__ldg(Mt + j * P + k), fx[j], fa);
-    double v = a.v[base + task];
-    if (a.fix_u && k == 0) v -= a.fix_u[d];   // the last step's fixcom
-    v = fma(a.half * (__ldg(a.inv_mm + i) * __ldg(a.mt.imu + k)), fa + fb, v);
-    if (a.integrator == 1 && a.thermo) {
-      const double c1 = __ldg(a.mt.c1 + k), c2s = __ldg(a.mt.c2 + k) * __ldg(a.sigv + i);
-      v = fma(c1, v, c2s * gauss1(a.seed, (uint32_t)i, (uint32_t)k, kStreamO2, step, d));
-    }
-    a.v[base + task] = v;
   }
 }
 
@@ -502,24 +482,58 @@ __global__ void k_nap_to_pna(const double *src, double *dst, int N, int P) {
 }
 
 // --- host launchers --------------------------------------------------------
-size_t step_smem_bytes(int A, int P) { return ((size_t)6 * A * 3 * P + 3 * A) * sizeof(double); }
-size_t close_smem_bytes(int A, int P) { return (size_t)A * 3 * P * sizeof(double); }
+// Atoms per block of the normal-mode step: the smallest tile that fills its
+// warps best (A P close to a multiple of 32, at most 128 per component), as
+// long as the grid still has two blocks for every SM of the GPU.
+int step_tile_atoms(int N, int P) {
+  const int need = std::min(N, 304);
+  int best = 1;
+  double eff = 0.0;
+  for (int A = 1; A <= std::max(1, 128 / P); ++A) {
+    if (A > 1 && (N + A - 1) / A < need) break;
+    const double e = (double)A * P / ((A * P + 31) / 32 * 32);
+    if (e > 1.02 * eff) {
+      eff = e;
+      best = A;
+    }
+  }
+  return best;
+}
+
+int step_threads(int A, int P) { return 3 * ((A * P + 31) / 32 * 32); }
+
+static size_t step_smem_bytes(int A, int P) {
+  const size_t rows = 3 * (size_t)A, AP = (size_t)A * P;
+  return rows * 2 * fix_pairs(P) * sizeof(int4) * 2 +   // limbs of x and F
+         (2 * 3 * AP + rows) * sizeof(long long) +      // rows, centroids
+         4 * AP * sizeof(double) + 3 * rows * sizeof(int) + 3 * AP * sizeof(float);
+}
+
+static size_t cart_smem_bytes(int A, int P) { return ((size_t)4 * A * 3 * P + 3 * A) * sizeof(double); }
 
 cudaError_t launch_step(const StepArgs &a0, int threads, cudaStream_t s) {
   const int grid = (a0.N + a0.A - 1) / a0.A;
   StepArgs a = a0;
-  static int nsm = 0;   // SM count of the device (one GPU per process)
-  if (!nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 152;
-  }
-  a.noise_pre = grid >= 4 * nsm ? 1 : 0;
   if (a.method == 1) {
-    k_step_cart_f64<<<grid, threads, step_smem_bytes(a.A, a.P), s>>>(a);
+    static int nsm = 0;   // SM count of the device (one GPU per process)
+    if (!nsm) {
+      int dev = 0;
+      cudaGetDevice(&dev);
+      if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 152;
+    }
+    a.noise_pre = grid >= 4 * nsm ? 1 : 0;
+    k_step_cart_f64<<<grid, threads, cart_smem_bytes(a.A, a.P), s>>>(a);
     return cudaGetLastError();
   }
-  k_step_f64<<<grid, threads, step_smem_bytes(a.A, a.P), s>>>(a);
+  const size_t smem = step_smem_bytes(a.A, a.P);
+  if (a.integrator == 0)
+    k_step_f64<0, false><<<grid, threads, smem, s>>>(a);
+  else if (a.phase == 1)
+    k_step_f64<1, true><<<grid, threads, smem, s>>>(a);
+  else if (a.phase == 2)
+    k_step_f64<2, true><<<grid, threads, smem, s>>>(a);
+  else
+    k_step_f64<0, true><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -530,7 +544,11 @@ cudaError_t launch_close(const StepArgs &a, int threads, cudaStream_t s) {
     return cudaGetLastError();
   }
   const int grid = (a.N + a.A - 1) / a.A;
-  k_close_f64<<<grid, threads, close_smem_bytes(a.A, a.P), s>>>(a);
+  const size_t smem = step_smem_bytes(a.A, a.P);
+  if (a.integrator == 0)
+    k_step_f64<3, false><<<grid, threads, smem, s>>>(a);
+  else
+    k_step_f64<3, true><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -154,56 +154,57 @@ __global__ void __launch_bounds__(kSumThreads) k_baro_kick(BaroArgs a) {
     gauss3(a.seed, 0xffffffffu, a.step_follows ? 0u : 1u, 3u, a.step_follows ? step : step - 1, noise[0], noise[1],
            noise[2]);
   __syncthreads();
-  if (threadIdx.x != 0) return;
+  // the scalar work, one thread per edge (isotropic: the three do the same)
+  if (threadIdx.x >= 3) return;
+  const int c = threadIdx.x;
   const double *mv = tot, *sfv = tot + 3, *sf2 = tot + 6, *srcf = tot + 9, *svir = tot + 12;
   double *b = a.baro;
-  const double V = b[kBaroL] * b[kBaroL + 1] * b[kBaroL + 2];
-  const double tB = a.tB;
+  const double V = b[kBaroL] * b[kBaroL + 1] * b[kBaroL + 2], L = b[kBaroL + c];
+  __syncwarp(0x7u);   // V is formed before an edge changes below
+  const bool moves = !a.axes || (a.axes >> c & 1);
+  const double eta = a.axes ? noise[c] : noise[0];
   // O_W: v_W <- c1 v_W + sigW eta; each edge its own deviate, the isotropic
   // v_W the first
-  auto langevin = [&](double *w) {
-    if (a.axes) {
-      for (int c = 0; c < 3; ++c)
-        if (a.axes >> c & 1) w[c] = a.c1W * w[c] + a.sigW * noise[c];
-    } else {
-      w[0] = w[1] = w[2] = a.c1W * w[0] + a.sigW * noise[0];
-    }
-  };
-  double vW[3] = {b[kBaroV], b[kBaroV + 1], b[kBaroV + 2]};
-  if (a.obabo && a.step_follows && a.thermo) langevin(vW);   // this step's first O(h/2)
-  if (a.axes) {
-    for (int c = 0; c < 3; ++c)
-      vW[c] = (a.axes >> c & 1)
-                  ? vW[c] + tB / a.W * (mv[c] - srcf[c] + svir[c] - V * a.npext + a.nkT) +
-                        tB * tB / a.W * sfv[c] + tB * tB * tB / (3.0 * a.W) * sf2[c]
-                  : 0.0;
+  auto langevin = [&](double w) { return moves ? a.c1W * w + a.sigW * eta : w; };
+  double vW = b[kBaroV + c];
+  if (a.obabo && a.step_follows && a.thermo) vW = langevin(vW);   // this step's first O(h/2)
+  if (!moves) {
+    vW = 0.0;
+  } else if (a.axes) {
+    vW += a.k1 * (mv[c] - srcf[c] + svir[c] - V * a.npext + a.nkT) + a.k2 * sfv[c] + a.k3 * sf2[c];
   } else {
-    const double smv2 = mv[0] + mv[1] + mv[2], trcf = srcf[0] + srcf[1] + srcf[2];
-    const double tfv = sfv[0] + sfv[1] + sfv[2], tf2m = sf2[0] + sf2[1] + sf2[2];
-    const double w = vW[0] + 3.0 * tB / a.W * ((smv2 - trcf + svir[0]) / 3.0 - V * a.npext + a.nkT) +
-                     tB * tB / a.W * tfv + tB * tB * tB / (3.0 * a.W) * tf2m;
-    vW[0] = vW[1] = vW[2] = w;
+    vW += a.k1 * ((mv[0] + mv[1] + mv[2] - (srcf[0] + srcf[1] + srcf[2]) + svir[0]) * (1.0 / 3.0) - V * a.npext +
+                  a.nkT) +
+          a.k2 * (sfv[0] + sfv[1] + sfv[2]) + a.k3 * (sf2[0] + sf2[1] + sf2[2]);
   }
   if (!a.step_follows) {
     // OBABO: the closing O(h/2) of the step just completed (the counter has
     // already been advanced past it)
-    if (a.obabo && a.thermo) langevin(vW);
-    for (int c = 0; c < 3; ++c) b[kBaroV + c] = vW[c];
+    if (a.obabo && a.thermo) vW = langevin(vW);
+    b[kBaroV + c] = vW;
     return;
   }
-  double vO[3] = {vW[0], vW[1], vW[2]};
-  if (a.thermo && !a.obabo) langevin(vO);
-  for (int c = 0; c < 3; ++c) {
-    b[kBaroVA1 + c] = vW[c];
-    b[kBaroVA2 + c] = vO[c];
-    b[kBaroV + c] = vO[c];
-    // BAOAB: A(h/2) at v_W, O_W, A(h/2) at v_O; OBABO: one A(h) at v_W
-    const double L = a.obabo ? b[kBaroL + c] * exp(a.tA * vW[c])
-                             : b[kBaroL + c] * exp(a.tA * vW[c]) * exp(a.tA * vO[c]);
-    b[kBaroL + c] = L;
-    b[kBaroInvL + c] = 1.0 / L;
-    if (!(L > a.Lmin)) atomicOr(a.err, kErrBoxSmall);
+  double vO = vW;
+  if (a.thermo && !a.obabo) vO = langevin(vO);
+  b[kBaroVA1 + c] = vW;
+  b[kBaroVA2 + c] = vO;
+  b[kBaroV + c] = vO;
+  // the A factors of the centroid mode at v_W and (BAOAB) at v_O
+  double grow = 1.0;
+  for (int h = 0; h < (a.obabo ? 1 : 2); ++h) {
+    const double w = h ? vO : vW, x = a.tA * w;
+    const double ea = exp(x), ema = exp(-x);
+    double *f = b + (h ? kBaroA2 : kBaroA1) + 3 * c;
+    f[0] = ea;
+    f[1] = ema;
+    f[2] = fabs(x) < 1e-8 ? a.tA * (1.0 + x * x / 6.0) : (ea - ema) / (2.0 * w);
+    grow *= ea;
   }
+  // BAOAB: A(h/2) at v_W, O_W, A(h/2) at v_O; OBABO: one A(h) at v_W
+  const double Ln = L * grow;
+  b[kBaroL + c] = Ln;
+  b[kBaroInvL + c] = 1.0 / Ln;
+  if (!(Ln > a.Lmin)) atomicOr(a.err, kErrBoxSmall);
 }
 
 // fixcom: the mass-weighted mean velocity u of the centroid mode (normal
