@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "noise64.cuh"
+
 namespace pimd {
 
 // Metal units (A, ps, eV, amu, K).  h and mvv2e are the values printed in
@@ -71,28 +73,19 @@ __device__ __forceinline__ uint4 noise_words(uint64_t seed, uint32_t atom, uint3
                        make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
 }
 
-// Box-Muller on u = (w + 1/2) 2^-32: radius sqrt(-2 ln u), and sine and cosine
-// of the angle 2 pi u.
-__device__ __forceinline__ double bm_radius64(uint32_t w) {
-  return sqrt(-2.0 * log(((double)w + 0.5) * 2.3283064365386962890625e-10));
-}
-
-__device__ __forceinline__ void bm_angle64(uint32_t w, double &sn, double &cs) {
-  sincospi(2.0 * (((double)w + 0.5) * 2.3283064365386962890625e-10), &sn, &cs);
-}
-
-// Three standard normal deviates of (atom, mode, stream, step): (eta_x, eta_y)
-// = r0 (cos, sin)(2 pi u1), eta_z = r1 cos(2 pi u3).
+// Three standard normal deviates of (atom, mode, stream, step): Box-Muller on
+// u = (w + 1/2) 2^-32, (eta_x, eta_y) = r0 (cos, sin)(2 pi u1), eta_z = r1
+// cos(2 pi u3), r = sqrt(-2 ln u).
 __device__ __forceinline__ void gauss3(uint64_t seed, uint32_t atom, uint32_t mode, uint32_t stream,
                                        uint64_t step, double &e0, double &e1, double &e2) {
   const uint4 w = noise_words(seed, atom, mode, stream, step);
-  const double r0 = bm_radius64(w.x), r1 = bm_radius64(w.z);
-  double sn, cs, s3, c3;
-  bm_angle64(w.y, sn, cs);
-  bm_angle64(w.w, s3, c3);
-  e0 = r0 * cs;
-  e1 = r0 * sn;
-  e2 = r1 * c3;
+  const uint64_t r0 = bm_radius_fix(w.x), r1 = bm_radius_fix(w.z);
+  int64_t sn, cs, s3, c3;
+  bm_angle_fix(w.y, sn, cs);
+  bm_angle_fix(w.w, s3, c3);
+  e0 = bm_deviate(r0, cs);
+  e1 = bm_deviate(r0, sn);
+  e2 = bm_deviate(r1, c3);
 }
 
 // One standard normal deviate of the triple above (component d = 0, 1, 2),
@@ -100,9 +93,9 @@ __device__ __forceinline__ void gauss3(uint64_t seed, uint32_t atom, uint32_t mo
 __device__ __forceinline__ double gauss1(uint64_t seed, uint32_t atom, uint32_t mode, uint32_t stream,
                                          uint64_t step, int d) {
   const uint4 w = noise_words(seed, atom, mode, stream, step);
-  double sn, cs;
-  bm_angle64(d < 2 ? w.y : w.w, sn, cs);
-  return bm_radius64(d < 2 ? w.x : w.z) * (d == 1 ? sn : cs);
+  int64_t sn, cs;
+  bm_angle_fix(d < 2 ? w.y : w.w, sn, cs);
+  return bm_deviate(bm_radius_fix(d < 2 ? w.x : w.z), d == 1 ? sn : cs);
 }
 
 // Compensated running sum: (s, c) holds s + c, every addition keeping its

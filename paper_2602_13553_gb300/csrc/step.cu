@@ -84,8 +84,8 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
   long long *rX = reinterpret_cast<long long *>(uF + 3 * A * (rs >> 1));   // [3][AP]
   long long *rF = rX + 3 * AP;
   long long *sC = rF + 3 * AP;                                // [3A] centroids, fixed point
-  double *sR = reinterpret_cast<double *>(sC + 3 * A);        // [2][AP] Box-Muller radius of x, y
-  double *sCs = sR + 2 * AP;                                  // [2][AP] cosine of their angle
+  uint64_t *sR = reinterpret_cast<uint64_t *>(sC + 3 * A);    // [2][AP] Box-Muller radius of x, y
+  int64_t *sCs = reinterpret_cast<int64_t *>(sR + 2 * AP);    // [2][AP] cosine of their angle
   int *sE = reinterpret_cast<int *>(sCs + 2 * AP);            // [3][3A] largest exponents of x, F, q~
   float *sD = reinterpret_cast<float *>(sE + 9 * A);          // [3][AP] bead deviations
   __shared__ float sred[2][12];
@@ -103,18 +103,20 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
   const bool d1 = a.thermo && (kPhase == 0 || kPhase == 1);
   const bool d2 = kObabo && a.thermo && kPhase != 2 && (kPhase == 3 || !a.first);
   double eta[2] = {0.0, 0.0};
+  uint64_t part[2] = {0, 0};   // this thread's share: radius (c = 0) or sine (c = 1)
   auto draw = [&](int d, uint32_t stream, uint64_t st) {
     const uint4 w = noise_words(a.seed, (uint32_t)i, (uint32_t)k, stream, st);
     if (c == 0) {
-      sR[d * AP + u] = eta[d] = bm_radius64(w.x);
-    } else if (c == 1) {
-      double cs;
-      bm_angle64(w.y, eta[d], cs);
-      sCs[d * AP + u] = cs;
+      sR[d * AP + u] = part[d] = bm_radius_fix(w.x);
     } else {
-      double sn, cs;
-      bm_angle64(w.w, sn, cs);
-      eta[d] = bm_radius64(w.z) * cs;
+      int64_t sn, cs;
+      bm_angle_fix(c == 1 ? w.y : w.w, sn, cs);
+      if (c == 1) {
+        part[d] = (uint64_t)sn;
+        sCs[d * AP + u] = cs;
+      } else {
+        eta[d] = bm_deviate(bm_radius_fix(w.z), cs);
+      }
     }
   };
   if (on && d1) draw(0, kStreamO1, step);
@@ -123,13 +125,12 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
   if (on) {
     if (kX) atomicMax(sE + row, exp_field(x));
     if (needF) atomicMax(sE + 3 * A + row, exp_field(f));
-  }
-  if (c == 0) {   // e_x = r cos, e_y = r sin
-    if (on && d1) eta[0] *= sCs[u];
-    if (on && d2) eta[1] *= sCs[AP + u];
-  } else if (c == 1) {
-    if (on && d1) eta[0] *= sR[u];
-    if (on && d2) eta[1] *= sR[AP + u];
+    if (c < 2) {   // e_x = r cos, e_y = r sin
+#pragma unroll
+      for (int d = 0; d < 2; ++d)
+        if (d ? d2 : d1)
+          eta[d] = c == 0 ? bm_deviate(part[d], sCs[d * AP + u]) : bm_deviate(sR[d * AP + u], (int64_t)part[d]);
+    }
   }
   __syncthreads();
   const int Ex = sE[row], Ef = sE[3 * A + row];

@@ -42,3 +42,21 @@ def test_device_words_match_published_vector(pimd):
     assert ctr == [0, 0, 0, 0] and key == [0, 0]
     words, _ = pimd.noise_sample(0, 0, 0, 1, 1)
     assert list(map(int, words[0, 0])) == out
+
+
+def test_deviates_near_extended_precision(pimd):
+    """A quarter of a million draws (every table interval and both ends of
+    the unit interval occur) against extended precision: the radius is taken
+    to 2^-54, sine and cosine to 2^-56.5, and the deviate rounds once; half
+    as much again is allowed."""
+    n_atoms, n_modes = 4096, 64
+    words, eta = pimd.noise_sample(11, 1, 77, n_atoms, n_modes)
+    u = (words.astype(np.longdouble) + np.longdouble(0.5)) / np.longdouble(2.0) ** 32
+    r = np.sqrt(-2 * np.log(u[..., [0, 2]]))
+    two_pi = 2 * np.longdouble("3.14159265358979323846264338327950288")
+    ang = two_pi * u[..., [1, 3]]
+    want = np.stack([r[..., 0] * np.cos(ang[..., 0]), r[..., 0] * np.sin(ang[..., 0]),
+                     r[..., 1] * np.cos(ang[..., 1])], axis=-1)
+    rr = r[..., [0, 0, 1]].astype(np.float64)
+    tol = 1.5 * (2.0 ** -54 + rr * 2.0 ** -56.5 + 0.5 * np.spacing(rr))
+    assert np.all(np.abs((eta - want).astype(np.float64)) <= tol)
