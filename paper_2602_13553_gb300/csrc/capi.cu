@@ -25,7 +25,6 @@ int est_rows(int N, int A);
 cudaError_t launch_step(const StepArgs &a, int threads, cudaStream_t s);
 cudaError_t launch_close(const StepArgs &a, int threads, cudaStream_t s);
 cudaError_t launch_advance(int64_t *step, int n, cudaStream_t s);
-cudaError_t launch_to_f32(const double *src, float *dst, size_t n, cudaStream_t s);
 cudaError_t launch_thermal_v(double *v, const double *sigv, const double *imu, uint64_t seed, int N, int P,
                              cudaStream_t s);
 cudaError_t launch_fixcom(const FixcomArgs &a, cudaStream_t s);
@@ -35,6 +34,10 @@ cudaError_t launch_pna_to_nap(const double *src, double *dst, int N, int P, cuda
 cudaError_t launch_nap_to_pna(const double *src, double *dst, int N, int P, cudaStream_t s);
 cudaError_t launch_force_harmonic(const ForceArgs &a, cudaStream_t s);
 cudaError_t launch_force_water(const ForceArgs &a, cudaStream_t s);
+cudaError_t launch_fix_positions(const ForceArgs &a, long long *xi, cudaStream_t s);
+cudaError_t force_water_prepare();
+bool water_lists_apart(int nmol, int P);
+cudaError_t launch_nbr_f64(const ForceArgs &a, cudaStream_t s);
 cudaError_t launch_nbr_build(const NbrArgs &a, const double *ccur, cudaStream_t s);
 cudaError_t launch_centroids(const NbrArgs &a, double *ccur, cudaStream_t s);
 cudaError_t launch_est(const EstArgs &a, int threads, cudaStream_t s);
@@ -162,7 +165,8 @@ struct pimd_handle {
   size_t arena_bytes = 0;
   // device state, layout [N][3][P]
   double *x = nullptr, *v = nullptr, *F = nullptr, *tmp = nullptr;
-  float *x32 = nullptr;   // FP32 copy of x (water-like: the force kernel's cutoff prefilter)
+  long long *xi = nullptr;   // water-like FP64: wrapped fixed-point positions of the oxygens, [nmol][3][P]
+  LjFix lj = {};
   // split precision: FP64 centroids, FP32 deviations / internal modes / forces
   // (x, v, F above then only serve as FP64 staging for estimators and state copies)
   double *xc = nullptr, *v0 = nullptr;
@@ -350,7 +354,12 @@ static StepArgs step_args(pimd_handle *h) {
   a.step = h->d_step;
   a.step_off = 0;
   const bool water = h->potential == PIMD_POT_WATERLIKE;
-  a.x32 = water ? h->x32 : nullptr;
+  a.xi = water ? h->xi : nullptr;
+  for (int d = 0; d < 3; ++d) {
+    a.box[d] = h->box[d];
+    a.invbox[d] = h->box[d] > 0 ? 1.0 / h->box[d] : 0.0;
+  }
+  a.dbox = h->baro ? h->baro + kBaroL : nullptr;
   a.cref = water ? h->cref : nullptr;
   a.ccur = water ? h->ccur : nullptr;
   a.blkmax = water ? h->blkmax : nullptr;
@@ -370,7 +379,8 @@ static ForceArgs force_args(pimd_handle *h) {
   a.P = h->P;
   a.nmol = h->nmol;
   a.x = h->x;
-  a.x32 = h->x32;
+  a.xi = reinterpret_cast<const int64_t *>(h->xi);
+  a.lj = h->lj;
   a.step_inc = nullptr;
   a.F = h->F;
   a.Upart = h->Upart;
@@ -540,7 +550,7 @@ static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, bool advanc
     pimd_status st;
     if (from_outside) {
       st = enqueue(h, PIMD_KIND_OTHER, 2, [&] {
-        cudaError_t e = launch_to_f32(h->x, h->x32, (size_t)h->N * 3 * h->P, h->stream);
+        cudaError_t e = launch_fix_positions(fa, h->xi, h->stream);
         if (e != cudaSuccess) return e;
         return launch_centroids(nbr_args(h, true), h->ccur, h->stream);
       });
@@ -552,7 +562,11 @@ static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, bool advanc
       });
       if (st != PIMD_OK) return st;
     } else {
-      fa.check_nbr = 1;   // the skin test and any rebuild run inside the force kernel
+      fa.check_nbr = 1;   // the skin test and any rebuild: inside the force kernel of a small system
+      if (water_lists_apart(h->nmol, h->P)) {
+        st = enqueue(h, PIMD_KIND_NBR, 1, [&] { return launch_nbr_f64(fa, h->stream); });
+        if (st != PIMD_OK) return st;
+      }
     }
     return enqueue(h, PIMD_KIND_FORCE, 1, [&] { return launch_force_water(fa, h->stream); });
   }
@@ -774,7 +788,8 @@ static void carve(pimd_handle *h, Carver &c) {
   h->v = c.take<double>(len);
   h->F = c.take<double>(len);
   h->tmp = c.take<double>(len);
-  if (h->potential == PIMD_POT_WATERLIKE) h->x32 = c.take<float>(len);
+  if (h->potential == PIMD_POT_WATERLIKE && h->precision == PIMD_PREC_FP64)
+    h->xi = c.take<long long>((size_t)h->nmol * 3 * P);
   h->inv_mm = c.take<double>(N);
   h->sigv = c.take<double>(N);
   h->mass_mm = c.take<double>(N);
@@ -1076,6 +1091,14 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
   for (int d = 0; d < 3; ++d) h->box[d] = sys->box[d];
   for (int q = 0; q < 8; ++q) h->ff[q] = sys->ff[q];
   h->rlist = h->ff[6] + h->skin;
+  if (h->potential == PIMD_POT_WATERLIKE && h->precision == PIMD_PREC_FP64) {
+    h->lj = lj_fix_setup(h->ff[4], h->ff[5], h->ff[6], h->box);
+    const cudaError_t e = force_water_prepare();
+    if (e != cudaSuccess) {
+      delete h;
+      return fail(PIMD_ECUDA, "force kernel set-up failed: %s", cudaGetErrorString(e));
+    }
+  }
   h->alloc = current_allocator();
   if (stream) {
     h->stream = (cudaStream_t)stream;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ljfix.cuh"
 #include "noise64.cuh"
 
 namespace pimd {
@@ -173,7 +174,9 @@ struct StepArgs {
   const double *F;             // [N][3][P] Cartesian forces
   const int64_t *step;         // device step counter (step index of this step = *step + step_off)
   int step_off;
-  float *x32;                  // [N][3][P] FP32 copy of x for the force kernel's cutoff prefilter, or null
+  long long *xi;               // water: [nmol][3][P] wrapped fixed-point positions of the oxygens, or null
+  double box[3], invbox[3];    // water
+  const double *dbox;          // device box (barostat state at kBaroL), overriding box/invbox, or null
   // water-like systems: neighbour-list skin check of the oxygens (atoms 3m)
   const double *cref;          // [nmol][3] centroids at the last list build, or null
   double *ccur;                // [nmol][3] current centroids (written)
@@ -261,7 +264,8 @@ struct ForceArgs {
   int N, P, nmol;
   const double *dbox;          // device box (barostat state at kBaroL), overriding box/invbox, or null
   const double *x;             // [N][3][P]
-  const float *x32;            // [N][3][P] FP32 copy of x (water prefilter)
+  const int64_t *xi;           // water: [nmol][3][P] wrapped fixed-point positions of the oxygens
+  LjFix lj;                    // water: fixed-point pairs
   int64_t *step_inc;           // if not null, block 0 advances the step counter by one
   double *F;                   // [N][3][P]
   double *Upart, *Wpart;       // [rows][P] bead sums of U and Tr Xi (rows: blocks or molecules)

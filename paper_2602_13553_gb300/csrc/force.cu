@@ -4,17 +4,15 @@
 // estimators of App. A need.
 //
 // Harmonic well: thread (atom i, bead k), F = -m mvv2e w^2 x.
-// Water-like model: one block per (molecule, chunk of beads); the beads of the
+// Water-like model: warps over (molecule, chunk of beads); the beads of the
 // chunk sit in adjacent lanes, so each lane's gather of a neighbour's bead is
 // a contiguous segment of that neighbour's bead row.  O-O Lennard-Jones runs
 // over a centroid neighbour list (cutoff + skin) shared by all beads.  Each
 // molecule sums its full neighbour list (no atomics), so forces are
 // deterministic and independent of what else is on the GPU.
-#include <cooperative_groups.h>
+#include <algorithm>
 
 #include "common.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace pimd {
 
@@ -61,326 +59,385 @@ __global__ void __launch_bounds__(256) k_force_harmonic_f64(ForceArgs a) {
   if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
 }
 
-// Water-like model, FP64.  A cluster of kForceBlocks (4) blocks x 4 warps
-// serves one (molecule m, chunk of Bk = min(P, 32) beads).  Lane = (group u,
-// bead kl): beads of the chunk in adjacent lanes (coalesced gathers of a
-// neighbour's bead row), G = 32 / Bk groups when P < 32.  Warps s = 0 ..
-// kLJWarps - 1 split the molecule's O-O neighbour list: warp s, group u owns
-// bucket b = s G + u, the neighbours j with j mod (kLJWarps G) = b, in index
-// order -- every lane of a warp runs the same loop (no divergent filtering),
-// and because a pair's bucket depends on j alone, every sum depends only on
-// the set of interacting pairs: a rebuilt list cannot change a bit.  Warp
-// kLJWarps evaluates the two O-H bonds, warp kLJWarps + 1 the H-O-H angle.
-// A neighbour is first tested in FP32 against (rc + 0.05 A)^2 -- a
-// conservative bound, FP32 rounding of a <100 A coordinate being ~1e-5 A --
-// and only survivors are evaluated in FP64 with the exact r < rc test, so the
-// FP64 result is that of an all-FP64 loop; the FP32 image shift is exact for
-// every pair that can be inside rc (their |d| is well below L/2).
-// Reduction: warps and groups in shared memory, then the blocks of the
-// cluster through distributed shared memory in rank order -- deterministic,
-// no atomics, no global scratch.
-// kDiag (anisotropic barostat) also accumulates the diagonal of the virial
-// tensor, Xi_aa = sum d_a f_a, into W3part.
+// Water-like model, FP64.  A unit of work is one molecule and a chunk of
+// Bk = min(P, 32) beads, or G = 32 / Bk molecules where the beads leave lanes
+// free: lane = (molecule u of the unit, bead kl), beads in adjacent lanes, so
+// a gather of a neighbour's bead row is a contiguous segment.
+//
+// What bounds it is the FP64 pipe (a warp instruction in 64 clocks per SM
+// partition) and, in small systems, the length of one warp's chain:
+//  * the O-O pairs run in 64-bit fixed point on the integer pipe (ljfix.cuh),
+//    positions from a wrapped fixed-point copy of the oxygens' beads; pairs
+//    closer than its range, and systems it does not fit, take the FP64
+//    expressions on the FP64 positions;
+//  * a system with many units takes them whole, one warp each (split = 1: no
+//    reduction, four units to a block); a small one splits a unit's neighbour
+//    list over `split` warps and gives its bonds and its angle to two more, one
+//    unit to a block, partial sums joined in shared memory in a fixed order.
+// A neighbour's bucket (j mod NS) decides its warp, so every sum depends only on
+// the set of interacting pairs: a rebuilt list cannot change a bit.
+// kDiag (anisotropic barostat) also sums the diagonal of the virial tensor,
+// Xi_aa = sum d_a f_a, into W3part.
+struct Bonded {
+  double fO[3], fH[2][3], U, W, w3[3];
+};
+
+// O-H bonds, U = 1/2 kb (r - r0)^2 each (what & 1), and the H-O-H angle, U =
+// 1/2 kth (theta - th0)^2 (what & 2), of molecule m at bead k.
 template <bool kDiag>
-__global__ void __cluster_dims__(kForceBlocks, 1, 1) __launch_bounds__(128) k_force_water_f64(ForceArgs a) {
-  constexpr int NC = kDiag ? 14 : 11;   // F (9), U, Tr Xi, then Xi_xx, Xi_yy, Xi_zz
-  __shared__ double sacc[NC][128];
-  __shared__ double gath[kForceBlocks][NC][32];   // rank 0: every block's partial sums
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
+__device__ __forceinline__ void bonded_f64(const ForceArgs &a, int m, int k, const double (&L)[3],
+                                           const double (&iL)[3], int what, Bonded &o) {
   const int P = a.P;
-  const int Bk = P < 32 ? P : 32;
-  const int G = a.nbr_groups;
-  const int NS = kLJWarps * G;
+  const double *x = a.x + (size_t)9 * m * P + k;
+  double d[2][3], r2[2], ir[2];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double xo = x[c * P];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      double e = x[(3 + 3 * h + c) * P] - xo;
+      // the minimum image, only where a component reaches half a box (the
+      // comparison of high words may fall to either side of a tie, as rint may)
+      if ((__double2hiint(e) & 0x7fffffff) >= __double2hiint(0.5 * L[c])) e = mic(e, L[c], iL[c]);
+      d[h][c] = e;
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    r2[h] = d[h][0] * d[h][0] + d[h][1] * d[h][1] + d[h][2] * d[h][2];
+    ir[h] = rsqrt(r2[h]);
+  }
+  o.U = o.W = 0.0;
+  // H force h: gd[h] d_h + ga[h] d_{1-h}
+  double gd[2] = {0.0, 0.0}, ga = 0.0;
+  if (what & 1) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      // r - r0 with r = r2 ir corrected by half a Newton step of its square
+      const double r = r2[h] * ir[h];
+      const double dr = fma(0.5 * ir[h], fma(-r, r, r2[h]), r - a.r0), kd = a.kb * dr;
+      o.U = fma(0.5 * kd, dr, o.U);
+      gd[h] = -kd * ir[h];
+      o.W = fma(gd[h], r2[h], o.W);
+    }
+  }
+  if (what & 2) {
+    // F_h = kth (theta - th0) / sin(theta) d cos(theta) / d r_h; the virial of
+    // an angle is zero (it does not change with the scale)
+    const double ir01 = ir[0] * ir[1];
+    const double dot = d[0][0] * d[1][0] + d[0][1] * d[1][1] + d[0][2] * d[1][2];
+    const double cth = fmin(1.0, fmax(-1.0, dot * ir01));
+    const double dth = acos(cth) - a.th0, kd = a.kth * dth;
+    o.U = fma(0.5 * kd, dth, o.U);
+    const double pref = kd * rsqrt(fma(-cth, cth, 1.0));
+    ga = pref * ir01;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) gd[h] = fma(-pref * cth * ir[h], ir[h], gd[h]);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    o.fH[0][c] = fma(ga, d[1][c], gd[0] * d[0][c]);
+    o.fH[1][c] = fma(ga, d[0][c], gd[1] * d[1][c]);
+    o.fO[c] = -(o.fH[0][c] + o.fH[1][c]);
+    if (kDiag) o.w3[c] = fma(d[1][c], o.fH[1][c], d[0][c] * o.fH[0][c]);
+  }
+}
+
+// A pair in FP64, from the FP64 positions: forces on i, U, Tr Xi (and Xi_aa).
+struct PairF64 {
+  double f[3] = {0.0, 0.0, 0.0}, U = 0.0, W = 0.0, w3[3] = {0.0, 0.0, 0.0};
+};
+
+template <bool kDiag>
+__device__ __noinline__ void pair_f64(const ForceArgs &a, const double *L, const double *iL, int m, int j, int k,
+                                      PairF64 &s) {
+  const int P = a.P;
+  const double *xi = a.x + (size_t)9 * m * P + k, *xj = a.x + (size_t)9 * j * P + k;
+  double d[3], r2 = 0.0;
+  for (int c = 0; c < 3; ++c) {
+    d[c] = mic(xj[c * P] - xi[c * P], L[c], iL[c]);
+    r2 = fma(d[c], d[c], r2);
+  }
+  if (!(r2 < a.rc * a.rc)) return;
+  const double inv = 1.0 / r2;
+  const double s2 = a.sig * a.sig * inv;
+  const double s6 = s2 * s2 * s2;
+  s.U = fma(4.0 * a.eps, fma(s6, s6, -s6), s.U);
+  const double fr = 24.0 * a.eps * fma(2.0 * s6, s6, -s6) * inv;   // force on j = fr * d
+  for (int c = 0; c < 3; ++c) {
+    s.f[c] = fma(-fr, d[c], s.f[c]);
+    if (kDiag) s.w3[c] = fma(fr * d[c], d[c], s.w3[c]);
+  }
+  s.W = fma(fr, r2, s.W);
+}
+
+// Number of neighbours of molecule m within rc + skin, listed by bucket (j mod
+// NS) and index, by one warp: FP32 test on the differences of the FP64
+// centroids, in FP64 where it is close.
+__device__ __forceinline__ int list_molecule(const ForceArgs &a, const double (&L)[3], const double (&iL)[3], int m,
+                                             int NS, int *nl, int *off) {
+  const int lane = threadIdx.x & 31;
+  const double c0 = a.ccur[3 * m], c1 = a.ccur[3 * m + 1], c2 = a.ccur[3 * m + 2];
+  const float rl = (float)a.rlist, lo = rl * rl * (1.0f - 1e-5f), hi = rl * rl * (1.0f + 1e-5f);
+  const float Lf[3] = {(float)L[0], (float)L[1], (float)L[2]};
+  const float If[3] = {(float)iL[0], (float)iL[1], (float)iL[2]};
+  auto near = [&](int j) {
+    const double e0 = a.ccur[3 * j] - c0, e1 = a.ccur[3 * j + 1] - c1, e2 = a.ccur[3 * j + 2] - c2;
+    const float f0 = fmaf(-rintf((float)e0 * If[0]), Lf[0], (float)e0);
+    const float f1 = fmaf(-rintf((float)e1 * If[1]), Lf[1], (float)e1);
+    const float f2 = fmaf(-rintf((float)e2 * If[2]), Lf[2], (float)e2);
+    const float r2 = f0 * f0 + f1 * f1 + f2 * f2;
+    // unwrapped differences of many boxes lose FP32 digits: FP64 there too
+    const float far = fmaxf(fmaxf(fabsf((float)e0), fabsf((float)e1)), fabsf((float)e2));
+    if (far < 8.0f * rl) {
+      if (r2 < lo) return true;
+      if (r2 > hi) return false;
+    }
+    const double d0 = mic(e0, L[0], iL[0]), d1 = mic(e1, L[1], iL[1]), d2 = mic(e2, L[2], iL[2]);
+    return d0 * d0 + d1 * d1 + d2 * d2 < a.rlist * a.rlist;
+  };
+  int total = 0;
+  const int n0 = (a.nmol + NS - 1) / NS;   // candidates of bucket 0, the longest
+  int seg = 1;                             // lanes per bucket, 32 / seg buckets a round
+  while (seg < n0 && seg < 32) seg <<= 1;
+  const int sg = lane / seg, tl = lane - sg * seg;
+  for (int b = 0; b < NS; b += 32 / seg) {
+    const int bb = b + sg;
+    for (int t0 = 0; t0 < n0; t0 += seg) {   // more than one round only with a whole warp per bucket
+      const int j = bb + (t0 + tl) * NS;
+      const bool hit = bb < NS && j < a.nmol && j != m && near(j);
+      const unsigned mask = __ballot_sync(0xffffffffu, hit);
+      const int pos = total + __popc(mask & ((1u << lane) - 1u));
+      if (t0 == 0 && tl == 0 && bb < NS) off[bb] = pos;
+      if (hit && pos < kMaxNeighbours) nl[pos] = j;
+      total += __popc(mask);
+    }
+  }
+  if (total > kMaxNeighbours) {   // report, and use an empty list
+    if (lane == 0) atomicOr(a.err, kErrNbrOverflow);
+    __syncwarp();
+    for (int b = lane; b < NS; b += 32) off[b] = 0;
+    total = -1;
+  }
+  if (lane == 0) off[NS] = total < 0 ? 0 : total;
+  __syncwarp();
+  return total;
+}
+
+// This step's rebuild decision from the step kernel's per-block maxima, by all
+// threads of a block.
+__device__ __forceinline__ bool skin_exceeded(const double *blkmax, int n, double skin) {
+  __shared__ double s_mx[2][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  // the maxima are non-negative: they compare as integers, off the FP64 pipe
+  long long md = 0, me = 0;
+  const longlong2 *bm = reinterpret_cast<const longlong2 *>(blkmax);
+#pragma unroll 4
+  for (int b = threadIdx.x; b < n; b += blockDim.x) {
+    const longlong2 e = bm[b];
+    md = max(md, e.x);
+    me = max(me, e.y);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    md = max(md, __shfl_xor_sync(0xffffffffu, md, o));
+    me = max(me, __shfl_xor_sync(0xffffffffu, me, o));
+  }
+  if (lane == 0) {
+    s_mx[0][warp] = __longlong_as_double(md);
+    s_mx[1][warp] = __longlong_as_double(me);
+  }
+  __syncthreads();
+  double d = 0.0, e = 0.0;
+  for (int w = 0; w < nw; ++w) {
+    if (__double_as_longlong(s_mx[0][w]) > __double_as_longlong(d)) d = s_mx[0][w];
+    if (__double_as_longlong(s_mx[1][w]) > __double_as_longlong(e)) e = s_mx[1][w];
+  }
+  return 2.0 * d + 2.0 * e > skin;
+}
+
+__device__ __forceinline__ void force_box(const ForceArgs &a, double (&L)[3], double (&iL)[3]) {
+  const bool db = a.dbox != nullptr;   // the barostat's box: edges, then their inverses
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    L[c] = db ? a.dbox[c] : a.box[c];
+    iL[c] = db ? a.dbox[3 + c] : a.invbox[c];
+  }
+}
+
+// Neighbour lists for the systems whose units go one to a warp: rebuilt here,
+// one warp per molecule, when this step's skin test fails (a small system's
+// blocks rebuild their own molecule's list).
+__global__ void __launch_bounds__(256) k_nbr_f64(ForceArgs a) {
+  if (!skin_exceeded(a.blkmax, a.nblk_check, a.skin)) return;
+  const int NS = kLJWarps * a.nbr_groups, lane = threadIdx.x & 31;
+  double L[3], iL[3];
+  force_box(a, L, iL);
+  for (int m = blockIdx.x * 8 + (threadIdx.x >> 5); m < a.nmol; m += gridDim.x * 8) {
+    const int total = list_molecule(a, L, iL, m, NS, a.nbr + (size_t)m * kMaxNeighbours,
+                                    a.nbr_off + (size_t)m * (NS + 1));
+    if (total >= 0 && lane < 3) a.cref[3 * m + lane] = a.ccur[3 * m + lane];
+  }
+}
+
+template <bool kDiag, bool kFar, bool kSplit>
+__global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArgs a, int split) {
+  constexpr int NC = kDiag ? 14 : 11;   // F (9), U, Tr Xi, then Xi_xx, Xi_yy, Xi_zz
+  extern __shared__ __align__(16) unsigned char fsm[];
+  const int P = a.P;
+  const int Bk = P < 32 ? P : 32, G = 32 / Bk;
   const int nchunk = (P + Bk - 1) / Bk;
-  const int cid = blockIdx.x / kForceBlocks;
-  const int m = cid / nchunk, chunk = cid % nchunk;
+  const int NS = kLJWarps * a.nbr_groups;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int s = rank * 4 + warp;     // 0..kLJWarps-1: LJ buckets; then bonds, angle
-  const int u = lane / Bk, kl = lane % Bk;
-  const int k = chunk * Bk + kl;
+  const int unit = kSplit ? blockIdx.x : blockIdx.x * 4 + warp;
+  const int role = kSplit ? warp : 0;   // 0 .. split - 1: the list; then bonds, angle
+  // chunk by chunk: the warps of an SM gather from one chunk's rows
+  const int nmg = (a.nmol + G - 1) / G;
+  const int chunk = unit / nmg, mg = unit - chunk * nmg;
+  const int u = lane / Bk, kl = lane - u * Bk;
+  const int m = mg * G + u, k = chunk * Bk + kl;
+  const bool on = u < G && m < a.nmol && k < P;   // (a last block's spare warps have k >= P)
+  double L[3], iL[3];
+  force_box(a, L, iL);
+  // a small system's blocks take the step's rebuild decision themselves (the
+  // same one from the same maxima) and list their own molecules in shared
+  // memory; the block of chunk 0 also keeps the lists and the new centroids
+  int *s_nl = reinterpret_cast<int *>(fsm);             // [G][kMaxNeighbours]
+  int *s_off = s_nl + G * kMaxNeighbours;               // [G][NS + 1]
+  bool own = false;
+  if (kSplit && a.check_nbr) {
+    own = skin_exceeded(a.blkmax, a.nblk_check, a.skin);
+    if (own) {
+      for (int q = warp; q < G; q += blockDim.x >> 5) {
+        const int mm = mg * G + q;
+        if (mm >= a.nmol) break;
+        int *nl = s_nl + q * kMaxNeighbours, *off = s_off + q * (NS + 1);
+        const int total = list_molecule(a, L, iL, mm, NS, nl, off);
+        if (chunk == 0) {
+          for (int e = lane; e < total; e += 32) a.nbr[(size_t)mm * kMaxNeighbours + e] = nl[e];
+          for (int b = lane; b <= NS; b += 32) a.nbr_off[(size_t)mm * (NS + 1) + b] = off[b];
+          if (lane < 3 && total >= 0) a.cref[3 * mm + lane] = a.ccur[3 * mm + lane];
+        }
+      }
+      __syncthreads();
+    }
+  }
   double acc[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) acc[c] = 0.0;
-  // the neighbour list of molecule m: the stored one, or rebuilt here when
-  // this step's skin test fails (every block takes the same decision from the
-  // same maxima and builds the same list into its own shared memory; the
-  // cluster of chunk 0 also stores it and the new reference centroid)
-  __shared__ int s_nl[kMaxNeighbours];
-  __shared__ int s_off[kMaxBuckets + 1];
-  __shared__ int s_go;
-  __shared__ double s_mx[4][2];
-  if (a.check_nbr) {
-    // the step kernel's per-block maxima: every thread loads its share (one
-    // 16-byte pair per block entry, all loads in flight at once), then warp
-    // and block maxima
-    double md = 0.0, me = 0.0;
-    const double2 *bm = reinterpret_cast<const double2 *>(a.blkmax);
-    int b = threadIdx.x;
-    for (; b + (int)blockDim.x < a.nblk_check; b += 2 * blockDim.x) {   // two entries in flight
-      const double2 e = bm[b], f = bm[b + blockDim.x];
-      md = fmax(md, fmax(e.x, f.x));
-      me = fmax(me, fmax(e.y, f.y));
+  if (on && role < split) {
+    // O-O Lennard-Jones: this warp's share of the buckets
+    const int *off = own ? s_off + u * (NS + 1) : a.nbr_off + (size_t)m * (NS + 1);
+    const int *nl = own ? s_nl + u * kMaxNeighbours : a.nbr + (size_t)m * kMaxNeighbours;
+    int q = off[kSplit ? role * NS / split : 0];
+    const int q1 = off[kSplit ? (role + 1) * NS / split : NS];
+    const LjFix &lj = a.lj;
+    int64_t LQ[3], xi[3];
+    const int64_t *__restrict__ xp = a.xi + k;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      LQ[c] = fix_pos(L[c]);
+      xi[c] = xp[(size_t)(3 * m + c) * P];
     }
-    if (b < a.nblk_check) {
-      const double2 e = bm[b];
-      md = fmax(md, e.x);
-      me = fmax(me, e.y);
-    }
-#pragma unroll
-    for (int o2 = 16; o2 > 0; o2 >>= 1) {
-      md = fmax(md, __shfl_xor_sync(0xffffffffu, md, o2));
-      me = fmax(me, __shfl_xor_sync(0xffffffffu, me, o2));
-    }
-    if (lane == 0) {
-      s_mx[warp][0] = md;
-      s_mx[warp][1] = me;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      md = fmax(fmax(s_mx[0][0], s_mx[1][0]), fmax(s_mx[2][0], s_mx[3][0]));
-      me = fmax(fmax(s_mx[0][1], s_mx[1][1]), fmax(s_mx[2][1], s_mx[3][1]));
-      int go = 2.0 * md + 2.0 * me > a.skin;
-      if (go && m < a.nmol) {
-        // bucket b holds the neighbours j = b mod NS in increasing j
-        const bool db0 = a.dbox != nullptr;
-        const double B0 = db0 ? a.dbox[0] : a.box[0], B1 = db0 ? a.dbox[1] : a.box[1], B2 = db0 ? a.dbox[2] : a.box[2];
-        const double I0 = db0 ? a.dbox[3] : a.invbox[0], I1 = db0 ? a.dbox[4] : a.invbox[1];
-        const double I2 = db0 ? a.dbox[5] : a.invbox[2];
-        const double c0 = a.ccur[3 * m], c1 = a.ccur[3 * m + 1], c2 = a.ccur[3 * m + 2];
-        const double rl2 = a.rlist * a.rlist;
-        int total = 0;
-        for (int b = 0; b < NS; ++b) {
-          if (lane == 0) s_off[b] = total;
-          for (int j0 = b; j0 < a.nmol; j0 += 32 * NS) {
-            const int j = j0 + lane * NS;
-            bool hit = false;
-            if (j < a.nmol && j != m) {
-              const double d0 = mic(a.ccur[3 * j] - c0, B0, I0);
-              const double d1 = mic(a.ccur[3 * j + 1] - c1, B1, I1);
-              const double d2 = mic(a.ccur[3 * j + 2] - c2, B2, I2);
-              hit = d0 * d0 + d1 * d1 + d2 * d2 < rl2;
-            }
-            const unsigned mask = __ballot_sync(0xffffffffu, hit);
-            const int pos = total + __popc(mask & ((1u << lane) - 1u));
-            if (hit && pos < kMaxNeighbours) s_nl[pos] = j;
-            total += __popc(mask);
-          }
-        }
-        if (total > kMaxNeighbours) {   // report, and use an empty list
-          if (lane == 0 && rank == 0 && chunk == 0) atomicOr(a.err, kErrNbrOverflow);
-          for (int b = lane; b <= NS; b += 32) s_off[b] = 0;
-          total = 0;
-        }
-        if (lane == 0) s_off[NS] = total;
-        __syncwarp();
-        if (rank == 0 && chunk == 0) {   // keep it for the following steps
-          for (int q = lane; q < total; q += 32) a.nbr[(size_t)m * kMaxNeighbours + q] = s_nl[q];
-          for (int b = lane; b <= NS; b += 32) a.nbr_off[(size_t)m * (NS + 1) + b] = s_off[b];
-          if (lane < 3 && total <= kMaxNeighbours) a.cref[3 * m + lane] = a.ccur[3 * m + lane];
-        }
-      }
-      if (lane == 0) s_go = go;
-    }
-    __syncthreads();
-  }
-  if (u < G && k < P && m < a.nmol) {
-    const int o = 3 * m;
-    const bool db = a.dbox != nullptr;
-    const double L0 = db ? a.dbox[0] : a.box[0], L1 = db ? a.dbox[1] : a.box[1], L2 = db ? a.dbox[2] : a.box[2];
-    const double i0 = db ? a.dbox[3] : a.invbox[0], i1 = db ? a.dbox[4] : a.invbox[1];
-    const double i2 = db ? a.dbox[5] : a.invbox[2];
-    const size_t so = (size_t)o * 3 * P + k;
-    const double xo0 = a.x[so], xo1 = a.x[so + P], xo2 = a.x[so + 2 * P];
-    if (s >= kLJWarps) {
-      // warp kLJWarps: the two O-H bonds; warp kLJWarps + 1: the H-O-H angle
-      if (u == 0) {
-        double dv[2][3], r[2], ir[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const size_t sh = (size_t)(o + 1 + h) * 3 * P + k;
-          dv[h][0] = mic(a.x[sh] - xo0, L0, i0);
-          dv[h][1] = mic(a.x[sh + P] - xo1, L1, i1);
-          dv[h][2] = mic(a.x[sh + 2 * P] - xo2, L2, i2);
-          r[h] = sqrt(dv[h][0] * dv[h][0] + dv[h][1] * dv[h][1] + dv[h][2] * dv[h][2]);
-          ir[h] = 1.0 / r[h];
-        }
-        if (s == kLJWarps) {
-          // U = 1/2 kb (r - r0)^2 per bond, force on H = -kb (r - r0) d / r
-          double uu = 0.0, w = 0.0;
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const double dr = r[h] - a.r0;
-            uu = fma(0.5 * a.kb * dr, dr, uu);
-            const double g = -a.kb * dr * ir[h];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const double fc = g * dv[h][c];
-              acc[3 + 3 * h + c] = fc;
-              acc[c] -= fc;
-              w = fma(dv[h][c], fc, w);
-              if (kDiag) acc[11 + c] = fma(dv[h][c], fc, acc[11 + c]);
-            }
-          }
-          acc[9] = uu;
-          acc[10] = w;
-        } else {
-          // U = 1/2 kth (theta - th0)^2; F_h = kth (theta - th0)/sin(theta) d cos(theta)/d r_h
-          const double ir01 = ir[0] * ir[1];
-          const double dot = dv[0][0] * dv[1][0] + dv[0][1] * dv[1][1] + dv[0][2] * dv[1][2];
-          const double cth = fmin(1.0, fmax(-1.0, dot * ir01));
-          const double th = acos(cth);
-          const double dth = th - a.th0;
-          // sin(acos c) = sqrt(1 - c^2): one square root on the FP64 pipe
-          // in place of a sine (the H-O-H angle stays far from 0 and pi)
-          const double pref = a.kth * dth / sqrt(fma(-cth, cth, 1.0));
-          double w = 0.0;
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int g = 1 - h;
-            const double ch = cth * ir[h] * ir[h];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const double fa = pref * fma(dv[g][c], ir01, -ch * dv[h][c]);
-              acc[3 + 3 * h + c] = fa;
-              acc[c] -= fa;
-              w = fma(dv[h][c], fa, w);
-              if (kDiag) acc[11 + c] = fma(dv[h][c], fa, acc[11 + c]);
-            }
-          }
-          acc[9] = 0.5 * a.kth * dth * dth;
-          acc[10] = w;
-        }
-      }
-    } else {
-    // O-O Lennard-Jones over bucket b of the neighbour list
-    const int b = s * G + u;          // neighbours j with j mod (kLJWarps G) = b
-    const bool own = a.check_nbr && s_go;   // rebuilt in this block's shared memory
-    const int *off = own ? s_off : a.nbr_off + (size_t)m * (NS + 1);
-    const int q0 = off[b], q1 = off[b + 1];
-    const int *nl = own ? s_nl : a.nbr + (size_t)m * kMaxNeighbours;
-    const float xf0 = a.x32[so], xf1 = a.x32[so + P], xf2 = a.x32[so + 2 * P];
-    const float Lf0 = (float)L0, Lf1 = (float)L1, Lf2 = (float)L2;
-    const float if0 = (float)i0, if1 = (float)i1, if2 = (float)i2;
-    const float rpre = (float)(a.rc + 0.05);
-    const float rpre2 = rpre * rpre;
-    const double rc2 = a.rc * a.rc;
-    const double sig2 = a.sig * a.sig;
-    const double e4 = 4.0 * a.eps, e24 = 24.0 * a.eps;
-    double f0 = 0.0, f1 = 0.0, f2 = 0.0, ulj = 0.0, wlj = 0.0;
-    double wx = 0.0, wy = 0.0, wz = 0.0;
-    // one candidate j from its FP32 and FP64 bead positions: the FP32
-    // prefilter, then the exact FP64 cutoff test and the pair terms
-    auto pair = [&](const float (&pf)[3], const double (&pd)[3]) {
-      float d0f = pf[0] - xf0, d1f = pf[1] - xf1, d2f = pf[2] - xf2;
-      const float n0 = rintf(d0f * if0), n1 = rintf(d1f * if1), n2 = rintf(d2f * if2);
-      d0f = fmaf(-n0, Lf0, d0f);
-      d1f = fmaf(-n1, Lf1, d1f);
-      d2f = fmaf(-n2, Lf2, d2f);
-      if (d0f * d0f + d1f * d1f + d2f * d2f >= rpre2) return;
-      const double d0 = fma(-(double)n0, L0, pd[0] - xo0);
-      const double d1 = fma(-(double)n1, L1, pd[1] - xo1);
-      const double d2 = fma(-(double)n2, L2, pd[2] - xo2);
-      const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
-      if (r2 < rc2) {
-        // 1 / r2 by Newton's iteration x <- x (2 - r2 x) from the FP32
-        // reciprocal: each step squares the relative error (2^-23 -> 2^-46
-        // -> below FP64 rounding), two FMAs each on the FP64 pipe
-        double inv = (double)__frcp_rn((float)r2);
-        inv = fma(inv, fma(-r2, inv, 1.0), inv);
-        inv = fma(inv, fma(-r2, inv, 1.0), inv);
-        const double s2 = sig2 * inv;
-        const double s6 = s2 * s2 * s2;
-        ulj = fma(e4, fma(s6, s6, -s6), ulj);
-        const double fr = e24 * fma(2.0 * s6, s6, -s6) * inv;   // force on j = fr * d
-        f0 = fma(-fr, d0, f0);
-        f1 = fma(-fr, d1, f1);
-        f2 = fma(-fr, d2, f2);
-        wlj = fma(fr, r2, wlj);
-        if (kDiag) {
-          wx = fma(fr * d0, d0, wx);
-          wy = fma(fr * d1, d1, wy);
-          wz = fma(fr * d2, d2, wz);
-        }
-      }
-    };
-    // four candidates per round: their indices, then their bead rows (FP32
-    // and FP64), are requested before any arithmetic, so the gathers of a
-    // round overlap; the candidates are then summed in list order
-    int q = q0;
-    for (; q + 4 <= q1; q += 4) {
-      int jj[4];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) jj[v] = nl[q + v];
-      float pf[4][3];
-      double pd[4][3];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const size_t sj = (size_t)(3 * jj[v]) * 3 * P + k;
+    LjSums s;
+    PairF64 far;
+    // fixed point holds edges below 8192 A (the barostat may change them)
+    const bool fixed = lj.on && L[0] < 4096.0 && L[1] < 4096.0 && L[2] < 4096.0;
+    auto pair = [&](const int64_t (&xj)[3], int j) {
+      if (fixed) {
+        int64_t d[3];
+        float h2 = 0.f;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          pf[v][c] = __ldg(a.x32 + sj + c * P);
-          pd[v][c] = a.x[sj + c * P];
+          d[c] = fix_mic(xj[c] - xi[c], LQ[c]);
+          const float h = (float)(int)(d[c] >> 32);
+          h2 = fmaf(h, h, h2);
         }
+        if (h2 >= lj.rpre2) return;
+        if (lj_fix_pair<kDiag, kFar>(lj, d, s)) return;
       }
+      pair_f64<kDiag>(a, L, iL, m, j, k, far);
+    };
+    // the next candidate's rows and the index after it are requested before
+    // this candidate's arithmetic
+    int j = q < q1 ? nl[q] : 0, jn = q + 1 < q1 ? nl[q + 1] : 0;
+    int64_t xj[3], xn[3];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) pair(pf[v], pd[v]);
-    }
+    for (int c = 0; c < 3; ++c) xn[c] = xj[c] = xp[(size_t)(3 * j + c) * P];
+#pragma unroll 1
     for (; q < q1; ++q) {
-      const size_t sj = (size_t)(3 * nl[q]) * 3 * P + k;
-      float pf[3];
-      double pd[3];
+      const int ja = q + 2 < q1 ? nl[q + 2] : 0;
+      if (q + 1 < q1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xn[c] = __ldg(xp + (size_t)(3 * jn + c) * P);
+      }
+      pair(xj, j);
+      j = jn;
+      jn = ja;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) xj[c] = xn[c];
+    }
+    // each molecule takes half of every pair's energy and virial; a pair's
+    // fixed-point force is the one on j
+    if (fixed) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        pf[c] = __ldg(a.x32 + sj + c * P);
-        pd[c] = a.x[sj + c * P];
+        acc[c] = fma(-lj.fs, fix_sum(s.f[c]), far.f[c]);
+        if (kDiag) acc[11 + c] = 0.5 * fma(lj.w3, fix_sum(s.w[c]), far.w3[c]);
       }
-      pair(pf, pd);
-    }
-    // each molecule takes half of every pair's energy and virial
-    acc[0] = f0;
-    acc[1] = f1;
-    acc[2] = f2;
-    acc[9] = 0.5 * ulj;
-    acc[10] = 0.5 * wlj;
-    if (kDiag) {
-      acc[11] = 0.5 * wx;
-      acc[12] = 0.5 * wy;
-      acc[13] = 0.5 * wz;
-    }
-    }
-  }
+      acc[9] = fma(lj.us, fix_energy<kFar>(s), 0.5 * far.U);
+      acc[10] = fma(lj.ws, fix_sum(s.T), 0.5 * far.W);
+    } else {
 #pragma unroll
-  for (int c = 0; c < NC; ++c) sacc[c][threadIdx.x] = acc[c];
-  __syncthreads();
-  // each block's partial sums go straight into rank 0's shared memory
-  // (distributed shared memory stores), so after one cluster barrier rank 0
-  // sums them locally in rank order and the other blocks may exit
-  for (int t = threadIdx.x; t < NC * Bk; t += blockDim.x) {
-    const int comp = t / Bk, kk = t % Bk;
-    double sum = 0.0;
-    for (int w = 0; w < 4; ++w)
-      for (int g = 0; g < G; ++g) sum += sacc[comp][w * 32 + g * Bk + kk];
-    *cluster.map_shared_rank(&gath[rank][comp][kk], 0) = sum;
-  }
-  cluster.sync();
-  if (rank == 0 && m < a.nmol) {
-    for (int t = threadIdx.x; t < NC * Bk; t += blockDim.x) {
-      const int comp = t / Bk, kk = t % Bk;
-      const int k2 = chunk * Bk + kk;
-      if (k2 >= P) continue;
-      double sum = 0.0;
-      for (int r = 0; r < kForceBlocks; ++r) sum += gath[r][comp][kk];
-      if (comp < 9)
-        a.F[(size_t)(3 * m + comp / 3) * 3 * P + (comp % 3) * P + k2] = sum;
-      else if (comp == 9)
-        a.Upart[(size_t)m * P + k2] = sum;
-      else if (comp == 10)
-        a.Wpart[(size_t)m * P + k2] = sum;
-      else
-        a.W3part[((size_t)m * P + k2) * 3 + (comp - 11)] = sum;
+      for (int c = 0; c < 3; ++c) {
+        acc[c] = far.f[c];
+        if (kDiag) acc[11 + c] = 0.5 * far.w3[c];
+      }
+      acc[9] = 0.5 * far.U;
+      acc[10] = 0.5 * far.W;
     }
-    if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
+  }
+  if (on && (!kSplit || role >= split)) {
+    Bonded b;
+    bonded_f64<kDiag>(a, m, k, L, iL, kSplit ? (role == split ? 1 : 2) : 3, b);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      acc[c] += b.fO[c];
+      acc[3 + c] = b.fH[0][c];
+      acc[6 + c] = b.fH[1][c];
+      if (kDiag) acc[11 + c] += b.w3[c];
+    }
+    acc[9] += b.U;
+    acc[10] += b.W;
+  }
+  auto store = [&](int comp, int mm, int kk, double v) {
+    if (comp < 9)
+      a.F[(size_t)(9 * mm + comp) * P + kk] = v;
+    else if (comp == 9)
+      a.Upart[(size_t)mm * P + kk] = v;
+    else if (comp == 10)
+      a.Wpart[(size_t)mm * P + kk] = v;
+    else
+      a.W3part[((size_t)mm * P + kk) * 3 + (comp - 11)] = v;
+  };
+  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
+  if (!kSplit) {
+    if (on)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) store(c, m, k, acc[c]);
+    return;
+  }
+  double *sacc = reinterpret_cast<double *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [warps][NC][32]
+#pragma unroll
+  for (int c = 0; c < NC; ++c) sacc[(warp * NC + c) * 32 + lane] = acc[c];
+  __syncthreads();
+  const int nw = split + 2;
+  for (int t = threadIdx.x; t < NC * 32; t += blockDim.x) {
+    const int comp = t >> 5;   // the lanes keep their (molecule, bead)
+    // the hydrogens' forces come from the bonded warps alone
+    double sum = 0.0;
+    for (int w = comp >= 3 && comp < 9 ? split : 0; w < nw; ++w) sum += sacc[(w * NC + comp) * 32 + lane];
+    if (on) store(comp, m, k, sum);
   }
 }
 
@@ -495,9 +552,22 @@ int force_blocks(int n_groups, int P) {
   return (n_groups + per - 1) / per;
 }
 
-int water_force_blocks(int nmol, int P) {
+int water_force_blocks(int nmol, int P) {   // split precision
   const int Bk = P < 32 ? P : 32;
   return kForceBlocks * nmol * ((P + Bk - 1) / Bk);
+}
+
+// Units of work of the FP64 water force, and the warps that share a unit's
+// neighbour list: 1 (a warp takes whole units) once there are enough of them
+// for every SM partition twice over.
+static int water_units(int nmol, int P) {
+  const int Bk = P < 32 ? P : 32, G = 32 / Bk;
+  return (nmol + G - 1) / G * ((P + Bk - 1) / Bk);
+}
+
+static int water_split(int nmol, int P) {
+  const int n = water_units(nmol, P);
+  return n >= 1024 ? 1 : (n >= 512 ? 2 : (n >= 256 ? 4 : 7));   // NS is a multiple of 14
 }
 
 // lane groups per warp of the water force kernel: the largest power of two
@@ -514,11 +584,65 @@ cudaError_t launch_force_harmonic(const ForceArgs &a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Whether the list check is a kernel of its own (the one-warp units).
+bool water_lists_apart(int nmol, int P) { return water_split(nmol, P) == 1; }
+
+cudaError_t launch_nbr_f64(const ForceArgs &a, cudaStream_t s) {
+  k_nbr_f64<<<std::min((a.nmol + 7) / 8, 304), 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <bool kDiag, bool kFar>
+static void force_water(const ForceArgs &a, cudaStream_t s) {
+  const int split = water_split(a.nmol, a.P), units = water_units(a.nmol, a.P);
+  if (split == 1) {
+    k_force_water_f64<kDiag, kFar, false><<<(units + 3) / 4, 128, 0, s>>>(a, 1);
+    return;
+  }
+  const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nbr_groups;
+  const size_t smem = (size_t)G * kMaxNeighbours * sizeof(int) + (((size_t)G * (NS + 1) + 3) & ~(size_t)3) * sizeof(int) +
+                      (size_t)(split + 2) * (kDiag ? 14 : 11) * 32 * sizeof(double);
+  k_force_water_f64<kDiag, kFar, true><<<units, 32 * (split + 2), smem, s>>>(a, split);
+}
+
+cudaError_t force_water_prepare() {   // a one-bead system's lists take more than 48 KB
+  const int most = 128 * 1024;
+  cudaError_t e = cudaFuncSetAttribute(k_force_water_f64<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  return e;
+}
+
 cudaError_t launch_force_water(const ForceArgs &a, cudaStream_t s) {
-  if (a.W3part)
-    k_force_water_f64<true><<<water_force_blocks(a.nmol, a.P), 128, 0, s>>>(a);
-  else
-    k_force_water_f64<false><<<water_force_blocks(a.nmol, a.P), 128, 0, s>>>(a);
+  if (a.W3part) {
+    if (a.lj.far)
+      force_water<true, true>(a, s);
+    else
+      force_water<true, false>(a, s);
+  } else if (a.lj.far) {
+    force_water<false, true>(a, s);
+  } else {
+    force_water<false, false>(a, s);
+  }
+  return cudaGetLastError();
+}
+
+// Wrapped fixed-point positions of the oxygens (the step kernels write them;
+// this is for positions from outside).
+__global__ void k_fix_positions(ForceArgs a, long long *xi) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= a.nmol * 3 * a.P) return;
+  const int k = t % a.P, mc = t / a.P, c = mc % 3, m = mc / 3;
+  double L[3], iL[3];
+  force_box(a, L, iL);
+  const double x = a.x[(size_t)(9 * m + c) * a.P + k];
+  xi[t] = fix_wrap(x, (float)x, (float)iL[c], fix_pos(L[c]));
+}
+
+cudaError_t launch_fix_positions(const ForceArgs &a, long long *xi, cudaStream_t s) {
+  const int n = a.nmol * 3 * a.P;
+  k_fix_positions<<<(n + 255) / 256, 256, 0, s>>>(a, xi);
   return cudaGetLastError();
 }
 

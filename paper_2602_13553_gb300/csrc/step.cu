@@ -56,8 +56,8 @@ __device__ __forceinline__ double warp_max(double v) {
 //  * A O A is one linear map of (q~, v~, eta) per mode (table map6);
 //  * one Philox draw's Box-Muller work is dealt to the three threads of an
 //    (atom, mode): the radius of the x, y pair, its angle, and all of z;
-//  * scalings are exponent additions; the skin test and the FP32 copy of x
-//    come from the integers.
+//  * scalings are exponent additions; the skin test and the force kernel's
+//    wrapped fixed-point positions of the oxygens come from the integers.
 // Threads are component-major (c = threadIdx.x / S, S whole warps), so a warp
 // has one component and its Box-Muller share does not diverge.
 //
@@ -248,9 +248,10 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
     const long long Sj = even ? (pj > H ? X + o : X) : o - X;
     const double xn = from_fixed(Sj, Eq, em);
     a.x[g] = xn;
-    const float sc = sh < -126 ? 0.f : (sh > 127 ? __int_as_float(0x7f800000) : __int_as_float((sh + 127) << 23));
-    if (a.x32) a.x32[g] = Eq > kFixMaxE ? __int_as_float(0x7fc00000) : (float)Sj * sc;
     if (oxy) {
+      const float sc = sh < -126 ? 0.f : (sh > 127 ? __int_as_float(0x7f800000) : __int_as_float((sh + 127) << 23));
+      const double Lc = a.dbox ? a.dbox[c] : a.box[c], iLc = a.dbox ? a.dbox[3 + c] : a.invbox[c];
+      a.xi[((size_t)i + c) * P + k] = fix_wrap(xn, (float)Sj * sc, (float)iLc, fix_pos(Lc));   // row 3 (i / 3) + c
       dev = Eq > kFixMaxE ? __int_as_float(0x7f800000) : (float)(Sj - sC[row]) * sc;
       sD[c * AP + u] = dev;
     }
@@ -369,7 +370,11 @@ __global__ void __launch_bounds__(256) k_step_cart_f64(StepArgs a) {
     }
     a.v[base + task] = v;
     a.x[base + task] = x;
-    if (a.x32) a.x32[base + task] = (float)x;
+    if (a.xi && i % 3 == 0) {
+      const int c = r % 3;
+      const double Lc = a.dbox ? a.dbox[c] : a.box[c], iLc = a.dbox ? a.dbox[3 + c] : a.invbox[c];
+      a.xi[((size_t)i + c) * P + k] = fix_wrap(x, (float)x, (float)iLc, fix_pos(Lc));   // row 3 (i / 3) + c
+    }
     sN[task] = x;
   }
   if (!a.blkmax) return;
@@ -434,11 +439,6 @@ __global__ void __launch_bounds__(256) k_close_cart_f64(StepArgs a) {
       v = fma(c1, v, c2 * __ldg(a.sigv + i) * gauss1(a.seed, (uint32_t)i, (uint32_t)k, kStreamO2, step, d));
     a.v[t] = v;
   }
-}
-
-__global__ void k_to_f32(const double *src, float *dst, size_t n) {
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) dst[t] = (float)src[t];
 }
 
 __global__ void k_advance(int64_t *step, int n) {
@@ -550,11 +550,6 @@ cudaError_t launch_close(const StepArgs &a, int threads, cudaStream_t s) {
     k_step_f64<3, false><<<grid, threads, smem, s>>>(a);
   else
     k_step_f64<3, true><<<grid, threads, smem, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_to_f32(const double *src, float *dst, size_t n, cudaStream_t s) {
-  k_to_f32<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(src, dst, n);
   return cudaGetLastError();
 }
 
