@@ -50,7 +50,7 @@ cudaError_t launch_thermal_v(double *v, const double *sigv, const double *imu, u
 cudaError_t launch_compress_split(const SplitStepArgs &a, const double *x, const double *v, cudaStream_t s);
 cudaError_t launch_expand_split(const SplitStepArgs &a, const float *F, double *x, double *v, double *Fd,
                                 cudaStream_t s);
-cudaError_t launch_centroids(const NbrArgs &a, double *ccur, cudaStream_t s);
+cudaError_t launch_centroids(int nmol, int P, const double *x, double *ccur, cudaStream_t s);
 int water_lane_groups(int P);
 
 constexpr int kTileMax = 3 * 512;   // largest A * 3 * P of a step tile (A P <= 512)
@@ -2810,14 +2810,7 @@ extern "C" pimd_status pimd_batch_add(pimd_batch *b, const pimd_system *sys, int
     }
   }
   if (e == cudaSuccess) e = launch_compress_split(replica_split_args(r), b->stg_x, b->stg_v, b->stream);
-  if (e == cudaSuccess) {
-    NbrArgs na{};
-    std::memset(&na, 0, sizeof(na));
-    na.nmol = r.nmol;
-    na.P = P;
-    na.x = b->stg_x;
-    e = launch_centroids(na, d.ccur, b->stream);
-  }
+  if (e == cudaSuccess) e = launch_centroids(r.nmol, P, b->stg_x, d.ccur, b->stream);
   // initial neighbour list and forces of this replica only
   if (e == cudaSuccess) {
     k_bpos<<<std::min(1024, (r.nmol * 3 * P + 255) / 256), 256, 0, b->stream>>>(b->d_reps, slot);

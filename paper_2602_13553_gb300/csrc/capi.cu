@@ -37,9 +37,10 @@ cudaError_t launch_force_water(const ForceArgs &a, cudaStream_t s);
 cudaError_t launch_fix_positions(const ForceArgs &a, long long *xi, cudaStream_t s);
 cudaError_t force_water_prepare();
 bool water_lists_apart(int nmol, int P);
-cudaError_t launch_nbr_f64(const ForceArgs &a, cudaStream_t s);
-cudaError_t launch_nbr_build(const NbrArgs &a, const double *ccur, cudaStream_t s);
-cudaError_t launch_centroids(const NbrArgs &a, double *ccur, cudaStream_t s);
+cudaError_t launch_nbr_lists(const NbrList &a, bool force, cudaStream_t s);
+cudaError_t launch_centroids(int nmol, int P, const double *x, double *ccur, cudaStream_t s);
+bool split_lists_apart(int nmol, int P);
+cudaError_t split_force_prepare();
 cudaError_t launch_est(const EstArgs &a, int threads, cudaStream_t s);
 cudaError_t launch_est_final(const EstFinalArgs &a, cudaStream_t s);
 int force_blocks(int n_groups, int P);
@@ -372,9 +373,30 @@ static StepArgs step_args(pimd_handle *h) {
   return a;
 }
 
+static NbrList nbr_list(pimd_handle *h) {
+  NbrList a{};
+  a.nmol = h->nmol;
+  a.dbox = h->baro ? h->baro + kBaroL : nullptr;
+  for (int d = 0; d < 3; ++d) {
+    a.box[d] = h->box[d];
+    a.invbox[d] = h->box[d] > 0 ? 1.0 / h->box[d] : 0.0;
+  }
+  a.ccur = h->ccur;
+  a.cref = h->cref;
+  a.blkmax = h->blkmax;
+  // the warp-item split step reports one (drift, spread) pair for the system
+  a.nblk_check = h->split_warp ? 1 : (h->N + h->A_step - 1) / h->A_step;
+  a.skin = h->skin;
+  a.rlist = h->rlist;
+  a.nbr = h->nbr;
+  a.off = h->nbr_off;
+  a.groups = h->nbr_groups;
+  a.err = h->d_err;
+  return a;
+}
+
 static ForceArgs force_args(pimd_handle *h) {
   ForceArgs a{};
-  a.dbox = h->baro ? h->baro + kBaroL : nullptr;
   a.N = h->N;
   a.P = h->P;
   a.nmol = h->nmol;
@@ -387,10 +409,6 @@ static ForceArgs force_args(pimd_handle *h) {
   a.Wpart = h->Wpart;
   a.W3part = h->W3part;
   a.kspring = h->kspring;
-  for (int d = 0; d < 3; ++d) {
-    a.box[d] = h->box[d];
-    a.invbox[d] = h->box[d] > 0 ? 1.0 / h->box[d] : 0.0;
-  }
   a.kb = h->ff[0];
   a.r0 = h->ff[1];
   a.kth = h->ff[2];
@@ -398,42 +416,8 @@ static ForceArgs force_args(pimd_handle *h) {
   a.eps = h->ff[4];
   a.sig = h->ff[5];
   a.rc = h->ff[6];
-  a.nbr = h->nbr;
-  a.nbr_off = h->nbr_off;
-  a.nbr_groups = h->nbr_groups;
+  a.nb = nbr_list(h);
   a.check_nbr = 0;
-  a.blkmax = h->blkmax;
-  // the warp-item split step reports one (drift, spread) pair for the system
-  a.nblk_check = h->split_warp ? 1 : (h->N + h->A_step - 1) / h->A_step;
-  a.skin = h->skin;
-  a.rlist = h->rlist;
-  a.ccur = h->ccur;
-  a.cref = h->cref;
-  a.err = h->d_err;
-  return a;
-}
-
-static NbrArgs nbr_args(pimd_handle *h, bool force) {
-  NbrArgs a;
-  a.nmol = h->nmol;
-  a.P = h->P;
-  a.x = h->x;
-  a.cref = h->cref;
-  a.blkmax = h->blkmax;
-  // the warp-item split step reports one (drift, spread) pair for the system
-  a.nblk_check = h->split_warp ? 1 : (h->N + h->A_step - 1) / h->A_step;
-  a.nbr = h->nbr;
-  a.nbr_off = h->nbr_off;
-  a.nbr_groups = h->nbr_groups;
-  a.err = h->d_err;
-  for (int d = 0; d < 3; ++d) {
-    a.box[d] = h->box[d];
-    a.invbox[d] = 1.0 / h->box[d];
-  }
-  a.dbox = h->baro ? h->baro + kBaroL : nullptr;
-  a.rlist = h->rlist;
-  a.skin = h->skin;
-  a.force = force ? 1 : 0;
   return a;
 }
 
@@ -499,10 +483,6 @@ static SplitForceArgs split_force_args(pimd_handle *h) {
   a.Wpart = h->Wpart;
   a.step_inc = nullptr;
   a.kspring = h->kspring;
-  for (int d = 0; d < 3; ++d) {
-    a.box[d] = f.box[d];
-    a.invbox[d] = f.invbox[d];
-  }
   a.kb = f.kb;
   a.r0 = f.r0;
   a.kth = f.kth;
@@ -510,9 +490,8 @@ static SplitForceArgs split_force_args(pimd_handle *h) {
   a.eps = f.eps;
   a.sig = f.sig;
   a.rc = f.rc;
-  a.nbr = h->nbr;
-  a.nbr_off = h->nbr_off;
-  a.nbr_groups = h->nbr_groups;
+  a.nb = f.nb;
+  a.check_nbr = 0;
   return a;
 }
 
@@ -533,14 +512,16 @@ static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, bool advanc
     if (water) {
       if (from_outside) {
         st = enqueue(h, PIMD_KIND_OTHER, 1, [&] {
-          return launch_centroids(nbr_args(h, true), h->ccur, h->stream);
+          return launch_centroids(h->nmol, h->P, h->x, h->ccur, h->stream);
         });
         if (st != PIMD_OK) return st;
+      } else {
+        sa.check_nbr = 1;   // the skin test and any rebuild: inside the force kernel of a small system
       }
-      st = enqueue(h, PIMD_KIND_NBR, 1, [&] {
-        return launch_nbr_build(nbr_args(h, from_outside), h->ccur, h->stream);
-      });
-      if (st != PIMD_OK) return st;
+      if (from_outside || split_lists_apart(h->nmol, h->P)) {
+        st = enqueue(h, PIMD_KIND_NBR, 1, [&] { return launch_nbr_lists(sa.nb, from_outside, h->stream); });
+        if (st != PIMD_OK) return st;
+      }
     }
     return enqueue(h, PIMD_KIND_FORCE, 1, [&] { return launch_force_split(sa, water, h->stream); });
   }
@@ -552,21 +533,15 @@ static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, bool advanc
       st = enqueue(h, PIMD_KIND_OTHER, 2, [&] {
         cudaError_t e = launch_fix_positions(fa, h->xi, h->stream);
         if (e != cudaSuccess) return e;
-        return launch_centroids(nbr_args(h, true), h->ccur, h->stream);
-      });
-      if (st != PIMD_OK) return st;
-    }
-    if (from_outside) {
-      st = enqueue(h, PIMD_KIND_NBR, 1, [&] {
-        return launch_nbr_build(nbr_args(h, true), h->ccur, h->stream);
+        return launch_centroids(h->nmol, h->P, h->x, h->ccur, h->stream);
       });
       if (st != PIMD_OK) return st;
     } else {
       fa.check_nbr = 1;   // the skin test and any rebuild: inside the force kernel of a small system
-      if (water_lists_apart(h->nmol, h->P)) {
-        st = enqueue(h, PIMD_KIND_NBR, 1, [&] { return launch_nbr_f64(fa, h->stream); });
-        if (st != PIMD_OK) return st;
-      }
+    }
+    if (from_outside || water_lists_apart(h->nmol, h->P)) {
+      st = enqueue(h, PIMD_KIND_NBR, 1, [&] { return launch_nbr_lists(fa.nb, from_outside, h->stream); });
+      if (st != PIMD_OK) return st;
     }
     return enqueue(h, PIMD_KIND_FORCE, 1, [&] { return launch_force_water(fa, h->stream); });
   }
@@ -1091,9 +1066,9 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
   for (int d = 0; d < 3; ++d) h->box[d] = sys->box[d];
   for (int q = 0; q < 8; ++q) h->ff[q] = sys->ff[q];
   h->rlist = h->ff[6] + h->skin;
-  if (h->potential == PIMD_POT_WATERLIKE && h->precision == PIMD_PREC_FP64) {
+  if (h->potential == PIMD_POT_WATERLIKE) {
     h->lj = lj_fix_setup(h->ff[4], h->ff[5], h->ff[6], h->box);
-    const cudaError_t e = force_water_prepare();
+    const cudaError_t e = h->precision == PIMD_PREC_FP64 ? force_water_prepare() : split_force_prepare();
     if (e != cudaSuccess) {
       delete h;
       return fail(PIMD_ECUDA, "force kernel set-up failed: %s", cudaGetErrorString(e));

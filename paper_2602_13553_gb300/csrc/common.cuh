@@ -20,14 +20,9 @@ constexpr double kPi = 3.14159265358979323846;
 
 constexpr int kMaxBeads = 128;
 constexpr int kMaxNeighbours = 192;     // per molecule, O-O list with skin
-// The single-system water force kernels run one cluster of kForceBlocks
-// blocks x 4 warps per (molecule, bead chunk): kLJWarps warps share the
-// molecule's O-O neighbour list, one takes the two bonds, one the angle.
-// (Two blocks per cluster -- one block per SM for a 64-molecule box, six
-// list warps -- measured slower: 25.1 against 21.5 us per FP64 launch.)
-constexpr int kForceBlocks = 4;
-constexpr int kLJWarps = 4 * kForceBlocks - 2;   // warps sharing one molecule's O-O neighbour list
-constexpr int kMaxBuckets = kLJWarps * 8;        // kLJWarps * max lane groups (8)
+// Neighbours are listed in NS = kLJWarps * groups buckets (j mod NS), which the
+// force kernels deal to up to seven warps.
+constexpr int kLJWarps = 14;
 
 // Bits of the device error word (read back at synchronising calls).
 enum : unsigned { kErrNbrOverflow = 1u, kErrNonFinite = 2u, kErrBoxSmall = 4u };
@@ -124,6 +119,18 @@ __device__ __forceinline__ CSum warp_csum(CSum v) {
     CSum w{__shfl_down_sync(0xffffffffu, v.s, o), __shfl_down_sync(0xffffffffu, v.c, o)};
     v.add(w);
   }
+  return v;
+}
+
+// Lanes per row: the smallest power of two >= min(P, 32).
+__host__ __device__ __forceinline__ int row_lanes(int P) {
+  int w = 1;
+  while (w < P && w < 32) w <<= 1;
+  return w;
+}
+
+__device__ __forceinline__ double group_sum(double v, int W) {
+  for (int o = W >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
@@ -260,9 +267,24 @@ struct FixcomArgs {
   const double *sigv;          // [N] sqrt(P kB T / (m mvv2e))
 };
 
+// O-O neighbour lists of a single water-like system (nbr.cuh).
+struct NbrList {
+  int nmol;
+  const double *dbox;          // device box (barostat state at kBaroL), overriding box/invbox, or null
+  double box[3], invbox[3];
+  const double *ccur;          // [nmol][3] current centroids of the oxygens
+  double *cref;                // [nmol][3] centroids at the last build (written on rebuild)
+  const double *blkmax;        // [nblk_check][2] per-block max |c - cref|, max_k |x^k - c|
+  int nblk_check;
+  double skin, rlist;          // rlist = rc + skin
+  int *nbr;                    // [nmol][kMaxNeighbours] neighbours grouped by bucket j mod NS
+  int *off;                    // [nmol][NS + 1] bucket offsets into the molecule's row
+  int groups;                  // NS = kLJWarps * groups buckets
+  unsigned *err;
+};
+
 struct ForceArgs {
   int N, P, nmol;
-  const double *dbox;          // device box (barostat state at kBaroL), overriding box/invbox, or null
   const double *x;             // [N][3][P]
   const int64_t *xi;           // water: [nmol][3][P] wrapped fixed-point positions of the oxygens
   LjFix lj;                    // water: fixed-point pairs
@@ -271,37 +293,11 @@ struct ForceArgs {
   double *Upart, *Wpart;       // [rows][P] bead sums of U and Tr Xi (rows: blocks or molecules)
   double *W3part;              // water: [nmol][P][3] diagonal Xi_aa as well, or null
   const double *kspring;       // harmonic: [N] m mvv2e omega^2
-  double box[3], invbox[3];
   double kb, r0, kth, th0, eps, sig, rc;
-  int *nbr;                    // [nmol][kMaxNeighbours] neighbours grouped by bucket j mod NS
-  int *nbr_off;                // [nmol][NS + 1] bucket offsets into the molecule's row
-  int nbr_groups;              // G: lane groups per warp; NS = kLJWarps * G buckets
-  // check_nbr: the force kernel itself takes the step's rebuild decision
-  // (the skin test of k_nbr_build on the step kernel's per-block maxima) and,
-  // when it rebuilds, lists its molecule's neighbours before the pair loop
+  NbrList nb;
+  // a small system's force blocks take the step's rebuild decision themselves
+  // and list their molecules' neighbours before the pair loop
   int check_nbr;
-  const double *blkmax;        // [nblk_check][2]
-  int nblk_check;
-  double skin, rlist;
-  const double *ccur;          // [nmol][3] current centroids of the oxygens
-  double *cref;                // [nmol][3] centroids at the last build (written on rebuild)
-  unsigned *err;
-};
-
-struct NbrArgs {
-  int nmol, P;
-  const double *x;             // [N][3][P]
-  double *cref;                // [nmol][3] centroids of the oxygens at the last build
-  const double *blkmax;        // [nblk_check][2] per-block max |c - cref|, max_k |x^k - c|
-  int nblk_check;
-  int *nbr, *nbr_off;
-  int nbr_groups;
-  unsigned *err;
-  double box[3], invbox[3];
-  const double *dbox;          // device box (barostat state at kBaroL), overriding box/invbox, or null
-  double rlist;                // rc + skin
-  double skin;
-  int force;                   // rebuild unconditionally
 };
 
 // Split precision (split.cu): FP64 centroid xc, v~_0 [N][3]; FP32 deviations
@@ -337,10 +333,9 @@ struct SplitForceArgs {
   double *Upart, *Wpart;
   int64_t *step_inc;
   const double *kspring;
-  double box[3], invbox[3];
   double kb, r0, kth, th0, eps, sig, rc;
-  const int *nbr, *nbr_off;
-  int nbr_groups;
+  NbrList nb;
+  int check_nbr;               // as ForceArgs::check_nbr
 };
 
 // Columns of an estimator row: K, S, U and Tr Xi per mode or bead, then

@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "nbr.cuh"
 
 namespace pimd {
 
@@ -171,123 +172,13 @@ __device__ __noinline__ void pair_f64(const ForceArgs &a, const double *L, const
   s.W = fma(fr, r2, s.W);
 }
 
-// Number of neighbours of molecule m within rc + skin, listed by bucket (j mod
-// NS) and index, by one warp: FP32 test on the differences of the FP64
-// centroids, in FP64 where it is close.
-__device__ __forceinline__ int list_molecule(const ForceArgs &a, const double (&L)[3], const double (&iL)[3], int m,
-                                             int NS, int *nl, int *off) {
-  const int lane = threadIdx.x & 31;
-  const double c0 = a.ccur[3 * m], c1 = a.ccur[3 * m + 1], c2 = a.ccur[3 * m + 2];
-  const float rl = (float)a.rlist, lo = rl * rl * (1.0f - 1e-5f), hi = rl * rl * (1.0f + 1e-5f);
-  const float Lf[3] = {(float)L[0], (float)L[1], (float)L[2]};
-  const float If[3] = {(float)iL[0], (float)iL[1], (float)iL[2]};
-  auto near = [&](int j) {
-    const double e0 = a.ccur[3 * j] - c0, e1 = a.ccur[3 * j + 1] - c1, e2 = a.ccur[3 * j + 2] - c2;
-    const float f0 = fmaf(-rintf((float)e0 * If[0]), Lf[0], (float)e0);
-    const float f1 = fmaf(-rintf((float)e1 * If[1]), Lf[1], (float)e1);
-    const float f2 = fmaf(-rintf((float)e2 * If[2]), Lf[2], (float)e2);
-    const float r2 = f0 * f0 + f1 * f1 + f2 * f2;
-    // unwrapped differences of many boxes lose FP32 digits: FP64 there too
-    const float far = fmaxf(fmaxf(fabsf((float)e0), fabsf((float)e1)), fabsf((float)e2));
-    if (far < 8.0f * rl) {
-      if (r2 < lo) return true;
-      if (r2 > hi) return false;
-    }
-    const double d0 = mic(e0, L[0], iL[0]), d1 = mic(e1, L[1], iL[1]), d2 = mic(e2, L[2], iL[2]);
-    return d0 * d0 + d1 * d1 + d2 * d2 < a.rlist * a.rlist;
-  };
-  int total = 0;
-  const int n0 = (a.nmol + NS - 1) / NS;   // candidates of bucket 0, the longest
-  int seg = 1;                             // lanes per bucket, 32 / seg buckets a round
-  while (seg < n0 && seg < 32) seg <<= 1;
-  const int sg = lane / seg, tl = lane - sg * seg;
-  for (int b = 0; b < NS; b += 32 / seg) {
-    const int bb = b + sg;
-    for (int t0 = 0; t0 < n0; t0 += seg) {   // more than one round only with a whole warp per bucket
-      const int j = bb + (t0 + tl) * NS;
-      const bool hit = bb < NS && j < a.nmol && j != m && near(j);
-      const unsigned mask = __ballot_sync(0xffffffffu, hit);
-      const int pos = total + __popc(mask & ((1u << lane) - 1u));
-      if (t0 == 0 && tl == 0 && bb < NS) off[bb] = pos;
-      if (hit && pos < kMaxNeighbours) nl[pos] = j;
-      total += __popc(mask);
-    }
-  }
-  if (total > kMaxNeighbours) {   // report, and use an empty list
-    if (lane == 0) atomicOr(a.err, kErrNbrOverflow);
-    __syncwarp();
-    for (int b = lane; b < NS; b += 32) off[b] = 0;
-    total = -1;
-  }
-  if (lane == 0) off[NS] = total < 0 ? 0 : total;
-  __syncwarp();
-  return total;
-}
-
-// This step's rebuild decision from the step kernel's per-block maxima, by all
-// threads of a block.
-__device__ __forceinline__ bool skin_exceeded(const double *blkmax, int n, double skin) {
-  __shared__ double s_mx[2][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  // the maxima are non-negative: they compare as integers, off the FP64 pipe
-  long long md = 0, me = 0;
-  const longlong2 *bm = reinterpret_cast<const longlong2 *>(blkmax);
-#pragma unroll 4
-  for (int b = threadIdx.x; b < n; b += blockDim.x) {
-    const longlong2 e = bm[b];
-    md = max(md, e.x);
-    me = max(me, e.y);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    md = max(md, __shfl_xor_sync(0xffffffffu, md, o));
-    me = max(me, __shfl_xor_sync(0xffffffffu, me, o));
-  }
-  if (lane == 0) {
-    s_mx[0][warp] = __longlong_as_double(md);
-    s_mx[1][warp] = __longlong_as_double(me);
-  }
-  __syncthreads();
-  double d = 0.0, e = 0.0;
-  for (int w = 0; w < nw; ++w) {
-    if (__double_as_longlong(s_mx[0][w]) > __double_as_longlong(d)) d = s_mx[0][w];
-    if (__double_as_longlong(s_mx[1][w]) > __double_as_longlong(e)) e = s_mx[1][w];
-  }
-  return 2.0 * d + 2.0 * e > skin;
-}
-
-__device__ __forceinline__ void force_box(const ForceArgs &a, double (&L)[3], double (&iL)[3]) {
-  const bool db = a.dbox != nullptr;   // the barostat's box: edges, then their inverses
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    L[c] = db ? a.dbox[c] : a.box[c];
-    iL[c] = db ? a.dbox[3 + c] : a.invbox[c];
-  }
-}
-
-// Neighbour lists for the systems whose units go one to a warp: rebuilt here,
-// one warp per molecule, when this step's skin test fails (a small system's
-// blocks rebuild their own molecule's list).
-__global__ void __launch_bounds__(256) k_nbr_f64(ForceArgs a) {
-  if (!skin_exceeded(a.blkmax, a.nblk_check, a.skin)) return;
-  const int NS = kLJWarps * a.nbr_groups, lane = threadIdx.x & 31;
-  double L[3], iL[3];
-  force_box(a, L, iL);
-  for (int m = blockIdx.x * 8 + (threadIdx.x >> 5); m < a.nmol; m += gridDim.x * 8) {
-    const int total = list_molecule(a, L, iL, m, NS, a.nbr + (size_t)m * kMaxNeighbours,
-                                    a.nbr_off + (size_t)m * (NS + 1));
-    if (total >= 0 && lane < 3) a.cref[3 * m + lane] = a.ccur[3 * m + lane];
-  }
-}
-
 template <bool kDiag, bool kFar, bool kSplit>
 __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArgs a, int split) {
   constexpr int NC = kDiag ? 14 : 11;   // F (9), U, Tr Xi, then Xi_xx, Xi_yy, Xi_zz
   extern __shared__ __align__(16) unsigned char fsm[];
   const int P = a.P;
   const int Bk = P < 32 ? P : 32, G = 32 / Bk;
-  const int nchunk = (P + Bk - 1) / Bk;
-  const int NS = kLJWarps * a.nbr_groups;
+  const int NS = kLJWarps * a.nb.groups;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = kSplit ? blockIdx.x : blockIdx.x * 4 + warp;
   const int role = kSplit ? warp : 0;   // 0 .. split - 1: the list; then bonds, angle
@@ -298,7 +189,7 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
   const int m = mg * G + u, k = chunk * Bk + kl;
   const bool on = u < G && m < a.nmol && k < P;   // (a last block's spare warps have k >= P)
   double L[3], iL[3];
-  force_box(a, L, iL);
+  list_box(a.nb, L, iL);
   // a small system's blocks take the step's rebuild decision themselves (the
   // same one from the same maxima) and list their own molecules in shared
   // memory; the block of chunk 0 also keeps the lists and the new centroids
@@ -306,18 +197,14 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
   int *s_off = s_nl + G * kMaxNeighbours;               // [G][NS + 1]
   bool own = false;
   if (kSplit && a.check_nbr) {
-    own = skin_exceeded(a.blkmax, a.nblk_check, a.skin);
+    own = skin_exceeded(a.nb.blkmax, a.nb.nblk_check, a.nb.skin);
     if (own) {
       for (int q = warp; q < G; q += blockDim.x >> 5) {
         const int mm = mg * G + q;
         if (mm >= a.nmol) break;
         int *nl = s_nl + q * kMaxNeighbours, *off = s_off + q * (NS + 1);
-        const int total = list_molecule(a, L, iL, mm, NS, nl, off);
-        if (chunk == 0) {
-          for (int e = lane; e < total; e += 32) a.nbr[(size_t)mm * kMaxNeighbours + e] = nl[e];
-          for (int b = lane; b <= NS; b += 32) a.nbr_off[(size_t)mm * (NS + 1) + b] = off[b];
-          if (lane < 3 && total >= 0) a.cref[3 * mm + lane] = a.ccur[3 * mm + lane];
-        }
+        const int total = list_molecule(a.nb, L, iL, mm, NS, nl, off);
+        if (chunk == 0) keep_list(a.nb, mm, NS, total, nl, off);
       }
       __syncthreads();
     }
@@ -327,8 +214,8 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
   for (int c = 0; c < NC; ++c) acc[c] = 0.0;
   if (on && role < split) {
     // O-O Lennard-Jones: this warp's share of the buckets
-    const int *off = own ? s_off + u * (NS + 1) : a.nbr_off + (size_t)m * (NS + 1);
-    const int *nl = own ? s_nl + u * kMaxNeighbours : a.nbr + (size_t)m * kMaxNeighbours;
+    const int *off = own ? s_off + u * (NS + 1) : a.nb.off + (size_t)m * (NS + 1);
+    const int *nl = own ? s_nl + u * kMaxNeighbours : a.nb.nbr + (size_t)m * kMaxNeighbours;
     int q = off[kSplit ? role * NS / split : 0];
     const int q1 = off[kSplit ? (role + 1) * NS / split : NS];
     const LjFix &lj = a.lj;
@@ -441,100 +328,29 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
   }
 }
 
-// --- O-O neighbour list on ring-polymer centroids ---------------------------
-// A pair (m, j) can interact at some bead only if its centroid distance at
-// the last build was below rc + skin, as long as
-//   2 max_m |c_m - c_m(build)| + 2 max_{m,k} |x_O^k - c_m| <= skin
-// (triangle inequality on the minimum-image metric: a pair's bead distance
-// is at least its build-time centroid distance minus both centroid drifts
-// and both bead deviations).  The step kernel writes per-block maxima of the
-// two terms and the current centroids; this kernel rebuilds when the bound
-// exceeds the skin (or when forced), listing neighbours in index order.
-__global__ void k_nbr_build(NbrArgs a, const double *ccur) {
-  __shared__ double sd[128], se[128];
-  __shared__ int s_go;
-  double md = 0.0, me = 0.0;
-  for (int b = threadIdx.x; b < a.nblk_check; b += blockDim.x) {
-    md = fmax(md, a.blkmax[2 * b]);
-    me = fmax(me, a.blkmax[2 * b + 1]);
+// The lists of a system's molecules, one warp each: on this step's skin test,
+// or (force) always.  Small systems' force blocks do this themselves.
+__global__ void __launch_bounds__(256) k_nbr_lists(NbrList a, int force) {
+  if (!force && !skin_exceeded(a.blkmax, a.nblk_check, a.skin)) return;
+  const int NS = kLJWarps * a.groups, lane = threadIdx.x & 31;
+  double L[3], iL[3];
+  list_box(a, L, iL);
+  for (int m = blockIdx.x * 8 + (threadIdx.x >> 5); m < a.nmol; m += gridDim.x * 8) {
+    const int total = list_molecule(a, L, iL, m, NS, a.nbr + (size_t)m * kMaxNeighbours, a.off + (size_t)m * (NS + 1));
+    if (total >= 0 && lane < 3) a.cref[3 * m + lane] = a.ccur[3 * m + lane];
   }
-  sd[threadIdx.x] = md;
-  se[threadIdx.x] = me;
-  __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) {
-      sd[threadIdx.x] = fmax(sd[threadIdx.x], sd[threadIdx.x + st]);
-      se[threadIdx.x] = fmax(se[threadIdx.x], se[threadIdx.x + st]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) s_go = a.force || (2.0 * sd[0] + 2.0 * se[0] > a.skin);
-  __syncthreads();
-  if (!s_go) return;
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= a.nmol) return;
-  const int NS = kLJWarps * a.nbr_groups;
-  const double c0 = ccur[3 * m], c1 = ccur[3 * m + 1], c2 = ccur[3 * m + 2];
-  const double rl2 = a.rlist * a.rlist;
-  const bool db = a.dbox != nullptr;
-  const double L0 = db ? a.dbox[0] : a.box[0], L1 = db ? a.dbox[1] : a.box[1], L2 = db ? a.dbox[2] : a.box[2];
-  const double i0 = db ? a.dbox[3] : a.invbox[0], i1 = db ? a.dbox[4] : a.invbox[1];
-  const double i2 = db ? a.dbox[5] : a.invbox[2];
-  int cnt[kMaxBuckets];
-  for (int b = 0; b < NS; ++b) cnt[b] = 0;
-  int n = 0;
-  for (int j = 0; j < a.nmol; ++j) {
-    if (j == m) continue;
-    const double d0 = mic(ccur[3 * j] - c0, L0, i0);
-    const double d1 = mic(ccur[3 * j + 1] - c1, L1, i1);
-    const double d2 = mic(ccur[3 * j + 2] - c2, L2, i2);
-    if (d0 * d0 + d1 * d1 + d2 * d2 < rl2) {
-      ++cnt[j % NS];
-      ++n;
-    }
-  }
-  int *off = a.nbr_off + (size_t)m * (NS + 1);
-  if (n > kMaxNeighbours) {
-    // leave an empty list and report: the forces of this step are incomplete
-    atomicOr(a.err, kErrNbrOverflow);
-    for (int b = 0; b <= NS; ++b) off[b] = 0;
-    return;
-  }
-  int acc = 0;
-  for (int b = 0; b < NS; ++b) {
-    off[b] = acc;
-    acc += cnt[b];
-    cnt[b] = 0;
-  }
-  off[NS] = acc;
-  int *nl = a.nbr + (size_t)m * kMaxNeighbours;
-  for (int j = 0; j < a.nmol; ++j) {
-    if (j == m) continue;
-    const double d0 = mic(ccur[3 * j] - c0, L0, i0);
-    const double d1 = mic(ccur[3 * j + 1] - c1, L1, i1);
-    const double d2 = mic(ccur[3 * j + 2] - c2, L2, i2);
-    if (d0 * d0 + d1 * d1 + d2 * d2 < rl2) {
-      const int b = j % NS;
-      nl[off[b] + cnt[b]++] = j;
-    }
-  }
-  a.cref[3 * m] = c0;
-  a.cref[3 * m + 1] = c1;
-  a.cref[3 * m + 2] = c2;
 }
 
 // Centroids of the oxygens from the positions (used when the positions were
-// set from outside the step kernel: create, set_state), and a forced build.
-__global__ void k_centroids(NbrArgs a, double *ccur) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= a.nmol) return;
-  const int P = a.P;
-  const size_t so = (size_t)(3 * m) * 3 * P;
-  for (int d = 0; d < 3; ++d) {
-    double s = 0.0;
-    for (int k = 0; k < P; ++k) s += a.x[so + d * P + k];
-    ccur[3 * m + d] = s / P;
-  }
+// set from outside the step kernel: create, set_state), one lane group a row.
+__global__ void k_centroids(int nmol, int P, const double *x, double *ccur) {
+  const int W = row_lanes(P), l = threadIdx.x % W;
+  const int r = (blockIdx.x * blockDim.x + threadIdx.x) / W;   // row 3 m + d
+  double s = 0.0;
+  if (r < 3 * nmol)
+    for (int k = l; k < P; k += W) s += x[((size_t)9 * (r / 3) + r % 3) * P + k];
+  s = group_sum(s, W);
+  if (r < 3 * nmol && l == 0) ccur[r] = s / P;
 }
 
 // --- host launchers --------------------------------------------------------
@@ -552,15 +368,10 @@ int force_blocks(int n_groups, int P) {
   return (n_groups + per - 1) / per;
 }
 
-int water_force_blocks(int nmol, int P) {   // split precision
-  const int Bk = P < 32 ? P : 32;
-  return kForceBlocks * nmol * ((P + Bk - 1) / Bk);
-}
-
 // Units of work of the FP64 water force, and the warps that share a unit's
 // neighbour list: 1 (a warp takes whole units) once there are enough of them
 // for every SM partition twice over.
-static int water_units(int nmol, int P) {
+int water_units(int nmol, int P) {
   const int Bk = P < 32 ? P : 32, G = 32 / Bk;
   return (nmol + G - 1) / G * ((P + Bk - 1) / Bk);
 }
@@ -587,11 +398,6 @@ cudaError_t launch_force_harmonic(const ForceArgs &a, cudaStream_t s) {
 // Whether the list check is a kernel of its own (the one-warp units).
 bool water_lists_apart(int nmol, int P) { return water_split(nmol, P) == 1; }
 
-cudaError_t launch_nbr_f64(const ForceArgs &a, cudaStream_t s) {
-  k_nbr_f64<<<std::min((a.nmol + 7) / 8, 304), 256, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
 template <bool kDiag, bool kFar>
 static void force_water(const ForceArgs &a, cudaStream_t s) {
   const int split = water_split(a.nmol, a.P), units = water_units(a.nmol, a.P);
@@ -599,7 +405,7 @@ static void force_water(const ForceArgs &a, cudaStream_t s) {
     k_force_water_f64<kDiag, kFar, false><<<(units + 3) / 4, 128, 0, s>>>(a, 1);
     return;
   }
-  const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nbr_groups;
+  const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nb.groups;
   const size_t smem = (size_t)G * kMaxNeighbours * sizeof(int) + (((size_t)G * (NS + 1) + 3) & ~(size_t)3) * sizeof(int) +
                       (size_t)(split + 2) * (kDiag ? 14 : 11) * 32 * sizeof(double);
   k_force_water_f64<kDiag, kFar, true><<<units, 32 * (split + 2), smem, s>>>(a, split);
@@ -635,7 +441,7 @@ __global__ void k_fix_positions(ForceArgs a, long long *xi) {
   if (t >= a.nmol * 3 * a.P) return;
   const int k = t % a.P, mc = t / a.P, c = mc % 3, m = mc / 3;
   double L[3], iL[3];
-  force_box(a, L, iL);
+  list_box(a.nb, L, iL);
   const double x = a.x[(size_t)(9 * m + c) * a.P + k];
   xi[t] = fix_wrap(x, (float)x, (float)iL[c], fix_pos(L[c]));
 }
@@ -646,13 +452,14 @@ cudaError_t launch_fix_positions(const ForceArgs &a, long long *xi, cudaStream_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_nbr_build(const NbrArgs &a, const double *ccur, cudaStream_t s) {
-  k_nbr_build<<<(a.nmol + 127) / 128, 128, 0, s>>>(a, ccur);
+cudaError_t launch_nbr_lists(const NbrList &a, bool force, cudaStream_t s) {
+  k_nbr_lists<<<std::min((a.nmol + 7) / 8, 304), 256, 0, s>>>(a, force ? 1 : 0);
   return cudaGetLastError();
 }
 
-cudaError_t launch_centroids(const NbrArgs &a, double *ccur, cudaStream_t s) {
-  k_centroids<<<(a.nmol + 127) / 128, 128, 0, s>>>(a, ccur);
+cudaError_t launch_centroids(int nmol, int P, const double *x, double *ccur, cudaStream_t s) {
+  const long long threads = (long long)3 * nmol * row_lanes(P);
+  k_centroids<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(nmol, P, x, ccur);
   return cudaGetLastError();
 }
 

@@ -13,11 +13,8 @@
 // HBM per bead-atom and step: step kernel reads F, d, v~ (36 B) and writes
 // d, v~ (24 B), plus 96 B per atom for xc, v~_0; force kernel reads d (12 B)
 // and writes F (12 B).
-#include <cooperative_groups.h>
-
 #include "common.cuh"
-
-namespace cg = cooperative_groups;
+#include "nbr.cuh"
 
 namespace pimd {
 
@@ -369,170 +366,213 @@ __global__ void __launch_bounds__(256) k_force_harmonic_split(SplitForceArgs a) 
 
 __device__ __forceinline__ float micf(float d, float L, float invL) { return fmaf(-rintf(d * invL), L, d); }
 
-// Water-like model in FP32, same decomposition as the FP64 kernel: a
-// kForceBlocks-block cluster per (molecule, bead chunk), warps 0 ..
-// kLJWarps - 1 own buckets of the O-O neighbour list, warp kLJWarps the
-// bonds, warp kLJWarps + 1 the angle; partials are
-// reduced through distributed shared memory in rank order.  A pair vector is
-// the minimum-image difference of the wrapped FP32 centroids plus the
-// difference of the FP32 deviations.
-__global__ void __cluster_dims__(kForceBlocks, 1, 1) __launch_bounds__(128) k_force_water_split(SplitForceArgs a) {
-  __shared__ float sacc[9][128];
-  __shared__ double saccd[2][128];
-  __shared__ float red[9][32];
-  __shared__ double redd[2][32];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
+// Water-like model in FP32.  Work as in the FP64 kernel: a unit is one molecule
+// and a chunk of Bk = min(P, 32) beads (G = 32 / Bk molecules where the beads
+// leave lanes free), beads in adjacent lanes.  Many units: one warp each, four
+// to a block; otherwise a block per unit, whose list `split` warps share and one
+// more takes the bonds and the angle.  A pair vector is the minimum-image
+// difference of the wrapped FP32 centroids plus the difference of the FP32
+// deviations.  Candidates go two at a time on packed FP32 (each element rounds
+// as a scalar would), eight to a partial sum.
+//
+// What bounds it is the latency of the gathers: the rows of the next two
+// candidates are requested before the arithmetic of these.  A four-block cluster
+// per unit (whose fixed cost this replaces) with a list check of its own took
+// 38.5 + 3 us a step at 512 molecules x 64 beads, 10.8 + 8.4 us at 216 x 20.
+template <bool kSplit>
+__global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitForceArgs a, int split) {
+  extern __shared__ __align__(16) unsigned char fsm[];
   const int P = a.P;
-  const int Bk = P < 32 ? P : 32;
-  const int G = a.nbr_groups;
-  const int NS = kLJWarps * G;
-  const int nchunk = (P + Bk - 1) / Bk;
-  const int cid = blockIdx.x / kForceBlocks;
-  const int m = cid / nchunk, chunk = cid % nchunk;
+  const int Bk = P < 32 ? P : 32, G = 32 / Bk;
+  const int NS = kLJWarps * a.nb.groups;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int s = rank * 4 + warp;
-  const int u = lane / Bk, kl = lane % Bk;
-  const int k = chunk * Bk + kl;
-  float acc[9];
+  const int unit = kSplit ? blockIdx.x : blockIdx.x * 4 + warp;
+  const int role = kSplit ? warp : 0;   // 0 .. split - 1: the list; then bonds and angle
+  const int nmg = (a.nmol + G - 1) / G;
+  const int chunk = unit / nmg, mg = unit - chunk * nmg;
+  const int u = lane / Bk, kl = lane - u * Bk;
+  const int m = mg * G + u, k = chunk * Bk + kl;
+  const bool on = u < G && m < a.nmol && k < P;   // (a last block's spare warps have k >= P)
+  int *s_nl = reinterpret_cast<int *>(fsm);             // [G][kMaxNeighbours]
+  int *s_off = s_nl + G * kMaxNeighbours;               // [G][NS + 1]
+  bool own = false;
+  if (kSplit && a.check_nbr) {
+    own = skin_exceeded(a.nb.blkmax, a.nb.nblk_check, a.nb.skin);
+    if (own) {
+      double L[3], iL[3];
+      list_box(a.nb, L, iL);
+      for (int q = warp; q < G; q += blockDim.x >> 5) {
+        const int mm = mg * G + q;
+        if (mm >= a.nmol) break;
+        int *nl = s_nl + q * kMaxNeighbours, *off = s_off + q * (NS + 1);
+        const int total = list_molecule(a.nb, L, iL, mm, NS, nl, off);
+        if (chunk == 0) keep_list(a.nb, mm, NS, total, nl, off);
+      }
+      __syncthreads();
+    }
+  }
+  float F[9];
 #pragma unroll
-  for (int c = 0; c < 9; ++c) acc[c] = 0.f;
+  for (int c = 0; c < 9; ++c) F[c] = 0.f;
   double ue = 0.0, we = 0.0;
-  if (u < G && k < P && m < a.nmol) {
-    const int o = 3 * m;
-    const float L0 = (float)a.box[0], L1 = (float)a.box[1], L2 = (float)a.box[2];
-    const float i0 = (float)a.invbox[0], i1 = (float)a.invbox[1], i2 = (float)a.invbox[2];
-    const size_t so = (size_t)o * 3 * P + k;
-    const float co0 = a.xcw[3 * o], co1 = a.xcw[3 * o + 1], co2 = a.xcw[3 * o + 2];
-    const float do0 = a.d[so], do1 = a.d[so + P], do2 = a.d[so + 2 * P];
-    if (s >= kLJWarps) {
-      if (u == 0) {
-        float dv[2][3], r[2], ir[2];
+  const float L[3] = {(float)a.nb.box[0], (float)a.nb.box[1], (float)a.nb.box[2]};
+  const float iL[3] = {(float)a.nb.invbox[0], (float)a.nb.invbox[1], (float)a.nb.invbox[2]};
+  float co[3] = {0.f, 0.f, 0.f}, dO[3] = {0.f, 0.f, 0.f};
+  if (on) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int hh = o + 1 + h;
-          const size_t sh = (size_t)hh * 3 * P + k;
-          dv[h][0] = micf(a.xcw[3 * hh] - co0, L0, i0) + (a.d[sh] - do0);
-          dv[h][1] = micf(a.xcw[3 * hh + 1] - co1, L1, i1) + (a.d[sh + P] - do1);
-          dv[h][2] = micf(a.xcw[3 * hh + 2] - co2, L2, i2) + (a.d[sh + 2 * P] - do2);
-          r[h] = sqrtf(dv[h][0] * dv[h][0] + dv[h][1] * dv[h][1] + dv[h][2] * dv[h][2]);
-          ir[h] = 1.f / r[h];
-        }
-        float uu = 0.f, w = 0.f;
-        if (s == kLJWarps) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float dr = r[h] - (float)a.r0;
-            uu = fmaf(0.5f * (float)a.kb * dr, dr, uu);
-            const float g = -(float)a.kb * dr * ir[h];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const float fc = g * dv[h][c];
-              acc[3 + 3 * h + c] = fc;
-              acc[c] -= fc;
-              w = fmaf(dv[h][c], fc, w);
-            }
-          }
-        } else {
-          const float ir01 = ir[0] * ir[1];
-          const float dot = dv[0][0] * dv[1][0] + dv[0][1] * dv[1][1] + dv[0][2] * dv[1][2];
-          const float cth = fminf(1.f, fmaxf(-1.f, dot * ir01));
-          const float th = acosf(cth);
-          const float dth = th - (float)a.th0;
-          const float pref = (float)a.kth * dth / sinf(th);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int g = 1 - h;
-            const float ch = cth * ir[h] * ir[h];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const float fa = pref * fmaf(dv[g][c], ir01, -ch * dv[h][c]);
-              acc[3 + 3 * h + c] = fa;
-              acc[c] -= fa;
-              w = fmaf(dv[h][c], fa, w);
-            }
-          }
-          uu = 0.5f * (float)a.kth * dth * dth;
-        }
-        ue = uu;
-        we = w;
-      }
-    } else {
-      const int b = s * G + u;
-      const int *off = a.nbr_off + (size_t)m * (NS + 1);
-      const int q0 = __ldg(off + b), q1 = __ldg(off + b + 1);
-      const int *nl = a.nbr + (size_t)m * kMaxNeighbours;
-      const float rc2 = (float)(a.rc * a.rc);
-      const float sig2 = (float)(a.sig * a.sig);
-      const float e4 = (float)(4.0 * a.eps), e24 = (float)(24.0 * a.eps);
-      float f0 = 0.f, f1 = 0.f, f2 = 0.f, ulj = 0.f, wlj = 0.f;
-      for (int q = q0; q < q1; ++q) {
-        const int j = __ldg(nl + q);
-        const size_t sj = (size_t)(3 * j) * 3 * P + k;
-        const float d0 = micf(__ldg(a.xcw + 9 * j) - co0, L0, i0) + (__ldg(a.d + sj) - do0);
-        const float d1 = micf(__ldg(a.xcw + 9 * j + 1) - co1, L1, i1) + (__ldg(a.d + sj + P) - do1);
-        const float d2 = micf(__ldg(a.xcw + 9 * j + 2) - co2, L2, i2) + (__ldg(a.d + sj + 2 * P) - do2);
-        const float r2 = d0 * d0 + d1 * d1 + d2 * d2;
-        if (r2 < rc2) {
-          const float inv = 1.f / r2;
-          const float s2 = sig2 * inv;
-          const float s6 = s2 * s2 * s2;
-          ulj = fmaf(e4, fmaf(s6, s6, -s6), ulj);
-          const float fr = e24 * fmaf(2.f * s6, s6, -s6) * inv;
-          f0 = fmaf(-fr, d0, f0);
-          f1 = fmaf(-fr, d1, f1);
-          f2 = fmaf(-fr, d2, f2);
-          wlj = fmaf(fr, r2, wlj);
-        }
-      }
-      acc[0] = f0;
-      acc[1] = f1;
-      acc[2] = f2;
-      ue = 0.5 * (double)ulj;
-      we = 0.5 * (double)wlj;
+    for (int c = 0; c < 3; ++c) {
+      co[c] = a.xcw[9 * m + c];
+      dO[c] = a.d[(size_t)(9 * m + c) * P + k];
     }
   }
+  if (on && role < split) {
+    const int *off = own ? s_off + u * (NS + 1) : a.nb.off + (size_t)m * (NS + 1);
+    const int *nl = own ? s_nl + u * kMaxNeighbours : a.nb.nbr + (size_t)m * kMaxNeighbours;
+    int q = off[kSplit ? role * NS / split : 0];
+    const int q1 = off[kSplit ? (role + 1) * NS / split : NS];
+    const float rc2 = (float)(a.rc * a.rc);
+    const float2 sig2 = make_float2((float)(a.sig * a.sig), (float)(a.sig * a.sig));
+    const float e4 = (float)(4.0 * a.eps), e24 = (float)(24.0 * a.eps);
+    const float2 e4v = make_float2(e4, e4), ne4 = make_float2(-e4, -e4);
+    const float2 e48 = make_float2(2.f * e24, 2.f * e24), ne24 = make_float2(-e24, -e24);
+    const float2 zero = make_float2(0.f, 0.f);
+    struct Cand { float c[2][3], d[2][3]; };
+    auto load = [&](int j0, int j1, Cand &v) {
 #pragma unroll
-  for (int c = 0; c < 9; ++c) sacc[c][threadIdx.x] = acc[c];
-  saccd[0][threadIdx.x] = ue;
-  saccd[1][threadIdx.x] = we;
-  __syncthreads();
-  for (int t = threadIdx.x; t < 11 * Bk; t += blockDim.x) {
-    const int comp = t / Bk, kk = t % Bk;
-    if (comp < 9) {
-      float sum = 0.f;
-      for (int w = 0; w < 4; ++w)
-        for (int g = 0; g < G; ++g) sum += sacc[comp][w * 32 + g * Bk + kk];
-      red[comp][kk] = sum;
-    } else {
-      double sum = 0.0;
-      for (int w = 0; w < 4; ++w)
-        for (int g = 0; g < G; ++g) sum += saccd[comp - 9][w * 32 + g * Bk + kk];
-      redd[comp - 9][kk] = sum;
+      for (int c = 0; c < 3; ++c) {
+        v.c[0][c] = __ldg(a.xcw + 9 * j0 + c);
+        v.c[1][c] = __ldg(a.xcw + 9 * j1 + c);
+        v.d[0][c] = __ldg(a.d + (size_t)(9 * j0 + c) * P + k);
+        v.d[1][c] = __ldg(a.d + (size_t)(9 * j1 + c) * P + k);
+      }
+    };
+    Cand cur, nxt;
+    // a list's odd end pairs its last candidate with itself, masked
+    if (q < q1) load(nl[q], nl[min(q + 1, q1 - 1)], cur);
+    float2 S[5] = {zero, zero, zero, zero, zero};   // F on this molecule (3), U, W
+    while (q < q1) {
+      float2 s[5] = {zero, zero, zero, zero, zero};
+#pragma unroll 1
+      for (int t = 0; t < 4 && q < q1; ++t, q += 2) {
+        if (q + 2 < q1) load(nl[q + 2], nl[min(q + 3, q1 - 1)], nxt);
+        float2 d[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          float2 e = make_float2(cur.c[0][c] - co[c], cur.c[1][c] - co[c]);
+          const float2 n = make_float2(-rintf(e.x * iL[c]), -rintf(e.y * iL[c]));
+          e = __ffma2_rn(n, make_float2(L[c], L[c]), e);
+          d[c] = __fadd2_rn(e, make_float2(cur.d[0][c] - dO[c], cur.d[1][c] - dO[c]));
+        }
+        const float2 r2 = __ffma2_rn(d[2], d[2], __ffma2_rn(d[1], d[1], __fmul2_rn(d[0], d[0])));
+        const bool i0 = r2.x < rc2, i1 = r2.y < rc2 && q + 1 < q1;
+        if (i0 || i1) {
+          // a candidate outside the cutoff gets 1 / r^2 = 0: it adds exact zeros
+          const float2 inv = make_float2(i0 ? __frcp_rn(r2.x) : 0.f, i1 ? __frcp_rn(r2.y) : 0.f);
+          const float2 s2 = __fmul2_rn(sig2, inv);
+          const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
+          s[3] = __ffma2_rn(s6, __ffma2_rn(e4v, s6, ne4), s[3]);
+          const float2 fr = __fmul2_rn(__fmul2_rn(__ffma2_rn(e48, s6, ne24), s6), inv);
+          const float2 nf = make_float2(-fr.x, -fr.y);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) s[c] = __ffma2_rn(nf, d[c], s[c]);
+          if (i0) s[4].x = fmaf(fr.x, r2.x, s[4].x);
+          if (i1) s[4].y = fmaf(fr.y, r2.y, s[4].y);
+        }
+        cur = nxt;
+      }
+#pragma unroll
+      for (int c = 0; c < 5; ++c) S[c] = __fadd2_rn(S[c], s[c]);
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) F[c] = S[c].x + S[c].y;
+    ue = 0.5 * (double)(S[3].x + S[3].y);
+    we = 0.5 * (double)(S[4].x + S[4].y);
   }
-  cluster.sync();
-  if (rank == 0 && m < a.nmol) {
-    for (int t = threadIdx.x; t < 11 * Bk; t += blockDim.x) {
-      const int comp = t / Bk, kk = t % Bk;
-      const int k2 = chunk * Bk + kk;
-      if (k2 >= P) continue;
-      if (comp < 9) {
-        float sum = 0.f;
-        for (int r = 0; r < kForceBlocks; ++r) sum += cluster.map_shared_rank(&red[0][0], r)[comp * 32 + kk];
-        a.F[(size_t)(3 * m + comp / 3) * 3 * P + (comp % 3) * P + k2] = sum;
-      } else {
-        double sum = 0.0;
-        for (int r = 0; r < kForceBlocks; ++r) sum += cluster.map_shared_rank(&redd[0][0], r)[(comp - 9) * 32 + kk];
-        if (comp == 9)
-          a.Upart[(size_t)m * P + k2] = sum;
-        else
-          a.Wpart[(size_t)m * P + k2] = sum;
+  if (on && (!kSplit || role == split)) {
+    float dv[2][3], r[2], ir[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int row = 9 * m + 3 * (1 + h) + c;
+        dv[h][c] = micf(a.xcw[row] - co[c], L[c], iL[c]) + (a.d[(size_t)row * P + k] - dO[c]);
+      }
+      r[h] = sqrtf(dv[h][0] * dv[h][0] + dv[h][1] * dv[h][1] + dv[h][2] * dv[h][2]);
+      ir[h] = 1.f / r[h];
+    }
+    // bonds
+    float uu = 0.f, w = 0.f, fO[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float dr = r[h] - (float)a.r0;
+      uu = fmaf(0.5f * (float)a.kb * dr, dr, uu);
+      const float g = -(float)a.kb * dr * ir[h];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float fc = g * dv[h][c];
+        F[3 + 3 * h + c] = fc;
+        fO[c] -= fc;
+        w = fmaf(dv[h][c], fc, w);
       }
     }
-    if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
+    ue += (double)uu;
+    we += (double)w;
+    // angle
+    const float ir01 = ir[0] * ir[1];
+    const float dot = dv[0][0] * dv[1][0] + dv[0][1] * dv[1][1] + dv[0][2] * dv[1][2];
+    const float cth = fminf(1.f, fmaxf(-1.f, dot * ir01));
+    const float th = acosf(cth);
+    const float dth = th - (float)a.th0;
+    const float pref = (float)a.kth * dth / sinf(th);
+    w = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int g = 1 - h;
+      const float ch = cth * ir[h] * ir[h];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float fa = pref * fmaf(dv[g][c], ir01, -ch * dv[h][c]);
+        F[3 + 3 * h + c] += fa;
+        fO[c] -= fa;
+        w = fmaf(dv[h][c], fa, w);
+      }
+    }
+    ue += (double)(0.5f * (float)a.kth * dth * dth);
+    we += (double)w;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) F[c] += fO[c];
   }
-  cluster.sync();
+  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
+  if (kSplit) {
+    // partial sums of the warps, joined in order by the last warp
+    float *sF = reinterpret_cast<float *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [split][3][32]
+    double *sU = reinterpret_cast<double *>(sF + split * 96);                   // [split][2][32]
+    if (role < split) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) sF[(role * 3 + c) * 32 + lane] = F[c];
+      sU[(role * 2) * 32 + lane] = ue;
+      sU[(role * 2 + 1) * 32 + lane] = we;
+    }
+    __syncthreads();
+    if (role < split) return;
+    float sum[3] = {0.f, 0.f, 0.f};
+    double su = 0.0, sw = 0.0;
+    for (int w = 0; w < split; ++w) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) sum[c] += sF[(w * 3 + c) * 32 + lane];
+      su += sU[(w * 2) * 32 + lane];
+      sw += sU[(w * 2 + 1) * 32 + lane];
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) F[c] += sum[c];
+    ue += su;
+    we += sw;
+  }
+  if (!on) return;
+#pragma unroll
+  for (int c = 0; c < 9; ++c) a.F[(size_t)(9 * m + c) * P + k] = F[c];
+  a.Upart[(size_t)m * P + k] = ue;
+  a.Wpart[(size_t)m * P + k] = we;
 }
 
 // --- conversions between the split state and FP64 [N][3][P] arrays ----------
@@ -549,22 +589,33 @@ __global__ void k_expand_split(SplitStepArgs a, const float *F, double *x, doubl
   if (Fd) Fd[t] = (double)F[t];
 }
 
-// xc = bead average, d = x - xc, v~_0 and v~_k from FP64 [N][3][P] arrays
-__global__ void k_compress_split(SplitStepArgs a, const double *x, const double *v) {
-  const size_t ic = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (ic >= (size_t)a.N * 3) return;
-  const int P = a.P;
+// xc = bead average, d = x - xc, v~_0 and v~_k from FP64 [N][3][P] arrays; one
+// lane group a row (at most four beads a lane).
+__global__ void __launch_bounds__(128) k_compress_split(SplitStepArgs a, const double *x, const double *v) {
+  const int P = a.P, W = row_lanes(P), l = threadIdx.x % W;
+  const size_t ic = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
+  const bool on = ic < (size_t)a.N * 3;
+  double xv[4], s = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int k = l + q * W;
+    xv[q] = on && k < P ? x[ic * P + k] : 0.0;
+    s += xv[q];
+  }
+  const double xc = group_sum(s, W) / P;
+  if (!on) return;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int k = l + q * W;
+    if (k >= P) continue;
+    a.d[ic * P + k] = (float)(xv[q] - xc);
+    a.vk[ic * P + k] = k == 0 ? 0.f : (float)v[ic * P + k];
+  }
+  if (l) return;
   const int c = (int)(ic % 3);
-  double s = 0.0;
-  for (int k = 0; k < P; ++k) s += x[ic * P + k];
-  const double xc = s / P;
   a.xc[ic] = xc;
   a.v0[ic] = v[ic * P];
   if (a.xcw) a.xcw[ic] = wrapf(xc, a.box[c], a.invbox[c]);
-  for (int k = 0; k < P; ++k) {
-    a.d[ic * P + k] = (float)(x[ic * P + k] - xc);
-    a.vk[ic * P + k] = k == 0 ? 0.f : (float)v[ic * P + k];
-  }
 }
 
 // --- host launchers ----------------------------------------------------------
@@ -592,12 +643,34 @@ cudaError_t launch_close_split(const SplitStepArgs &a, int threads, cudaStream_t
 
 int force_blocks(int n_groups, int P);
 int force_block_threads(int P);
-int water_force_blocks(int nmol, int P);
+int water_units(int nmol, int P);
+
+// Warps that share a unit's neighbour list (1: a warp takes whole units).
+static int split_water_warps(int nmol, int P) {
+  const int n = water_units(nmol, P);
+  return n >= 4096 ? 1 : (n >= 2048 ? 2 : (n >= 512 ? 4 : 7));   // NS is a multiple of 14
+}
+
+// Whether the list check is a kernel of its own (the one-warp units).
+bool split_lists_apart(int nmol, int P) { return split_water_warps(nmol, P) == 1; }
+
+cudaError_t split_force_prepare() {   // a one-bead system's lists take more than 48 KB
+  return cudaFuncSetAttribute(k_force_water_split<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+}
 
 cudaError_t launch_force_split(const SplitForceArgs &a, bool water, cudaStream_t s) {
-  if (water)
-    k_force_water_split<<<water_force_blocks(a.nmol, a.P), 128, 0, s>>>(a);
-  else
+  if (water) {
+    const int split = split_water_warps(a.nmol, a.P), units = water_units(a.nmol, a.P);
+    if (split == 1) {
+      k_force_water_split<false><<<(units + 3) / 4, 128, 0, s>>>(a, 1);
+    } else {
+      const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nb.groups;
+      const size_t smem = (size_t)G * kMaxNeighbours * sizeof(int) +
+                          (((size_t)G * (NS + 1) + 3) & ~(size_t)3) * sizeof(int) +
+                          (size_t)split * 32 * (3 * sizeof(float) + 2 * sizeof(double));
+      k_force_water_split<true><<<units, 32 * (split + 1), smem, s>>>(a, split);
+    }
+  } else
     k_force_harmonic_split<<<force_blocks(a.N, a.P), force_block_threads(a.P), 0, s>>>(a);
   return cudaGetLastError();
 }
@@ -611,7 +684,7 @@ cudaError_t launch_expand_split(const SplitStepArgs &a, const float *F, double *
 
 cudaError_t launch_compress_split(const SplitStepArgs &a, const double *x, const double *v,
                                   cudaStream_t s) {
-  const size_t n = (size_t)a.N * 3;
+  const size_t n = (size_t)a.N * 3 * row_lanes(a.P);
   k_compress_split<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(a, x, v);
   return cudaGetLastError();
 }

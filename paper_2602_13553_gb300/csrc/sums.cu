@@ -22,18 +22,6 @@ namespace pimd {
 
 constexpr int kSumThreads = 256;
 
-// Lanes per row: the smallest power of two >= min(P, 32).
-__host__ __device__ __forceinline__ int row_lanes(int P) {
-  int w = 1;
-  while (w < P && w < 32) w <<= 1;
-  return w;
-}
-
-__device__ __forceinline__ double group_sum(double v, int W) {
-  for (int o = W >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 __device__ __forceinline__ double warp_sum(double v) { return group_sum(v, 32); }
 
 // True in every thread of the block that finishes last; the others' partial
