@@ -96,6 +96,7 @@ struct RepDesc {
   float *pO;                  // [nmol][3][P] oxygen bead positions xcw + d (FP32), for the pair loop
   const double *inv_mm, *sigv, *mass_mm;
   const float *inv_mmf, *sigvf;   // FP32 copies for the FP32 mode updates
+  const float *ksf;               // harmonic well (single systems): [N] m mvv2e omega^2, F is not read
   const float *Mf, *Mtf, *cAf, *sAf, *wsAf, *c1f, *c2f;
   const double *Mt64, *lam;
   // tensor-core path (P % 8 == 0): M (forward) and M^T (inverse) as TF32
@@ -431,6 +432,7 @@ constexpr int kWAtoms = 8;      // atoms per warp item
 constexpr int kWWarps = 4;      // warps per block
 constexpr int kWMaxP = 64;
 __host__ __device__ constexpr int wslot_floats(int P) { return 48 * (P + 4) + 128; }
+__host__ __device__ constexpr int wslot_floats_harm(int P) { return 24 * (P + 4) + 128; }   // no forces
 __host__ __device__ constexpr bool warp_class(int P) { return P == 8 || P == 16 || P == 32 || P == 64; }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
@@ -507,7 +509,9 @@ __device__ __forceinline__ void fwd_tile(const float4 *__restrict__ thi, const f
 // and deviations (the latter reused as q~' [c][mode][atom]), row stride P + 4
 // (conflict-free B fragments); then F~_0, the centroid-mode noise of both
 // streams per (atom, component) and the new FP64 centroids.
-template <int P>
+// kHarm (single systems in a harmonic well): F~ = -k q~, so no forces are read,
+// staged or transformed.
+template <int P, bool kHarm = false>
 __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__restrict__ slot, uint64_t step,
                            int first) {
   constexpr int PS = P + 4, MT = (P + 15) / 16, KS = P / 8;
@@ -516,8 +520,8 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
   const int na = min(kWAtoms, Rp->N - tile0);
   const size_t base = (size_t)tile0 * 3 * P;
   float *sF = slot;
-  float *sX = slot + 24 * PS;
-  float *__restrict__ sf0 = slot + 48 * PS;
+  float *sX = slot + (kHarm ? 0 : 24 * PS);
+  float *__restrict__ sf0 = sX + 24 * PS;
   float *__restrict__ se = sf0 + 24;
   float *__restrict__ se2 = se + 24;
   double *__restrict__ sxc = reinterpret_cast<double *>(se2 + 24);
@@ -530,14 +534,14 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
       const int row = q / CPR, col = (q - row * CPR) * 4;
       const int a = row / 3, c = row - 3 * a;
       const int so = (c * 8 + a) * PS + col;
-      cp_async16(sF + so, gF + (size_t)row * P + col);
+      if (!kHarm) cp_async16(sF + so, gF + (size_t)row * P + col);
       cp_async16(sX + so, gX + (size_t)row * P + col);
     }
     cp_async_commit();
     for (int q = lane; q < (kWAtoms - na) * 3 * P; q += 32) {   // rows of missing atoms
       const int r = q / P, j = q - r * P;
       const int a = na + r / 3, c = r - 3 * (r / 3);
-      sF[(c * 8 + a) * PS + j] = 0.f;
+      if (!kHarm) sF[(c * 8 + a) * PS + j] = 0.f;
       sX[(c * 8 + a) * PS + j] = 0.f;
     }
   }
@@ -553,10 +557,11 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
   const float *__restrict__ c2f = Rp->c2f;
   float *__restrict__ vkg = Rp->vk + base;
   // per-lane atom constants (atoms 2t, 2t + 1) and the centroid prefetch
-  float imv[2], sgv[2];
+  float imv[2], sgv[2], ksv[2];
 #pragma unroll
   for (int aa = 0; aa < 2; ++aa) {
     const int a = min(2 * t + aa, na - 1);
+    ksv[aa] = kHarm ? __ldg(Rp->ksf + tile0 + a) : 0.f;
     imv[aa] = __ldg(Rp->inv_mmf + tile0 + a);
     sgv[aa] = __ldg(Rp->sigvf + tile0 + a);
   }
@@ -594,9 +599,10 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
     }
   // forward transform of the forces: F~_c = M F_c, then F~ [c][mode][atom]
   // over the staged forces
+  float *sG = sF;
+  if (!kHarm) {
   fwd_tile<P>(fhi, flo, sF, C);
   __syncwarp();   // every lane is done with the staged forces
-  float *sG = sF;
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
@@ -606,6 +612,7 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
       if (k + 8 < P)
         *reinterpret_cast<float2 *>(sG + (c * P + k + 8) * 8 + 2 * t) = make_float2(C[mt][c][2], C[mt][c][3]);
     }
+  }
   // mode update: lane (g, t) owns modes {16 mt + g, 16 mt + g + 8} of atoms
   // {2t, 2t + 1}, the same (mode, atom) slots it wrote; q~' replaces q~
   load_v(0, vv);
@@ -632,7 +639,8 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       qv[c] = *reinterpret_cast<const float2 *>(sQ + (c * P + k) * 8 + 2 * t);
-      fv[c] = *reinterpret_cast<const float2 *>(sG + (c * P + k) * 8 + 2 * t);
+      fv[c] = kHarm ? make_float2(-ksv[0] * qv[c].x, -ksv[1] * qv[c].y)
+                    : *reinterpret_cast<const float2 *>(sG + (c * P + k) * 8 + 2 * t);
     }
 #pragma unroll
     for (int aa = 0; aa < 2; ++aa) {
@@ -705,7 +713,8 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
     const double dr = Rp->dr0, c1_0 = Rp->c1_0;
     const float kbf = (integ == 0 ? kick : half) * __ldg(Rp->inv_mmf + i);
     const float c2sf = __ldg(c2f) * __ldg(Rp->sigvf + i);
-    const float f0 = sf0[lane];
+    // q~_0 = sqrt(P) xc
+    const float f0 = kHarm ? -__ldg(Rp->ksf + i) * (float)(sqrt((double)P) * xpre) : sf0[lane];
     const float e = se[lane], e2 = se2[lane];
     double x = xpre, v = vpre;
     if (integ == 0) {
@@ -883,7 +892,7 @@ __global__ void __launch_bounds__(kWWarps * 32, 1) k_bstep_w128(const RepDesc *_
 // block's share of registers), 3 the 8- and 16-bead one (one mode tile, six
 // blocks: its short items leave the memory waits exposed unless more warps
 // share an SM; 8 and 16 beads step 15% and 10% faster than at four blocks).
-template <int kClass>
+template <int kClass, bool kHarm>
 __global__ void __launch_bounds__(kWWarps * 32, kClass == 3 ? 6 : (kClass == 0 ? 4 : (kClass == 1 ? 3 : 1)))
     k_sstep_w(const RepDesc *__restrict__ Rp, const int64_t *__restrict__ stepp, int step_off, int first,
               int slot_floats, double *blkmax, unsigned *done) {
@@ -896,15 +905,15 @@ __global__ void __launch_bounds__(kWWarps * 32, kClass == 3 ? 6 : (kClass == 0 ?
   for (int tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; tile < ntiles; tile += nw) {
     if (kClass == 3) {
       if (Rp->P == 8)
-        bstep_warp<8>(Rp, tile, slot, step, first);
+        bstep_warp<8, kHarm>(Rp, tile, slot, step, first);
       else if (Rp->P == 16)
-        bstep_warp<16>(Rp, tile, slot, step, first);
+        bstep_warp<16, kHarm>(Rp, tile, slot, step, first);
     } else if (kClass == 2) {
-      if (Rp->P == 128) bstep_warp<128>(Rp, tile, slot, step, first);
+      if (Rp->P == 128) bstep_warp<128, kHarm>(Rp, tile, slot, step, first);
     } else if (kClass == 1) {
-      if (Rp->P == 64) bstep_warp<64>(Rp, tile, slot, step, first);
+      if (Rp->P == 64) bstep_warp<64, kHarm>(Rp, tile, slot, step, first);
     } else if (Rp->P == 32) {
-      bstep_warp<32>(Rp, tile, slot, step, first);
+      bstep_warp<32, kHarm>(Rp, tile, slot, step, first);
     }
   }
   if (!blkmax) return;
@@ -2342,14 +2351,17 @@ cudaError_t split_warp_prepare() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void *)k_sstep_w<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute((const void *)k_sstep_w<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kWWarps * wslot_floats(32) * sizeof(float)));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void *)k_sstep_w<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute((const void *)k_sstep_w<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kWWarps * wslot_floats(64) * sizeof(float)));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void *)k_sstep_w<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute((const void *)k_sstep_w<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kWWarps * wslot_floats(128) * sizeof(float)));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute((const void *)k_sstep_w<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kWWarps * wslot_floats_harm(128) * sizeof(float)));
   if (e == cudaSuccess) g_sw_nsm = nsm > 0 ? nsm : 152;
   return e;
 }
@@ -2389,6 +2401,7 @@ cudaError_t split_warp_setup(const SplitWarpSetup &w, cudaStream_t st) {
   d.sigv = w.sigv;
   d.inv_mmf = w.inv_mmf;
   d.sigvf = w.sigvf;
+  d.ksf = w.ksf;
   d.cAf = w.cAf;
   d.sAf = w.sAf;
   d.wsAf = w.wsAf;
@@ -2408,10 +2421,11 @@ cudaError_t split_warp_setup(const SplitWarpSetup &w, cudaStream_t st) {
   std::vector<float> fh, fl, ih, il;
   fragment_tables(M, P, fh, fl);
   fragment_tables(Mt, P, ih, il);
-  std::vector<float> imf(N), sgf(N);
+  std::vector<float> imf(N), sgf(N), ksf(w.ksf ? N : 0);
   for (int i = 0; i < N; ++i) {
     imf[i] = (float)w.inv_mm_host[i];
     sgf[i] = (float)w.sigv_host[i];
+    if (w.ksf) ksf[i] = (float)w.kspring_host[i];
   }
   long long ctl[kCtlWords] = {0};
   const struct {
@@ -2426,9 +2440,11 @@ cudaError_t split_warp_setup(const SplitWarpSetup &w, cudaStream_t st) {
       {w.frag + 3 * one, il.data(), one * sizeof(float4)},
       {w.inv_mmf, imf.data(), N * sizeof(float)},
       {w.sigvf, sgf.data(), N * sizeof(float)},
+      {w.ksf, ksf.data(), ksf.size() * sizeof(float)},
       {w.ctl, ctl, sizeof(ctl)},
   };
   for (const auto &u : ups) {
+    if (!u.bytes) continue;
     // pageable sources: the copy completes before the call returns
     const cudaError_t e = cudaMemcpyAsync(u.dst, u.src, u.bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
@@ -2439,12 +2455,12 @@ cudaError_t split_warp_setup(const SplitWarpSetup &w, cudaStream_t st) {
 }
 
 cudaError_t launch_step_split_warp(const void *desc, int N, int P, const int64_t *step, int step_off, int first,
-                                   double *blkmax, unsigned *done, cudaStream_t s) {
+                                   double *blkmax, unsigned *done, bool harm, cudaStream_t s) {
   const cudaError_t pe = split_warp_prepare();
   if (pe != cudaSuccess) return pe;
   const int nsm = g_sw_nsm;
   const int cls = P == 128 ? 2 : (P == 64 ? 1 : (P == 32 ? 0 : 3));
-  const int slot = wslot_floats(P);
+  const int slot = harm ? wslot_floats_harm(P) : wslot_floats(P);
   // resident blocks per SM (registers, shared memory)
   const int per_sm = cls == 2 ? 2 : (cls == 1 ? 3 : (cls == 0 ? 4 : 6));
   const int smem = (int)(kWWarps * slot * sizeof(float));
@@ -2452,14 +2468,13 @@ cudaError_t launch_step_split_warp(const void *desc, int N, int P, const int64_t
   const int warps = std::min(ntiles, nsm * per_sm * kWWarps);
   const int grid = std::max(1, (warps + kWWarps - 1) / kWWarps);
   const RepDesc *d = reinterpret_cast<const RepDesc *>(desc);
-  if (cls == 3)
-    k_sstep_w<3><<<grid, kWWarps * 32, smem, s>>>(d, step, step_off, first, slot, blkmax, done);
-  else if (cls == 2)
-    k_sstep_w<2><<<grid, kWWarps * 32, smem, s>>>(d, step, step_off, first, slot, blkmax, done);
-  else if (cls == 1)
-    k_sstep_w<1><<<grid, kWWarps * 32, smem, s>>>(d, step, step_off, first, slot, blkmax, done);
-  else
-    k_sstep_w<0><<<grid, kWWarps * 32, smem, s>>>(d, step, step_off, first, slot, blkmax, done);
+  auto go = [&](auto kernel) { kernel<<<grid, kWWarps * 32, smem, s>>>(d, step, step_off, first, slot, blkmax, done); };
+  switch (cls) {
+    case 0: harm ? go(k_sstep_w<0, true>) : go(k_sstep_w<0, false>); break;
+    case 1: harm ? go(k_sstep_w<1, true>) : go(k_sstep_w<1, false>); break;
+    case 2: harm ? go(k_sstep_w<2, true>) : go(k_sstep_w<2, false>); break;
+    default: harm ? go(k_sstep_w<3, true>) : go(k_sstep_w<3, false>); break;
+  }
   return cudaGetLastError();
 }
 

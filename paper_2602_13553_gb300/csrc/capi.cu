@@ -161,6 +161,9 @@ struct pimd_handle {
   double ff[8] = {0};
   cudaStream_t stream = nullptr;
   bool own_stream = false;
+  // harmonic wells: the step forms F~ = -k q~ itself, so the force kernel runs
+  // (and the step counter advances) once a call, not once a step
+  bool fused_well = false;
   DevAllocator alloc;
   void *arena = nullptr;
   size_t arena_bytes = 0;
@@ -181,7 +184,7 @@ struct pimd_handle {
   bool split_warp = false;
   char *sw_desc = nullptr;
   float4 *sw_frag = nullptr;
-  float *sw_imf = nullptr, *sw_sgf = nullptr;
+  float *sw_imf = nullptr, *sw_sgf = nullptr, *sw_ksf = nullptr;
   long long *sw_ctl = nullptr;
   unsigned *sw_done = nullptr;
   double *inv_mm = nullptr, *sigv = nullptr, *mass_mm = nullptr, *kspring = nullptr;
@@ -346,6 +349,7 @@ static StepArgs step_args(pimd_handle *h) {
   a.x = h->x;
   a.v = h->v;
   a.F = h->F;
+  a.kspring = h->fused_well ? h->kspring : nullptr;
   a.method = h->method;
   a.ifmass = 1.0 / h->fmass;
   a.wn2 = h->wn * h->wn;
@@ -449,6 +453,7 @@ static SplitStepArgs split_args(pimd_handle *h) {
   a.d = h->dev;
   a.vk = h->vk;
   a.F = h->F32;
+  a.kspring = h->fused_well ? h->kspring : nullptr;
   const bool water = h->potential == PIMD_POT_WATERLIKE;
   a.xcw = water ? h->xcw : nullptr;
   for (int d = 0; d < 3; ++d) {
@@ -503,11 +508,13 @@ static pimd_status expand_split(pimd_handle *h, bool with_forces) {
   });
 }
 
-static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, bool advance) {
+// advance: steps by which the force kernel also advances the counter.
+static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, int advance) {
   if (h->precision == PIMD_PREC_SPLIT) {
     const bool water = h->potential == PIMD_POT_WATERLIKE;
     SplitForceArgs sa = split_force_args(h);
     sa.step_inc = advance ? h->d_step : nullptr;
+    sa.inc = advance;
     pimd_status st;
     if (water) {
       if (from_outside) {
@@ -527,6 +534,7 @@ static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, bool advanc
   }
   ForceArgs fa = force_args(h);
   fa.step_inc = advance ? h->d_step : nullptr;
+  fa.inc = advance;
   if (h->potential == PIMD_POT_WATERLIKE) {
     pimd_status st;
     if (from_outside) {
@@ -591,26 +599,29 @@ static pimd_status enqueue_baro(pimd_handle *h, double t0, double tB, bool step_
 }
 
 // One full step: the fused integrator kernel, the forces of the new
-// positions, and the step counter.
-static pimd_status enqueue_step(pimd_handle *h, bool first) {
+// positions, and the step counter; in a harmonic well (fused_well) the
+// integrator alone, off steps after the counter.
+static pimd_status enqueue_step(pimd_handle *h, bool first, int off = 0) {
   if (h->precision == PIMD_PREC_SPLIT) {
     pimd_status st;
     if (h->split_warp) {
       const bool water = h->potential == PIMD_POT_WATERLIKE;
       st = enqueue(h, PIMD_KIND_STEP, 1, [&] {
-        return launch_step_split_warp(h->sw_desc, h->N, h->P, h->d_step, 0, first ? 1 : 0,
-                                      water ? h->blkmax : nullptr, h->sw_done, h->stream);
+        return launch_step_split_warp(h->sw_desc, h->N, h->P, h->d_step, off, first ? 1 : 0,
+                                      water ? h->blkmax : nullptr, h->sw_done, h->fused_well, h->stream);
       });
     } else {
       SplitStepArgs a = split_args(h);
+      a.step_off = off;
       a.first = first ? 1 : 0;
       a.kick = first ? 0.5 * h->dt : h->dt;
       st = enqueue(h, PIMD_KIND_STEP, 1, [&] { return launch_step_split(a, h->threads_step, h->stream); });
     }
-    if (st != PIMD_OK) return st;
-    return enqueue_forces(h, false, true);
+    if (st != PIMD_OK || h->fused_well) return st;
+    return enqueue_forces(h, false, 1);
   }
   StepArgs a = step_args(h);
+  a.step_off = off;
   a.first = first ? 1 : 0;
   a.kick = first ? 0.5 * h->dt : h->dt;
   // BAOAB merges the closing B(h/2) of the previous step into its kick
@@ -639,7 +650,8 @@ static pimd_status enqueue_step(pimd_handle *h, bool first) {
     st = enqueue(h, PIMD_KIND_STEP, 1, [&] { return launch_step(a, h->threads_step, h->stream); });
     if (st != PIMD_OK) return st;
   }
-  st = enqueue_forces(h, false, true);
+  if (h->fused_well) return PIMD_OK;
+  st = enqueue_forces(h, false, 1);
   if (st != PIMD_OK) return st;
   // the B_W beside this step's closing B(h/2) (applied by the next kernel)
   if (h->baro && (st = enqueue_baro(h, 0.0, 0.5 * h->dt, false, false)) != PIMD_OK) return st;
@@ -677,9 +689,14 @@ static pimd_status enqueue_close(pimd_handle *h) {
     return enqueue(h, PIMD_KIND_CLOSE, 1, [&] { return launch_close_split(a, h->threads_step, h->stream); });
   }
   StepArgs a = step_args(h);
-  a.step_off = -1;
+  a.step_off = h->method == PIMD_METHOD_PIMD ? -1 : 0;   // the normal-mode kernel counts back itself
   a.fix_u = h->fixcom ? h->fix_u : nullptr;
   return enqueue(h, PIMD_KIND_CLOSE, 1, [&] { return launch_close(a, h->threads_step, h->stream); });
+}
+
+// Advance the device step counter.
+static pimd_status enqueue_advance(pimd_handle *h, int n) {
+  return enqueue(h, PIMD_KIND_OTHER, 1, [&] { return launch_advance(h->d_step, n, h->stream); });
 }
 
 static pimd_status build_graph(pimd_handle *h, int nsteps) {
@@ -688,7 +705,8 @@ static pimd_status build_graph(pimd_handle *h, int nsteps) {
   h->capturing = true;
   const int64_t before = h->launches;
   pimd_status st = PIMD_OK;
-  for (int s = 0; s < nsteps && st == PIMD_OK; ++s) st = enqueue_step(h, false);
+  for (int s = 0; s < nsteps && st == PIMD_OK; ++s) st = enqueue_step(h, false, h->fused_well ? s : 0);
+  if (h->fused_well && st == PIMD_OK) st = enqueue_advance(h, nsteps);
   h->capturing = false;
   h->graph_kernels = h->launches - before;
   h->launches = before;
@@ -830,6 +848,7 @@ static void carve(pimd_handle *h, Carver &c) {
       h->sw_frag = c.take<float4>(split_warp_frag_float4(P));
       h->sw_imf = c.take<float>(N);
       h->sw_sgf = c.take<float>(N);
+      if (h->fused_well) h->sw_ksf = c.take<float>(N);
       h->sw_ctl = c.take<long long>(8);
       h->sw_done = c.take<unsigned>(1);
     }
@@ -1084,6 +1103,7 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
     }
     h->own_stream = true;
   }
+  h->fused_well = h->potential == PIMD_POT_HARMONIC && h->method == PIMD_METHOD_NMPIMD && !h->fixcom;
   if (prm.precision == PIMD_PREC_FP64 && prm.method == PIMD_METHOD_NMPIMD) {
     h->A_step = step_tile_atoms(N, P);
     h->threads_step = step_threads(h->A_step, P);
@@ -1214,6 +1234,8 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
       w.M_host = M.data();
       w.inv_mm_host = inv_mm.data();
       w.sigv_host = sigv.data();
+      w.kspring_host = ksp.data();
+      w.ksf = h->sw_ksf;
       w.desc = h->sw_desc;
       w.frag = h->sw_frag;
       w.inv_mmf = h->sw_imf;
@@ -1244,7 +1266,7 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
     }
     pimd_status s2 = upload_state(h, sys->pos, sys->vel);
     if (s2 != PIMD_OK) return s2;
-    s2 = enqueue_forces(h, true, false);
+    s2 = enqueue_forces(h, true, 0);
     if (s2 != PIMD_OK) return s2;
     return check_device_errors(h);
   };
@@ -1264,6 +1286,7 @@ extern "C" pimd_status pimd_step(pimd_handle *h, int64_t n) {
   pimd_status st = enqueue_step(h, true);
   if (st != PIMD_OK) return st;
   int64_t left = n - 1;
+  int off = 1;   // fused_well: steps enqueued since the counter last advanced
   // steps per graph replay (8: 31.1, 32: 30.8 us per MD step on 64 x 32 water)
   const int G = 32;
   if (h->use_graph && !h->timing && left >= G) {
@@ -1271,6 +1294,8 @@ extern "C" pimd_status pimd_step(pimd_handle *h, int64_t n) {
       st = build_graph(h, G);
       if (st != PIMD_OK) return st;
     }
+    if (h->fused_well && (st = enqueue_advance(h, off)) != PIMD_OK) return st;
+    off = 0;
     while (left >= h->graph_steps) {
       CK(cudaGraphLaunch(h->graph, h->stream));
       h->launches += h->graph_kernels;
@@ -1278,9 +1303,14 @@ extern "C" pimd_status pimd_step(pimd_handle *h, int64_t n) {
     }
   }
   for (; left > 0; --left) {
-    st = enqueue_step(h, false);
+    st = enqueue_step(h, false, h->fused_well ? off++ : 0);
     if (st != PIMD_OK) return st;
+    if (h->fused_well && off == (1 << 20)) {
+      if ((st = enqueue_advance(h, off)) != PIMD_OK) return st;
+      off = 0;
+    }
   }
+  if (h->fused_well && (st = enqueue_forces(h, false, off)) != PIMD_OK) return st;
   st = enqueue_close(h);
   if (st != PIMD_OK) return st;
   h->step += n;
@@ -1426,7 +1456,7 @@ extern "C" pimd_status pimd_set_barostat(pimd_handle *h, const double *vW, const
     h->h_baro[kBaroInvL + c] = 1.0 / box[c];
   }
   CK(cudaMemcpyAsync(h->baro, h->h_baro, sizeof(h->h_baro), cudaMemcpyHostToDevice, h->stream));
-  pimd_status st = enqueue_forces(h, true, false);
+  pimd_status st = enqueue_forces(h, true, 0);
   if (st != PIMD_OK) return st;
   return check_device_errors(h);
 }
@@ -1460,7 +1490,7 @@ extern "C" pimd_status pimd_set_state(pimd_handle *h, const double *x, const dou
   if (st != PIMD_OK) return st;
   h->step = step;
   CK(cudaMemcpyAsync(h->d_step, &h->step, sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
-  st = enqueue_forces(h, true, false);
+  st = enqueue_forces(h, true, 0);
   if (st != PIMD_OK) return st;
   return check_device_errors(h);
 }

@@ -179,6 +179,7 @@ struct StepArgs {
   double *x;                   // [N][3][P] Cartesian positions
   double *v;                   // [N][3][P] normal-mode velocities
   const double *F;             // [N][3][P] Cartesian forces
+  const double *kspring;       // normal modes in a harmonic well: [N] m mvv2e omega^2, F is not read; or null
   const int64_t *step;         // device step counter (step index of this step = *step + step_off)
   int step_off;
   long long *xi;               // water: [nmol][3][P] wrapped fixed-point positions of the oxygens, or null
@@ -288,7 +289,8 @@ struct ForceArgs {
   const double *x;             // [N][3][P]
   const int64_t *xi;           // water: [nmol][3][P] wrapped fixed-point positions of the oxygens
   LjFix lj;                    // water: fixed-point pairs
-  int64_t *step_inc;           // if not null, block 0 advances the step counter by one
+  int64_t *step_inc;           // if not null, block 0 advances the step counter by inc
+  int inc;
   double *F;                   // [N][3][P]
   double *Upart, *Wpart;       // [rows][P] bead sums of U and Tr Xi (rows: blocks or molecules)
   double *W3part;              // water: [nmol][P][3] diagonal Xi_aa as well, or null
@@ -312,6 +314,7 @@ struct SplitStepArgs {
   double *xc, *v0;             // [N][3]
   float *d, *vk;               // [N][3][P]
   const float *F;              // [N][3][P]
+  const double *kspring;       // harmonic well: [N] m mvv2e omega^2, F is not read; or null
   float *xcw;                  // [N][3] centroids wrapped into the box, FP32 (water), or null
   double box[3], invbox[3];
   const int64_t *step;
@@ -331,7 +334,8 @@ struct SplitForceArgs {
   const float *d;              // [N][3][P]
   float *F;                    // [N][3][P]
   double *Upart, *Wpart;
-  int64_t *step_inc;
+  int64_t *step_inc;           // if not null, block 0 advances the step counter by inc
+  int inc;
   const double *kspring;
   double kb, r0, kth, th0, eps, sig, rc;
   NbrList nb;

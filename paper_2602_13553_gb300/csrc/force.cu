@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(256) k_force_harmonic_f64(ForceArgs a) {
   }
   const int groups = min(per, a.N - blockIdx.x * per);
   block_bead_sums(u, w, P, groups, a.Upart, a.Wpart);
-  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
+  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += a.inc;
 }
 
 // Water-like model, FP64.  A unit of work is one molecule and a chunk of
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
     else
       a.W3part[((size_t)mm * P + kk) * 3 + (comp - 11)] = v;
   };
-  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
+  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += a.inc;
   if (!kSplit) {
     if (on)
 #pragma unroll

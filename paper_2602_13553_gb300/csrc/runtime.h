@@ -56,10 +56,10 @@ struct SplitWarpSetup {
   const double *inv_mm, *sigv;                  // device [N]
   const float *cAf, *sAf, *wsAf, *c1f, *c2f;    // device [P]
   double *cref, *ccur;                          // water-like: skin test, else null
-  const double *M_host, *inv_mm_host, *sigv_host;
+  const double *M_host, *inv_mm_host, *sigv_host, *kspring_host;
   void *desc;
   float4 *frag;
-  float *inv_mmf, *sigvf;
+  float *inv_mmf, *sigvf, *ksf;                 // ksf: harmonic well, else null
   long long *ctl;
   unsigned *done;
 };
@@ -68,7 +68,7 @@ size_t split_warp_frag_float4(int P);
 bool split_warp_class(int P);
 cudaError_t split_warp_setup(const SplitWarpSetup &w, cudaStream_t st);
 cudaError_t launch_step_split_warp(const void *desc, int N, int P, const int64_t *step, int step_off, int first,
-                                   double *blkmax, unsigned *done, cudaStream_t s);
+                                   double *blkmax, unsigned *done, bool harm, cudaStream_t s);
 
 pimd_status fail(pimd_status s, const char *fmt, ...);
 void set_last_error(const char *msg);

@@ -99,13 +99,15 @@ __global__ void __launch_bounds__(256) k_step_split(SplitStepArgs a) {
   // the forward transforms then sum one half of a row (rows of M are even
   // for modes k <= H = P/2, odd above), as in the FP64 step kernel
   const int H = P >> 1;
+  // a harmonic well's F~_k is -k q~_k: neither read nor transformed
+  const bool harm = a.kspring != nullptr;
   for (int t = threadIdx.x; t < len; t += blockDim.x) {
     const int j = t % P, pj = j == 0 ? 0 : P - j;
     const size_t g = base + t, gp = g - j + pj;
-    const float da = a.d[g], fa = a.F[g];
+    const float da = a.d[g], fa = harm ? 0.f : a.F[g];
     float du = da, fu = fa;
     if (pj != j) {
-      const float db = a.d[gp], fb = a.F[gp];
+      const float db = a.d[gp], fb = harm ? 0.f : a.F[gp];
       du = j < pj ? da + db : db - da;
       fu = j < pj ? fa + fb : fb - fa;
     }
@@ -141,24 +143,32 @@ __global__ void __launch_bounds__(256) k_step_split(SplitStepArgs a) {
     const float *tf = Tf + k;
     float fa = 0.f, fb = 0.f, qa = 0.f, qb = 0.f;
     int j = 0;
-    for (; j + 1 < n; j += 2) {
-      const float m0 = __ldg(tf + j * P), m1 = __ldg(tf + (j + 1) * P);
-      fa = fmaf(m0, fx[j], fa);
-      fb = fmaf(m1, fx[j + 1], fb);
-      qa = fmaf(m0, xx[j], qa);
-      qb = fmaf(m1, xx[j + 1], qb);
+    if (harm) {
+      for (; j + 1 < n; j += 2) {
+        qa = fmaf(__ldg(tf + j * P), xx[j], qa);
+        qb = fmaf(__ldg(tf + (j + 1) * P), xx[j + 1], qb);
+      }
+      if (j < n) qa = fmaf(__ldg(tf + j * P), xx[j], qa);
+    } else {
+      for (; j + 1 < n; j += 2) {
+        const float m0 = __ldg(tf + j * P), m1 = __ldg(tf + (j + 1) * P);
+        fa = fmaf(m0, fx[j], fa);
+        fb = fmaf(m1, fx[j + 1], fb);
+        qa = fmaf(m0, xx[j], qa);
+        qb = fmaf(m1, xx[j + 1], qb);
+      }
+      if (j < n) {
+        const float m0 = __ldg(tf + j * P);
+        fa = fmaf(m0, fx[j], fa);
+        qa = fmaf(m0, xx[j], qa);
+      }
     }
-    if (j < n) {
-      const float m0 = __ldg(tf + j * P);
-      fa = fmaf(m0, fx[j], fa);
-      qa = fmaf(m0, xx[j], qa);
-    }
-    const float f = fa + fb;
+    float q = qa + qb;
+    const float f = harm ? -(float)__ldg(a.kspring + i) * q : fa + fb;
     if (k == 0) {
       sQ[task] = f;      // F~_0, consumed by the centroid task below
       continue;
     }
-    float q = qa + qb;
     float v = sV[task];
     const float im = (float)__ldg(a.inv_mm + i);
     const float cA = __ldg(a.cAf + k), sA = __ldg(a.sAf + k), wsA = __ldg(a.wsAf + k);
@@ -188,9 +198,9 @@ __global__ void __launch_bounds__(256) k_step_split(SplitStepArgs a) {
     const int al = t / 3, c = t % 3;
     const int i = tile0 + al;
     const size_t ic = (size_t)i * 3 + c;
-    const double f0 = (double)sQ[t * P];
     double x = a.xc[ic], v = a.v0[ic];
     const double im = __ldg(a.inv_mm + i);
+    const double f0 = harm ? -__ldg(a.kspring + i) * x / rsp : (double)sQ[t * P];   // q~_0 = sqrt(P) xc
     const double dr = a.tA * rsp;
     if (a.integrator == 0) {
       v = fma(a.kick * im, f0, v);
@@ -361,7 +371,7 @@ __global__ void __launch_bounds__(256) k_force_harmonic_split(SplitForceArgs a) 
     a.Upart[(size_t)blockIdx.x * P + kk] = su;
     a.Wpart[(size_t)blockIdx.x * P + kk] = sw;
   }
-  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
+  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += a.inc;
 }
 
 __device__ __forceinline__ float micf(float d, float L, float invL) { return fmaf(-rintf(d * invL), L, d); }
@@ -542,7 +552,7 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
 #pragma unroll
     for (int c = 0; c < 3; ++c) F[c] += fO[c];
   }
-  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
+  if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += a.inc;
   if (kSplit) {
     // partial sums of the warps, joined in order by the last warp
     float *sF = reinterpret_cast<float *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [split][3][32]

@@ -61,14 +61,18 @@ __device__ __forceinline__ double warp_max(double v) {
 // Threads are component-major (c = threadIdx.x / S, S whole warps), so a warp
 // has one component and its Box-Muller share does not diverge.
 //
+// In a harmonic well (kHarm) F = -k x, so F~ = -k q~ and the forces are neither
+// read nor transformed; the force kernel runs once, after a call's last step.
+//
 // kPhase 0: the whole step.  1, 2: a step in two launches around the barostat's
 // OBABO kick (velocities only; then B(h/2), A(h) and the positions).  3: the
 // closing B(h/2) (OBABO: and O(h/2)) of a call's last step.
 //
 // Measured (GB300, per launch): see k_step_f64's rows in the design table.
-template <int kPhase, bool kObabo>
+template <int kPhase, bool kObabo, bool kHarm>
 __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
   constexpr bool kX = kPhase == 0 || kPhase == 2;   // positions move
+  constexpr bool kQ = kX || kHarm;                  // q~ is formed
   extern __shared__ __align__(16) unsigned char smraw[];
   const int P = a.P, H = P >> 1, A = a.A, AP = A * P, np = fix_pairs(P), rs = 4 * np;
   const int S = blockDim.x / 3;
@@ -89,15 +93,15 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
   int *sE = reinterpret_cast<int *>(sCs + 2 * AP);            // [3][3A] largest exponents of x, F, q~
   float *sD = reinterpret_cast<float *>(sE + 9 * A);          // [3][AP] bead deviations
   __shared__ float sred[2][12];
-  const bool needF = kPhase != 1 || !a.first;
+  const bool needF = !kHarm && (kPhase != 1 || !a.first);
   double x = 0.0, f = 0.0, v = 0.0;
   if (on) {
-    if (kX) x = a.x[g];
+    if (kQ) x = a.x[g];
     if (needF) f = a.F[g];
     v = a.v[g];
   }
   for (int t = threadIdx.x; t < 9 * A; t += blockDim.x) sE[t] = kFixMinE;
-  const uint64_t step = (uint64_t)*a.step;
+  const uint64_t step = (uint64_t)(*a.step + a.step_off);
   // the noise does not wait for the loads above: stream O1 of this step, O2 of
   // the previous one
   const bool d1 = a.thermo && (kPhase == 0 || kPhase == 1);
@@ -123,7 +127,7 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
   if (on && d2) draw(1, kStreamO2, step - 1);
   __syncthreads();
   if (on) {
-    if (kX) atomicMax(sE + row, exp_field(x));
+    if (kQ) atomicMax(sE + row, exp_field(x));
     if (needF) atomicMax(sE + 3 * A + row, exp_field(f));
     if (c < 2) {   // e_x = r cos, e_y = r sin
 #pragma unroll
@@ -140,12 +144,12 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
   const int half_row = row * (rs >> 1) + (even ? 0 : np);        // the terms of mode (bead) k
   long long X = 0, F = 0;
   if (on) {
-    if (kX) rX[c * AP + u] = X = to_fixed(x, Ex);
+    if (kQ) rX[c * AP + u] = X = to_fixed(x, Ex);
     if (needF) rF[c * AP + u] = F = to_fixed(f, Ef);
   }
   __syncthreads();
   if (on) {
-    if (kX) {
+    if (kQ) {
       const long long o = pj != k ? rX[c * AP + u - k + pj] : 0;
       reinterpret_cast<int2 *>(uX)[fold] = fix_limbs(even ? X + o : o - X);
     }
@@ -160,7 +164,11 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
   double q = 0.0;
   if (on) {
     FixSum sx, sf;
-    if (kX && needF) {
+    if (kHarm) {
+#pragma unroll 3
+      for (int p = 0; p < np; ++p) sx.add2(uX[half_row + p], __ldg(tf + p * P));
+      q = from_fixed(sx.value(), Ex, em);
+    } else if (kX && needF) {
 #pragma unroll 3
       for (int p = 0; p < np; ++p) {
         const int4 m = __ldg(tf + p * P);
@@ -172,7 +180,7 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
 #pragma unroll 3
       for (int p = 0; p < np; ++p) sf.add2(uF[half_row + p], __ldg(tf + p * P));
     }
-    f = needF ? from_fixed(sf.value(), Ef, em) : 0.0;
+    f = kHarm ? -__ldg(a.kspring + i) * q : (needF ? from_fixed(sf.value(), Ef, em) : 0.0);
     if (!a.mu_one) f *= __ldg(a.mt.imu + k);   // 1 / m^(k) = imu_k / (m mvv2e)
     if (k == 0 && a.fix_u) v -= a.fix_u[c];    // the previous step's fixcom
     const double km = __ldg(a.kmm + i);        // this kick's time / (m mvv2e)
@@ -527,14 +535,18 @@ cudaError_t launch_step(const StepArgs &a0, int threads, cudaStream_t s) {
     return cudaGetLastError();
   }
   const size_t smem = step_smem_bytes(a.A, a.P);
-  if (a.integrator == 0)
-    k_step_f64<0, false><<<grid, threads, smem, s>>>(a);
+  if (a.kspring && a.integrator == 0)
+    k_step_f64<0, false, true><<<grid, threads, smem, s>>>(a);
+  else if (a.kspring)
+    k_step_f64<0, true, true><<<grid, threads, smem, s>>>(a);
+  else if (a.integrator == 0)
+    k_step_f64<0, false, false><<<grid, threads, smem, s>>>(a);
   else if (a.phase == 1)
-    k_step_f64<1, true><<<grid, threads, smem, s>>>(a);
+    k_step_f64<1, true, false><<<grid, threads, smem, s>>>(a);
   else if (a.phase == 2)
-    k_step_f64<2, true><<<grid, threads, smem, s>>>(a);
+    k_step_f64<2, true, false><<<grid, threads, smem, s>>>(a);
   else
-    k_step_f64<0, true><<<grid, threads, smem, s>>>(a);
+    k_step_f64<0, true, false><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -546,10 +558,14 @@ cudaError_t launch_close(const StepArgs &a, int threads, cudaStream_t s) {
   }
   const int grid = (a.N + a.A - 1) / a.A;
   const size_t smem = step_smem_bytes(a.A, a.P);
-  if (a.integrator == 0)
-    k_step_f64<3, false><<<grid, threads, smem, s>>>(a);
+  if (a.kspring && a.integrator == 0)
+    k_step_f64<3, false, true><<<grid, threads, smem, s>>>(a);
+  else if (a.kspring)
+    k_step_f64<3, true, true><<<grid, threads, smem, s>>>(a);
+  else if (a.integrator == 0)
+    k_step_f64<3, false, false><<<grid, threads, smem, s>>>(a);
   else
-    k_step_f64<3, true><<<grid, threads, smem, s>>>(a);
+    k_step_f64<3, true, false><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
