@@ -151,6 +151,7 @@ struct pimd_handle {
   // fixcom and barostat: partial sums, the mean velocity that the next kernel
   // subtracts ([P][3]), the total mass (m mvv2e)
   double *sums_part = nullptr, *fix_u = nullptr;
+  double *baro_mm = nullptr;   // barostat: [2][N] centroid masses m^(0) mvv2e and their inverses
   double msum = 0;
   double *W3part = nullptr;   // anisotropic barostat: [nmol][P][3] diagonal virial rows
   double T = 0, dt = 0, tau = 0, scale = 0, sp = 0, fmass = 1.0, pext = 0, taup = 0;
@@ -572,7 +573,9 @@ static pimd_status enqueue_baro(pimd_handle *h, double t0, double tB, bool step_
   b.v = h->v;
   b.F = h->F;
   b.Mt = h->Mt;
-  b.mass_mm = h->mass_mm;
+  b.mass_mm = h->baro_mm;
+  b.inv_mm = h->baro_mm + h->N;
+  b.invP = 1.0 / h->P;
   b.Wpart = h->Wpart;
   b.W3part = h->W3part;
   b.axes = h->baro_axes;
@@ -587,7 +590,6 @@ static pimd_status enqueue_baro(pimd_handle *h, double t0, double tB, bool step_
   b.k3 = tB * tB * tB / (3.0 * W);
   b.nkT = h->P * kT;
   b.npext = h->P * h->pext;
-  b.mu0 = h->fmass;
   b.thermo = h->thermostat == PIMD_THERMO_PILE_L;
   b.c1W = std::exp(-(b.obabo ? 0.5 * h->dt : h->dt) / h->tau);   // the O_W's own duration
   b.sigW = std::sqrt(1.0 - b.c1W * b.c1W) * std::sqrt(b.nkT / W);
@@ -667,7 +669,8 @@ static pimd_status enqueue_step(pimd_handle *h, bool first, int off = 0) {
   f.F = h->F;
   f.v = h->v;
   f.u = h->fix_u;
-  f.msum = h->msum;
+  f.imsum = 1.0 / h->msum;
+  f.rsp = 1.0 / std::sqrt((double)h->P);
   f.part = h->sums_part;
   f.count = h->d_err + 2;
   f.half = 0.5 * h->dt;
@@ -822,6 +825,7 @@ static void carve(pimd_handle *h, Carver &c) {
   h->d_step = c.take<int64_t>(1);
   h->d_err = c.take<unsigned>(4);
   if (h->barostat) h->baro = c.take<double>(kBaroWords);
+  if (h->barostat) h->baro_mm = c.take<double>((size_t)2 * N);
   if (h->barostat || h->fixcom) {
     h->sums_part = c.take<double>(sums_part_doubles(N, P, h->method));
     h->fix_u = c.take<double>((size_t)3 * P);
@@ -1176,6 +1180,17 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
     for (int i = 0; i < N; ++i) {
       kmm[i] = 0.5 * dt * inv_mm[i];
       kmm[N + i] = dt * inv_mm[i];
+    }
+    if (h->barostat) {   // mu_0 = fmass
+      std::vector<double> bm(2 * (size_t)N);
+      for (int i = 0; i < N; ++i) {
+        bm[i] = mass_mm[i] * h->fmass;
+        bm[N + i] = 1.0 / bm[i];
+      }
+      if ((st = up(h->baro_mm, bm))) {
+        release(h);
+        return st;
+      }
     }
     h->mu_one = std::all_of(tb.imu.begin(), tb.imu.end(), [](double m) { return m == 1.0; });
     auto upi = [&](int4 *dst, const std::vector<int4> &src) -> pimd_status {

@@ -219,7 +219,8 @@ struct BaroArgs {
   int N, P, nmol;
   const double *x, *v, *F;     // [N][3][P]
   const double *Mt;            // [P][P]
-  const double *mass_mm;       // [N] m mvv2e
+  const double *mass_mm, *inv_mm;   // [N] m^(0) mvv2e (fictitious masses included), and its inverse
+  double invP;
   const double *Wpart;         // [nmol][P] Tr Xi rows of the force kernel
   const double *W3part;        // [nmol][P][3] diagonal Xi_aa rows (anisotropic), or null
   int axes;                    // 0: isotropic; else the mask of edges with their own v_W
@@ -230,7 +231,7 @@ struct BaroArgs {
   // scales the box once by exp(tA v_W), tA = h; the end-of-step call applies
   // the closing O_W (mode 1, keyed on the step just completed) after its B_W
   int obabo;
-  double nkT, npext, mu0;      // n kB T; n P_ext; mu_0
+  double nkT, npext;           // n kB T; n P_ext
   // weights of B_W's three terms: 3 tB / W (per edge tB / W), tB^2 / W and
   // tB^3 / 3W, W = 3 n N kB T taup^2 (n N kB T taup^2 per edge)
   double k1, k2, k3;
@@ -252,7 +253,8 @@ struct BaroArgs {
 struct FixcomArgs {
   int N, P, method;
   const double *mass_mm;       // [N] m mvv2e
-  double msum;                 // their sum
+  double imsum;                // 1 / their sum
+  double rsp;                  // 1 / sqrt(P)
   const double *x, *F, *v;     // [N][3][P]
   double *u;                   // out: [nb][3], subtracted by the next kernel
   double *part;                // partial sums (sums_part_doubles)

@@ -80,18 +80,19 @@ __global__ void __launch_bounds__(kSumThreads) k_baro_kick(BaroArgs a) {
       sx += x[q];
       sf += f[q];
     }
-    const double mm = on ? a.mass_mm[r / 3] * a.mu0 : 1.0;
+    const double mm = on ? a.mass_mm[r / 3] : 1.0, im = on ? a.inv_mm[r / 3] : 1.0;
     const double v = on ? a.v[row] - (a.fix_u ? a.fix_u[r % 3] : 0.0) : 0.0;
-    const double xm = group_sum(sx, W) / P;
+    const double xm = group_sum(sx, W) * a.invP;
     const double f0 = rp * group_sum(sf, W);
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       if (l + q * W < P) rcf = fma(x[q] - xm, f[q], rcf);
     if (l == 0 && on) {
-      const double v0 = fma(a.t0, f0 / mm, v);   // at t0 into the kick
+      const double fm = f0 * im;
+      const double v0 = fma(a.t0, fm, v);   // at t0 into the kick
       mv2 = fma(mm * v0, v0, mv2);
       fv = fma(f0, v0, fv);
-      f2m += f0 * f0 / mm;
+      f2m = fma(f0, fm, f2m);
     }
   }
   rcf = group_sum(rcf, W);
@@ -142,19 +143,20 @@ __global__ void __launch_bounds__(kSumThreads) k_baro_kick(BaroArgs a) {
     gauss3(a.seed, 0xffffffffu, a.step_follows ? 0u : 1u, 3u, a.step_follows ? step : step - 1, noise[0], noise[1],
            noise[2]);
   __syncthreads();
-  // the scalar work, one thread per edge (isotropic: the three do the same)
-  if (threadIdx.x >= 3) return;
-  const int c = threadIdx.x;
+  // the scalar work, one warp: lane = (edge c, sign of the exponent, which A);
+  // the lanes of an edge do the same up to their exponential (isotropic: all do)
+  if (threadIdx.x >= 12) return;
+  const int c = threadIdx.x % 3, sgn = threadIdx.x / 3 % 2, h = threadIdx.x / 6;
   const double *mv = tot, *sfv = tot + 3, *sf2 = tot + 6, *srcf = tot + 9, *svir = tot + 12;
   double *b = a.baro;
   const double V = b[kBaroL] * b[kBaroL + 1] * b[kBaroL + 2], L = b[kBaroL + c];
-  __syncwarp(0x7u);   // V is formed before an edge changes below
   const bool moves = !a.axes || (a.axes >> c & 1);
   const double eta = a.axes ? noise[c] : noise[0];
+  double vW = b[kBaroV + c];
+  __syncwarp(0xfffu);   // every lane has read the state that lanes change below
   // O_W: v_W <- c1 v_W + sigW eta; each edge its own deviate, the isotropic
   // v_W the first
   auto langevin = [&](double w) { return moves ? a.c1W * w + a.sigW * eta : w; };
-  double vW = b[kBaroV + c];
   if (a.obabo && a.step_follows && a.thermo) vW = langevin(vW);   // this step's first O(h/2)
   if (!moves) {
     vW = 0.0;
@@ -169,27 +171,28 @@ __global__ void __launch_bounds__(kSumThreads) k_baro_kick(BaroArgs a) {
     // OBABO: the closing O(h/2) of the step just completed (the counter has
     // already been advanced past it)
     if (a.obabo && a.thermo) vW = langevin(vW);
-    b[kBaroV + c] = vW;
+    if (threadIdx.x < 3) b[kBaroV + c] = vW;
     return;
   }
   double vO = vW;
   if (a.thermo && !a.obabo) vO = langevin(vO);
+  // the A factors of the centroid mode at v_W (h = 0) and, BAOAB, at v_O (h = 1)
+  const double w = h ? vO : vW, x = a.tA * w;
+  const double ex = exp(sgn ? -x : x);
+  const double other = __shfl_sync(0xfffu, ex, (threadIdx.x + 3) % 12);   // sgn 0: the lane's e^-x
+  const double grow2 = __shfl_sync(0xfffu, ex, (threadIdx.x + 6) % 12);   // h 0: e^x of the second A
+  if (sgn == 0) {
+    double *f = b + (h ? kBaroA2 : kBaroA1) + 3 * c;
+    f[0] = ex;
+    f[1] = other;
+    f[2] = fabs(x) < 1e-8 ? a.tA * (1.0 + x * x / 6.0) : (ex - other) / (2.0 * w);
+  }
+  if (threadIdx.x >= 3) return;
   b[kBaroVA1 + c] = vW;
   b[kBaroVA2 + c] = vO;
   b[kBaroV + c] = vO;
-  // the A factors of the centroid mode at v_W and (BAOAB) at v_O
-  double grow = 1.0;
-  for (int h = 0; h < (a.obabo ? 1 : 2); ++h) {
-    const double w = h ? vO : vW, x = a.tA * w;
-    const double ea = exp(x), ema = exp(-x);
-    double *f = b + (h ? kBaroA2 : kBaroA1) + 3 * c;
-    f[0] = ea;
-    f[1] = ema;
-    f[2] = fabs(x) < 1e-8 ? a.tA * (1.0 + x * x / 6.0) : (ea - ema) / (2.0 * w);
-    grow *= ea;
-  }
   // BAOAB: A(h/2) at v_W, O_W, A(h/2) at v_O; OBABO: one A(h) at v_W
-  const double Ln = L * grow;
+  const double Ln = a.obabo ? L * ex : L * ex * grow2;
   b[kBaroL + c] = Ln;
   b[kBaroInvL + c] = 1.0 / Ln;
   if (!(Ln > a.Lmin)) atomicOr(a.err, kErrBoxSmall);
@@ -199,7 +202,8 @@ __global__ void __launch_bounds__(kSumThreads) k_baro_kick(BaroArgs a) {
 // modes, nb = 1) or of every bead (Cartesian, nb = P) as it will stand after
 // the closing B(h/2) (and O(h/2)) that the next kernel applies; that kernel
 // subtracts u when it loads v.  Partial row of a block: [q][c][k] for
-// q = m v, F, m x (Cartesian), m sigv eta (OBABO's closing O(h/2)).
+// q = m v, F, m (2 x_k - x_{k-1} - x_{k+1}) (Cartesian: the springs, from the
+// small differences), m sigv eta (OBABO's closing O(h/2)).
 __global__ void __launch_bounds__(kSumThreads) k_fixcom_f64(FixcomArgs a) {
   __shared__ double sh[4 * 1024];   // [q][group][k]; then the totals [q][c][k]
   const int P = a.P, W = row_lanes(P), gpb = kSumThreads / W;
@@ -222,7 +226,11 @@ __global__ void __launch_bounds__(kSumThreads) k_fixcom_f64(FixcomArgs a) {
       pf[q] += a.F[row + k];
       if (k >= nb) continue;
       pv[q] = fma(mm, a.v[row + k], pv[q]);
-      if (a.method == 1) px[q] = fma(mm, a.x[row + k], px[q]);
+      if (a.method == 1) {
+        const double xk = a.x[row + k];
+        const double xm = a.x[row + (k == 0 ? P - 1 : k - 1)], xp = a.x[row + (k == P - 1 ? 0 : k + 1)];
+        px[q] = fma(mm, (xk - xm) + (xk - xp), px[q]);
+      }
       if (a.obabo_thermo)
         pn[q] = fma(mm * a.sigv[i], gauss1(a.seed, (uint32_t)i, (uint32_t)k, kStreamO2, s, c), pn[q]);
     }
@@ -251,25 +259,38 @@ __global__ void __launch_bounds__(kSumThreads) k_fixcom_f64(FixcomArgs a) {
     part[t] = sum;
   }
   if (!last_block(a.count)) return;
-  for (int t = threadIdx.x; t < ncol; t += kSumThreads) {
-    double sum = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) sum += __ldcg(a.part + (size_t)b * ncol + t);
-    sh[t] = sum;
+  const int rows_p = (int)gridDim.x;
+  if (nb == 1) {   // twelve columns: a warp each
+    for (int t = threadIdx.x >> 5; t < ncol; t += kSumThreads / 32) {
+      double sum = 0.0;
+      for (int b = threadIdx.x & 31; b < rows_p; b += 32) sum += __ldcg(a.part + (size_t)b * ncol + t);
+      sum = warp_sum(sum);
+      if ((threadIdx.x & 31) == 0) sh[t] = sum;
+    }
+  } else {         // a thread each, four loads in flight and four partial sums
+    for (int t = threadIdx.x; t < ncol; t += kSumThreads) {
+      double s4[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int b = 0; b < rows_p; b += 4) {
+        double v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = b + q < rows_p ? __ldcg(a.part + (size_t)(b + q) * ncol + t) : 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s4[q] += v[q];
+      }
+      sh[t] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+    }
   }
   __syncthreads();
   for (int kc = threadIdx.x; kc < 3 * nb; kc += kSumThreads) {
     const int c = kc / nb, k = kc % nb;
-    const double *sx = sh + 6 * nb + c * nb;
     double p = sh[kc], f = sh[3 * nb + kc];
-    if (a.method == 0) {
-      f /= sqrt((double)P);
-    } else {
-      const int km = k == 0 ? P - 1 : k - 1, kp = k == P - 1 ? 0 : k + 1;
-      f -= a.wn2 * (2.0 * sx[k] - sx[km] - sx[kp]);
-    }
+    if (a.method == 0)
+      f *= a.rsp;   // F~_0
+    else
+      f = fma(-a.wn2, sh[6 * nb + kc], f);
     // the closing O(h/2) scales by c1 and adds c2 sigv eta: remove its mean too
-    if (a.obabo_thermo) p += a.c2[k] * sh[9 * nb + kc] / a.c1[k];
-    a.u[3 * k + c] = fma(a.half * a.imu0, f, p) / a.msum;
+    if (a.obabo_thermo) p = fma(a.c2[k] / a.c1[k], sh[9 * nb + kc], p);
+    a.u[3 * k + c] = fma(a.half * a.imu0, f, p) * a.imsum;
   }
 }
 
