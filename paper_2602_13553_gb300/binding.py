@@ -86,17 +86,28 @@ class Estimates(ctypes.Structure):
     ]
 
     def as_dict(self) -> dict:
-        P = self.P
-        out = {k: getattr(self, k) for k in ("H", "K_PR", "K_VR", "K_CV", "P_PR", "P_MD", "P_CV",
-                                             "T_ring", "volume", "vir_sum", "vW", "K_W", "U_W",
-                                             "J_W", "enthalpy")}
-        out["box"] = np.array(list(self.box))
-        out["vWa"] = np.array(list(self.vWa))
-        out["step"] = int(self.step)
-        out["K_mode"] = np.array(self.K_mode[:P])
-        out["S_mode"] = np.array(self.S_mode[:P])
-        out["U_bead"] = np.array(self.U_bead[:P])
-        return out
+        return _estimates_dict(np.frombuffer(self, dtype=np.float64), int(self.step), self.P)
+
+
+# pimd_estimates as doubles: step and (P, N) take one each, then K_mode,
+# S_mode, U_bead, the scalars, box and vWa
+_EST_SCALARS = ("H", "K_PR", "K_VR", "K_CV", "P_PR", "P_MD", "P_CV", "T_ring", "volume", "vir_sum", "vW", "K_W", "U_W",
+                "J_W", "enthalpy")
+_EST_DOUBLES = ctypes.sizeof(Estimates) // 8
+
+
+def _estimates_dict(a, step: int, P: int) -> dict:
+    """The dictionary of one pimd_estimates, from its words as doubles (its own
+    arrays: the words may be reused)."""
+    at = 2 + 3 * MAX_BEADS
+    out = dict(zip(_EST_SCALARS, a[at:at + len(_EST_SCALARS)].tolist()))
+    at += len(_EST_SCALARS)
+    out["box"] = a[at:at + 3].copy()
+    out["vWa"] = a[at + 3:at + 6].copy()
+    out["step"] = step
+    for q, k in enumerate(("K_mode", "S_mode", "U_bead")):
+        out[k] = a[2 + q * MAX_BEADS:2 + q * MAX_BEADS + P].copy()
+    return out
 
 
 class _EstimatesMap(collections.abc.Mapping):
@@ -104,9 +115,13 @@ class _EstimatesMap(collections.abc.Mapping):
     a slot's dict is built when it is first read (a batch holds hundreds of
     replicas; building every dict costs milliseconds of host time)."""
 
-    def __init__(self, arr, slots):
+    def __init__(self, arr):
         self._arr = arr
-        self._slots = list(slots)
+        self._words = np.frombuffer(arr, dtype=np.float64).reshape(-1, _EST_DOUBLES)
+        ints = np.frombuffer(arr, dtype=np.int64).reshape(-1, _EST_DOUBLES)
+        self._steps = ints[:, 0].tolist()
+        self._beads = np.frombuffer(arr, dtype=np.int32).reshape(-1, 2 * _EST_DOUBLES)[:, 2].tolist()
+        self._slots = [s for s, step in enumerate(self._steps) if step >= 0]
         self._live = set(self._slots)
         self._cache = {}
 
@@ -114,7 +129,7 @@ class _EstimatesMap(collections.abc.Mapping):
         if slot not in self._live:
             raise KeyError(slot)
         if slot not in self._cache:
-            self._cache[slot] = self._arr[slot].as_dict()
+            self._cache[slot] = _estimates_dict(self._words[slot], self._steps[slot], self._beads[slot])
         return self._cache[slot]
 
     def __iter__(self):
@@ -489,7 +504,7 @@ class Batch:
         """slot -> estimator dict of every live replica (converted on first access)."""
         arr = (Estimates * self.capacity)()
         check(_batch_lib().pimd_batch_estimators(self._h, arr))
-        return _EstimatesMap(arr, [s for s in range(self.capacity) if arr[s].step >= 0])
+        return _EstimatesMap(arr)
 
     def get_state(self, slot: int):
         P, N = self.shapes[slot]

@@ -98,7 +98,7 @@ struct RepDesc {
   const float *inv_mmf, *sigvf;   // FP32 copies for the FP32 mode updates
   const float *ksf;               // harmonic well (single systems): [N] m mvv2e omega^2, F is not read
   const float *Mf, *Mtf, *cAf, *sAf, *wsAf, *c1f, *c2f;
-  const double *Mt64, *lam;
+  const double *lam;
   // tensor-core path (P % 8 == 0): M (forward) and M^T (inverse) as TF32
   // hi/lo halves in m16n8k8 A-fragment order [mode tile][k step][lane][4]
   const float4 *mfa_hi, *mfa_lo, *mia_hi, *mia_lo;
@@ -1929,6 +1929,7 @@ struct Replica {
   int2 *d_items_step = nullptr, *d_items_nbr = nullptr;
   int4 *d_items_clu = nullptr;
   int *d_counts = nullptr;   // [4] own item counts: step, cluster, nbr, est
+  char *up_lo = nullptr, *up_hi = nullptr;   // the part of the arena that admission uploads
 };
 
 template <typename T>
@@ -1947,7 +1948,6 @@ size_t layout_replica(Replica &r, char *base) {
   const int NS = kLJWarps * r.G;
   RepDesc &d = r.desc;
   size_t off = 0;
-  d.ctl = carve_ptr<long long>(base, off, kCtlWords);
   d.xc = carve_ptr<double>(base, off, N * 3);
   d.v0 = carve_ptr<double>(base, off, N * 3);
   d.d = carve_ptr<float>(base, off, len);
@@ -1955,6 +1955,16 @@ size_t layout_replica(Replica &r, char *base) {
   d.F = carve_ptr<float>(base, off, len);
   d.xcw = carve_ptr<float>(base, off, N * 3);
   d.pO = carve_ptr<float>(base, off, nmol * 3 * P);
+  d.cref = carve_ptr<double>(base, off, nmol * 3);
+  d.ccur = carve_ptr<double>(base, off, nmol * 3);
+  d.nbr = carve_ptr<int>(base, off, nmol * kMaxNeighbours);
+  d.nbr_off = carve_ptr<int>(base, off, nmol * (NS + 1));
+  d.Upart = carve_ptr<double>(base, off, nmol * P);
+  d.Wpart = carve_ptr<double>(base, off, nmol * P);
+  d.epart = carve_ptr<double>(base, off, kEstItems * (2 * P + 4));
+  // what admission uploads, in one copy
+  d.ctl = carve_ptr<long long>(base, off, kCtlWords);
+  r.up_lo = reinterpret_cast<char *>(d.ctl);
   d.inv_mm = carve_ptr<double>(base, off, N);
   d.sigv = carve_ptr<double>(base, off, N);
   d.mass_mm = carve_ptr<double>(base, off, N);
@@ -1965,20 +1975,13 @@ size_t layout_replica(Replica &r, char *base) {
   d.wsAf = carve_ptr<float>(base, off, P);
   d.c1f = carve_ptr<float>(base, off, P);
   d.c2f = carve_ptr<float>(base, off, P);
-  d.Mt64 = carve_ptr<double>(base, off, P * P);
   d.lam = carve_ptr<double>(base, off, P);
-  d.cref = carve_ptr<double>(base, off, nmol * 3);
-  d.ccur = carve_ptr<double>(base, off, nmol * 3);
-  d.nbr = carve_ptr<int>(base, off, nmol * kMaxNeighbours);
-  d.nbr_off = carve_ptr<int>(base, off, nmol * (NS + 1));
-  d.Upart = carve_ptr<double>(base, off, nmol * P);
-  d.Wpart = carve_ptr<double>(base, off, nmol * P);
-  d.epart = carve_ptr<double>(base, off, kEstItems * (2 * P + 4));
   d.mperm = carve_ptr<int>(base, off, nmol);
   r.d_items_step = carve_ptr<int2>(base, off, N);
   r.d_items_nbr = carve_ptr<int2>(base, off, (nmol + kNbrMolPerItem - 1) / kNbrMolPerItem);
   r.d_items_clu = carve_ptr<int4>(base, off, nmol * ((P + 31) / 32));
   r.d_counts = carve_ptr<int>(base, off, 4);
+  r.up_hi = base ? base + off : nullptr;
   return off + 256;
 }
 
@@ -2339,9 +2342,8 @@ size_t split_warp_desc_bytes() { return sizeof(RepDesc); }
 size_t split_warp_frag_float4(int P) { return 4 * (size_t)((P + 15) / 16) * (P / 8) * 32; }
 bool split_warp_class(int P) { return warp_class(P) || P == 128; }
 
-// Fill a descriptor for the handle's own arrays and upload it with the FP32
-// per-atom constants and the TF32 fragment tables of M and M^T into the
-// device buffers the handle carved for them.
+// Fill a descriptor for the handle's own arrays and put it and the TF32
+// fragment tables of M and M^T into the handle's table image.
 namespace {
 int g_sw_nsm = 0;   // SM count of the device, read at set-up (one GPU per process)
 
@@ -2367,16 +2369,16 @@ cudaError_t split_warp_prepare() {
 }
 }  // namespace
 
-cudaError_t split_warp_setup(const SplitWarpSetup &w, cudaStream_t st) {
+cudaError_t split_warp_setup(const SplitWarpSetup &w, const std::function<void(void *, const void *, size_t)> &put) {
   const cudaError_t pe = split_warp_prepare();   // outside any stream capture
   if (pe != cudaSuccess) return pe;
-  const int N = w.N, P = w.P;
+  const int P = w.P;
   RepDesc d;
   std::memset(&d, 0, sizeof(d));
   d.live = 1;
-  d.N = N;
+  d.N = w.N;
   d.P = P;
-  d.nmol = w.cref ? N / 3 : 0;
+  d.nmol = w.cref ? w.N / 3 : 0;
   d.integrator = w.integrator;
   d.thermo = w.thermo;
   d.seed = w.seed;
@@ -2414,44 +2416,16 @@ cudaError_t split_warp_setup(const SplitWarpSetup &w, cudaStream_t st) {
   d.mfa_lo = w.frag + one;
   d.mia_hi = w.frag + 2 * one;
   d.mia_lo = w.frag + 3 * one;
-  std::vector<double> Mt((size_t)P * P);
-  std::vector<double> M(w.M_host, w.M_host + (size_t)P * P);
-  for (int k = 0; k < P; ++k)
-    for (int j = 0; j < P; ++j) Mt[(size_t)j * P + k] = M[(size_t)k * P + j];
+  const std::vector<double> M(w.M_host, w.M_host + (size_t)P * P), Mt(w.Mt_host, w.Mt_host + (size_t)P * P);
   std::vector<float> fh, fl, ih, il;
   fragment_tables(M, P, fh, fl);
   fragment_tables(Mt, P, ih, il);
-  std::vector<float> imf(N), sgf(N), ksf(w.ksf ? N : 0);
-  for (int i = 0; i < N; ++i) {
-    imf[i] = (float)w.inv_mm_host[i];
-    sgf[i] = (float)w.sigv_host[i];
-    if (w.ksf) ksf[i] = (float)w.kspring_host[i];
-  }
-  long long ctl[kCtlWords] = {0};
-  const struct {
-    void *dst;
-    const void *src;
-    size_t bytes;
-  } ups[] = {
-      {w.desc, &d, sizeof(RepDesc)},
-      {w.frag, fh.data(), one * sizeof(float4)},
-      {w.frag + one, fl.data(), one * sizeof(float4)},
-      {w.frag + 2 * one, ih.data(), one * sizeof(float4)},
-      {w.frag + 3 * one, il.data(), one * sizeof(float4)},
-      {w.inv_mmf, imf.data(), N * sizeof(float)},
-      {w.sigvf, sgf.data(), N * sizeof(float)},
-      {w.ksf, ksf.data(), ksf.size() * sizeof(float)},
-      {w.ctl, ctl, sizeof(ctl)},
-  };
-  for (const auto &u : ups) {
-    if (!u.bytes) continue;
-    // pageable sources: the copy completes before the call returns
-    const cudaError_t e = cudaMemcpyAsync(u.dst, u.src, u.bytes, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return e;
-  }
-  const cudaError_t e = cudaMemsetAsync(w.done, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
-  return cudaStreamSynchronize(st);
+  put(w.desc, &d, sizeof(RepDesc));
+  put(w.frag, fh.data(), one * sizeof(float4));
+  put(w.frag + one, fl.data(), one * sizeof(float4));
+  put(w.frag + 2 * one, ih.data(), one * sizeof(float4));
+  put(w.frag + 3 * one, il.data(), one * sizeof(float4));
+  return cudaSuccess;
 }
 
 cudaError_t launch_step_split_warp(const void *desc, int N, int P, const int64_t *step, int step_off, int first,
@@ -2800,18 +2774,19 @@ extern "C" pimd_status pimd_batch_add(pimd_batch *b, const pimd_system *sys, int
       {(void *)d.wsAf, wsAf.data(), P * sizeof(float)},
       {(void *)d.c1f, c1f.data(), P * sizeof(float)},
       {(void *)d.c2f, c2f.data(), P * sizeof(float)},
-      {(void *)d.Mt64, tb.Mt.data(), (size_t)P * P * sizeof(double)},
       {(void *)d.lam, tb.lam.data(), P * sizeof(double)},
       {r.d_items_step, r.items_step.data(), r.items_step.size() * sizeof(int2)},
       {r.d_items_nbr, r.items_nbr.data(), r.items_nbr.size() * sizeof(int2)},
       {r.d_items_clu, r.items_clu.data(), r.items_clu.size() * sizeof(int4)},
       {(void *)d.mperm, mperm.data(), nmol * sizeof(int)},
       {r.d_counts, counts, sizeof(counts)},
-      {b->d_reps + slot, &d, sizeof(RepDesc)},
   };
+  std::vector<char> img((size_t)(r.up_hi - r.up_lo), 0);
   for (const auto &u : ups)
-    if (u.bytes && cudaMemcpyAsync(u.dst, u.src, u.bytes, cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
-      return cleanup(fail(PIMD_ECUDA, "replica upload failed"));
+    if (u.bytes) std::memcpy(img.data() + (static_cast<char *>(u.dst) - r.up_lo), u.src, u.bytes);
+  if (cudaMemcpyAsync(r.up_lo, img.data(), img.size(), cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+      cudaMemcpyAsync(b->d_reps + slot, &d, sizeof(RepDesc), cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
+    return cleanup(fail(PIMD_ECUDA, "replica upload failed"));
   const size_t len = (size_t)N * 3 * P;
   if ((st = ensure_staging(b, len)) != PIMD_OK) return cleanup(st);
   cudaError_t e = cudaMemcpyAsync(b->stg_t, sys->pos, len * sizeof(double), cudaMemcpyHostToDevice, b->stream);

@@ -176,7 +176,7 @@ struct pimd_handle {
   // (x, v, F above then only serve as FP64 staging for estimators and state copies)
   double *xc = nullptr, *v0 = nullptr;
   float *dev = nullptr, *vk = nullptr, *F32 = nullptr, *xcw = nullptr;
-  float *Mf = nullptr, *Mtf = nullptr, *cAf = nullptr, *sAf = nullptr, *wsAf = nullptr;
+  float *Mtf = nullptr, *cAf = nullptr, *sAf = nullptr, *wsAf = nullptr;
   float *Tff = nullptr, *Tif = nullptr;   // split: FP32 folded transforms
   float *c1f = nullptr, *c2f = nullptr;
   double tA = 0.0, c1_0 = 0.0, c2_0 = 0.0;
@@ -189,9 +189,10 @@ struct pimd_handle {
   long long *sw_ctl = nullptr;
   unsigned *sw_done = nullptr;
   double *inv_mm = nullptr, *sigv = nullptr, *mass_mm = nullptr, *kspring = nullptr;
-  double *M = nullptr, *Mt = nullptr, *cA = nullptr, *sA = nullptr, *wsA = nullptr;
+  double *cA = nullptr, *sA = nullptr, *wsA = nullptr;
   double *c1 = nullptr, *c2 = nullptr, *lam = nullptr, *mu = nullptr, *imu = nullptr;
-  double *Tf = nullptr, *Ti = nullptr;   // folded transforms, [P/2 + 1][P]
+  double *Tf = nullptr;   // folded forward transform, [P/2 + 1][P]
+  char *tab_lo = nullptr, *tab_hi = nullptr;   // the tables' part of the arena
   // FP64 normal-mode step: folded transforms in fixed point, A O A as one map
   // per mode, [2][N] B(h/2) and B(h) durations over m mvv2e
   int4 *fTf = nullptr, *fTi = nullptr;
@@ -292,20 +293,26 @@ void dev_free(const DevAllocator &a, void *p, cudaStream_t s) {
 
 // Eq. (A1), with cos rows 1 <= i <= floor((P-1)/2), the alternating row at
 // i = P/2 for even P, and sin rows i > P/2.
+// The entries depend on i j mod P alone: P cosines and sines, the
+// angles reduced exactly (P^2 of unreduced angles took 0.3 ms at 128 beads and
+// were up to 2e-14 off).
 static void build_nm_matrix(int P, std::vector<double> &M) {
   M.assign((size_t)P * P, 0.0);
   const double rp = 1.0 / std::sqrt((double)P), r2p = std::sqrt(2.0 / P);
+  std::vector<double> cs(P), sn(P);
+  for (int r = 0; r < P; ++r) {
+    cs[r] = r2p * std::cos(2.0 * kPi * r / P);
+    sn[r] = r2p * std::sin(2.0 * kPi * r / P);
+  }
   for (int i = 0; i < P; ++i)
-    for (int j = 0; j < P; ++j) {
+    for (int j = 0, r = 0; j < P; ++j, r = r + i >= P ? r + i - P : r + i) {
       double val;
       if (i == 0)
         val = rp;
       else if (P % 2 == 0 && 2 * i == P)
         val = (j & 1) ? -rp : rp;
-      else if (2 * i < P)
-        val = r2p * std::cos(2.0 * kPi * (double)i * j / P);
       else
-        val = r2p * std::sin(2.0 * kPi * (double)i * j / P);
+        val = 2 * i < P ? cs[r] : sn[r];
       M[(size_t)i * P + j] = val;
     }
 }
@@ -341,7 +348,7 @@ static StepArgs step_args(pimd_handle *h) {
   a.N = h->N;
   a.P = h->P;
   a.A = h->A_step;
-  a.mt = ModeTables{h->M, h->Mt, h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf, h->Ti,
+  a.mt = ModeTables{h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf,
                     h->fTf, h->fTi, h->fem, h->map6, 1.0 / std::sqrt((double)h->P)};
   a.inv_mm = h->inv_mm;
   a.mu_one = h->mu_one;
@@ -435,7 +442,6 @@ static SplitStepArgs split_args(pimd_handle *h) {
   a.N = h->N;
   a.P = h->P;
   a.A = h->A_step;
-  a.Mf = h->Mf;
   a.Mtf = h->Mtf;
   a.Tff = h->Tff;
   a.Tif = h->Tif;
@@ -572,7 +578,7 @@ static pimd_status enqueue_baro(pimd_handle *h, double t0, double tB, bool step_
   b.x = h->x;
   b.v = h->v;
   b.F = h->F;
-  b.Mt = h->Mt;
+  b.rsp = 1.0 / std::sqrt((double)h->P);
   b.mass_mm = h->baro_mm;
   b.inv_mm = h->baro_mm + h->N;
   b.invP = 1.0 / h->P;
@@ -758,7 +764,6 @@ static void release(pimd_handle *h) {
   if (h->graph) cudaGraphExecDestroy(h->graph);
   dev_free(h->alloc, h->arena, h->stream);
   if (h->h_est) cudaFreeHost(h->h_est);
-  if (h->h_err) cudaFreeHost(h->h_err);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }
@@ -786,12 +791,12 @@ static void carve(pimd_handle *h, Carver &c) {
   h->tmp = c.take<double>(len);
   if (h->potential == PIMD_POT_WATERLIKE && h->precision == PIMD_PREC_FP64)
     h->xi = c.take<long long>((size_t)h->nmol * 3 * P);
+  // the tables, filled in one copy (TableImage)
   h->inv_mm = c.take<double>(N);
+  h->tab_lo = reinterpret_cast<char *>(h->inv_mm);
   h->sigv = c.take<double>(N);
   h->mass_mm = c.take<double>(N);
   h->kspring = c.take<double>(N);
-  h->M = c.take<double>((size_t)P * P);
-  h->Mt = c.take<double>((size_t)P * P);
   h->cA = c.take<double>(P);
   h->sA = c.take<double>(P);
   h->wsA = c.take<double>(P);
@@ -801,11 +806,31 @@ static void carve(pimd_handle *h, Carver &c) {
   h->mu = c.take<double>(P);
   h->imu = c.take<double>(P);
   h->Tf = c.take<double>((size_t)(P / 2 + 1) * P);
-  h->Ti = c.take<double>((size_t)(P / 2 + 1) * P);
   h->fTf = c.take<int4>((size_t)fix_pairs(P) * P);
   h->fTi = c.take<int4>((size_t)fix_pairs(P) * P);
   h->map6 = c.take<double>((size_t)6 * P);
   h->kmm = c.take<double>((size_t)2 * N);
+  if (h->barostat) h->baro_mm = c.take<double>((size_t)2 * N);
+  if (h->precision == PIMD_PREC_SPLIT) {
+    h->Mtf = c.take<float>((size_t)P * P);
+    h->Tff = c.take<float>((size_t)(P / 2 + 1) * P);
+    h->Tif = c.take<float>((size_t)(P / 2 + 1) * P);
+    h->cAf = c.take<float>(P);
+    h->sAf = c.take<float>(P);
+    h->wsAf = c.take<float>(P);
+    h->c1f = c.take<float>(P);
+    h->c2f = c.take<float>(P);
+    if (h->split_warp) {
+      h->sw_desc = c.take<char>(split_warp_desc_bytes());
+      h->sw_frag = c.take<float4>(split_warp_frag_float4(P));
+      h->sw_imf = c.take<float>(N);
+      h->sw_sgf = c.take<float>(N);
+      if (h->fused_well) h->sw_ksf = c.take<float>(N);
+      h->sw_ctl = c.take<long long>(8);
+      h->sw_done = c.take<unsigned>(1);
+    }
+  }
+  h->tab_hi = c.base ? c.base + c.off : nullptr;
   // rows of per-bead U / Tr Xi sums: one per molecule (water) or per block
   h->nblk_force = h->potential == PIMD_POT_WATERLIKE ? h->nmol : force_blocks(h->N, P);
   h->Upart = c.take<double>((size_t)h->nblk_force * P);
@@ -825,7 +850,6 @@ static void carve(pimd_handle *h, Carver &c) {
   h->d_step = c.take<int64_t>(1);
   h->d_err = c.take<unsigned>(4);
   if (h->barostat) h->baro = c.take<double>(kBaroWords);
-  if (h->barostat) h->baro_mm = c.take<double>((size_t)2 * N);
   if (h->barostat || h->fixcom) {
     h->sums_part = c.take<double>(sums_part_doubles(N, P, h->method));
     h->fix_u = c.take<double>((size_t)3 * P);
@@ -838,26 +862,25 @@ static void carve(pimd_handle *h, Carver &c) {
     h->vk = c.take<float>(len);
     h->F32 = c.take<float>(len);
     h->xcw = c.take<float>((size_t)N * 3);
-    h->Mf = c.take<float>((size_t)P * P);
-    h->Mtf = c.take<float>((size_t)P * P);
-    h->Tff = c.take<float>((size_t)(P / 2 + 1) * P);
-    h->Tif = c.take<float>((size_t)(P / 2 + 1) * P);
-    h->cAf = c.take<float>(P);
-    h->sAf = c.take<float>(P);
-    h->wsAf = c.take<float>(P);
-    h->c1f = c.take<float>(P);
-    h->c2f = c.take<float>(P);
-    if (h->split_warp) {
-      h->sw_desc = c.take<char>(split_warp_desc_bytes());
-      h->sw_frag = c.take<float4>(split_warp_frag_float4(P));
-      h->sw_imf = c.take<float>(N);
-      h->sw_sgf = c.take<float>(N);
-      if (h->fused_well) h->sw_ksf = c.take<float>(N);
-      h->sw_ctl = c.take<long long>(8);
-      h->sw_done = c.take<unsigned>(1);
-    }
   }
 }
+
+// Host image of the tables' part of a handle's arena: every table is put at
+// its device address, one copy uploads them (twenty small synchronous copies
+// were a third of a small handle's creation).
+struct TableImage {
+  char *lo;
+  std::vector<char> bytes;
+  TableImage(char *lo_, char *hi) : lo(lo_), bytes((size_t)(hi - lo_), 0) {}
+  void put(void *dst, const void *src, size_t n) {
+    if (n) std::memcpy(bytes.data() + (static_cast<char *>(dst) - lo), src, n);
+  }
+  template <typename T, typename U>
+  void put(T *dst, const std::vector<U> &src) {
+    T *d = reinterpret_cast<T *>(bytes.data() + (reinterpret_cast<char *>(dst) - lo));
+    for (size_t i = 0; i < src.size(); ++i) d[i] = (T)src[i];
+  }
+};
 
 static pimd_status upload_state(pimd_handle *h, const double *x, const double *v) {
   const size_t bytes = (size_t)h->N * 3 * h->P * sizeof(double);
@@ -1131,93 +1154,77 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
   }
   Carver c1{(char *)h->arena};
   carve(h, c1);
-  if (cudaMallocHost(&h->h_est, sizeof(double) * (3 * P + 12)) != cudaSuccess ||
-      cudaMallocHost(&h->h_err, sizeof(unsigned) * 4) != cudaSuccess) {
+  if (cudaMallocHost(&h->h_est, sizeof(double) * (3 * P + 12) + sizeof(unsigned) * 4) != cudaSuccess) {
     release(h);
     return fail(PIMD_ENOMEM, "pinned host allocation failed");
   }
+  h->h_err = reinterpret_cast<unsigned *>(h->h_est + 3 * P + 12);
 
   // ---- host tables (App. B, App. D), FP64 ----
   HostTables tb;
   build_tables(P, T, dt, prm, tb);
   h->wn = tb.wn;
-  const std::vector<double> &M = tb.M, &Mt = tb.Mt, &cA = tb.cA, &sA = tb.sA, &wsA = tb.wsA;
-  const std::vector<double> &c1v = tb.c1, &c2v = tb.c2, &lam = tb.lam;
-  const double tA = tb.tA;
-  std::vector<double> inv_mm(N), sigv(N), mass_mm(N), ksp(N);
+  std::vector<double> inv_mm(N), sigv(N), mass_mm(N), ksp(N), kmm(2 * (size_t)N), map6;
   for (int i = 0; i < N; ++i) {
     const double mm = sys->mass[i] * kMvv2e;
     mass_mm[i] = mm;
     inv_mm[i] = 1.0 / mm;
     sigv[i] = std::sqrt(P * kBoltzmann * T / mm);
     ksp[i] = mm * sys->ff[0] * sys->ff[0];
+    kmm[i] = 0.5 * dt * inv_mm[i];
+    kmm[N + i] = dt * inv_mm[i];
     h->msum += mm;
   }
-  pimd_status st = PIMD_OK;
-  auto up = [&](double *dst, const std::vector<double> &src) -> pimd_status {
-    CK(cudaMemcpy(dst, src.data(), src.size() * sizeof(double), cudaMemcpyHostToDevice));
-    return PIMD_OK;
-  };
-  if ((st = up(h->M, M)) || (st = up(h->Mt, Mt)) || (st = up(h->cA, cA)) || (st = up(h->sA, sA)) ||
-      (st = up(h->wsA, wsA)) || (st = up(h->c1, c1v)) || (st = up(h->c2, c2v)) ||
-      (st = up(h->lam, lam)) || (st = up(h->mu, tb.mu)) || (st = up(h->imu, tb.imu)) ||
-      (st = up(h->Tf, tb.Tf)) || (st = up(h->Ti, tb.Ti)) ||
-      (st = up(h->inv_mm, inv_mm)) || (st = up(h->sigv, sigv)) ||
-      (st = up(h->mass_mm, mass_mm)) || (st = up(h->kspring, ksp))) {
-    release(h);
-    return st;
-  }
+  TableImage img(h->tab_lo, h->tab_hi);
+  img.put(h->inv_mm, inv_mm);
+  img.put(h->sigv, sigv);
+  img.put(h->mass_mm, mass_mm);
+  img.put(h->kspring, ksp);
+  img.put(h->kmm, kmm);
+  img.put(h->cA, tb.cA);
+  img.put(h->sA, tb.sA);
+  img.put(h->wsA, tb.wsA);
+  img.put(h->c1, tb.c1);
+  img.put(h->c2, tb.c2);
+  img.put(h->lam, tb.lam);
+  img.put(h->mu, tb.mu);
+  img.put(h->imu, tb.imu);
+  img.put(h->Tf, tb.Tf);
+  h->mu_one = std::all_of(tb.imu.begin(), tb.imu.end(), [](double m) { return m == 1.0; });
+  aoa_map(P, tb, h->thermostat == PIMD_THERMO_PILE_L, map6);
+  img.put(h->map6, map6);
   {
-    std::vector<int4> fTf, fTi;
-    h->fem = fixed_table(P, tb.Tf, fTf);
-    const int fi = fixed_table(P, tb.Ti, fTi);
+    std::vector<int4> fT;
+    h->fem = fixed_table(P, tb.Tf, fT);
+    img.put(h->fTf, fT);
+    const int fi = fixed_table(P, tb.Ti, fT);
+    img.put(h->fTi, fT);
     if (fi != h->fem) {   // the entries of both are those of M
       release(h);
       return fail(PIMD_EINVAL, "internal: transform scales %d and %d differ", h->fem, fi);
     }
-    std::vector<double> map6, kmm(2 * (size_t)N);
-    aoa_map(P, tb, h->thermostat == PIMD_THERMO_PILE_L, map6);
-    for (int i = 0; i < N; ++i) {
-      kmm[i] = 0.5 * dt * inv_mm[i];
-      kmm[N + i] = dt * inv_mm[i];
-    }
-    if (h->barostat) {   // mu_0 = fmass
-      std::vector<double> bm(2 * (size_t)N);
-      for (int i = 0; i < N; ++i) {
-        bm[i] = mass_mm[i] * h->fmass;
-        bm[N + i] = 1.0 / bm[i];
-      }
-      if ((st = up(h->baro_mm, bm))) {
-        release(h);
-        return st;
-      }
-    }
-    h->mu_one = std::all_of(tb.imu.begin(), tb.imu.end(), [](double m) { return m == 1.0; });
-    auto upi = [&](int4 *dst, const std::vector<int4> &src) -> pimd_status {
-      CK(cudaMemcpy(dst, src.data(), src.size() * sizeof(int4), cudaMemcpyHostToDevice));
-      return PIMD_OK;
-    };
-    if ((st = up(h->map6, map6)) || (st = up(h->kmm, kmm)) || (st = upi(h->fTf, fTf)) || (st = upi(h->fTi, fTi))) {
-      release(h);
-      return st;
-    }
   }
-  if (h->precision == PIMD_PREC_SPLIT) {
-    auto upf = [&](float *dst, const std::vector<double> &src) -> pimd_status {
-      std::vector<float> f(src.begin(), src.end());
-      CK(cudaMemcpy(dst, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
-      return PIMD_OK;
-    };
-    if ((st = upf(h->Mf, M)) || (st = upf(h->Mtf, Mt)) || (st = upf(h->Tff, tb.Tf)) ||
-        (st = upf(h->Tif, tb.Ti)) || (st = upf(h->cAf, cA)) ||
-        (st = upf(h->sAf, sA)) || (st = upf(h->wsAf, wsA)) || (st = upf(h->c1f, c1v)) ||
-        (st = upf(h->c2f, c2v))) {
-      release(h);
-      return st;
+  if (h->barostat) {   // mu_0 = fmass
+    std::vector<double> bm(2 * (size_t)N);
+    for (int i = 0; i < N; ++i) {
+      bm[i] = mass_mm[i] * h->fmass;
+      bm[N + i] = 1.0 / bm[i];
     }
-    h->tA = tA;
-    h->c1_0 = c1v[0];
-    h->c2_0 = c2v[0];
+    img.put(h->baro_mm, bm);
+  }
+  pimd_status st = PIMD_OK;
+  if (h->precision == PIMD_PREC_SPLIT) {
+    img.put(h->Mtf, tb.Mt);
+    img.put(h->Tff, tb.Tf);
+    img.put(h->Tif, tb.Ti);
+    img.put(h->cAf, tb.cA);
+    img.put(h->sAf, tb.sA);
+    img.put(h->wsAf, tb.wsA);
+    img.put(h->c1f, tb.c1);
+    img.put(h->c2f, tb.c2);
+    h->tA = tb.tA;
+    h->c1_0 = tb.c1[0];
+    h->c2_0 = tb.c2[0];
     if (h->split_warp) {
       SplitWarpSetup w{};
       w.N = N;
@@ -1226,9 +1233,9 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
       w.thermo = h->thermostat == PIMD_THERMO_PILE_L;
       w.seed = h->seed;
       w.dt = h->dt;
-      w.tA = tA;
-      w.c1_0 = c1v[0];
-      w.c2_0 = c2v[0];
+      w.tA = tb.tA;
+      w.c1_0 = tb.c1[0];
+      w.c2_0 = tb.c2[0];
       for (int c = 0; c < 3; ++c) w.box[c] = h->potential == PIMD_POT_WATERLIKE ? h->box[c] : 0.0;
       w.xc = h->xc;
       w.v0 = h->v0;
@@ -1246,18 +1253,20 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
       const bool water = h->potential == PIMD_POT_WATERLIKE;
       w.cref = water ? h->cref : nullptr;
       w.ccur = water ? h->ccur : nullptr;
-      w.M_host = M.data();
-      w.inv_mm_host = inv_mm.data();
-      w.sigv_host = sigv.data();
-      w.kspring_host = ksp.data();
-      w.ksf = h->sw_ksf;
+      w.M_host = tb.M.data();
+      w.Mt_host = tb.Mt.data();
       w.desc = h->sw_desc;
       w.frag = h->sw_frag;
       w.inv_mmf = h->sw_imf;
       w.sigvf = h->sw_sgf;
+      w.ksf = h->sw_ksf;
       w.ctl = h->sw_ctl;
-      w.done = h->sw_done;
-      const cudaError_t e = split_warp_setup(w, h->stream);
+      img.put(h->sw_imf, inv_mm);
+      img.put(h->sw_sgf, sigv);
+      if (h->sw_ksf) img.put(h->sw_ksf, ksp);
+      // control words and the completion counter start at zero, as the image does
+      const cudaError_t e =
+          split_warp_setup(w, [&](void *dst, const void *src, size_t n) { img.put(dst, src, n); });
       if (e != cudaSuccess) {
         release(h);
         return fail(PIMD_ECUDA, "split step set-up failed: %s", cudaGetErrorString(e));
@@ -1265,6 +1274,7 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
     }
   }
   auto init = [&]() -> pimd_status {
+    CK(cudaMemcpyAsync(h->tab_lo, img.bytes.data(), img.bytes.size(), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemsetAsync(h->d_step, 0, sizeof(int64_t), h->stream));
     CK(cudaMemsetAsync(h->d_err, 0, 4 * sizeof(unsigned), h->stream));
     if (h->baro) {
@@ -1351,7 +1361,7 @@ extern "C" pimd_status pimd_estimators(pimd_handle *h, pimd_estimates *out) {
   a.P = P;
   a.A = h->A_est;
   a.method = h->method;
-  a.mt = ModeTables{h->M, h->Mt, h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf, h->Ti,
+  a.mt = ModeTables{h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf,
                     h->fTf, h->fTi, h->fem, h->map6, 1.0 / std::sqrt((double)P)};
   a.mass_mm = h->mass_mm;
   a.x = h->x;

@@ -144,8 +144,6 @@ __device__ __forceinline__ double mic(double d, double L, double invL) {
 // bead/mode), i.e. every atom's P beads are contiguous per component.
 // ---------------------------------------------------------------------------
 struct ModeTables {
-  const double *M;     // [P][P]  M[k][j]  (mode k, bead j), Eq. (A1)
-  const double *Mt;    // [P][P]  Mt[j][k] = M[k][j]
   const double *cA;    // [P] cos(w_k tA)
   const double *sA;    // [P] sin(w_k tA)/w_k   (tA for k = 0)
   const double *wsA;   // [P] w_k sin(w_k tA)   (0 for k = 0)
@@ -154,13 +152,12 @@ struct ModeTables {
   const double *lam;   // [P] lambda_k (Eq. A2)
   const double *mu;    // [P] fictitious-mass factor mu_k: m^(k) = mu_k m (fmmode, fmass)
   const double *imu;   // [P] 1 / mu_k
-  // folded transforms (H = floor(P/2)), [H + 1][P] each:
+  // folded forward transform (H = floor(P/2)), [H + 1][P]:
   //   Tf[i][k]: k <= H: M[k][i]; k > H: M[k][P - (H + 1 + i)] (0 past the row)
-  //   Ti[i][j]: j <= H: M[i][j]; j > H: M[H + 1 + i][P - j] (0 past the modes)
   const double *Tf;
-  const double *Ti;
   // the folded transforms in fixed point (fixed.cuh): [fix_pairs(P)][P], limbs
-  // (h, l) of terms 2p and 2p + 1, scaled by 2^(55 - fem)
+  // (h, l) of terms 2p and 2p + 1, scaled by 2^(55 - fem); the inverse's terms
+  // for bead j are Ti[i][j]: j <= H: M[i][j]; j > H: M[H + 1 + i][P - j]
   const int4 *fTf, *fTi;
   int fem;
   // A(h/2) O(h) A(h/2) of BAOAB per mode, [6][P]: q' = m0 q + m1 v + m2 n,
@@ -218,7 +215,7 @@ struct StepArgs {
 struct BaroArgs {
   int N, P, nmol;
   const double *x, *v, *F;     // [N][3][P]
-  const double *Mt;            // [P][P]
+  double rsp;                  // 1 / sqrt(P)
   const double *mass_mm, *inv_mm;   // [N] m^(0) mvv2e (fictitious masses included), and its inverse
   double invP;
   const double *Wpart;         // [nmol][P] Tr Xi rows of the force kernel
@@ -308,7 +305,7 @@ struct ForceArgs {
 // d = x - xc and internal-mode velocities v~_k (k >= 1) [N][3][P]; FP32 forces.
 struct SplitStepArgs {
   int N, P, A;
-  const float *Mf, *Mtf;       // [P][P] FP32 copies of M and M^T
+  const float *Mtf;            // [P][P] FP32 copy of M^T
   const float *Tff, *Tif;      // [P/2 + 1][P] FP32 folded forward / inverse tables (as ModeTables::Tf, Ti)
   const float *cAf, *sAf, *wsAf, *c1f, *c2f;   // FP32 mode coefficients (k >= 1)
   double tA, c1_0, c2_0;       // centroid: drift time of one A, O coefficients

@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <functional>
 #include <vector>
 
 #include "pimd.h"
@@ -56,17 +57,17 @@ struct SplitWarpSetup {
   const double *inv_mm, *sigv;                  // device [N]
   const float *cAf, *sAf, *wsAf, *c1f, *c2f;    // device [P]
   double *cref, *ccur;                          // water-like: skin test, else null
-  const double *M_host, *inv_mm_host, *sigv_host, *kspring_host;
+  const double *M_host, *Mt_host;               // [P][P]
   void *desc;
   float4 *frag;
-  float *inv_mmf, *sigvf, *ksf;                 // ksf: harmonic well, else null
+  const float *inv_mmf, *sigvf, *ksf;           // device [N], filled by the handle; ksf: harmonic well, else null
   long long *ctl;
-  unsigned *done;
 };
 size_t split_warp_desc_bytes();
 size_t split_warp_frag_float4(int P);
 bool split_warp_class(int P);
-cudaError_t split_warp_setup(const SplitWarpSetup &w, cudaStream_t st);
+// put(device address, host source, bytes): into the handle's table image
+cudaError_t split_warp_setup(const SplitWarpSetup &w, const std::function<void(void *, const void *, size_t)> &put);
 cudaError_t launch_step_split_warp(const void *desc, int N, int P, const int64_t *step, int step_off, int first,
                                    double *blkmax, unsigned *done, bool harm, cudaStream_t s);
 

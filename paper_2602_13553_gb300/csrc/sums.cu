@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kSumThreads) k_baro_kick(BaroArgs a) {
   const int g = blockIdx.x * gpb + lg;
   const int S = (int)gridDim.x * gpb / 3 * 3;
   const int rows = a.N * 3;
-  const double rp = a.Mt[0];   // F~0 = (M F)_0 = sum_j F_j / sqrt(P)
+  const double rp = a.rsp;   // F~0 = (M F)_0 = sum_j F_j / sqrt(P)
   double mv2 = 0.0, fv = 0.0, f2m = 0.0, rcf = 0.0;
   // every lane of a warp runs the same rounds (the shuffles need them all)
   for (int r0 = 0; r0 < rows; r0 += S) {
