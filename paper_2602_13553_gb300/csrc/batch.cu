@@ -432,6 +432,8 @@ constexpr int kWAtoms = 8;      // atoms per warp item
 constexpr int kWWarps = 4;      // warps per block
 constexpr int kWMaxP = 64;
 __host__ __device__ constexpr int wslot_floats(int P) { return 48 * (P + 4) + 128; }
+__host__ __device__ constexpr int est_slot_floats(int P) { return 48 * (P + 4) + 32; }     // and 24 bead means
+__host__ __device__ constexpr int close_slot_floats(int P) { return 24 * (P + 4); }        // forces alone
 __host__ __device__ constexpr int wslot_floats_harm(int P) { return 24 * (P + 4) + 128; }   // no forces
 __host__ __device__ constexpr bool warp_class(int P) { return P == 8 || P == 16 || P == 32 || P == 64; }
 
@@ -1212,11 +1214,11 @@ __global__ void __launch_bounds__(128, 4) k_bstep(const RepDesc *__restrict__ re
 }
 
 // Closing B(h/2) (O(h/2) for OBABO) of the replicas that stepped since their
-// last closing kick, over step items.
-__global__ void __launch_bounds__(128) k_bclose(const RepDesc *reps, const int2 *items, const int *count) {
+// last closing kick, over the block items [counts[7], counts[0]).
+__global__ void __launch_bounds__(128) k_bclose(const RepDesc *reps, const int2 *items, const int *counts) {
   __shared__ float sF[kTileMax];
-  const int n = *count;
-  for (int it = blockIdx.x; it < n; it += gridDim.x) {
+  const int n = counts[0];
+  for (int it = counts[7] + blockIdx.x; it < n; it += gridDim.x) {
     const int2 w = items[it];
     const RepDesc &R = reps[w.x];
     if (!R.ctl[kCtlClose]) continue;
@@ -1265,6 +1267,99 @@ __global__ void __launch_bounds__(128) k_bclose(const RepDesc *reps, const int2 
       R.vk[base + task] = v;
     }
     __syncthreads();
+    }
+  }
+}
+
+// The closing kick of one warp item on tensor cores: F~ = M F as in the step,
+// then B(h/2) (and O(h/2)) on the velocities; lane (g, t) holds modes 16 mt + g
+// (+ 8) of atoms 2t, 2t + 1.
+template <int P>
+__device__ __forceinline__ void bclose_warp(const RepDesc &R, int tile, float *__restrict__ sF, uint64_t step) {
+  constexpr int PS = P + 4, MT = (P + 15) / 16, CPR = P / 4;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int tile0 = tile * kWAtoms, na = min(kWAtoms, R.N - tile0);
+  const size_t base = (size_t)tile0 * 3 * P;
+  const float *__restrict__ gF = R.F + base;
+  for (int q = lane; q < na * 3 * CPR; q += 32) {
+    const int row = q / CPR, col = (q - row * CPR) * 4;
+    const int a = row / 3, c = row - 3 * a;
+    cp_async16(sF + (c * 8 + a) * PS + col, gF + (size_t)row * P + col);
+  }
+  cp_async_commit();
+  for (int q = lane; q < (kWAtoms - na) * 3 * P; q += 32) {   // rows of missing atoms
+    const int r = q / P, j = q - r * P;
+    sF[((r % 3) * 8 + na + r / 3) * PS + j] = 0.f;
+  }
+  cp_async_wait_all();
+  __syncwarp();
+  float C[MT][3][4];
+  fwd_tile<P>(R.mfa_hi, R.mfa_lo, sF, C);
+  const bool bath = R.integrator == 1 && R.thermo;
+  const float half = 0.5f * (float)R.dt;
+  float *__restrict__ vkg = R.vk + base;
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = 16 * mt + g + 8 * h;
+      if (k >= P) continue;
+#pragma unroll
+      for (int aa = 0; aa < 2; ++aa) {
+        const int a = 2 * t + aa, i = tile0 + a;
+        if (a >= na) continue;
+        float e[3] = {0.f, 0.f, 0.f};
+        if (bath) gauss3f_b(R.seed, (uint32_t)i, (uint32_t)k, kStreamO2, step, e[0], e[1], e[2]);
+        if (k == 0) {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const size_t ic = (size_t)i * 3 + c;
+            double v = fma(0.5 * R.dt * __ldg(R.inv_mm + i), (double)C[mt][c][2 * h + aa], R.v0[ic]);
+            if (bath) v = fma(R.c1_0, v, R.c2_0 * __ldg(R.sigv + i) * (double)e[c]);
+            R.v0[ic] = v;
+          }
+        } else {
+          const float kb = half * __ldg(R.inv_mmf + i);
+          const float c1 = __ldg(R.c1f + k), c2s = __ldg(R.c2f + k) * __ldg(R.sigvf + i);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            float *v = vkg + (a * 3 + c) * P + k;
+            float w = fmaf(kb, C[mt][c][2 * h + aa], *v);
+            if (bath) w = fmaf(c1, w, c2s * e[c]);
+            *v = w;
+          }
+        }
+      }
+    }
+  __syncwarp();   // the slot is free for the next item
+}
+
+// Closing kicks of the warp items (bead counts 8, 16, 32, 64, 128), the range
+// [0, counts[7]) of the step list.  The block form above read the mode matrix
+// once per element: 432 us on the 256-replica mix.
+template <bool k128>
+__global__ void __launch_bounds__(kWWarps * 32) k_bclose_w(const RepDesc *__restrict__ reps,
+                                                          const int2 *__restrict__ items,
+                                                          const int *__restrict__ counts, int slot_floats) {
+  extern __shared__ __align__(16) float wsm[];
+  float *slot = wsm + (threadIdx.x >> 5) * slot_floats;
+  const int lo = k128 ? counts[4] : 0, hi = k128 ? counts[7] : counts[4];
+  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+  for (int it = lo + gw; it < hi; it += nw) {
+    const int2 w = items[it];
+    const RepDesc &R = reps[w.x];
+    if (!R.ctl[kCtlClose]) continue;
+    const uint64_t step = (uint64_t)R.ctl[kCtlStep] - 1;
+    if (k128) {
+      bclose_warp<128>(R, w.y, slot, step);
+    } else {
+      switch (R.P) {
+        case 8: bclose_warp<8>(R, w.y, slot, step); break;
+        case 16: bclose_warp<16>(R, w.y, slot, step); break;
+        case 32: bclose_warp<32>(R, w.y, slot, step); break;
+        case 64: bclose_warp<64>(R, w.y, slot, step); break;
+        default: break;
+      }
     }
   }
 }
@@ -1699,12 +1794,175 @@ __global__ void __launch_bounds__(128, 6) k_bforce(const RepDesc *__restrict__ r
   }
 }
 
-// Estimators, pass 1: work items (replica, e-block); e-block b walks the
-// replica's tiles b, b + ne, ... (x = xc + d in FP64; q~_k = (M d)_k and the
-// bead mean of d in FP32 from the FP32 deviations, relative error ~P 2^-24;
-// r - r_c = d - mean_j d_j); products and sums in FP64.
-__global__ void __launch_bounds__(128) k_best(const RepDesc *reps, const int2 *items, const int *count) {
+// s + c += x, an FP32 sum with its rounding errors kept (two-sum).
+__device__ __forceinline__ void ff_add(float &s, float &c, float x) {
+  const float t = __fadd_rn(s, x), z = __fadd_rn(t, -s);
+  c += __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(x, -z));
+  s = t;
+}
+
+// s + c += a b, the product exact (its rounding error by a fused multiply-add).
+__device__ __forceinline__ void ff_fma(float &s, float &c, float a, float b) {
+  const float p = __fmul_rn(a, b);
+  ff_add(s, c, p);
+  c += fmaf(a, b, -p);
+}
+
+// Estimator sums of the 8-atom tiles e 4 + warp, + 4 ne, ... of one replica, one
+// warp.  As lane r < 24 it holds the beads of row (component r / 8, atom r % 8);
+// then the rows are folded by the parity of the modes (e_j = d_j + d_{P-j} kept at
+// j, o_j = d_j - d_{P-j} at P - j) and lane (atom group, mode) forms q~ = M d in
+// FP32.  Products of FP32 quantities are summed in FP32 with their errors kept
+// (an FP64 instruction costs a warp 64 clocks); whatever has an FP64 factor --
+// masses, centroids, the centroid-mode velocity -- joins in FP64 (masses as two
+// floats).  3xTF32 transforms, whose accumulation truncates, were as fast but
+// put the modes' spring energies 20% further from their FP64 values.  K and S of
+// this warp go to sKS [2 P].
+template <int P>
+__device__ void best_warp(const RepDesc &R, int e, float *__restrict__ slot, double *__restrict__ sKS, double &rF,
+                          double &rcF) {
+  constexpr int PS = P + 4, CPR = P / 4, H = P / 2;
+  constexpr int PL = P < 32 ? P : 32, NG = 32 / PL, NCH = (P + 31) / 32;
+  const int lane = threadIdx.x & 31, grp = lane / PL, kl = lane % PL, warp = threadIdx.x >> 5;
+  float *sF = slot, *sX = slot + 24 * PS, *sM = slot + 48 * PS;   // sM [24]: bead means of the deviations
+  float K[NCH][2], S[NCH][2];
+#pragma unroll
+  for (int cc = 0; cc < NCH; ++cc) K[cc][0] = K[cc][1] = S[cc][0] = S[cc][1] = 0.f;
+  double kk0 = 0.0;
+  const float rsp = rsqrtf((float)P);
+  const int ntiles = (R.N + kWAtoms - 1) / kWAtoms;
+  for (int tile = e * 4 + warp; tile < ntiles; tile += R.ne * 4) {
+    const int tile0 = tile * kWAtoms, na = min(kWAtoms, R.N - tile0);
+    const size_t base = (size_t)tile0 * 3 * P;
+    for (int q = lane; q < na * 3 * CPR; q += 32) {
+      const int row = q / CPR, col = (q - row * CPR) * 4;
+      const int a = row / 3, c = row - 3 * a;
+      const int so = (c * 8 + a) * PS + col;
+      cp_async16(sF + so, R.F + base + (size_t)row * P + col);
+      cp_async16(sX + so, R.d + base + (size_t)row * P + col);
+    }
+    cp_async_commit();
+    const float *__restrict__ vkg = R.vk + base;
+    cp_async_wait_all();
+    __syncwarp();
+    // x.F = x_c.F + d.F, (x - r_c).F = d.F - <d>.F over the row's beads
+    const bool bead = lane < 24 && (lane & 7) < na;
+    double sumF = 0.0, dF = 0.0;
+    if (bead) {
+      const float *f = sF + lane * PS, *d = sX + lane * PS;
+      float fs = 0.f, fc = 0.f, ds = 0.f, dc = 0.f;
+#pragma unroll 4
+      for (int j = 0; j < P; ++j) {
+        ff_add(fs, fc, f[j]);
+        ff_fma(ds, dc, d[j], f[j]);
+      }
+      sumF = (double)fs + (double)fc;
+      dF = (double)ds + (double)dc;
+    }
+    __syncwarp();
+    for (int q = lane; q < 24 * (H - 1); q += 32) {
+      const int row = q / (H - 1), j = 1 + q - row * (H - 1);
+      if ((row & 7) >= na) continue;
+      float *x = sX + row * PS;
+      const float u = x[j], w = x[P - j];
+      x[j] = u + w;
+      x[P - j] = u - w;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int cc = 0; cc < NCH; ++cc) {
+      const int k = kl + 32 * cc;
+      const bool even = k <= H;
+      // even modes: terms j = 4 b + q at j, and j = H; odd ones: j = 4 b + 4 - q at P - j
+      float m[H];
+#pragma unroll
+      for (int b = 0; b < H / 4; ++b)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int jt = even ? 4 * b + q : 4 * b + 4 - q;
+          m[4 * b + q] = !even && jt == H ? 0.f : __ldg(R.Mtf + jt * P + k);
+        }
+      const float mH = even ? __ldg(R.Mtf + H * P + k) : 0.f;
+      for (int a = grp; a < na; a += NG) {
+        float q2 = 0.f, qc[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const float *x = sX + (c * 8 + a) * PS;
+          float qa = mH * x[H], qb = 0.f;
+#pragma unroll
+          for (int b = 0; b < H / 4; ++b) {
+            const float4 v = *reinterpret_cast<const float4 *>(x + (even ? 4 * b : P - 4 - 4 * b));
+            qa = fmaf(m[4 * b], v.x, qa);
+            qb = fmaf(m[4 * b + 1], v.y, qb);
+            qa = fmaf(m[4 * b + 2], v.z, qa);
+            qb = fmaf(m[4 * b + 3], v.w, qb);
+          }
+          qc[c] = qa + qb;
+          q2 = fmaf(qc[c], qc[c], q2);
+        }
+        const double md = __ldg(R.mass_mm + tile0 + a);
+        if (k == 0) {
+          double v2 = 0.0;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const double v = R.v0[(size_t)(tile0 + a) * 3 + c];
+            v2 = fma(v, v, v2);
+            sM[c * 8 + a] = qc[c] * rsp;   // <d> = (M d)_0 / sqrt(P)
+          }
+          kk0 = fma(0.5 * md, v2, kk0);
+        } else {
+          const float mh = (float)md, ml = (float)(md - (double)mh);
+          float v2 = 0.f;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float v = vkg[(a * 3 + c) * P + k];
+            v2 = fmaf(v, v, v2);
+          }
+          ff_fma(K[cc][0], K[cc][1], mh, v2);
+          K[cc][1] = fmaf(ml, v2, K[cc][1]);
+          ff_fma(S[cc][0], S[cc][1], mh, q2);
+          S[cc][1] = fmaf(ml, q2, S[cc][1]);
+        }
+      }
+    }
+    __syncwarp();
+    if (bead) {
+      rF += fma(R.xc[(size_t)(tile0 + (lane & 7)) * 3 + (lane >> 3)], sumF, dF);
+      rcF += fma(-(double)sM[lane], sumF, dF);
+    }
+    __syncwarp();   // the slot is free for the next tile
+  }
+  // the lanes that share a mode
+#pragma unroll
+  for (int cc = 0; cc < NCH; ++cc) {
+    const int k = kl + 32 * cc;
+    double kd = 0.5 * ((double)K[cc][0] + (double)K[cc][1]), sd = (double)S[cc][0] + (double)S[cc][1];
+    if (k == 0) kd = kk0;
+#pragma unroll
+    for (int o = PL; o < 32; o <<= 1) {
+      kd += __shfl_xor_sync(0xffffffffu, kd, o);
+      sd += __shfl_xor_sync(0xffffffffu, sd, o);
+    }
+    if (grp == 0) {
+      sKS[k] = kd;
+      sKS[P + k] = k ? 0.5 * R.wn2 * __ldg(R.lam + k) * sd : 0.0;
+    }
+  }
+}
+
+// Estimators, pass 1: work items (replica, e-block); e-block b takes the
+// replica's tiles b, b + ne, ... and its share of the force kernel's rows of
+// U^(k) and Tr Xi^(k).  Bead counts of the warp items go through best_warp; the
+// others walk tiles of A P <= 128 (atom, mode) tasks (x = xc + d in FP64; q~_k
+// and the bead mean of d in FP32 from the FP32 deviations).  One row of
+// est_columns(P) sums per e-block.  A thread-per-task form with every product
+// converted to FP64, and the rows of U and Tr Xi left to pass 2, took 694 +
+// 246 us on the 256-replica mix.
+__global__ void __launch_bounds__(128) k_best(const RepDesc *reps, const int2 *items, const int *count,
+                                              int slot_floats) {
+  extern __shared__ __align__(16) float wsm[];
   __shared__ CSum sK[128], sS[128];
+  __shared__ double sKS[4][2 * kMaxBeads];
   __shared__ CSum sred[3][4];
   __shared__ float sDv[3 * 128];   // the tile's deviation rows (A atoms x 3 x P <= 384)
   const int n = *count;
@@ -1712,77 +1970,129 @@ __global__ void __launch_bounds__(128) k_best(const RepDesc *reps, const int2 *i
     const int2 w = items[it];
     const RepDesc &R = reps[w.x];
     const int P = R.P, N = R.N;
+    const int warp = threadIdx.x >> 5;
+    double *out = R.epart + (size_t)w.y * est_columns(P);
+    const bool items_w = warp_class(P) || P == 128;
     const int A = P >= 128 ? 1 : 128 / P;       // estimator tile: A P <= 128 tasks
     const int ntiles = (N + A - 1) / A;
     const int ntask = A * P;
-    // per thread a handful of tiles (plain FP64 sums: a few tens of terms);
-    // every combination across threads and blocks below is compensated
-    double kk = 0.0, ss = 0.0, rF = 0.0, rcF = 0.0, mv0 = 0.0;
-    for (int tile = w.y; tile < ntiles; tile += R.ne) {
-      const int tile0 = tile * A;
-      // stage the tile's deviations (contiguous in [N][3][P]) once: every
-      // mode's transform reads the whole row
-      const int nrow = min(A, N - tile0) * 3 * P;
+    double rF = 0.0, rcF = 0.0, mv0 = 0.0;
+    if (items_w) {
+      float *slot = wsm + warp * slot_floats;
+      switch (P) {
+        case 8: best_warp<8>(R, w.y, slot, sKS[warp], rF, rcF); break;
+        case 16: best_warp<16>(R, w.y, slot, sKS[warp], rF, rcF); break;
+        case 32: best_warp<32>(R, w.y, slot, sKS[warp], rF, rcF); break;
+        case 64: best_warp<64>(R, w.y, slot, sKS[warp], rF, rcF); break;
+        default: best_warp<128>(R, w.y, slot, sKS[warp], rF, rcF); break;
+      }
       __syncthreads();
-      for (int t = threadIdx.x; t < nrow; t += blockDim.x) sDv[t] = R.d[(size_t)tile0 * 3 * P + t];
-      __syncthreads();
-      for (int task = threadIdx.x; task < ntask; task += blockDim.x) {
-        const int k = task % P, al = task / P;
-        const int i = tile0 + al;
-        if (i >= N) continue;
-        // the FP64 pipe is the scarce unit: products of FP32 quantities stay
-        // in FP32 and are converted once per task; only terms with an FP64
-        // factor (the centroid x_c, the centroid-mode velocity, the masses)
-        // are formed in FP64.  x.F = x_c.F + d.F, (x - x_c).F = (d - <d>).F.
-        const double mm = __ldg(R.mass_mm + i);
-        double v2 = 0.0, xcF = 0.0;
-        float v2f = 0.f, q2f = 0.f, dF = 0.f, dcF = 0.f;
-        const float invP = 1.0f / (float)P;
-        for (int c = 0; c < 3; ++c) {
-          const size_t row = ((size_t)i * 3 + c) * P;
-          if (k == 0) {
-            const double v = R.v0[(size_t)i * 3 + c];
-            v2 = fma(v, v, v2);
-          } else {
-            const float v = R.vk[row + k];
-            v2f = fmaf(v, v, v2f);
+      for (int q = threadIdx.x; q < 2 * P; q += blockDim.x) {
+        CSum a{sKS[0][q], 0.0};
+        for (int v = 1; v < 4; ++v) a.add(sKS[v][q]);
+        out[q] = a.value();
+        if (q == 0) mv0 = 2.0 * a.value();   // m |v~_0|^2 = 2 K^(0)
+      }
+    } else {
+      // per thread a handful of tiles (plain FP64 sums: a few tens of terms);
+      // every combination across threads and blocks below is compensated
+      double kk = 0.0, ss = 0.0;
+      for (int tile = w.y; tile < ntiles; tile += R.ne) {
+        const int tile0 = tile * A;
+        // stage the tile's deviations (contiguous in [N][3][P]) once: every
+        // mode's transform reads the whole row
+        const int nrow = min(A, N - tile0) * 3 * P;
+        __syncthreads();
+        for (int t = threadIdx.x; t < nrow; t += blockDim.x) sDv[t] = R.d[(size_t)tile0 * 3 * P + t];
+        __syncthreads();
+        for (int task = threadIdx.x; task < ntask; task += blockDim.x) {
+          const int k = task % P, al = task / P;
+          const int i = tile0 + al;
+          if (i >= N) continue;
+          // the FP64 pipe is the scarce unit: products of FP32 quantities stay
+          // in FP32 and are converted once per task; only terms with an FP64
+          // factor (the centroid x_c, the centroid-mode velocity, the masses)
+          // are formed in FP64.  x.F = x_c.F + d.F, (x - x_c).F = (d - <d>).F.
+          const double mm = __ldg(R.mass_mm + i);
+          double v2 = 0.0, xcF = 0.0;
+          float v2f = 0.f, q2f = 0.f, dF = 0.f, dcF = 0.f;
+          const float invP = 1.0f / (float)P;
+          for (int c = 0; c < 3; ++c) {
+            const size_t row = ((size_t)i * 3 + c) * P;
+            if (k == 0) {
+              const double v = R.v0[(size_t)i * 3 + c];
+              v2 = fma(v, v, v2);
+            } else {
+              const float v = R.vk[row + k];
+              v2f = fmaf(v, v, v2f);
+            }
+            float qa = 0.f, qb = 0.f, dma = 0.f, dmb = 0.f;
+            const float *__restrict__ dr = sDv + (al * 3 + c) * P;
+            const float *__restrict__ mc = R.Mtf + k;
+            int j = 0;
+            for (; j + 1 < P; j += 2) {
+              const float d0 = dr[j], d1 = dr[j + 1];
+              qa = fmaf(__ldg(mc + j * P), d0, qa);
+              qb = fmaf(__ldg(mc + (j + 1) * P), d1, qb);
+              dma += d0;
+              dmb += d1;
+            }
+            if (j < P) {
+              qa = fmaf(__ldg(mc + j * P), dr[j], qa);
+              dma += dr[j];
+            }
+            const float q = qa + qb;
+            if (k > 0) q2f = fmaf(q, q, q2f);
+            const float dk = dr[k];
+            const float fk = R.F[row + k];
+            xcF = fma(R.xc[(size_t)i * 3 + c], (double)fk, xcF);
+            dF = fmaf(dk, fk, dF);
+            dcF = fmaf(dk - (dma + dmb) * invP, fk, dcF);
           }
-          float qa = 0.f, qb = 0.f, dma = 0.f, dmb = 0.f;
-          const float *__restrict__ dr = sDv + (al * 3 + c) * P;
-          const float *__restrict__ mc = R.Mtf + k;
-          int j = 0;
-          for (; j + 1 < P; j += 2) {
-            const float d0 = dr[j], d1 = dr[j + 1];
-            qa = fmaf(__ldg(mc + j * P), d0, qa);
-            qb = fmaf(__ldg(mc + (j + 1) * P), d1, qb);
-            dma += d0;
-            dmb += d1;
-          }
-          if (j < P) {
-            qa = fmaf(__ldg(mc + j * P), dr[j], qa);
-            dma += dr[j];
-          }
-          const float q = qa + qb;
-          if (k > 0) q2f = fmaf(q, q, q2f);
-          const float dk = dr[k];
-          const float fk = R.F[row + k];
-          xcF = fma(R.xc[(size_t)i * 3 + c], (double)fk, xcF);
-          dF = fmaf(dk, fk, dF);
-          dcF = fmaf(dk - (dma + dmb) * invP, fk, dcF);
+          v2 += (double)v2f;
+          rF += xcF + (double)dF;
+          rcF += (double)dcF;
+          kk = fma(0.5 * mm, v2, kk);
+          ss = fma(0.5 * mm * R.wn2 * __ldg(R.lam + k), (double)q2f, ss);
+          if (k == 0) mv0 = fma(mm, v2, mv0);
         }
-        v2 += (double)v2f;
-        rF += xcF + (double)dF;
-        rcF += (double)dcF;
-        kk = fma(0.5 * mm, v2, kk);
-        ss = fma(0.5 * mm * R.wn2 * __ldg(R.lam + k), (double)q2f, ss);
-        if (k == 0) mv0 = fma(mm, v2, mv0);
+      }
+      sK[threadIdx.x] = CSum{kk, 0.0};
+      sS[threadIdx.x] = CSum{ss, 0.0};
+      __syncthreads();
+      // tile tasks never exceed the 128 threads, so thread t always held task
+      // t, i.e. mode t mod P; sum over atoms in order
+      for (int k = threadIdx.x; k < P; k += blockDim.x) {
+        CSum a{0.0, 0.0}, b2{0.0, 0.0};
+        for (int t = k; t < ntask; t += P) {
+          a.add(sK[t]);
+          b2.add(sS[t]);
+        }
+        out[k] = a.value();
+        out[P + k] = b2.value();
       }
     }
-    // per-mode sums: tile tasks never exceed the 128 threads, so thread t
-    // always held task t, i.e. mode t mod P; sum over atoms in order
-    double *out = R.epart + (size_t)w.y * (2 * P + 4);
-    sK[threadIdx.x] = CSum{kk, 0.0};
-    sS[threadIdx.x] = CSum{ss, 0.0};
+    // U and Tr Xi: thread (row r0, bead k) of the e-block's rows
+    CSum cu{0.0, 0.0}, cw{0.0, 0.0};
+    if (threadIdx.x < ntask) {
+      const int r0 = threadIdx.x / P, k = threadIdx.x - r0 * P;
+      for (int m = w.y * A + r0; m < R.nmol; m += R.ne * A) {
+        cu.add(R.Upart[(size_t)m * P + k]);
+        cw.add(R.Wpart[(size_t)m * P + k]);
+      }
+    }
+    const CSum crF = warp_csum(CSum{rF, 0.0}), crcF = warp_csum(CSum{rcF, 0.0});
+    // only one thread of a warp item's block, but many of a block item's, hold
+    // centroid terms
+    const CSum cmv0 = items_w ? CSum{mv0, 0.0} : warp_csum(CSum{mv0, 0.0});
+    __syncthreads();   // everyone is done with sK, sS
+    sK[threadIdx.x] = cu;
+    sS[threadIdx.x] = cw;
+    if ((threadIdx.x & 31) == 0) {
+      sred[0][warp] = crF;
+      sred[1][warp] = crcF;
+      sred[2][warp] = cmv0;
+    }
     __syncthreads();
     for (int k = threadIdx.x; k < P; k += blockDim.x) {
       CSum a{0.0, 0.0}, b2{0.0, 0.0};
@@ -1790,23 +2100,14 @@ __global__ void __launch_bounds__(128) k_best(const RepDesc *reps, const int2 *i
         a.add(sK[t]);
         b2.add(sS[t]);
       }
-      out[k] = a.value();
-      out[P + k] = b2.value();
+      out[2 * P + k] = a.value();
+      out[3 * P + k] = b2.value();
     }
-    const CSum crF = warp_csum(CSum{rF, 0.0}), crcF = warp_csum(CSum{rcF, 0.0}), cmv0 = warp_csum(CSum{mv0, 0.0});
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
-      sred[0][threadIdx.x >> 5] = crF;
-      sred[1][threadIdx.x >> 5] = crcF;
-      sred[2][threadIdx.x >> 5] = cmv0;
-    }
-    __syncthreads();
     if (threadIdx.x < 3) {
       CSum sum{0.0, 0.0};
       for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) sum.add(sred[threadIdx.x][ww]);
-      out[2 * P + threadIdx.x] = sum.value();
+      out[4 * P + threadIdx.x] = sum.value();
     }
-    if (threadIdx.x == 3) out[2 * P + 3] = 0.0;
     __syncthreads();
   }
 }
@@ -1830,80 +2131,49 @@ __global__ void k_bgather_ctl(const RepDesc *reps, int nslots, long long *out) {
   for (int w = 0; w < kCtlWords; ++w) out[(size_t)r * kCtlWords + w] = reps[r].live ? reps[r].ctl[w] : -1;
 }
 
-__device__ double neumaier_b(const double *p, int n, size_t stride) {
-  double s = 0.0, c = 0.0;
-  for (int b = 0; b < n; ++b) {
-    const double x = p[(size_t)b * stride];
-    const double t = s + x;
-    c += (fabs(s) >= fabs(x)) ? (s - t) + x : (x - t) + s;
-    s = t;
-  }
-  return s + c;
-}
-
-// Estimators, pass 2: one block per replica; output in the pimd_estimates
-// layout from K_mode on.
-__global__ void k_best_final(const RepDesc *reps, int nslots, double *eout) {
-  __shared__ double tot[2 * kMaxBeads + 4];
-  __shared__ double U[kMaxBeads], Wv[kMaxBeads];
-  __shared__ CSum cu[128], cw[128];
+// Estimators, pass 2: one block per replica sums the e-blocks' rows, one
+// compensated chain per column; output in the pimd_estimates layout from K_mode
+// on.
+__global__ void __launch_bounds__(256) k_best_final(const RepDesc *reps, int nslots, double *eout) {
+  __shared__ double tot[est_columns(kMaxBeads)];
+  __shared__ double stot[4];
   const int r = blockIdx.x;
   if (r >= nslots) return;
   const RepDesc &R = reps[r];
   if (!R.live) return;
-  const int P = R.P;
-  const int W = 2 * P + 4;
-  for (int s = threadIdx.x; s < W; s += blockDim.x) tot[s] = neumaier_b(R.epart + s, R.ne, W);
-  // the bead sums of U and Tr Xi over the molecules: thread t sums bead
-  // t mod P over the molecule rows of chunk t / P (compensated), then the
-  // chunks are added in order -- a fixed decomposition for a given P
-  const int nch = P >= 128 ? 1 : 128 / P;
-  const int per = (R.nmol + nch - 1) / nch;
-  if (threadIdx.x < nch * P) {
-    const int k = threadIdx.x % P, ch = threadIdx.x / P;
-    CSum su{0.0, 0.0}, sw{0.0, 0.0};
-    const int m1 = min(R.nmol, (ch + 1) * per);
-    for (int m = ch * per; m < m1; ++m) {
-      su.add(R.Upart[(size_t)m * P + k]);
-      sw.add(R.Wpart[(size_t)m * P + k]);
-    }
-    cu[threadIdx.x] = su;
-    cw[threadIdx.x] = sw;
+  const int P = R.P, W = est_columns(P);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int s = threadIdx.x; s < W; s += blockDim.x) {
+    CSum a{0.0, 0.0};
+    for (int b = 0; b < R.ne; ++b) a.add(R.epart[(size_t)b * W + s]);
+    tot[s] = a.value();
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < P; k += blockDim.x) {
-    CSum su{0.0, 0.0}, sw{0.0, 0.0};
-    for (int ch = 0; ch < nch; ++ch) {
-      su.add(cu[ch * P + k]);
-      sw.add(cw[ch * P + k]);
-    }
-    U[k] = su.value();
-    Wv[k] = sw.value();
-  }
   double *o = eout + (size_t)r * kOutStride;
-  for (int k = threadIdx.x; k < 3 * kMaxBeads; k += blockDim.x) o[k] = 0.0;
+  for (int t = threadIdx.x; t < 3 * kMaxBeads; t += blockDim.x) {
+    const int q = t / kMaxBeads, k = t - q * kMaxBeads;
+    o[t] = k < P ? tot[q * P + k] : 0.0;
+  }
+  if (warp < 4) {   // sums over the modes (beads) of K, S, U and Tr Xi, one warp each
+    CSum a{0.0, 0.0};
+    for (int k = lane; k < P; k += 32) a.add(tot[warp * P + k]);
+    a = warp_csum(a);
+    if (lane == 0) stot[warp] = a.value();
+  }
   __syncthreads();
   if (threadIdx.x) return;
-  double Kt = 0.0, St = 0.0, Ut = 0.0, Wt = 0.0;
-  for (int k = 0; k < P; ++k) {
-    o[k] = tot[k];
-    o[kMaxBeads + k] = tot[P + k];
-    o[2 * kMaxBeads + k] = U[k];
-    Kt += tot[k];
-    St += tot[P + k];
-    Ut += U[k];
-    Wt += Wv[k];
-  }
-  const double rF = tot[2 * P], rcF = tot[2 * P + 1], mv0 = tot[2 * P + 2];
+  const double Kt = stot[0], St = stot[1], Ut = stot[2], Wt = stot[3];
+  const double rF = tot[4 * P], rcF = tot[4 * P + 1], mv0 = tot[4 * P + 2];
   const double Nd = R.N, Pd = P, kT = R.kT, V = R.volume, spring = 2.0 * St;
+  const double iP = 1.0 / Pd, i3V = 1.0 / (3.0 * V);
   double *g = o + 3 * kMaxBeads;
   g[0] = Kt + St + Ut;
-  g[1] = 1.5 * Pd * Nd * kT - 0.5 * spring / Pd;
-  g[2] = -rF / (2.0 * Pd);
-  g[3] = 1.5 * Nd * kT - rcF / (2.0 * Pd);
-  g[4] = (3.0 * Pd * Nd * kT - spring / Pd + Wt / Pd) / (3.0 * V);
-  g[5] = (2.0 * Kt + Wt) / (3.0 * V);
-  g[6] = (mv0 - rcF + Wt) / (3.0 * Pd * V);
+  g[1] = 1.5 * Pd * Nd * kT - 0.5 * spring * iP;
+  g[2] = -0.5 * rF * iP;
+  g[3] = 1.5 * Nd * kT - 0.5 * rcF * iP;
+  g[4] = (3.0 * Pd * Nd * kT - spring * iP + Wt * iP) * i3V;
+  g[5] = (2.0 * Kt + Wt) * i3V;
+  g[6] = (mv0 - rcF + Wt) * i3V * iP;
   g[7] = 2.0 * Kt / (3.0 * Nd * Pd * kBoltzmann);
   g[8] = V;
   g[9] = Wt;
@@ -1961,7 +2231,7 @@ size_t layout_replica(Replica &r, char *base) {
   d.nbr_off = carve_ptr<int>(base, off, nmol * (NS + 1));
   d.Upart = carve_ptr<double>(base, off, nmol * P);
   d.Wpart = carve_ptr<double>(base, off, nmol * P);
-  d.epart = carve_ptr<double>(base, off, kEstItems * (2 * P + 4));
+  d.epart = carve_ptr<double>(base, off, kEstItems * est_columns((int)P));
   // what admission uploads, in one copy
   d.ctl = carve_ptr<long long>(base, off, kCtlWords);
   r.up_lo = reinterpret_cast<char *>(d.ctl);
@@ -2036,6 +2306,7 @@ struct pimd_batch {
   // [7] end of the 128-bead warp items, [8] their claim counter, [9] end of
   // the 64-bead warp items, [10] claim counter of the smaller warp items
   int h_counts[16] = {0};
+  int est_slot = 0;   // floats of shared memory per warp of the estimator pass
   int wslot = wslot_floats(64);   // floats of shared memory per warp of the 64-bead warp-item kernel
   int grid_w = 0;         // its blocks (persistent grid)
   int grid_ws = 0;        // blocks of the 8-, 16-, 32-bead warp-item kernel
@@ -2082,7 +2353,6 @@ void replica_items(pimd_batch *b, int slot, Replica &r) {
     r.A = (warp_class(r.P) || r.P == 128) ? kWAtoms : (b->tileA[r.P] > 0 ? b->tileA[r.P] : default_tile(r.P));
   r.desc.ffma = b->ffma ? 1 : 0;
   r.ntiles = (r.N + r.A - 1) / r.A;
-  r.ne = std::min(r.ntiles, kEstItems);
   r.items_step.clear();
   for (int t = 0; t < r.ntiles; ++t) r.items_step.push_back(make_int2(slot, t));
   r.items_nbr.clear();
@@ -2096,9 +2366,9 @@ void replica_items(pimd_batch *b, int slot, Replica &r) {
   const int per = r.P < cb ? 32 / ((r.P % 2 == 0) ? r.P / 2 : r.P) : 1;   // molecules per warp
   for (int m = 0; m < r.nmol; m += per)
     for (int c = 0; c < nchunk; ++c) r.items_clu.push_back(make_int4(slot, m, c, 0));
+  // e-blocks of about 64 atoms (two 8-atom tiles a warp), by the replica alone
   r.items_est.clear();
-  const int Ae = r.P >= 128 ? 1 : 128 / r.P;
-  r.ne = std::min((r.N + Ae - 1) / Ae, kEstItems);
+  r.ne = std::max(1, std::min((r.N + 63) / 64, kEstItems));
   for (int e = 0; e < r.ne; ++e) r.items_est.push_back(make_int2(slot, e));
   r.desc.A = r.A;
   r.desc.nstep_items = r.ntiles;
@@ -2163,6 +2433,10 @@ pimd_status upload(pimd_batch *b) {
   b->h_counts[8] = 0;
   b->h_counts[9] = n64;
   b->h_counts[10] = 0;
+  int pe = 8;   // the estimators' warp tiles: the largest bead count of their classes
+  for (int s = 0; s < b->capacity; ++s)
+    if (b->reps[s].live && (warp_class(b->reps[s].P) || b->reps[s].P == 128)) pe = std::max(pe, b->reps[s].P);
+  b->est_slot = est_slot_floats(pe);
   const bool blk = b->h_counts[0] > nw128, w128 = nw128 > nw, w64 = n64 > 0, wsm = nw > n64;
   if (blk != b->block_items || w128 != b->w128_items || w64 != b->w64_items || wsm != b->wsmall_items) {
     b->block_items = blk;
@@ -2221,6 +2495,29 @@ void launch_step_kernels(pimd_batch *b) {
 void launch_nbr_kernels(pimd_batch *b) {
   k_bdecide<<<b->nsm, 256, 0, b->stream>>>(b->d_reps, b->d_nbr, b->d_counts + 2, b->d_nbr_go, b->d_counts + 6);
   k_bnbr<<<b->grid_nbr, kNbrThreads, kNbrSmem, b->stream>>>(b->d_reps, b->d_nbr_go, b->d_counts + 6);
+}
+
+// The closing kicks, by class of bead count present; returns their number.
+int launch_close_kernels(pimd_batch *b) {
+  int n = 0;
+  auto grid = [&](int items) { return std::max(1, std::min((items + kWWarps - 1) / kWWarps, 16 * b->nsm)); };
+  if (b->w64_items || b->wsmall_items) {
+    const int slot = close_slot_floats(b->w64_items ? 64 : 32);
+    k_bclose_w<false><<<grid(b->h_counts[4]), kWWarps * 32, (size_t)kWWarps * slot * sizeof(float), b->stream>>>(
+        b->d_reps, b->d_step, b->d_counts, slot);
+    ++n;
+  }
+  if (b->w128_items) {
+    const int slot = close_slot_floats(128);
+    k_bclose_w<true><<<grid(b->h_counts[7] - b->h_counts[4]), kWWarps * 32, (size_t)kWWarps * slot * sizeof(float),
+                       b->stream>>>(b->d_reps, b->d_step, b->d_counts, slot);
+    ++n;
+  }
+  if (b->block_items) {
+    k_bclose<<<b->grid_step, 128, 0, b->stream>>>(b->d_reps, b->d_step, b->d_counts);
+    ++n;
+  }
+  return n;
 }
 
 // Kernels launched per MD step: control, warp-item step, 128-bead warp-item
@@ -2508,7 +2805,11 @@ extern "C" pimd_status pimd_batch_create(int32_t max_replicas, void *stream, pim
       cudaFuncSetAttribute((const void *)k_bstep_w<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(kWWarps * wslot_floats(32) * sizeof(float))) != cudaSuccess ||
       cudaFuncSetAttribute((const void *)k_bstep_w128, cudaFuncAttributeMaxDynamicSharedMemorySize, wsmem128) !=
-          cudaSuccess) {
+          cudaSuccess ||
+      cudaFuncSetAttribute((const void *)k_bclose_w<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(kWWarps * close_slot_floats(128) * sizeof(float))) != cudaSuccess ||
+      cudaFuncSetAttribute((const void *)k_best, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(4 * est_slot_floats(128) * sizeof(float))) != cudaSuccess) {
     cudaGetLastError();
     pimd_batch_destroy(b);
     return fail(PIMD_ECUDA, "cannot enable %d bytes of shared memory for the step kernels", wsmem128);
@@ -2861,9 +3162,8 @@ extern "C" pimd_status pimd_batch_run(pimd_batch *b, int64_t nsteps) {
   }
   const int cg = (b->capacity + 127) / 128;
   k_bctl<<<cg, 128, 0, b->stream>>>(b->d_reps, b->capacity, 1, nullptr);
-  k_bclose<<<b->grid_step, 128, 0, b->stream>>>(b->d_reps, b->d_step, b->d_counts + 0);
+  b->launches += 2 + launch_close_kernels(b);
   k_bctl<<<cg, 128, 0, b->stream>>>(b->d_reps, b->capacity, 2, nullptr);
-  b->launches += 3;
   BK(cudaGetLastError());
   return PIMD_OK;
 }
@@ -2899,8 +3199,9 @@ extern "C" pimd_status pimd_batch_estimators(pimd_batch *b, pimd_estimates *out)
   pimd_status st;
   if (b->dirty && (st = upload(b)) != PIMD_OK) return st;
   if (b->h_counts[3] > 0) {
-    k_best<<<std::min(b->grid_est, b->h_counts[3]), 128, 0, b->stream>>>(b->d_reps, b->d_est, b->d_counts + 3);
-    k_best_final<<<b->capacity, 128, 0, b->stream>>>(b->d_reps, b->capacity, b->d_eout);
+    k_best<<<std::min(b->grid_est, b->h_counts[3]), 128, (size_t)4 * b->est_slot * sizeof(float), b->stream>>>(
+        b->d_reps, b->d_est, b->d_counts + 3, b->est_slot);
+    k_best_final<<<b->capacity, 256, 0, b->stream>>>(b->d_reps, b->capacity, b->d_eout);
     b->launches += 2;
     BK(cudaGetLastError());
   }
@@ -3104,9 +3405,8 @@ extern "C" pimd_status pimd_batch_autotune(pimd_batch *b, int32_t steps_per_tria
   if (st == PIMD_OK) {
     const int cg = (b->capacity + 127) / 128;
     k_bctl<<<cg, 128, 0, b->stream>>>(b->d_reps, b->capacity, 1, nullptr);
-    k_bclose<<<b->grid_step, 128, 0, b->stream>>>(b->d_reps, b->d_step, b->d_counts + 0);
+    b->launches += 2 + launch_close_kernels(b);
     k_bctl<<<cg, 128, 0, b->stream>>>(b->d_reps, b->capacity, 2, nullptr);
-    b->launches += 3;
     if (cudaGetLastError() != cudaSuccess) st = fail(PIMD_ECUDA, "autotune close failed");
   }
   cudaEventDestroy(e0);
