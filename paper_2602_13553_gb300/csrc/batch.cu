@@ -430,8 +430,10 @@ __device__ __forceinline__ void bstep_mma(const RepDesc *__restrict__ Rp, int P,
 // q~' back from shared memory as its B operand.  3xTF32 throughout.
 constexpr int kWAtoms = 8;      // atoms per warp item
 constexpr int kWWarps = 4;      // warps per block
-constexpr int kWMaxP = 64;
 __host__ __device__ constexpr int wslot_floats(int P) { return 48 * (P + 4) + 128; }
+constexpr size_t item_smem(int P) {   // of a block: one slot per group of P / 32 warps (64 and 128 beads)
+  return (size_t)kWWarps / (P / 32) * wslot_floats(P) * sizeof(float);
+}
 __host__ __device__ constexpr int est_slot_floats(int P) { return 48 * (P + 4) + 32; }     // and 24 bead means
 __host__ __device__ constexpr int close_slot_floats(int P) { return 24 * (P + 4); }        // forces alone
 __host__ __device__ constexpr int wslot_floats_harm(int P) { return 24 * (P + 4) + 128; }   // no forces
@@ -474,14 +476,14 @@ __device__ __forceinline__ void frag_u32(const float4 &v, uint32_t (&a)[4]) {
 }
 
 // C_c[mode][atom] = M[mode][bead] S_c[bead][atom] for the three components of
-// a staged tile S ([c*8 + atom][bead], row stride P + 4), all mode tiles.
-template <int P>
+// a staged tile S ([c*8 + atom][bead], row stride P + 4), MTW mode tiles from mt0.
+template <int P, int MTW>
 __device__ __forceinline__ void fwd_tile(const float4 *__restrict__ thi, const float4 *__restrict__ tlo,
-                                         const float *__restrict__ S, float (&C)[(P + 15) / 16][3][4]) {
-  constexpr int PS = P + 4, MT = (P + 15) / 16, KS = P / 8;
+                                         const float *__restrict__ S, int mt0, float (&C)[MTW][3][4]) {
+  constexpr int PS = P + 4, KS = P / 8;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
-  for (int mt = 0; mt < MT; ++mt)
+  for (int mt = 0; mt < MTW; ++mt)
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -496,15 +498,32 @@ __device__ __forceinline__ void fwd_tile(const float4 *__restrict__ thi, const f
       split_tf32(S[so + 4], bh[c][1], bl[c][1]);
     }
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
+    for (int mt = 0; mt < MTW; ++mt) {
       uint32_t ah[4], al[4];
-      const int o = (mt * KS + ks) * 32 + lane;
+      const int o = ((mt0 + mt) * KS + ks) * 32 + lane;
       frag_u32(ld_frag(thi + o), ah);
       frag_u32(ld_frag(tlo + o), al);
 #pragma unroll
       for (int c = 0; c < 3; ++c) mma3(C[mt][c], ah, al, bh[c][0], bh[c][1], bl[c][0], bl[c][1]);
     }
   }
+}
+
+// Warps that share an item (8-atom tile): each takes two of its 16-row mode
+// (and bead) tiles, so every bead count keeps the accumulators, and with them
+// the registers, of 32 beads, and a few large items still fill an SM.  One warp
+// with four or eight tiles (168 and 255 registers, 12 and 8 warps an SM) took
+// 21.4 us a step at 512 molecules x 64 beads (15.7 so) and 59 us for a handful
+// of 128-bead items (34); many 64-bead items at once run as fast either way.
+__host__ __device__ constexpr int item_warps(int P) { return P <= 32 ? 1 : P / 32; }
+
+// Barrier of the W warps of an item (group `grp` of its block).
+template <int W>
+__device__ __forceinline__ void item_sync(int grp) {
+  if (W == 1)
+    __syncwarp();
+  else
+    asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(32 * W) : "memory");
 }
 
 // Shared-memory slot of one warp (floats): staged forces [c*8 + atom][bead]
@@ -516,8 +535,10 @@ __device__ __forceinline__ void fwd_tile(const float4 *__restrict__ thi, const f
 template <int P, bool kHarm = false>
 __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__restrict__ slot, uint64_t step,
                            int first) {
-  constexpr int PS = P + 4, MT = (P + 15) / 16, KS = P / 8;
+  constexpr int PS = P + 4, KS = P / 8, W = item_warps(P), MT = (P + 15) / 16 / W;   // MT: this warp's mode tiles
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int warp = threadIdx.x >> 5, wi = warp % W, grp = warp / W, mt0 = wi * MT;
+  const int il = wi * 32 + lane;   // thread of the item
   const int tile0 = tile * kWAtoms;
   const int na = min(kWAtoms, Rp->N - tile0);
   const size_t base = (size_t)tile0 * 3 * P;
@@ -532,7 +553,7 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
     const float *__restrict__ gF = Rp->F + base;
     const float *__restrict__ gX = Rp->d + base;
     const int nchunk = na * 3 * CPR;
-    for (int q = lane; q < nchunk; q += 32) {
+    for (int q = il; q < nchunk; q += 32 * W) {
       const int row = q / CPR, col = (q - row * CPR) * 4;
       const int a = row / 3, c = row - 3 * a;
       const int so = (c * 8 + a) * PS + col;
@@ -540,7 +561,7 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
       cp_async16(sX + so, gX + (size_t)row * P + col);
     }
     cp_async_commit();
-    for (int q = lane; q < (kWAtoms - na) * 3 * P; q += 32) {   // rows of missing atoms
+    for (int q = il; q < (kWAtoms - na) * 3 * P; q += 32 * W) {   // rows of missing atoms
       const int r = q / P, j = q - r * P;
       const int a = na + r / 3, c = r - 3 * (r / 3);
       if (!kHarm) sF[(c * 8 + a) * PS + j] = 0.f;
@@ -568,12 +589,12 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
     sgv[aa] = __ldg(Rp->sigvf + tile0 + a);
   }
   cp_async_wait_all();
-  __syncwarp();
+  item_sync<W>(grp);
 
-  // v~ of update iteration j (modes 16 (j/2) + g + 8 (j%2), atoms 2t, 2t + 1),
+  // v~ of update iteration j (modes 16 (mt0 + j/2) + g + 8 (j%2), atoms 2t, 2t + 1),
   // loaded one iteration ahead; the centroid mode and padding rows read none
   auto load_v = [&](int j, float (&vv)[2][3]) {
-    const int k = 16 * (j >> 1) + g + 8 * (j & 1);
+    const int k = 16 * (mt0 + (j >> 1)) + g + 8 * (j & 1);
     const bool on = k < P && k != 0;
 #pragma unroll
     for (int aa = 0; aa < 2; ++aa) {
@@ -588,13 +609,13 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
   float *sQ = sX;   // q~ [c][mode][atom] once the deviations are transformed
   float C[MT][3][4];
   // forward transform of the deviations: q~_c = M d_c
-  fwd_tile<P>(fhi, flo, sX, C);
-  __syncwarp();   // every lane is done with the staged deviations
+  fwd_tile<P, MT>(fhi, flo, sX, mt0, C);
+  item_sync<W>(grp);   // everyone is done with the staged deviations
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const int k = 16 * mt + g;
+      const int k = 16 * (mt0 + mt) + g;
       *reinterpret_cast<float2 *>(sQ + (c * P + k) * 8 + 2 * t) = make_float2(C[mt][c][0], C[mt][c][1]);
       if (k + 8 < P)
         *reinterpret_cast<float2 *>(sQ + (c * P + k + 8) * 8 + 2 * t) = make_float2(C[mt][c][2], C[mt][c][3]);
@@ -603,13 +624,13 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
   // over the staged forces
   float *sG = sF;
   if (!kHarm) {
-  fwd_tile<P>(fhi, flo, sF, C);
-  __syncwarp();   // every lane is done with the staged forces
+  fwd_tile<P, MT>(fhi, flo, sF, mt0, C);
+  item_sync<W>(grp);   // everyone is done with the staged forces
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const int k = 16 * mt + g;
+      const int k = 16 * (mt0 + mt) + g;
       *reinterpret_cast<float2 *>(sG + (c * P + k) * 8 + 2 * t) = make_float2(C[mt][c][0], C[mt][c][1]);
       if (k + 8 < P)
         *reinterpret_cast<float2 *>(sG + (c * P + k + 8) * 8 + 2 * t) = make_float2(C[mt][c][2], C[mt][c][3]);
@@ -619,14 +640,14 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
   // {2t, 2t + 1}, the same (mode, atom) slots it wrote; q~' replaces q~
   load_v(0, vv);
   double xpre = 0.0, vpre = 0.0;   // this lane's centroid entry, used after the update
-  if (lane < 3 * na) {
+  if (wi == 0 && lane < 3 * na) {
     xpre = Rp->xc[(size_t)tile0 * 3 + lane];
     vpre = Rp->v0[(size_t)tile0 * 3 + lane];
   }
 #pragma unroll 1
   for (int j = 0; j < 2 * MT; ++j) {
     if (j + 1 < 2 * MT) load_v(j + 1, vn);
-    const int k = 16 * (j >> 1) + g + 8 * (j & 1);
+    const int k = 16 * (mt0 + (j >> 1)) + g + 8 * (j & 1);
     if (k >= P) {
 #pragma unroll
       for (int aa = 0; aa < 2; ++aa)
@@ -704,9 +725,9 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
 #pragma unroll
       for (int c = 0; c < 3; ++c) vv[aa][c] = vn[aa][c];
   }
-  __syncwarp();
+  item_sync<W>(grp);
   // centroid mode in FP64, one (atom, component) per lane: q~_0 = sqrt(P) xc
-  if (lane < 3 * na) {
+  if (wi == 0 && lane < 3 * na) {
     const int a = lane / 3, c = lane - 3 * a;
     const int i = tile0 + a;
     const size_t ic = (size_t)tile0 * 3 + lane;
@@ -740,7 +761,7 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
     sxc[lane] = x;
     sf0[lane] = xw;   // this lane's own entry, read above
   }
-  // inverse: d'_c = M^T q~'_c, bead tiles of 16 as the M dimension
+  // inverse: d'_c = M^T q~'_c, bead tiles of 16 as the M dimension, this warp's two
   const float4 *__restrict__ ihi = Rp->mia_hi;
   const float4 *__restrict__ ilo = Rp->mia_lo;
   float D[MT][3][4];
@@ -762,14 +783,14 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
 #pragma unroll
     for (int bt = 0; bt < MT; ++bt) {
       uint32_t ah[4], al[4];
-      const int o = (bt * KS + ks) * 32 + lane;
+      const int o = ((mt0 + bt) * KS + ks) * 32 + lane;
       frag_u32(ld_frag(ihi + o), ah);
       frag_u32(ld_frag(ilo + o), al);
 #pragma unroll
       for (int c = 0; c < 3; ++c) mma3(D[bt][c], ah, al, bh[c][0], bh[c][1], bl[c][0], bl[c][1]);
     }
   }
-  __syncwarp();   // the centroids in sxc are visible to every lane
+  item_sync<W>(grp);   // the centroids in sxc are visible to everyone
   // new deviations, and the skin criterion: bead spread of the oxygens
   // (water-like systems, which carry reference centroids)
   const bool water = Rp->cref != nullptr;
@@ -779,7 +800,7 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
   for (int bt = 0; bt < MT; ++bt)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int bead = 16 * bt + g + 8 * (q >> 1);
+      const int bead = 16 * (mt0 + bt) + g + 8 * (q >> 1);
       const int a = 2 * t + (q & 1);
       if (bead < P && a < na) {
 #pragma unroll
@@ -797,7 +818,7 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
     }
   // centroid drift of the oxygens since the last rebuild
   float vdisp = 0.f;
-  if (water && lane < na && (tile0 + lane) % 3 == 0) {
+  if (water && wi == 0 && lane < na && (tile0 + lane) % 3 == 0) {
     const int m = (tile0 + lane) / 3;
     double s2 = 0.0;
 #pragma unroll
@@ -815,28 +836,38 @@ __device__ void bstep_warp(const RepDesc *__restrict__ Rp, int tile, float *__re
     vdev = fmaxf(vdev, __shfl_xor_sync(0xffffffffu, vdev, o));
   }
   if (water && lane < 2) skin_max(Rp->ctl, lane, lane == 0 ? vdisp : vdev);
-  __syncwarp();   // the slot is free for the next item
+  item_sync<W>(grp);   // the slot is free for the next item
 }
 
-// Warp items (replica, 8-atom tile) of the bead counts in {8, 16, 32, 64}:
-// the 64-bead items are the range [0, counts[9]) of the step list, claimed
-// from *next; the 8-, 16- and 32-bead items the range [counts[9], counts[4]),
-// run by the kSmall instance, whose smaller accumulator tiles fit four blocks
-// per SM (128 registers, 7.4 KB warp slots) where the 64-bead instance fits
-// three.  Lane 0 of each warp claims the next item (counters reset by k_bctl).
-template <bool kSmall>
-__global__ void __launch_bounds__(kWWarps * 32, kSmall ? 4 : 3) k_bstep_w(const RepDesc *__restrict__ reps,
-                                                                         const int2 *__restrict__ items,
-                                                                         const int *__restrict__ counts, int *next,
-                                                                         int slot_floats) {
+// Items (replica, 8-atom tile) of the bead counts in {8, 16, 32, 64, 128}, claimed
+// from *next (reset by k_bctl) by the warps that share one: kClass 0 the 8-, 16-
+// and 32-bead items, the range [counts[9], counts[4]) of the step list, one warp
+// each; 1 the 64-bead ones, [0, counts[9]), two; 2 the 128-bead ones, [counts[4],
+// counts[7]), four.
+template <int kClass>
+__global__ void __launch_bounds__(kWWarps * 32, 4) k_bstep_w(const RepDesc *__restrict__ reps,
+                                                            const int2 *__restrict__ items,
+                                                            const int *__restrict__ counts, int *next,
+                                                            int slot_floats) {
   extern __shared__ __align__(16) float wsm[];
-  float *slot = wsm + (threadIdx.x >> 5) * slot_floats;
-  const int lo = kSmall ? counts[9] : 0, hi = kSmall ? counts[4] : counts[9];
+  constexpr int W = kClass == 0 ? 1 : (kClass == 1 ? 2 : 4);
+  __shared__ int s_it[kWWarps];
+  const int warp = threadIdx.x >> 5, grp = warp / W;
+  float *slot = wsm + grp * slot_floats;
+  const int lo = kClass == 0 ? counts[9] : (kClass == 1 ? 0 : counts[4]);
+  const int hi = kClass == 0 ? counts[4] : (kClass == 1 ? counts[9] : counts[7]);
   const int lane = threadIdx.x & 31;
   for (;;) {
     int it = 0;
-    if (lane == 0) it = lo + atomicAdd(next, 1);
-    it = __shfl_sync(0xffffffffu, it, 0);
+    if (W == 1) {
+      if (lane == 0) it = lo + atomicAdd(next, 1);
+      it = __shfl_sync(0xffffffffu, it, 0);
+    } else {
+      if (warp % W == 0 && lane == 0) s_it[grp] = lo + atomicAdd(next, 1);
+      item_sync<W>(grp);
+      it = s_it[grp];
+      item_sync<W>(grp);   // read by all before the next claim
+    }
     if (it >= hi) break;
     const int2 w = items[it];
     const RepDesc *__restrict__ Rp = reps + w.x;
@@ -844,67 +875,44 @@ __global__ void __launch_bounds__(kWWarps * 32, kSmall ? 4 : 3) k_bstep_w(const 
     if (!ctl[kCtlActive]) continue;
     const uint64_t step = (uint64_t)ctl[kCtlStep];
     const int first = (int)ctl[kCtlFirst];
-    if (kSmall) {
+    if (kClass == 0) {
       switch (Rp->P) {
         case 8: bstep_warp<8>(Rp, w.y, slot, step, first); break;
         case 16: bstep_warp<16>(Rp, w.y, slot, step, first); break;
         case 32: bstep_warp<32>(Rp, w.y, slot, step, first); break;
         default: break;
       }
-    } else if (Rp->P == 64) {
-      bstep_warp<64>(Rp, w.y, slot, step, first);
+    } else if (kClass == 1) {
+      if (Rp->P == 64) bstep_warp<64>(Rp, w.y, slot, step, first);
+    } else if (Rp->P == 128) {
+      bstep_warp<128>(Rp, w.y, slot, step, first);
     }
-  }
-}
-
-// Warp items of bead count 128, the range [counts[4], counts[7]) of the step
-// list: the same per-item arithmetic as k_bstep_w in a kernel of its own,
-// whose larger accumulator tiles (eight mode tiles) and 26 KB warp slots
-// would otherwise set the register and shared-memory budget of the smaller
-// bead counts; claimed from the counter *next (reset by k_bctl).
-__global__ void __launch_bounds__(kWWarps * 32, 1) k_bstep_w128(const RepDesc *__restrict__ reps,
-                                                               const int2 *__restrict__ items,
-                                                               const int *__restrict__ counts, int *next) {
-  extern __shared__ __align__(16) float wsm[];
-  float *slot = wsm + (threadIdx.x >> 5) * wslot_floats(128);
-  const int lo = counts[4], hi = counts[7];
-  const int lane = threadIdx.x & 31;
-  for (;;) {
-    int it = 0;
-    if (lane == 0) it = lo + atomicAdd(next, 1);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= hi) break;
-    const int2 w = items[it];
-    const RepDesc *__restrict__ Rp = reps + w.x;
-    const long long *ctl = Rp->ctl;
-    if (!ctl[kCtlActive] || Rp->P != 128) continue;
-    bstep_warp<128>(Rp, w.y, slot, (uint64_t)ctl[kCtlStep], (int)ctl[kCtlFirst]);
   }
 }
 
 // The warp-item step of one system (a single-system handle in split
 // precision, bead counts 8, 16, 32, 64, 128): the same per-item arithmetic as
-// k_bstep_w, with the step index read from the handle's counter.  Warps take
-// the 8-atom tiles in turn.  For water-like systems the last warp to finish
+// k_bstep_w, with the step index read from the handle's counter.  Items (8-atom
+// tiles) are taken in turn.  For water-like systems the last warp to finish
 // turns the step's skin maxima (squared FP32 bit patterns in ctl) into the
 // one conservative (drift, spread) pair that the neighbour-list check reads,
 // and clears them for the next step (threadfence-and-count, no waiting).
-// kClass: 0 the 32-bead instance (128 registers, four blocks per SM), 1 the
-// 64-bead one (three blocks), 2 the 128-bead one (eight mode tiles, one
-// block's share of registers), 3 the 8- and 16-bead one (one mode tile, six
+// kClass: 0, 1, 2 the 32-, 64- and 128-bead instances (one, two and four warps an
+// item, four blocks per SM), 3 the 8- and 16-bead one (one mode tile, six
 // blocks: its short items leave the memory waits exposed unless more warps
 // share an SM; 8 and 16 beads step 15% and 10% faster than at four blocks).
 template <int kClass, bool kHarm>
-__global__ void __launch_bounds__(kWWarps * 32, kClass == 3 ? 6 : (kClass == 0 ? 4 : (kClass == 1 ? 3 : 1)))
+__global__ void __launch_bounds__(kWWarps * 32, kClass == 3 ? 6 : 4)
     k_sstep_w(const RepDesc *__restrict__ Rp, const int64_t *__restrict__ stepp, int step_off, int first,
               int slot_floats, double *blkmax, unsigned *done) {
   extern __shared__ __align__(16) float wsm[];
-  float *slot = wsm + (threadIdx.x >> 5) * slot_floats;
+  constexpr int W = kClass == 1 ? 2 : (kClass == 2 ? 4 : 1);
+  float *slot = wsm + (threadIdx.x >> 5) / W * slot_floats;
   const int lane = threadIdx.x & 31;
   const int ntiles = (Rp->N + kWAtoms - 1) / kWAtoms;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   const uint64_t step = (uint64_t)(*stepp + step_off);
-  for (int tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; tile < ntiles; tile += nw) {
+  for (int tile = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) / W; tile < ntiles; tile += nw / W) {
     if (kClass == 3) {
       if (Rp->P == 8)
         bstep_warp<8, kHarm>(Rp, tile, slot, step, first);
@@ -1294,7 +1302,7 @@ __device__ __forceinline__ void bclose_warp(const RepDesc &R, int tile, float *_
   cp_async_wait_all();
   __syncwarp();
   float C[MT][3][4];
-  fwd_tile<P>(R.mfa_hi, R.mfa_lo, sF, C);
+  fwd_tile<P, MT>(R.mfa_hi, R.mfa_lo, sF, 0, C);
   const bool bath = R.integrator == 1 && R.thermo;
   const float half = 0.5f * (float)R.dt;
   float *__restrict__ vkg = R.vk + base;
@@ -2307,7 +2315,6 @@ struct pimd_batch {
   // the 64-bead warp items, [10] claim counter of the smaller warp items
   int h_counts[16] = {0};
   int est_slot = 0;   // floats of shared memory per warp of the estimator pass
-  int wslot = wslot_floats(64);   // floats of shared memory per warp of the 64-bead warp-item kernel
   int grid_w = 0;         // its blocks (persistent grid)
   int grid_ws = 0;        // blocks of the 8-, 16-, 32-bead warp-item kernel
   bool w64_items = false, wsmall_items = false;   // which warp-item kernels have items
@@ -2476,14 +2483,14 @@ void launch_step_kernels(pimd_batch *b) {
     cudaStreamWaitEvent(b->side, b->fork_ev, 0);
   }
   if (b->w64_items)
-    k_bstep_w<false><<<b->grid_w, kWWarps * 32, (size_t)kWWarps * b->wslot * sizeof(float), b->stream>>>(
-        b->d_reps, b->d_step, b->d_counts, b->d_counts + 5, b->wslot);
+    k_bstep_w<1><<<b->grid_w, kWWarps * 32, item_smem(64), b->stream>>>(
+        b->d_reps, b->d_step, b->d_counts, b->d_counts + 5, wslot_floats(64));
   if (b->wsmall_items)
-    k_bstep_w<true><<<b->grid_ws, kWWarps * 32, (size_t)kWWarps * wslot_floats(32) * sizeof(float), s2>>>(
+    k_bstep_w<0><<<b->grid_ws, kWWarps * 32, (size_t)kWWarps * wslot_floats(32) * sizeof(float), s2>>>(
         b->d_reps, b->d_step, b->d_counts, b->d_counts + 10, wslot_floats(32));
   if (b->w128_items)
-    k_bstep_w128<<<b->grid_w128, kWWarps * 32, (size_t)kWWarps * wslot_floats(128) * sizeof(float), b->stream>>>(
-        b->d_reps, b->d_step, b->d_counts, b->d_counts + 8);
+    k_bstep_w<2><<<b->grid_w128, kWWarps * 32, item_smem(128), b->stream>>>(
+        b->d_reps, b->d_step, b->d_counts, b->d_counts + 8, wslot_floats(128));
   if (b->block_items) k_bstep<<<b->grid_step, 128, 0, s2>>>(b->d_reps, b->d_step, b->d_counts);
   if (fork) {
     cudaEventRecord(b->join_ev, b->side);
@@ -2649,18 +2656,6 @@ cudaError_t split_warp_prepare() {
   int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void *)k_sstep_w<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kWWarps * wslot_floats(32) * sizeof(float)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void *)k_sstep_w<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kWWarps * wslot_floats(64) * sizeof(float)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void *)k_sstep_w<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kWWarps * wslot_floats(128) * sizeof(float)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void *)k_sstep_w<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kWWarps * wslot_floats_harm(128) * sizeof(float)));
   if (e == cudaSuccess) g_sw_nsm = nsm > 0 ? nsm : 152;
   return e;
 }
@@ -2732,12 +2727,11 @@ cudaError_t launch_step_split_warp(const void *desc, int N, int P, const int64_t
   const int nsm = g_sw_nsm;
   const int cls = P == 128 ? 2 : (P == 64 ? 1 : (P == 32 ? 0 : 3));
   const int slot = harm ? wslot_floats_harm(P) : wslot_floats(P);
-  // resident blocks per SM (registers, shared memory)
-  const int per_sm = cls == 2 ? 2 : (cls == 1 ? 3 : (cls == 0 ? 4 : 6));
-  const int smem = (int)(kWWarps * slot * sizeof(float));
+  // resident blocks per SM (registers, shared memory); items per block
+  const int per_sm = cls == 3 ? 6 : 4, per_blk = kWWarps / item_warps(P);
+  const int smem = (int)(per_blk * slot * sizeof(float));
   const int ntiles = (N + kWAtoms - 1) / kWAtoms;
-  const int warps = std::min(ntiles, nsm * per_sm * kWWarps);
-  const int grid = std::max(1, (warps + kWWarps - 1) / kWWarps);
+  const int grid = std::max(1, std::min((ntiles + per_blk - 1) / per_blk, nsm * per_sm));
   const RepDesc *d = reinterpret_cast<const RepDesc *>(desc);
   auto go = [&](auto kernel) { kernel<<<grid, kWWarps * 32, smem, s>>>(d, step, step_off, first, slot, blkmax, done); };
   switch (cls) {
@@ -2798,21 +2792,15 @@ extern "C" pimd_status pimd_batch_create(int32_t max_replicas, void *stream, pim
     pimd_batch_destroy(b);
     return fail(PIMD_ECUDA, "cannot enable %zu bytes of shared memory for the neighbour kernel", kNbrSmem);
   }
-  const int wsmem = (int)(kWWarps * wslot_floats(kWMaxP) * sizeof(float));
-  const int wsmem128 = (int)(kWWarps * wslot_floats(128) * sizeof(float));
-  if (cudaFuncSetAttribute((const void *)k_bstep_w<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, wsmem) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute((const void *)k_bstep_w<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute((const void *)k_bstep_w<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(kWWarps * wslot_floats(32) * sizeof(float))) != cudaSuccess ||
-      cudaFuncSetAttribute((const void *)k_bstep_w128, cudaFuncAttributeMaxDynamicSharedMemorySize, wsmem128) !=
-          cudaSuccess ||
       cudaFuncSetAttribute((const void *)k_bclose_w<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(kWWarps * close_slot_floats(128) * sizeof(float))) != cudaSuccess ||
       cudaFuncSetAttribute((const void *)k_best, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(4 * est_slot_floats(128) * sizeof(float))) != cudaSuccess) {
     cudaGetLastError();
     pimd_batch_destroy(b);
-    return fail(PIMD_ECUDA, "cannot enable %d bytes of shared memory for the step kernels", wsmem128);
+    return fail(PIMD_ECUDA, "cannot enable the shared memory of the step kernels");
   }
   b->nsm = nsm;
   // persistent grids: every SM filled to the kernel's occupancy limit
@@ -2822,13 +2810,13 @@ extern "C" pimd_status pimd_batch_create(int32_t max_replicas, void *stream, pim
     return nsm * n;
   };
   b->grid_step = occ((const void *)k_bstep);
-  b->grid_w128 = occ((const void *)k_bstep_w128, (size_t)kWWarps * wslot_floats(128) * sizeof(float));
-  b->grid_ws = occ((const void *)k_bstep_w<true>, (size_t)kWWarps * wslot_floats(32) * sizeof(float));
+  b->grid_w128 = occ((const void *)k_bstep_w<2>, item_smem(128));
+  b->grid_ws = occ((const void *)k_bstep_w<0>, (size_t)kWWarps * wslot_floats(32) * sizeof(float));
   b->wblocks_sm = 0;
   {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void *)k_bstep_w<false>, kWWarps * 32,
-                                                      (size_t)kWWarps * b->wslot * sizeof(float)) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void *)k_bstep_w<1>, kWWarps * 32, item_smem(64)) !=
+            cudaSuccess ||
         nb < 1)
       nb = 1;
     b->wblocks_sm = nb;
@@ -3343,15 +3331,17 @@ extern "C" pimd_status pimd_batch_autotune(pimd_batch *b, int32_t steps_per_tria
   if (!b->ffma && std::find(classes.begin(), classes.end(), 64) != classes.end()) {
     if (b->dirty && (st = upload(b)) != PIMD_OK) return st;
     int nbmax = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbmax, (const void *)k_bstep_w<false>, kWWarps * 32,
-                                                      (size_t)kWWarps * b->wslot * sizeof(float)) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbmax, (const void *)k_bstep_w<1>, kWWarps * 32, item_smem(64)) !=
+            cudaSuccess ||
         nbmax < 1)
       nbmax = 1;
-    // each candidate: one untimed step (caches and clocks settle), then the
-    // faster of two timed trials; a smaller grid than the occupancy limit must
-    // win by more than 3% (the timings are a few milliseconds and noisy)
+    // each candidate, the occupancy limit and the two below it: one untimed
+    // step (caches and clocks settle), then the faster of two timed trials; a
+    // smaller grid than the limit must win by more than 3% (the timings are a
+    // few milliseconds and noisy)
+    const int nbmin = std::max(1, nbmax - 2);
     std::vector<float> tms(nbmax + 1, 1e30f);
-    for (int nb = nbmax; nb >= 1 && st == PIMD_OK; --nb) {
+    for (int nb = nbmax; nb >= nbmin && st == PIMD_OK; --nb) {
       b->wblocks_sm = nb;
       b->grid_w = b->nsm * nb;
       if (launch_one_step(b, nullptr, nullptr) != cudaSuccess) return fail(PIMD_ECUDA, "autotune step failed");
@@ -3363,7 +3353,7 @@ extern "C" pimd_status pimd_batch_autotune(pimd_batch *b, int32_t steps_per_tria
       }
     }
     int best = nbmax;
-    for (int nb = nbmax - 1; nb >= 1; --nb)
+    for (int nb = nbmax - 1; nb >= nbmin; --nb)
       if (tms[nb] < 0.97f * tms[best]) best = nb;
     b->wblocks_sm = best;
     b->wtuned = best;
