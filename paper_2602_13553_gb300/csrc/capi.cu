@@ -191,7 +191,6 @@ struct pimd_handle {
   double *inv_mm = nullptr, *sigv = nullptr, *mass_mm = nullptr, *kspring = nullptr;
   double *cA = nullptr, *sA = nullptr, *wsA = nullptr;
   double *c1 = nullptr, *c2 = nullptr, *lam = nullptr, *mu = nullptr, *imu = nullptr;
-  double *Tf = nullptr;   // folded forward transform, [P/2 + 1][P]
   char *tab_lo = nullptr, *tab_hi = nullptr;   // the tables' part of the arena
   // FP64 normal-mode step: folded transforms in fixed point, A O A as one map
   // per mode, [2][N] B(h/2) and B(h) durations over m mvv2e
@@ -348,7 +347,7 @@ static StepArgs step_args(pimd_handle *h) {
   a.N = h->N;
   a.P = h->P;
   a.A = h->A_step;
-  a.mt = ModeTables{h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf,
+  a.mt = ModeTables{h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu,
                     h->fTf, h->fTi, h->fem, h->map6, 1.0 / std::sqrt((double)h->P)};
   a.inv_mm = h->inv_mm;
   a.mu_one = h->mu_one;
@@ -805,7 +804,6 @@ static void carve(pimd_handle *h, Carver &c) {
   h->lam = c.take<double>(P);
   h->mu = c.take<double>(P);
   h->imu = c.take<double>(P);
-  h->Tf = c.take<double>((size_t)(P / 2 + 1) * P);
   h->fTf = c.take<int4>((size_t)fix_pairs(P) * P);
   h->fTi = c.take<int4>((size_t)fix_pairs(P) * P);
   h->map6 = c.take<double>((size_t)6 * P);
@@ -1189,7 +1187,6 @@ extern "C" pimd_status pimd_create(const pimd_system *sys, int32_t P, double T, 
   img.put(h->lam, tb.lam);
   img.put(h->mu, tb.mu);
   img.put(h->imu, tb.imu);
-  img.put(h->Tf, tb.Tf);
   h->mu_one = std::all_of(tb.imu.begin(), tb.imu.end(), [](double m) { return m == 1.0; });
   aoa_map(P, tb, h->thermostat == PIMD_THERMO_PILE_L, map6);
   img.put(h->map6, map6);
@@ -1361,7 +1358,7 @@ extern "C" pimd_status pimd_estimators(pimd_handle *h, pimd_estimates *out) {
   a.P = P;
   a.A = h->A_est;
   a.method = h->method;
-  a.mt = ModeTables{h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu, h->Tf,
+  a.mt = ModeTables{h->cA, h->sA, h->wsA, h->c1, h->c2, h->lam, h->mu, h->imu,
                     h->fTf, h->fTi, h->fem, h->map6, 1.0 / std::sqrt((double)P)};
   a.mass_mm = h->mass_mm;
   a.x = h->x;

@@ -152,12 +152,10 @@ struct ModeTables {
   const double *lam;   // [P] lambda_k (Eq. A2)
   const double *mu;    // [P] fictitious-mass factor mu_k: m^(k) = mu_k m (fmmode, fmass)
   const double *imu;   // [P] 1 / mu_k
-  // folded forward transform (H = floor(P/2)), [H + 1][P]:
-  //   Tf[i][k]: k <= H: M[k][i]; k > H: M[k][P - (H + 1 + i)] (0 past the row)
-  const double *Tf;
-  // the folded transforms in fixed point (fixed.cuh): [fix_pairs(P)][P], limbs
-  // (h, l) of terms 2p and 2p + 1, scaled by 2^(55 - fem); the inverse's terms
-  // for bead j are Ti[i][j]: j <= H: M[i][j]; j > H: M[H + 1 + i][P - j]
+  // the folded transforms (H = floor(P/2)) in fixed point (fixed.cuh):
+  // [fix_pairs(P)][P], limbs (h, l) of terms i = 2p and 2p + 1, scaled by
+  // 2^(55 - fem).  Term i of mode k is M[k][i] (k <= H) or M[k][P - (H + 1 + i)]
+  // (k > H; 0 past the row); of bead j, M[i][j] (j <= H) or M[H + 1 + i][P - j]
   const int4 *fTf, *fTi;
   int fem;
   // A(h/2) O(h) A(h/2) of BAOAB per mode, [6][P]: q' = m0 q + m1 v + m2 n,
@@ -306,7 +304,7 @@ struct ForceArgs {
 struct SplitStepArgs {
   int N, P, A;
   const float *Mtf;            // [P][P] FP32 copy of M^T
-  const float *Tff, *Tif;      // [P/2 + 1][P] FP32 folded forward / inverse tables (as ModeTables::Tf, Ti)
+  const float *Tff, *Tif;      // [P/2 + 1][P] FP32 folded forward / inverse tables (terms as of ModeTables::fTf, fTi)
   const float *cAf, *sAf, *wsAf, *c1f, *c2f;   // FP32 mode coefficients (k >= 1)
   double tA, c1_0, c2_0;       // centroid: drift time of one A, O coefficients
   const double *inv_mm, *sigv; // [N]

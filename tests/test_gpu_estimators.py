@@ -40,3 +40,20 @@ def test_estimators_match_oracle(orc, pimd, N, P, method):
         assert scalar_err(got[k], want[k]) < TOL, k
     # K_PR is a difference of its kinetic term 3 P N kB T / 2 and the springs
     assert abs(got["K_PR"] - want["K_PR"]) < TOL * 1.5 * P * N * 8.617333262e-5 * 300.0
+
+
+@pytest.mark.parametrize("N,P,method", [(1, 3, 0), (701, 8, 0), (333, 9, 1)])
+def test_sums_over_a_wide_range(orc, pimd, N, P, method):
+    """Kinetic terms over 24 decades, largest first, last and in between: every
+    sum is rounded once, its terms within 2^-51 of themselves, so 1e-14 leaves
+    a factor of 20."""
+    x0, mass = inputs.harmonic(N, P, seed=N, std=0.1)
+    g = np.random.default_rng(N + P)
+    mass = mass * 10.0 ** g.uniform(-6.0, 6.0, N)
+    v0 = g.standard_normal(x0.shape) * 10.0 ** g.uniform(-6.0, 6.0, (1, N, 1))
+    kw = dict(T=300.0, dt=2.5e-4, potential=0, ff=(OMEGA_HO,), seed=3, method=method)
+    s = pimd.Simulation(x0, mass, v0=v0, **kw)
+    got = s.estimators()
+    s.close()
+    want = orc.Sim(x0, mass, v0=v0, **kw).estimators()
+    assert coord_err(got["K_mode"], want["K_mode"]) < 1e-14
