@@ -494,13 +494,18 @@ static SplitForceArgs split_force_args(pimd_handle *h) {
   a.Wpart = h->Wpart;
   a.step_inc = nullptr;
   a.kspring = h->kspring;
-  a.kb = f.kb;
-  a.r0 = f.r0;
-  a.kth = f.kth;
-  a.th0 = f.th0;
-  a.eps = f.eps;
-  a.sig = f.sig;
-  a.rc = f.rc;
+  for (int c = 0; c < 3; ++c) {
+    a.ff.L[c] = (float)f.nb.box[c];
+    a.ff.iL[c] = (float)f.nb.invbox[c];
+  }
+  a.ff.rc2 = (float)(f.rc * f.rc);
+  a.ff.sig2 = (float)(f.sig * f.sig);
+  a.ff.e4 = (float)(4.0 * f.eps);
+  a.ff.e24 = (float)(24.0 * f.eps);
+  a.ff.kb = (float)f.kb;
+  a.ff.r0 = (float)f.r0;
+  a.ff.kth = (float)f.kth;
+  a.ff.th0 = (float)f.th0;
   a.nb = f.nb;
   a.check_nbr = 0;
   return a;
@@ -529,7 +534,8 @@ static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, int advance
         });
         if (st != PIMD_OK) return st;
       } else {
-        sa.check_nbr = 1;   // the skin test and any rebuild: inside the force kernel of a small system
+        // a small system's skin test and any rebuild are inside its force kernel
+        sa.check_nbr = !split_lists_apart(h->nmol, h->P);
       }
       if (from_outside || split_lists_apart(h->nmol, h->P)) {
         st = enqueue(h, PIMD_KIND_NBR, 1, [&] { return launch_nbr_lists(sa.nb, from_outside, h->stream); });
@@ -551,7 +557,8 @@ static pimd_status enqueue_forces(pimd_handle *h, bool from_outside, int advance
       });
       if (st != PIMD_OK) return st;
     } else {
-      fa.check_nbr = 1;   // the skin test and any rebuild: inside the force kernel of a small system
+      // a small system's skin test and any rebuild are inside its force kernel
+      fa.check_nbr = !water_lists_apart(h->nmol, h->P);
     }
     if (from_outside || water_lists_apart(h->nmol, h->P)) {
       st = enqueue(h, PIMD_KIND_NBR, 1, [&] { return launch_nbr_lists(fa.nb, from_outside, h->stream); });

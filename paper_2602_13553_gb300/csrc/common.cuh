@@ -324,6 +324,14 @@ struct SplitStepArgs {
   uint64_t seed;
 };
 
+// The water-like model's constants in FP32 (rounded once on the host: an FP64
+// conversion in the kernel costs a slot of the FP64 pipe in every warp).
+struct SplitFF {
+  float L[3], iL[3];
+  float rc2, sig2, e4, e24;    // rc^2, sigma^2, 4 eps, 24 eps
+  float kb, r0, kth, th0;
+};
+
 struct SplitForceArgs {
   int N, P, nmol;
   const double *xc;            // [N][3]
@@ -334,7 +342,7 @@ struct SplitForceArgs {
   int64_t *step_inc;           // if not null, block 0 advances the step counter by inc
   int inc;
   const double *kspring;
-  double kb, r0, kth, th0, eps, sig, rc;
+  SplitFF ff;                  // water
   NbrList nb;
   int check_nbr;               // as ForceArgs::check_nbr
 };

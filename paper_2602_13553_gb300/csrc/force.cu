@@ -72,9 +72,15 @@ __global__ void __launch_bounds__(256) k_force_harmonic_f64(ForceArgs a) {
 //    closer than its range, and systems it does not fit, take the FP64
 //    expressions on the FP64 positions;
 //  * a system with many units takes them whole, one warp each (split = 1: no
-//    reduction, four units to a block); a small one splits a unit's neighbour
-//    list over `split` warps and gives its bonds and its angle to two more, one
-//    unit to a block, partial sums joined in shared memory in a fixed order.
+//    reduction, four units to a block); a smaller one splits a unit's neighbour
+//    list over `split` warps, which also take the step's list check, and gives
+//    its bonds and angle to one more that starts at once; the partial sums are
+//    joined as integers, a component to a warp, and converted once.
+// Measured, us a launch: 512 molecules x 64 beads 172 in FP64, now about 37 (FP64
+// instructions 10.6 and integer issue 11 of it; three blocks fit an SM).  With
+// seven list warps, FP64 partial sums and two bonded warps behind the list check
+// against now: 64 x 32 beads 11.1 / 10.4 (16.7 in FP64), 100 x 12 13.2 / 11.1,
+// 125 x 16 with the diagonal virial 16.1 / 13.5.
 // A neighbour's bucket (j mod NS) decides its warp, so every sum depends only on
 // the set of interacting pairs: a rebuilt list cannot change a bit.
 // kDiag (anisotropic barostat) also sums the diagonal of the virial tensor,
@@ -83,11 +89,11 @@ struct Bonded {
   double fO[3], fH[2][3], U, W, w3[3];
 };
 
-// O-H bonds, U = 1/2 kb (r - r0)^2 each (what & 1), and the H-O-H angle, U =
-// 1/2 kth (theta - th0)^2 (what & 2), of molecule m at bead k.
+// O-H bonds, U = 1/2 kb (r - r0)^2 each, and the H-O-H angle, U = 1/2 kth
+// (theta - th0)^2, of molecule m at bead k.
 template <bool kDiag>
 __device__ __forceinline__ void bonded_f64(const ForceArgs &a, int m, int k, const double (&L)[3],
-                                           const double (&iL)[3], int what, Bonded &o) {
+                                           const double (&iL)[3], Bonded &o) {
   const int P = a.P;
   const double *x = a.x + (size_t)9 * m * P + k;
   double d[2][3], r2[2], ir[2];
@@ -99,7 +105,7 @@ __device__ __forceinline__ void bonded_f64(const ForceArgs &a, int m, int k, con
       double e = x[(3 + 3 * h + c) * P] - xo;
       // the minimum image, only where a component reaches half a box (the
       // comparison of high words may fall to either side of a tie, as rint may)
-      if ((__double2hiint(e) & 0x7fffffff) >= __double2hiint(0.5 * L[c])) e = mic(e, L[c], iL[c]);
+      if ((__double2hiint(e) & 0x7fffffff) >= __double2hiint(L[c]) - 0x100000) e = mic(e, L[c], iL[c]);
       d[h][c] = e;
     }
   }
@@ -109,32 +115,27 @@ __device__ __forceinline__ void bonded_f64(const ForceArgs &a, int m, int k, con
     ir[h] = rsqrt(r2[h]);
   }
   o.U = o.W = 0.0;
-  // H force h: gd[h] d_h + ga[h] d_{1-h}
-  double gd[2] = {0.0, 0.0}, ga = 0.0;
-  if (what & 1) {
+  double gd[2], ga;   // H force h: gd[h] d_h + ga d_{1-h}
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      // r - r0 with r = r2 ir corrected by half a Newton step of its square
-      const double r = r2[h] * ir[h];
-      const double dr = fma(0.5 * ir[h], fma(-r, r, r2[h]), r - a.r0), kd = a.kb * dr;
-      o.U = fma(0.5 * kd, dr, o.U);
-      gd[h] = -kd * ir[h];
-      o.W = fma(gd[h], r2[h], o.W);
-    }
+  for (int h = 0; h < 2; ++h) {
+    // r - r0 with r = r2 ir corrected by half a Newton step of its square
+    const double r = r2[h] * ir[h];
+    const double dr = fma(0.5 * ir[h], fma(-r, r, r2[h]), r - a.r0), kd = a.kb * dr;
+    o.U = fma(0.5 * kd, dr, o.U);
+    gd[h] = -kd * ir[h];
+    o.W = fma(gd[h], r2[h], o.W);
   }
-  if (what & 2) {
-    // F_h = kth (theta - th0) / sin(theta) d cos(theta) / d r_h; the virial of
-    // an angle is zero (it does not change with the scale)
-    const double ir01 = ir[0] * ir[1];
-    const double dot = d[0][0] * d[1][0] + d[0][1] * d[1][1] + d[0][2] * d[1][2];
-    const double cth = fmin(1.0, fmax(-1.0, dot * ir01));
-    const double dth = acos(cth) - a.th0, kd = a.kth * dth;
-    o.U = fma(0.5 * kd, dth, o.U);
-    const double pref = kd * rsqrt(fma(-cth, cth, 1.0));
-    ga = pref * ir01;
+  // F_h = kth (theta - th0) / sin(theta) d cos(theta) / d r_h; the virial of
+  // an angle is zero (it does not change with the scale)
+  const double ir01 = ir[0] * ir[1];
+  const double dot = d[0][0] * d[1][0] + d[0][1] * d[1][1] + d[0][2] * d[1][2];
+  const double cth = fmin(1.0, fmax(-1.0, dot * ir01));
+  const double dth = acos(cth) - a.th0, kd = a.kth * dth;
+  o.U = fma(0.5 * kd, dth, o.U);
+  const double pref = kd * rsqrt(fma(-cth, cth, 1.0));
+  ga = pref * ir01;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) gd[h] = fma(-pref * cth * ir[h], ir[h], gd[h]);
-  }
+  for (int h = 0; h < 2; ++h) gd[h] = fma(-pref * cth * ir[h], ir[h], gd[h]);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     o.fH[0][c] = fma(ga, d[1][c], gd[0] * d[0][c]);
@@ -147,6 +148,7 @@ __device__ __forceinline__ void bonded_f64(const ForceArgs &a, int m, int k, con
 // A pair in FP64, from the FP64 positions: forces on i, U, Tr Xi (and Xi_aa).
 struct PairF64 {
   double f[3] = {0.0, 0.0, 0.0}, U = 0.0, W = 0.0, w3[3] = {0.0, 0.0, 0.0};
+  bool any = false;
 };
 
 template <bool kDiag>
@@ -160,6 +162,7 @@ __device__ __noinline__ void pair_f64(const ForceArgs &a, const double *L, const
     r2 = fma(d[c], d[c], r2);
   }
   if (!(r2 < a.rc * a.rc)) return;
+  s.any = true;
   const double inv = 1.0 / r2;
   const double s2 = a.sig * a.sig * inv;
   const double s6 = s2 * s2 * s2;
@@ -173,7 +176,7 @@ __device__ __noinline__ void pair_f64(const ForceArgs &a, const double *L, const
 }
 
 template <bool kDiag, bool kFar, bool kSplit>
-__global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArgs a, int split) {
+__global__ void __launch_bounds__(kSplit ? 480 : 128) k_force_water_f64(ForceArgs a, int split) {
   constexpr int NC = kDiag ? 14 : 11;   // F (9), U, Tr Xi, then Xi_xx, Xi_yy, Xi_zz
   extern __shared__ __align__(16) unsigned char fsm[];
   const int P = a.P;
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
   const int NS = kLJWarps * a.nb.groups;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = kSplit ? blockIdx.x : blockIdx.x * 4 + warp;
-  const int role = kSplit ? warp : 0;   // 0 .. split - 1: the list; then bonds, angle
+  const int role = kSplit ? warp : 0;   // 0 .. split - 1: the list; then bonds and angle
   // chunk by chunk: the warps of an SM gather from one chunk's rows
   const int nmg = (a.nmol + G - 1) / G;
   const int chunk = unit / nmg, mg = unit - chunk * nmg;
@@ -196,19 +199,24 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
   int *s_nl = reinterpret_cast<int *>(fsm);             // [G][kMaxNeighbours]
   int *s_off = s_nl + G * kMaxNeighbours;               // [G][NS + 1]
   bool own = false;
-  if (kSplit && a.check_nbr) {
-    own = skin_exceeded(a.nb.blkmax, a.nb.nblk_check, a.nb.skin);
+  if (kSplit && a.check_nbr && role < split) {
+    own = skin_exceeded(a.nb.blkmax, a.nb.nblk_check, a.nb.skin, 32 * split);
     if (own) {
-      for (int q = warp; q < G; q += blockDim.x >> 5) {
+      for (int q = warp; q < G; q += split) {
         const int mm = mg * G + q;
         if (mm >= a.nmol) break;
         int *nl = s_nl + q * kMaxNeighbours, *off = s_off + q * (NS + 1);
         const int total = list_molecule(a.nb, L, iL, mm, NS, nl, off);
         if (chunk == 0) keep_list(a.nb, mm, NS, total, nl, off);
       }
-      __syncthreads();
+      block_part_sync(32 * split);
     }
   }
+  // each molecule takes half of every pair's energy and virial; a pair's
+  // fixed-point force is the one on j
+  const LjFix &lj = a.lj;
+  LjSums s;
+  bool took_f64 = false;
   double acc[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) acc[c] = 0.0;
@@ -218,7 +226,6 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
     const int *nl = own ? s_nl + u * kMaxNeighbours : a.nb.nbr + (size_t)m * kMaxNeighbours;
     int q = off[kSplit ? role * NS / split : 0];
     const int q1 = off[kSplit ? (role + 1) * NS / split : NS];
-    const LjFix &lj = a.lj;
     int64_t LQ[3], xi[3];
     const int64_t *__restrict__ xp = a.xi + k;
 #pragma unroll
@@ -226,10 +233,11 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
       LQ[c] = fix_pos(L[c]);
       xi[c] = xp[(size_t)(3 * m + c) * P];
     }
-    LjSums s;
     PairF64 far;
     // fixed point holds edges below 8192 A (the barostat may change them)
-    const bool fixed = lj.on && L[0] < 4096.0 && L[1] < 4096.0 && L[2] < 4096.0;
+    const int top = __double2hiint(4096.0);
+    const bool fixed =
+        lj.on && __double2hiint(L[0]) < top && __double2hiint(L[1]) < top && __double2hiint(L[2]) < top;
     auto pair = [&](const int64_t (&xj)[3], int j) {
       if (fixed) {
         int64_t d[3];
@@ -264,29 +272,28 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
 #pragma unroll
       for (int c = 0; c < 3; ++c) xj[c] = xn[c];
     }
-    // each molecule takes half of every pair's energy and virial; a pair's
-    // fixed-point force is the one on j
-    if (fixed) {
+    // the pairs taken in FP64
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        acc[c] = fma(-lj.fs, fix_sum(s.f[c]), far.f[c]);
-        if (kDiag) acc[11 + c] = 0.5 * fma(lj.w3, fix_sum(s.w[c]), far.w3[c]);
-      }
-      acc[9] = fma(lj.us, fix_energy<kFar>(s), 0.5 * far.U);
-      acc[10] = fma(lj.ws, fix_sum(s.T), 0.5 * far.W);
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        acc[c] = far.f[c];
-        if (kDiag) acc[11 + c] = 0.5 * far.w3[c];
-      }
-      acc[9] = 0.5 * far.U;
-      acc[10] = 0.5 * far.W;
+    for (int c = 0; c < 3; ++c) {
+      acc[c] = far.f[c];
+      if (kDiag) acc[11 + c] = 0.5 * far.w3[c];
     }
+    acc[9] = 0.5 * far.U;
+    acc[10] = 0.5 * far.W;
+    took_f64 = far.any;
+  }
+  if (!kSplit) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      acc[c] = fma(-lj.fs, fix_sum(s.f[c]), acc[c]);
+      if (kDiag) acc[11 + c] = fma(0.5 * lj.w3, fix_sum(s.w[c]), acc[11 + c]);
+    }
+    acc[9] = fma(lj.us, fix_energy<kFar>(s), acc[9]);
+    acc[10] = fma(lj.ws, fix_sum(s.T), acc[10]);
   }
   if (on && (!kSplit || role >= split)) {
     Bonded b;
-    bonded_f64<kDiag>(a, m, k, L, iL, kSplit ? (role == split ? 1 : 2) : 3, b);
+    bonded_f64<kDiag>(a, m, k, L, iL, b);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       acc[c] += b.fO[c];
@@ -314,16 +321,54 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
       for (int c = 0; c < NC; ++c) store(c, m, k, acc[c]);
     return;
   }
-  double *sacc = reinterpret_cast<double *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [warps][NC][32]
+  // partial sums joined in a fixed order, a component to a warp: the list's
+  // fixed-point sums as integers (one conversion a component), its FP64 pairs
+  // where a warp met one, the bonded warp's terms
+  constexpr int NL = kDiag ? 8 : 5;    // f (3), T, y^3 (, w (3))
+  constexpr int NF = kDiag ? 8 : 5;    // f (3), U, Tr Xi (, Xi_aa (3))
+  __int128 *sI = reinterpret_cast<__int128 *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [split][NL][32]
+  double *sP = reinterpret_cast<double *>(sI + split * NL * 32);                    // [split][NF][32]
+  double *sB = sP + split * NF * 32;                                                // [NC][32]
+  __shared__ int s_f64[14];
+  if (role < split) {
+    const __int128 part[8] = {s.f[0], s.f[1], s.f[2], s.T, s.y3, s.w[0], s.w[1], s.w[2]};
 #pragma unroll
-  for (int c = 0; c < NC; ++c) sacc[(warp * NC + c) * 32 + lane] = acc[c];
+    for (int c = 0; c < NL; ++c) sI[(role * NL + c) * 32 + lane] = part[c];
+    const bool any = __any_sync(0xffffffffu, took_f64);
+    if (lane == 0) s_f64[role] = any;
+    if (any)
+#pragma unroll
+      for (int c = 0; c < NF; ++c) sP[(role * NF + c) * 32 + lane] = acc[c < 3 ? c : c + 6];
+  } else {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) sB[c * 32 + lane] = acc[c];
+  }
   __syncthreads();
-  const int nw = split + 2;
-  for (int t = threadIdx.x; t < NC * 32; t += blockDim.x) {
-    const int comp = t >> 5;   // the lanes keep their (molecule, bead)
-    // the hydrogens' forces come from the bonded warps alone
-    double sum = 0.0;
-    for (int w = comp >= 3 && comp < 9 ? split : 0; w < nw; ++w) sum += sacc[(w * NC + comp) * 32 + lane];
+  for (int comp = warp; comp < NC; comp += split + 1) {   // the lanes keep their (molecule, bead)
+    double sum = sB[comp * 32 + lane];
+    if (comp < 3 || comp > 8) {   // the hydrogens' forces come from the bonded warp alone
+      LjSums t;
+      auto total = [&](int c) {
+        __int128 v = 0;
+        for (int w = 0; w < split; ++w) v += sI[(w * NL + c) * 32 + lane];
+        return v;
+      };
+      double pair;
+      if (comp < 3) {
+        pair = -lj.fs * fix_sum(total(comp));
+      } else if (comp == 9) {
+        t.T = total(3);
+        t.y3 = total(4);
+        pair = lj.us * fix_energy<kFar>(t);
+      } else if (comp == 10) {
+        pair = lj.ws * fix_sum(total(3));
+      } else {
+        pair = 0.5 * lj.w3 * fix_sum(total(comp - 6));
+      }
+      sum += pair;
+      for (int w = 0; w < split; ++w)
+        if (s_f64[w]) sum += sP[(w * NF + (comp < 3 ? comp : comp - 6)) * 32 + lane];
+    }
     if (on) store(comp, m, k, sum);
   }
 }
@@ -331,7 +376,7 @@ __global__ void __launch_bounds__(kSplit ? 320 : 128) k_force_water_f64(ForceArg
 // The lists of a system's molecules, one warp each: on this step's skin test,
 // or (force) always.  Small systems' force blocks do this themselves.
 __global__ void __launch_bounds__(256) k_nbr_lists(NbrList a, int force) {
-  if (!force && !skin_exceeded(a.blkmax, a.nblk_check, a.skin)) return;
+  if (!force && !skin_exceeded(a.blkmax, a.nblk_check, a.skin, blockDim.x)) return;
   const int NS = kLJWarps * a.groups, lane = threadIdx.x & 31;
   double L[3], iL[3];
   list_box(a, L, iL);
@@ -368,17 +413,21 @@ int force_blocks(int n_groups, int P) {
   return (n_groups + per - 1) / per;
 }
 
-// Units of work of the FP64 water force, and the warps that share a unit's
-// neighbour list: 1 (a warp takes whole units) once there are enough of them
-// for every SM partition twice over.
+// Units of work of the water force (one molecule x 32 beads, or 32 / P molecules).
 int water_units(int nmol, int P) {
   const int Bk = P < 32 ? P : 32, G = 32 / Bk;
   return (nmol + G - 1) / G * ((P + Bk - 1) / Bk);
 }
 
+// Warps that share a unit's neighbour list (divisors of NS, a multiple of 14).
+// 1, a warp takes whole units and makes no reduction, from eight units an SM on:
+// us a step, split 1 against 4, 1024 units 69.8 against 65.4, 1400 units 87.3
+// against 91.1, 2048 equal.  Below, warps are short of work and the list's chain
+// is what counts: 4 against 7 at 432 units 33.8 against 41, at 160 24.5 against
+// 23.9; 7 against 14 at 125 units (a block has its SM to itself) 21.8 against 19.9.
 static int water_split(int nmol, int P) {
   const int n = water_units(nmol, P);
-  return n >= 1024 ? 1 : (n >= 512 ? 2 : (n >= 256 ? 4 : 7));   // NS is a multiple of 14
+  return n >= 1216 ? 1 : (n >= 192 ? 4 : (n > 152 ? 7 : 14));
 }
 
 // lane groups per warp of the water force kernel: the largest power of two
@@ -407,12 +456,12 @@ static void force_water(const ForceArgs &a, cudaStream_t s) {
   }
   const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nb.groups;
   const size_t smem = (size_t)G * kMaxNeighbours * sizeof(int) + (((size_t)G * (NS + 1) + 3) & ~(size_t)3) * sizeof(int) +
-                      (size_t)(split + 2) * (kDiag ? 14 : 11) * 32 * sizeof(double);
-  k_force_water_f64<kDiag, kFar, true><<<units, 32 * (split + 2), smem, s>>>(a, split);
+                      ((size_t)split * (kDiag ? 8 : 5) * 3 + (kDiag ? 14 : 11)) * 32 * sizeof(double);
+  k_force_water_f64<kDiag, kFar, true><<<units, 32 * (split + 1), smem, s>>>(a, split);
 }
 
 cudaError_t force_water_prepare() {   // a one-bead system's lists take more than 48 KB
-  const int most = 128 * 1024;
+  const int most = 160 * 1024;
   cudaError_t e = cudaFuncSetAttribute(k_force_water_f64<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);

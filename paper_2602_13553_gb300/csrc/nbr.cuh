@@ -20,6 +20,11 @@
 
 namespace pimd {
 
+// Barrier of a block's first `threads` threads (whole warps).
+__device__ __forceinline__ void block_part_sync(int threads) {
+  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+
 // Number of neighbours of molecule m within rc + skin, listed by bucket (j mod
 // NS) and index, by one warp: FP32 test on the differences of the FP64
 // centroids, in FP64 where it is close.
@@ -73,16 +78,26 @@ __device__ __forceinline__ int list_molecule(const NbrList &a, const double (&L)
   return total;
 }
 
-// This step's rebuild decision from the step kernel's per-block maxima, by all
-// threads of a block.
-__device__ __forceinline__ bool skin_exceeded(const double *blkmax, int n, double skin) {
-  __shared__ double s_mx[2][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// FP32 at or above a non-negative FP64 value, by its bits (a conversion takes a
+// slot of the FP64 pipe).
+__device__ __forceinline__ float float_above(double x) {
+  const int hi = __double2hiint(x), e = hi >> 20;
+  if (e >= 1151) return __int_as_float(0x7f800000);
+  if (e < 897) return __int_as_float(0x00800000);
+  return __int_as_float((((e - 896) << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)__double2loint(x) >> 29)) + 1);
+}
+
+// This step's rebuild decision from the step kernel's per-block maxima, by the
+// first `threads` threads of a block.  Taken in FP32, towards a rebuild: one
+// that comes early changes no sum.
+__device__ __forceinline__ bool skin_exceeded(const double *blkmax, int n, double skin, int threads) {
+  __shared__ longlong2 s_mx[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = threads >> 5;
   // the maxima are non-negative: they compare as integers, off the FP64 pipe
   long long md = 0, me = 0;
   const longlong2 *bm = reinterpret_cast<const longlong2 *>(blkmax);
 #pragma unroll 4
-  for (int b = threadIdx.x; b < n; b += blockDim.x) {
+  for (int b = threadIdx.x; b < n; b += threads) {
     const longlong2 e = bm[b];
     md = max(md, e.x);
     me = max(me, e.y);
@@ -92,17 +107,15 @@ __device__ __forceinline__ bool skin_exceeded(const double *blkmax, int n, doubl
     md = max(md, __shfl_xor_sync(0xffffffffu, md, o));
     me = max(me, __shfl_xor_sync(0xffffffffu, me, o));
   }
-  if (lane == 0) {
-    s_mx[0][warp] = __longlong_as_double(md);
-    s_mx[1][warp] = __longlong_as_double(me);
-  }
-  __syncthreads();
-  double d = 0.0, e = 0.0;
+  if (lane == 0) s_mx[warp] = make_longlong2(md, me);
+  block_part_sync(threads);
   for (int w = 0; w < nw; ++w) {
-    if (__double_as_longlong(s_mx[0][w]) > __double_as_longlong(d)) d = s_mx[0][w];
-    if (__double_as_longlong(s_mx[1][w]) > __double_as_longlong(e)) e = s_mx[1][w];
+    const longlong2 e = s_mx[w];
+    md = max(md, e.x);
+    me = max(me, e.y);
   }
-  return 2.0 * d + 2.0 * e > skin;
+  const float d2 = __fadd_ru(float_above(__longlong_as_double(md)), float_above(__longlong_as_double(me)));
+  return d2 >= float_above(skin) * 0.49999985f;
 }
 
 __device__ __forceinline__ void list_box(const NbrList &a, double (&L)[3], double (&iL)[3]) {

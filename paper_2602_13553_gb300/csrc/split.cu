@@ -376,6 +376,18 @@ __global__ void __launch_bounds__(256) k_force_harmonic_split(SplitForceArgs a) 
 
 __device__ __forceinline__ float micf(float d, float L, float invL) { return fmaf(-rintf(d * invL), L, d); }
 
+// Error-free sum of a few FP32 terms (Knuth's two-sum): the FP64 pipe would take
+// two slots a term.
+struct FloatPair {
+  float h, l;
+  __device__ __forceinline__ void add(float x) {
+    const float t = h + x, z = t - h;
+    l += (h - (t - z)) + (x - z);
+    h = t;
+  }
+  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
 // Water-like model in FP32.  Work as in the FP64 kernel: a unit is one molecule
 // and a chunk of Bk = min(P, 32) beads (G = 32 / Bk molecules where the beads
 // leave lanes free), beads in adjacent lanes.  Many units: one warp each, four
@@ -386,9 +398,11 @@ __device__ __forceinline__ float micf(float d, float L, float invL) { return fma
 // as a scalar would), eight to a partial sum.
 //
 // What bounds it is the latency of the gathers: the rows of the next two
-// candidates are requested before the arithmetic of these.  A four-block cluster
-// per unit (whose fixed cost this replaces) with a list check of its own took
-// 38.5 + 3 us a step at 512 molecules x 64 beads, 10.8 + 8.4 us at 216 x 20.
+// candidates are requested before the arithmetic of these.  No FP64 instruction
+// is left but the list build's and four at the end: constants come converted,
+// the list check compares in FP32, U and Tr Xi are joined as FP32 pairs (80 FP64
+// instructions a warp held 22 of 35.6 us at 512 molecules x 64 beads and 5 of
+// 13.4 at 216 x 20; now 15.5 and 8.1 us).
 template <bool kSplit>
 __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitForceArgs a, int split) {
   extern __shared__ __align__(16) unsigned char fsm[];
@@ -406,27 +420,27 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
   int *s_nl = reinterpret_cast<int *>(fsm);             // [G][kMaxNeighbours]
   int *s_off = s_nl + G * kMaxNeighbours;               // [G][NS + 1]
   bool own = false;
-  if (kSplit && a.check_nbr) {
-    own = skin_exceeded(a.nb.blkmax, a.nb.nblk_check, a.nb.skin);
+  if (kSplit && a.check_nbr && role < split) {
+    own = skin_exceeded(a.nb.blkmax, a.nb.nblk_check, a.nb.skin, 32 * split);
     if (own) {
-      double L[3], iL[3];
-      list_box(a.nb, L, iL);
-      for (int q = warp; q < G; q += blockDim.x >> 5) {
+      double Ld[3], iLd[3];
+      list_box(a.nb, Ld, iLd);
+      for (int q = warp; q < G; q += split) {
         const int mm = mg * G + q;
         if (mm >= a.nmol) break;
         int *nl = s_nl + q * kMaxNeighbours, *off = s_off + q * (NS + 1);
-        const int total = list_molecule(a.nb, L, iL, mm, NS, nl, off);
+        const int total = list_molecule(a.nb, Ld, iLd, mm, NS, nl, off);
         if (chunk == 0) keep_list(a.nb, mm, NS, total, nl, off);
       }
-      __syncthreads();
+      block_part_sync(32 * split);
     }
   }
+  const float *const L = a.ff.L, *const iL = a.ff.iL;
   float F[9];
 #pragma unroll
   for (int c = 0; c < 9; ++c) F[c] = 0.f;
-  double ue = 0.0, we = 0.0;
-  const float L[3] = {(float)a.nb.box[0], (float)a.nb.box[1], (float)a.nb.box[2]};
-  const float iL[3] = {(float)a.nb.invbox[0], (float)a.nb.invbox[1], (float)a.nb.invbox[2]};
+  float lu = 0.f, lw = 0.f;     // U and Tr Xi of the list (twice this molecule's)
+  float bu = 0.f, bw = 0.f, au = 0.f, aw = 0.f;   // of the bonds, of the angle
   float co[3] = {0.f, 0.f, 0.f}, dO[3] = {0.f, 0.f, 0.f};
   if (on) {
 #pragma unroll
@@ -440,9 +454,8 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
     const int *nl = own ? s_nl + u * kMaxNeighbours : a.nb.nbr + (size_t)m * kMaxNeighbours;
     int q = off[kSplit ? role * NS / split : 0];
     const int q1 = off[kSplit ? (role + 1) * NS / split : NS];
-    const float rc2 = (float)(a.rc * a.rc);
-    const float2 sig2 = make_float2((float)(a.sig * a.sig), (float)(a.sig * a.sig));
-    const float e4 = (float)(4.0 * a.eps), e24 = (float)(24.0 * a.eps);
+    const float rc2 = a.ff.rc2, e4 = a.ff.e4, e24 = a.ff.e24;
+    const float2 sig2 = make_float2(a.ff.sig2, a.ff.sig2);
     const float2 e4v = make_float2(e4, e4), ne4 = make_float2(-e4, -e4);
     const float2 e48 = make_float2(2.f * e24, 2.f * e24), ne24 = make_float2(-e24, -e24);
     const float2 zero = make_float2(0.f, 0.f);
@@ -495,8 +508,8 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) F[c] = S[c].x + S[c].y;
-    ue = 0.5 * (double)(S[3].x + S[3].y);
-    we = 0.5 * (double)(S[4].x + S[4].y);
+    lu = S[3].x + S[3].y;
+    lw = S[4].x + S[4].y;
   }
   if (on && (!kSplit || role == split)) {
     float dv[2][3], r[2], ir[2];
@@ -511,30 +524,27 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
       ir[h] = 1.f / r[h];
     }
     // bonds
-    float uu = 0.f, w = 0.f, fO[3] = {0.f, 0.f, 0.f};
+    float fO[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const float dr = r[h] - (float)a.r0;
-      uu = fmaf(0.5f * (float)a.kb * dr, dr, uu);
-      const float g = -(float)a.kb * dr * ir[h];
+      const float dr = r[h] - a.ff.r0;
+      bu = fmaf(0.5f * a.ff.kb * dr, dr, bu);
+      const float g = -a.ff.kb * dr * ir[h];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const float fc = g * dv[h][c];
         F[3 + 3 * h + c] = fc;
         fO[c] -= fc;
-        w = fmaf(dv[h][c], fc, w);
+        bw = fmaf(dv[h][c], fc, bw);
       }
     }
-    ue += (double)uu;
-    we += (double)w;
     // angle
     const float ir01 = ir[0] * ir[1];
     const float dot = dv[0][0] * dv[1][0] + dv[0][1] * dv[1][1] + dv[0][2] * dv[1][2];
     const float cth = fminf(1.f, fmaxf(-1.f, dot * ir01));
     const float th = acosf(cth);
-    const float dth = th - (float)a.th0;
-    const float pref = (float)a.kth * dth / sinf(th);
-    w = 0.f;
+    const float dth = th - a.ff.th0;
+    const float pref = a.ff.kth * dth / sinf(th);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int g = 1 - h;
@@ -544,45 +554,45 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
         const float fa = pref * fmaf(dv[g][c], ir01, -ch * dv[h][c]);
         F[3 + 3 * h + c] += fa;
         fO[c] -= fa;
-        w = fmaf(dv[h][c], fa, w);
+        aw = fmaf(dv[h][c], fa, aw);
       }
     }
-    ue += (double)(0.5f * (float)a.kth * dth * dth);
-    we += (double)w;
+    au = 0.5f * a.ff.kth * dth * dth;
 #pragma unroll
     for (int c = 0; c < 3; ++c) F[c] += fO[c];
   }
   if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += a.inc;
+  FloatPair U{0.5f * lu, 0.f}, W{0.5f * lw, 0.f};
   if (kSplit) {
     // partial sums of the warps, joined in order by the last warp
-    float *sF = reinterpret_cast<float *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [split][3][32]
-    double *sU = reinterpret_cast<double *>(sF + split * 96);                   // [split][2][32]
+    float *sF = reinterpret_cast<float *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [split][5][32]
     if (role < split) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) sF[(role * 3 + c) * 32 + lane] = F[c];
-      sU[(role * 2) * 32 + lane] = ue;
-      sU[(role * 2 + 1) * 32 + lane] = we;
+      for (int c = 0; c < 3; ++c) sF[(role * 5 + c) * 32 + lane] = F[c];
+      sF[(role * 5 + 3) * 32 + lane] = lu;
+      sF[(role * 5 + 4) * 32 + lane] = lw;
     }
     __syncthreads();
     if (role < split) return;
     float sum[3] = {0.f, 0.f, 0.f};
-    double su = 0.0, sw = 0.0;
     for (int w = 0; w < split; ++w) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) sum[c] += sF[(w * 3 + c) * 32 + lane];
-      su += sU[(w * 2) * 32 + lane];
-      sw += sU[(w * 2 + 1) * 32 + lane];
+      for (int c = 0; c < 3; ++c) sum[c] += sF[(w * 5 + c) * 32 + lane];
+      U.add(0.5f * sF[(w * 5 + 3) * 32 + lane]);
+      W.add(0.5f * sF[(w * 5 + 4) * 32 + lane]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) F[c] += sum[c];
-    ue += su;
-    we += sw;
   }
+  U.add(bu);
+  U.add(au);
+  W.add(bw);
+  W.add(aw);
   if (!on) return;
 #pragma unroll
   for (int c = 0; c < 9; ++c) a.F[(size_t)(9 * m + c) * P + k] = F[c];
-  a.Upart[(size_t)m * P + k] = ue;
-  a.Wpart[(size_t)m * P + k] = we;
+  a.Upart[(size_t)m * P + k] = U.value();
+  a.Wpart[(size_t)m * P + k] = W.value();
 }
 
 // --- conversions between the split state and FP64 [N][3][P] arrays ----------
@@ -655,10 +665,14 @@ int force_blocks(int n_groups, int P);
 int force_block_threads(int P);
 int water_units(int nmol, int P);
 
-// Warps that share a unit's neighbour list (1: a warp takes whole units).
+// Warps that share a unit's neighbour list (divisors of NS, a multiple of 14);
+// 1: a warp takes whole units.  us a step, 1 against 2: 1024 units 39.2 against
+// 32.4, 1400 units 40.2 against 40.8, 2048 units 49.7 against 52.4; 2 against 7:
+// 600 units 29.7 against 30.2; 4 against 7: 432 units 26.0 against 25.6, 216
+// units 18.3 against 17.2 (14: 19.5).
 static int split_water_warps(int nmol, int P) {
   const int n = water_units(nmol, P);
-  return n >= 4096 ? 1 : (n >= 2048 ? 2 : (n >= 512 ? 4 : 7));   // NS is a multiple of 14
+  return n >= 1216 ? 1 : (n >= 512 ? 2 : 7);
 }
 
 // Whether the list check is a kernel of its own (the one-warp units).
@@ -677,7 +691,7 @@ cudaError_t launch_force_split(const SplitForceArgs &a, bool water, cudaStream_t
       const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nb.groups;
       const size_t smem = (size_t)G * kMaxNeighbours * sizeof(int) +
                           (((size_t)G * (NS + 1) + 3) & ~(size_t)3) * sizeof(int) +
-                          (size_t)split * 32 * (3 * sizeof(float) + 2 * sizeof(double));
+                          (size_t)split * 32 * 5 * sizeof(float);
       k_force_water_split<true><<<units, 32 * (split + 1), smem, s>>>(a, split);
     }
   } else

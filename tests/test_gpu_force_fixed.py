@@ -90,3 +90,10 @@ def test_rebuilds(orc, pimd, nmol, P):
     assert 2.0 * np.abs(x[:, 0::3].mean(0) - x0[:, 0::3].mean(0)).max() > 1.5
     assert coord_err(x, c.x) < 1e-8 and coord_err(v, c.v) < 1e-8
     g.close()
+
+
+@pytest.mark.parametrize("nmol,P", [(160, 32), (610, 64)])
+def test_warps_per_unit(orc, pimd, nmol, P):
+    """Units of 7 list warps, and one-warp units with the list check apart, over
+    rebuilds of the lists (the bar of test_rebuilds)."""
+    test_rebuilds(orc, pimd, nmol, P)
