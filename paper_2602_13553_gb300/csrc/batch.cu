@@ -5,7 +5,7 @@
 // RepDesc in a device table.  Each MD step is a sequence of launches over all
 // replicas -- control; the step, one kernel per class of bead count present
 // (warp items of 64 beads; of 8, 16 or 32; of 128; block items of any other
-// count), the classes side by side on two streams; rebuild decision;
+// count), the classes side by side on streams of their own; rebuild decision;
 // rebuilds; forces -- each a persistent grid of fixed size that walks a
 // device-resident work list (step tiles, force clusters, neighbour blocks)
 // whose length it reads from device memory.  Because neither grid sizes nor
@@ -182,7 +182,7 @@ __device__ __forceinline__ float wrapb(double x, double L, double invL) {
   return (float)(x - L * floor(x * invL));
 }
 
-__device__ __forceinline__ float micb(float d, float L, float invL) { return fmaf(-rintf(d * invL), L, d); }
+__device__ __forceinline__ float micb(float d, float L, float invL) { return fmaf(-rint_mul(d, invL), L, d); }
 
 // Three standard normal deviates of (atom, mode, stream, step) in FP32 from
 // one Philox call (the same words and mapping as gauss1f_b per component).
@@ -1668,10 +1668,7 @@ __device__ __forceinline__ float2 ldg2(const float *p) { return __ldg(reinterpre
 
 // Minimum image of a pair of components: d - L rint(d / L), elementwise.
 __device__ __forceinline__ float2 micb2(float2 d, float2 invL, float2 nL) {
-  float2 t = __fmul2_rn(d, invL);
-  t.x = rintf(t.x);
-  t.y = rintf(t.y);
-  return __ffma2_rn(t, nL, d);
+  return __ffma2_rn(rint_mul2(d, invL), nL, d);
 }
 
 // The work item of k_bforce for an even bead count, two adjacent beads
@@ -2276,10 +2273,11 @@ struct pimd_batch {
   int capacity = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  // a second stream and two events: the step kernels of the bead classes run
-  // side by side (a fork and a join inside every step, captured into the graph)
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+  // side streams and their events: the step kernels of the bead classes run
+  // side by side (a fork and joins inside every step, captured into the graph)
+  static constexpr int kSides = 3;
+  cudaStream_t side[kSides] = {nullptr};
+  cudaEvent_t fork_ev = nullptr, join_ev[kSides] = {nullptr};
   DevAllocator alloc;
   std::vector<Replica> reps;
   RepDesc *d_reps = nullptr;
@@ -2470,32 +2468,41 @@ pimd_status upload(pimd_batch *b) {
   return PIMD_OK;
 }
 
-// The two step kernels: warp items, then block items.
-// The classes' step kernels touch disjoint replicas, so the 8-32-bead and
-// block-item kernels run on the side stream beside the 64- and 128-bead ones
-// (fork after the control kernel, join before the rebuild decision): one
-// kernel's tail fills with the other's work.
+// The step kernels of the bead classes present.  They touch disjoint replicas,
+// so each runs on a stream of its own (fork after the control kernel, joins
+// before the rebuild decision), the ones with the longest items first: an item
+// takes 20 to 35 us whatever its class (its transforms are one chain), so a few
+// replicas of every class finish with the longest of them and not with the sum,
+// and one kernel's tail fills with the other's work.  With two streams (64 after
+// 128 beads, the block items after the small ones) 24 replicas of six classes
+// took 13.6 ms a 30-step job, so 12.5.
 void launch_step_kernels(pimd_batch *b) {
-  const bool fork = (b->w64_items || b->w128_items) && (b->wsmall_items || b->block_items);
-  cudaStream_t s2 = fork ? b->side : b->stream;
-  if (fork) {
-    cudaEventRecord(b->fork_ev, b->stream);
-    cudaStreamWaitEvent(b->side, b->fork_ev, 0);
+  const bool present[4] = {b->w128_items, b->w64_items, b->wsmall_items, b->block_items};
+  const int classes = present[0] + present[1] + present[2] + present[3];
+  if (classes > 1) cudaEventRecord(b->fork_ev, b->stream);
+  int used = 0;
+  for (int q = 0; q < 4; ++q) {
+    if (!present[q]) continue;
+    cudaStream_t s = b->stream;
+    if (used > 0) {
+      s = b->side[used - 1];
+      cudaStreamWaitEvent(s, b->fork_ev, 0);
+    }
+    if (q == 0)
+      k_bstep_w<2><<<b->grid_w128, kWWarps * 32, item_smem(128), s>>>(
+          b->d_reps, b->d_step, b->d_counts, b->d_counts + 8, wslot_floats(128));
+    else if (q == 1)
+      k_bstep_w<1><<<b->grid_w, kWWarps * 32, item_smem(64), s>>>(
+          b->d_reps, b->d_step, b->d_counts, b->d_counts + 5, wslot_floats(64));
+    else if (q == 2)
+      k_bstep_w<0><<<b->grid_ws, kWWarps * 32, (size_t)kWWarps * wslot_floats(32) * sizeof(float), s>>>(
+          b->d_reps, b->d_step, b->d_counts, b->d_counts + 10, wslot_floats(32));
+    else
+      k_bstep<<<b->grid_step, 128, 0, s>>>(b->d_reps, b->d_step, b->d_counts);
+    if (used > 0) cudaEventRecord(b->join_ev[used - 1], s);
+    ++used;
   }
-  if (b->w64_items)
-    k_bstep_w<1><<<b->grid_w, kWWarps * 32, item_smem(64), b->stream>>>(
-        b->d_reps, b->d_step, b->d_counts, b->d_counts + 5, wslot_floats(64));
-  if (b->wsmall_items)
-    k_bstep_w<0><<<b->grid_ws, kWWarps * 32, (size_t)kWWarps * wslot_floats(32) * sizeof(float), s2>>>(
-        b->d_reps, b->d_step, b->d_counts, b->d_counts + 10, wslot_floats(32));
-  if (b->w128_items)
-    k_bstep_w<2><<<b->grid_w128, kWWarps * 32, item_smem(128), b->stream>>>(
-        b->d_reps, b->d_step, b->d_counts, b->d_counts + 8, wslot_floats(128));
-  if (b->block_items) k_bstep<<<b->grid_step, 128, 0, s2>>>(b->d_reps, b->d_step, b->d_counts);
-  if (fork) {
-    cudaEventRecord(b->join_ev, b->side);
-    cudaStreamWaitEvent(b->stream, b->join_ev, 0);
-  }
+  for (int q = 1; q < used; ++q) cudaStreamWaitEvent(b->stream, b->join_ev[q - 1], 0);
 }
 
 // The rebuild decision over all neighbour items, then the rebuilds listed.
@@ -2776,11 +2783,13 @@ extern "C" pimd_status pimd_batch_create(int32_t max_replicas, void *stream, pim
     }
     b->own_stream = true;
   }
-  if (cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&b->join_ev, cudaEventDisableTiming) != cudaSuccess) {
+  bool sides = cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming) == cudaSuccess;
+  for (int q = 0; q < pimd_batch::kSides; ++q)
+    sides = sides && cudaStreamCreateWithFlags(&b->side[q], cudaStreamNonBlocking) == cudaSuccess &&
+            cudaEventCreateWithFlags(&b->join_ev[q], cudaEventDisableTiming) == cudaSuccess;
+  if (!sides) {
     pimd_batch_destroy(b);
-    return fail(PIMD_ECUDA, "cannot create the batch's side stream");
+    return fail(PIMD_ECUDA, "cannot create the batch's side streams");
   }
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
@@ -2864,9 +2873,11 @@ extern "C" void pimd_batch_destroy(pimd_batch *b) {
   for (auto p : b->mtab) dev_free(b->alloc, p, b->stream);
   if (b->h_eout) cudaFreeHost(b->h_eout);
   if (b->h_ctl) cudaFreeHost(b->h_ctl);
-  if (b->side) cudaStreamDestroy(b->side);
+  for (auto q : b->side)
+    if (q) cudaStreamDestroy(q);
   if (b->fork_ev) cudaEventDestroy(b->fork_ev);
-  if (b->join_ev) cudaEventDestroy(b->join_ev);
+  for (auto q : b->join_ev)
+    if (q) cudaEventDestroy(q);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
   delete b;
 }

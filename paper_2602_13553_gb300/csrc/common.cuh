@@ -134,6 +134,14 @@ __device__ __forceinline__ double group_sum(double v, int W) {
   return v;
 }
 
+// rint(x y), |x y| < 2^22, by the FP32 adder: rintf is an instruction of the
+// special-function pipe (a warp in 8 clocks per SM partition).
+constexpr float kRintMagic = 12582912.0f;   // 1.5 2^23
+__device__ __forceinline__ float rint_mul(float x, float y) { return __fadd_rn(__fmaf_rn(x, y, kRintMagic), -kRintMagic); }
+__device__ __forceinline__ float2 rint_mul2(float2 x, float2 y) {
+  return __fadd2_rn(__ffma2_rn(x, y, make_float2(kRintMagic, kRintMagic)), make_float2(-kRintMagic, -kRintMagic));
+}
+
 // Minimum-image component (box edge L > 0; round half to even like rint).
 __device__ __forceinline__ double mic(double d, double L, double invL) {
   return d - L * rint(d * invL);

@@ -37,9 +37,9 @@ __device__ __forceinline__ int list_molecule(const NbrList &a, const double (&L)
   const float If[3] = {(float)iL[0], (float)iL[1], (float)iL[2]};
   auto near = [&](int j) {
     const double e0 = a.ccur[3 * j] - c0, e1 = a.ccur[3 * j + 1] - c1, e2 = a.ccur[3 * j + 2] - c2;
-    const float f0 = fmaf(-rintf((float)e0 * If[0]), Lf[0], (float)e0);
-    const float f1 = fmaf(-rintf((float)e1 * If[1]), Lf[1], (float)e1);
-    const float f2 = fmaf(-rintf((float)e2 * If[2]), Lf[2], (float)e2);
+    const float f0 = fmaf(-rint_mul((float)e0, If[0]), Lf[0], (float)e0);
+    const float f1 = fmaf(-rint_mul((float)e1, If[1]), Lf[1], (float)e1);
+    const float f2 = fmaf(-rint_mul((float)e2, If[2]), Lf[2], (float)e2);
     const float r2 = f0 * f0 + f1 * f1 + f2 * f2;
     // unwrapped differences of many boxes lose FP32 digits: FP64 there too
     const float far = fmaxf(fmaxf(fabsf((float)e0), fabsf((float)e1)), fabsf((float)e2));

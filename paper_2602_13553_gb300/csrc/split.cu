@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(256) k_force_harmonic_split(SplitForceArgs a) 
   if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += a.inc;
 }
 
-__device__ __forceinline__ float micf(float d, float L, float invL) { return fmaf(-rintf(d * invL), L, d); }
+__device__ __forceinline__ float micf(float d, float L, float invL) { return fmaf(-rint_mul(d, invL), L, d); }
 
 // Error-free sum of a few FP32 terms (Knuth's two-sum): the FP64 pipe would take
 // two slots a term.
@@ -482,8 +482,7 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           float2 e = make_float2(cur.c[0][c] - co[c], cur.c[1][c] - co[c]);
-          const float2 n = make_float2(-rintf(e.x * iL[c]), -rintf(e.y * iL[c]));
-          e = __ffma2_rn(n, make_float2(L[c], L[c]), e);
+          e = __ffma2_rn(rint_mul2(e, make_float2(iL[c], iL[c])), make_float2(-L[c], -L[c]), e);
           d[c] = __fadd2_rn(e, make_float2(cur.d[0][c] - dO[c], cur.d[1][c] - dO[c]));
         }
         const float2 r2 = __ffma2_rn(d[2], d[2], __ffma2_rn(d[1], d[1], __fmul2_rn(d[0], d[0])));
