@@ -98,6 +98,22 @@ __host__ __device__ __forceinline__ float rsqrt_seed(float x) {
 #endif
 }
 
+// leading zeros of y > 0; 2^e for a normal exponent
+__host__ __device__ __forceinline__ int lead_zeros(uint64_t y) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)y);
+#else
+  return __builtin_clzll(y);
+#endif
+}
+__host__ __device__ __forceinline__ float pow2f(int e) {
+#ifdef __CUDA_ARCH__
+  return __int_as_float((e + 127) << 23);
+#else
+  return ldexpf(1.0f, e);
+#endif
+}
+
 // sqrt(-2 ln u), Q60.
 __host__ __device__ __forceinline__ uint64_t bm_radius_fix(uint32_t w) {
   // n = 2 w + 1 = (2^32 + f) 2^-lz, u = n 2^-33: -ln u = a ln 2 + T_j - log1p(r)
@@ -139,14 +155,17 @@ __host__ __device__ __forceinline__ uint64_t bm_radius_fix(uint32_t w) {
   const uint64_t y = (uint64_t)(a * (noise_detail::kLn2 >> 4) + (tail >> 4));   // -ln u, Q58
   // s = sqrt(t), t = 2 y (y as Q57): FP32 seed, then two corrections
   // s += (t - s^2) / (2 s) whose residuals are exact
-  const float tf = (float)y * 6.938893903907228e-18f;   // 2^-57
+  // (from 32 bits each: a 64-bit conversion takes a slot of the FP64 pipe; the
+  // step of 20011 x 17 oscillator beads, OBABO, took 81 us with them, 76.5 so)
+  const int nz = lead_zeros(y);
+  const float tf = (float)(uint32_t)((y << nz) >> 32) * pow2f(-25 - nz);         // 2^-57 y
   const float rs = rsqrt_seed(tf);
   const uint32_t g0 = (uint32_t)(tf * rs * 268435456.0f);                    // Q28
-  const int64_t e0 = (int64_t)(y - (((uint64_t)g0 * g0) << 1));              // Q57
+  const int64_t e0 = (int64_t)(y - (((uint64_t)g0 * g0) << 1));              // Q57, below 2^42
   const float hr = 0.5f * rs;
-  const int64_t g1 = ((int64_t)g0 << 22) + (int)((float)e0 * hr * 0.0078125f);   // Q50: 2^(50 - 57)
-  const int64_t e1 = (int64_t)((y << 43) - (uint64_t)g1 * (uint64_t)g1);      // Q100, small
-  return (uint64_t)((g1 << 10) + (int)((float)e1 * hr * 9.094947017729282e-13f));   // Q60: 2^(60 - 100)
+  const int64_t g1 = ((int64_t)g0 << 22) + (int)((float)(int)(e0 >> 12) * hr * 32.0f);   // Q50: 2^(12 + 50 - 57)
+  const int64_t e1 = (int64_t)((y << 43) - (uint64_t)g1 * (uint64_t)g1);      // Q100, below 2^62
+  return (uint64_t)((g1 << 10) + (int)((float)(int)(e1 >> 32) * hr * 0.00390625f));   // Q60: 2^(32 + 60 - 100)
 }
 
 // sine and cosine of 2 pi u, Q62.

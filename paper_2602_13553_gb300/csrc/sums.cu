@@ -13,7 +13,9 @@
 // single blocks with one thread per atom (strided reads, N P serial terms)
 // they were most of a step: the barostat 72 us a call (two a step) for 125
 // molecules x 16 beads, fixcom 50 us for 91 molecules x 17 beads and 192 us
-// for 100 molecules x 12 Cartesian beads.
+// for 100 molecules x 12 Cartesian beads; now 11.6, 10.1 and 9.5.  (The factor
+// (e^a - e^-a) / (2 v_W) from the series of sinh would need no division and no
+// cancellation, but leaves the published form by its 1e-11 at small a.)
 #include "common.cuh"
 
 #include <algorithm>
@@ -113,7 +115,7 @@ __global__ void __launch_bounds__(kSumThreads) k_baro_kick(BaroArgs a) {
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    vir[c] = warp_sum(vir[c]);
+    if (c == 0 || a.axes) vir[c] = warp_sum(vir[c]);
     if (lane == 0) sv[c][warp] = vir[c];
   }
   __syncthreads();
@@ -129,31 +131,40 @@ __global__ void __launch_bounds__(kSumThreads) k_baro_kick(BaroArgs a) {
     a.part[blockIdx.x * kBaroCols + threadIdx.x] = s;
   }
   if (!last_block(a.count)) return;
-  // the rows of partials: one warp per column; one thread draws the noise
+  // the state the scalar work starts from, requested before the sums
+  double *b = a.baro;
+  const double V = b[kBaroL] * b[kBaroL + 1] * b[kBaroL + 2], L = b[kBaroL + threadIdx.x % 3];
+  double vW = b[kBaroV + threadIdx.x % 3];
+  const uint64_t step = (uint64_t)*a.step;
+  // the rows of partials: one warp per column
   for (int col = warp; col < kBaroCols; col += kSumThreads / 32) {
     double s = 0.0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(a.part + b * kBaroCols + col);
+    for (int r = lane; r < (int)gridDim.x; r += 32) s += __ldcg(a.part + r * kBaroCols + col);
     s = warp_sum(s);
     if (lane == 0) tot[col] = s;
   }
   // O_W's deviates: Philox atom 0xffffffff, stream 3, mode 0 (the O of BAOAB,
-  // the first O(h/2) of OBABO) or 1 (the second, of the step just completed)
-  const uint64_t step = (uint64_t)*a.step;
-  if (a.thermo && threadIdx.x == kSumThreads - 1 && (a.step_follows || a.obabo))
-    gauss3(a.seed, 0xffffffffu, a.step_follows ? 0u : 1u, 3u, a.step_follows ? step : step - 1, noise[0], noise[1],
-           noise[2]);
+  // the first O(h/2) of OBABO) or 1 (the second, of the step just completed).
+  // The last warp (one column): a lane for each radius and angle
+  if (a.thermo && threadIdx.x >= kSumThreads - 32 && (a.step_follows || a.obabo)) {
+    const uint4 w = noise_words(a.seed, 0xffffffffu, a.step_follows ? 0u : 1u, 3u, a.step_follows ? step : step - 1);
+    uint64_t radius = 0;
+    int64_t sn = 0, cs = 0;
+    if (lane == 0 || lane == 2) radius = bm_radius_fix(lane ? w.z : w.x);
+    if (lane == 1 || lane == 3) bm_angle_fix(lane == 1 ? w.y : w.w, sn, cs);
+    const int64_t c1 = __shfl_sync(0xffffffffu, cs, 1), s1 = __shfl_sync(0xffffffffu, sn, 1);
+    const int64_t c3 = __shfl_sync(0xffffffffu, cs, 3);
+    const uint64_t r0 = __shfl_sync(0xffffffffu, radius, 0), r2 = __shfl_sync(0xffffffffu, radius, 2);
+    if (lane < 3) noise[lane] = bm_deviate(lane == 2 ? r2 : r0, lane == 0 ? c1 : (lane == 1 ? s1 : c3));
+  }
   __syncthreads();
   // the scalar work, one warp: lane = (edge c, sign of the exponent, which A);
   // the lanes of an edge do the same up to their exponential (isotropic: all do)
   if (threadIdx.x >= 12) return;
   const int c = threadIdx.x % 3, sgn = threadIdx.x / 3 % 2, h = threadIdx.x / 6;
   const double *mv = tot, *sfv = tot + 3, *sf2 = tot + 6, *srcf = tot + 9, *svir = tot + 12;
-  double *b = a.baro;
-  const double V = b[kBaroL] * b[kBaroL + 1] * b[kBaroL + 2], L = b[kBaroL + c];
   const bool moves = !a.axes || (a.axes >> c & 1);
   const double eta = a.axes ? noise[c] : noise[0];
-  double vW = b[kBaroV + c];
-  __syncwarp(0xfffu);   // every lane has read the state that lanes change below
   // O_W: v_W <- c1 v_W + sigW eta; each edge its own deviate, the isotropic
   // v_W the first
   auto langevin = [&](double w) { return moves ? a.c1W * w + a.sigW * eta : w; };
