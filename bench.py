@@ -163,7 +163,9 @@ def step_flops_per_bead_atom(P):
     folded normal-mode transforms of 3 components, each output a sum over one
     half of its folded row (P/2 + 1 FMAs: 9 P + 18), the folding and
     recombination adds (9), the merged kick (6), two exact rotations (36) and
-    the O update (9); the Box-Muller noise is not counted."""
+    the O update (9); the Box-Muller noise is not counted.  The kernel takes
+    the sums in fixed point on the integer pipe, so this rate can exceed the
+    FP64 pipe's."""
     return 9 * P + 78
 
 

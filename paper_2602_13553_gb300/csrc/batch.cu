@@ -418,9 +418,10 @@ __device__ __forceinline__ void bstep_mma(const RepDesc *__restrict__ Rp, int P,
     for (int j = threadIdx.x & 31; j < P; j += 32) dg[r * P + j] = sF[r * PS + j];
 }
 
-// ---- warp-item step on tensor cores: P in {8, 16, 32, 64} --------------------
-// One warp advances a tile of 8 atoms x 3 components x P beads with no block
-// barrier, so the warps of an SM overlap one another's memory waits.  Per
+// ---- warp-item step on tensor cores: P in {8, 16, 32, 64, 128} ---------------
+// One warp (two at 64 beads, four at 128) advances a tile of 8 atoms x 3
+// components x P beads with no block barrier, so the warps of an SM overlap one
+// another's memory waits.  Per
 // component c the forward transforms are GEMMs C[mode][atom] = M[mode][bead]
 // X_c[bead][atom] whose B operand (8 atoms = one n-tile) is the staged tile;
 // the C fragment of lane (g, t) then holds modes {16 mt + g, 16 mt + g + 8} of
@@ -2281,9 +2282,7 @@ struct pimd_batch {
   DevAllocator alloc;
   std::vector<Replica> reps;
   RepDesc *d_reps = nullptr;
-  // [8]: step, cluster, nbr, est items (all replicas); [4] warp-item prefix
-  // of the step list; [5] the warp-item counter; [6] the rebuild-list length
-  int *d_counts = nullptr;
+  int *d_counts = nullptr;                 // as h_counts below
   int2 *d_step = nullptr, *d_nbr = nullptr, *d_est = nullptr;
   int2 *d_nbr_go = nullptr;                // this step's rebuild list
   size_t cap_nbr_go = 0;
