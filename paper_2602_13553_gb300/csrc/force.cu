@@ -76,8 +76,8 @@ __global__ void __launch_bounds__(256) k_force_harmonic_f64(ForceArgs a) {
 //    list over `split` warps, which also take the step's list check, and gives
 //    its bonds and angle to one more that starts at once; the partial sums are
 //    joined as integers, a component to a warp, and converted once.
-// Measured, us a launch: 512 molecules x 64 beads 172 in FP64, now about 37 (FP64
-// instructions 10.6 and integer issue 11 of it; three blocks fit an SM).  With
+// Measured, us a launch: 512 molecules x 64 beads 172 in FP64, now about 32 (FP64
+// instructions and integer issue 13.5 each of it).  With
 // seven list warps, FP64 partial sums and two bonded warps behind the list check
 // against now: 64 x 32 beads 11.1 / 10.4 (16.7 in FP64), 100 x 12 13.2 / 11.1,
 // 125 x 16 with the diagonal virial 16.1 / 13.5.
@@ -175,8 +175,13 @@ __device__ __noinline__ void pair_f64(const ForceArgs &a, const double *L, const
   s.W = fma(fr, r2, s.W);
 }
 
-template <bool kDiag, bool kFar, bool kSplit>
-__global__ void __launch_bounds__(kSplit ? 480 : 128) k_force_water_f64(ForceArgs a, int split) {
+// kSplit: 0 one warp a unit, 1 up to 14 list warps, 2 four of them, with the
+// registers (96) that put four blocks on an SM: a pass of 512 molecules x 64
+// beads, 20 steps, 1.66 ms with 101 registers and three blocks, 1.56 so; five
+// blocks (72, spills) are faster only at 1024 units and more (68.7 against 69.5 us
+// a step there, 35.4 against 33.3 at 400)
+template <bool kDiag, bool kFar, int kSplit>
+__global__ void __launch_bounds__(kSplit == 2 ? 160 : (kSplit ? 480 : 128), kSplit == 2 ? 4 : 1) k_force_water_f64(ForceArgs a, int split) {
   constexpr int NC = kDiag ? 14 : 11;   // F (9), U, Tr Xi, then Xi_xx, Xi_yy, Xi_zz
   extern __shared__ __align__(16) unsigned char fsm[];
   const int P = a.P;
@@ -451,21 +456,28 @@ template <bool kDiag, bool kFar>
 static void force_water(const ForceArgs &a, cudaStream_t s) {
   const int split = water_split(a.nmol, a.P), units = water_units(a.nmol, a.P);
   if (split == 1) {
-    k_force_water_f64<kDiag, kFar, false><<<(units + 3) / 4, 128, 0, s>>>(a, 1);
+    k_force_water_f64<kDiag, kFar, 0><<<(units + 3) / 4, 128, 0, s>>>(a, 1);
     return;
   }
   const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nb.groups;
   const size_t smem = (size_t)G * kMaxNeighbours * sizeof(int) + (((size_t)G * (NS + 1) + 3) & ~(size_t)3) * sizeof(int) +
                       ((size_t)split * (kDiag ? 8 : 5) * 3 + (kDiag ? 14 : 11)) * 32 * sizeof(double);
-  k_force_water_f64<kDiag, kFar, true><<<units, 32 * (split + 1), smem, s>>>(a, split);
+  if (split == 4)
+    k_force_water_f64<kDiag, kFar, 2><<<units, 32 * (split + 1), smem, s>>>(a, split);
+  else
+    k_force_water_f64<kDiag, kFar, 1><<<units, 32 * (split + 1), smem, s>>>(a, split);
 }
 
 cudaError_t force_water_prepare() {   // a one-bead system's lists take more than 48 KB
   const int most = 160 * 1024;
-  cudaError_t e = cudaFuncSetAttribute(k_force_water_f64<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaError_t e = cudaFuncSetAttribute(k_force_water_f64<false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   return e;
 }
 
