@@ -12,7 +12,7 @@
 // sum f_c (fix_energy joins the two formats).  "Qn" is a number with n fraction bits; sums are 128-bit integers,
 // exact and free of order.
 //
-// Rounding: y to 2^-62 of itself, T and f_c to 2^-58 absolutely, where the
+// Rounding: y to 2^-61 of itself plus 2^-64, T and f_c to 2^-58 absolutely, where the
 // terms of a molecule's sum are 2^-5 to 2^0; the FP64 expressions round each
 // term at 2^-53 of itself several times.  With a cutoff far beyond sigma
 // (e > 4) most terms are small: those with C y^3 < 2 then keep five more bits
@@ -36,7 +36,6 @@ struct LjFix {
   uint64_t rc2;                // cutoff, x Q64
   uint64_t xmin;               // closer pairs in FP64, x Q62
   uint64_t C;                  // Q58
-  float seed;                  // 2^(62 - e)
   float rpre2;                 // 1.008 rc^2 in units of 2^-18 A squared: the quick test
   int far;                     // kFar
   double fs, us, ws, w3;       // force, energy (half), virial (half), diagonal virial of the sums
@@ -60,7 +59,6 @@ inline LjFix lj_fix_setup(double eps, double sig, double rc, const double *box) 
   p.rc2 = (uint64_t)std::ldexp(rc * rc, 64 - 2 * b);
   p.xmin = (uint64_t)std::ldexp(1.0 + 1.0 / 1024, 62 - e);
   p.C = (uint64_t)std::ldexp(2.0 * c6, 58);
-  p.seed = (float)std::ldexp(1.0, 62 - e);
   p.rpre2 = (float)(1.008 * rc * rc * std::ldexp(1.0, 36));
   p.far = e > 4;
   const int q = p.far ? 63 : 58;   // fraction bits of the sums
@@ -73,11 +71,42 @@ inline LjFix lj_fix_setup(double eps, double sig, double rc, const double *box) 
 
 #ifdef __CUDA_ARCH__
 #define PIMD_MULHI(a, b) __umul64hi(a, b)
-#define PIMD_FDIV(a, b) __fdividef(a, b)
+__device__ __forceinline__ float lj_rcp(float x) {   // within one unit in the last place
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+#define PIMD_RCP(x) lj_rcp(x)
+#define PIMD_CLZ(x) __clzll((long long)(x))
+#define PIMD_FLOAT(bits) __uint_as_float(bits)
 #else   // the same arithmetic on the host, for checking it there
 #define PIMD_MULHI(a, b) ((uint64_t)(((unsigned __int128)(a) * (b)) >> 64))
-#define PIMD_FDIV(a, b) ((a) / (b))
+#ifndef PIMD_RCP
+#define PIMD_RCP(x) (1.0f / (x))
 #endif
+#define PIMD_CLZ(x) __builtin_clzll(x)
+inline float lj_float(uint32_t bits) {
+  float f;
+  __builtin_memcpy(&f, &bits, 4);
+  return f;
+}
+#define PIMD_FLOAT(bits) lj_float(bits)
+#endif
+
+// 1 / (4 X) of X = xn 2^-64 in [1/2, 1), Q64 in (2^62, 2^63], to 2^-61 of
+// itself: FP32 seed of the leading 24 bits, then two Newton steps v += v (1 - X v).
+// X and v are cut so that each residual, exact modulo 2^64, stays inside it: the
+// first is below 2^-21 (24 bits rounded, the seed two units off) of 2^-17, the
+// second below 2^-39.6 (v cut to Q40, and the first squared) of 2^-39.
+__host__ __device__ __forceinline__ uint64_t lj_recip(uint64_t xn) {
+  const float X = PIMD_FLOAT(0x3f000000u + (uint32_t)(((xn >> 39) + 1) >> 1) - 0x800000u);
+  const uint32_t v0 = (uint32_t)(PIMD_RCP(X) * 1073741824.0f);                               // Q30
+  const int64_t e0 = -(int64_t)((xn >> 14) * v0);                                            // Q80
+  const uint64_t v1 =
+      ((uint64_t)v0 << 10) + (uint64_t)(((int64_t)(int)(v0 >> 1) * (int)(e0 >> 32)) >> 37);   // Q40
+  const int64_t e1 = -(int64_t)((xn >> 2) * v1);                                             // Q102
+  return (v1 << 22) + (uint64_t)(((int64_t)(int)(v1 >> 11) * (int)(e1 >> 32)) >> 37);         // Q62
+}
 
 // x 2^50 modulo 2^64, rounded (positions are kept wrapped into the box, so the
 // modulus never shows).
@@ -135,15 +164,11 @@ __host__ __device__ __forceinline__ bool lj_fix_pair(const LjFix &p, const int64
     r2 += PIMD_MULHI(dn[c], dn[c]);
   }
   if (r2 >= p.rc2) return true;
-  const uint64_t x = r2 >> 2;   // Q62
-  if (x <= p.xmin) return false;
-  // y = 2^-e / x: FP32 seed (Q24), then two Newton steps y += y (1 - 2^e x y)
-  // whose residuals are exact modulo 2^64
-  const uint32_t y0 = (uint32_t)(PIMD_FDIV(p.seed, (float)x) * 16777216.0f);
-  const int64_t e0 = -(int64_t)(x * y0);                                     // Q(86 - e)
-  const uint64_t y1 = ((uint64_t)y0 << 16) + (uint64_t)(((int64_t)y0 * (int)(e0 >> 31)) >> (39 - p.e));   // Q40
-  const int64_t e1 = -(int64_t)(x * y1);                                     // Q(102 - e)
-  const uint64_t y = (y1 << 24) + (uint64_t)(((int64_t)(y1 >> 10) * (int)(e1 >> 31)) >> (37 - p.e));   // Q64
+  if ((r2 >> 2) <= p.xmin) return false;
+  // y = 2^-e / x from the reciprocal of the normalised x; y < 1 above xmin
+  const int nx = PIMD_CLZ(r2), m = p.e - nx;   // m >= 1
+  const uint64_t w = lj_recip(r2 << nx);       // y = w 2^(2 - m)
+  const uint64_t y = m > 1 ? w >> (m - 2) : w << 1;                          // Q64
   const uint64_t y3 = PIMD_MULHI(PIMD_MULHI(y, y), y);                       // Q64
   const uint64_t Cy = PIMD_MULHI(p.C, y3), one = (uint64_t)1 << 58;          // Q58
   const bool neg = Cy < one;
