@@ -180,7 +180,7 @@ __device__ __noinline__ void pair_f64(const ForceArgs &a, const double *L, const
 // beads, 20 steps, 1.66 ms with 101 registers and three blocks, 1.56 so; five
 // blocks (72, spills) are faster only at 1024 units and more (68.7 against 69.5 us
 // a step there, 35.4 against 33.3 at 400)
-template <bool kDiag, bool kFar, int kSplit>
+template <bool kDiag, int kSplit>
 __global__ void __launch_bounds__(kSplit == 2 ? 160 : (kSplit ? 480 : 128), kSplit == 2 ? 4 : 1) k_force_water_f64(ForceArgs a, int split) {
   constexpr int NC = kDiag ? 14 : 11;   // F (9), U, Tr Xi, then Xi_xx, Xi_yy, Xi_zz
   extern __shared__ __align__(16) unsigned char fsm[];
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kSplit == 2 ? 160 : (kSplit ? 480 : 128), kSpl
           h2 = fmaf(h, h, h2);
         }
         if (h2 >= lj.rpre2) return;
-        if (lj_fix_pair<kDiag, kFar>(lj, d, s)) return;
+        if (lj_fix_pair<kDiag>(lj, d, s)) return;
       }
       pair_f64<kDiag>(a, L, iL, m, j, k, far);
     };
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kSplit == 2 ? 160 : (kSplit ? 480 : 128), kSpl
       acc[c] = fma(-lj.fs, fix_sum(s.f[c]), acc[c]);
       if (kDiag) acc[11 + c] = fma(0.5 * lj.w3, fix_sum(s.w[c]), acc[11 + c]);
     }
-    acc[9] = fma(lj.us, fix_energy<kFar>(s), acc[9]);
+    acc[9] = fma(lj.us, fix_energy(s), acc[9]);
     acc[10] = fma(lj.ws, fix_sum(s.T), acc[10]);
   }
   if (on && (!kSplit || role >= split)) {
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kSplit == 2 ? 160 : (kSplit ? 480 : 128), kSpl
       } else if (comp == 9) {
         t.T = total(3);
         t.y3 = total(4);
-        pair = lj.us * fix_energy<kFar>(t);
+        pair = lj.us * fix_energy(t);
       } else if (comp == 10) {
         pair = lj.ws * fix_sum(total(3));
       } else {
@@ -452,46 +452,36 @@ cudaError_t launch_force_harmonic(const ForceArgs &a, cudaStream_t s) {
 // Whether the list check is a kernel of its own (the one-warp units).
 bool water_lists_apart(int nmol, int P) { return water_split(nmol, P) == 1; }
 
-template <bool kDiag, bool kFar>
+template <bool kDiag>
 static void force_water(const ForceArgs &a, cudaStream_t s) {
   const int split = water_split(a.nmol, a.P), units = water_units(a.nmol, a.P);
   if (split == 1) {
-    k_force_water_f64<kDiag, kFar, 0><<<(units + 3) / 4, 128, 0, s>>>(a, 1);
+    k_force_water_f64<kDiag, 0><<<(units + 3) / 4, 128, 0, s>>>(a, 1);
     return;
   }
   const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nb.groups;
   const size_t smem = (size_t)G * kMaxNeighbours * sizeof(int) + (((size_t)G * (NS + 1) + 3) & ~(size_t)3) * sizeof(int) +
                       ((size_t)split * (kDiag ? 8 : 5) * 3 + (kDiag ? 14 : 11)) * 32 * sizeof(double);
   if (split == 4)
-    k_force_water_f64<kDiag, kFar, 2><<<units, 32 * (split + 1), smem, s>>>(a, split);
+    k_force_water_f64<kDiag, 2><<<units, 32 * (split + 1), smem, s>>>(a, split);
   else
-    k_force_water_f64<kDiag, kFar, 1><<<units, 32 * (split + 1), smem, s>>>(a, split);
+    k_force_water_f64<kDiag, 1><<<units, 32 * (split + 1), smem, s>>>(a, split);
 }
 
 cudaError_t force_water_prepare() {   // a one-bead system's lists take more than 48 KB
   const int most = 160 * 1024;
-  cudaError_t e = cudaFuncSetAttribute(k_force_water_f64<false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaError_t e = cudaFuncSetAttribute(k_force_water_f64<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_force_water_f64<true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   return e;
 }
 
 cudaError_t launch_force_water(const ForceArgs &a, cudaStream_t s) {
-  if (a.W3part) {
-    if (a.lj.far)
-      force_water<true, true>(a, s);
-    else
-      force_water<true, false>(a, s);
-  } else if (a.lj.far) {
-    force_water<false, true>(a, s);
-  } else {
-    force_water<false, false>(a, s);
-  }
+  if (a.W3part)
+    force_water<true>(a, s);
+  else
+    force_water<false>(a, s);
   return cudaGetLastError();
 }
 

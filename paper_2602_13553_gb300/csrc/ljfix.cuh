@@ -4,21 +4,24 @@
 // a 32-bit multiply-add 2.4, so the pairs of the O-O sum are evaluated in
 // integers.  Lengths are scaled by the power of two 2^b above the cutoff and
 // x = r^2 / 2^2b; y = 2^-e / x is in (0, 1] down to the distance 2^(b - e/2),
-// which lies between 0.56 and 0.79 sigma (closer pairs, and systems whose
+// which lies between 0.56 and 0.79 sigma (farther out for sigma below a tenth of
+// the cutoff, where e is at its cap; closer pairs, and systems whose
 // scales do not fit, take the FP64 expressions).  With C = 2 (2^e sigma^2 /
 // 2^2b)^3 the pair's terms are, per component c,
 //   T = y^3 (C y^3 - 1),  f_c = y T d_c / 2^b,
 // energy, virial and force being constants times sum (T - y^3), sum T and
-// sum f_c (fix_energy joins the two formats).  "Qn" is a number with n fraction bits; sums are 128-bit integers,
+// sum f_c.  "Qn" is a number with n fraction bits; sums are 128-bit integers,
 // exact and free of order.
 //
-// Rounding: y to 2^-61 of itself plus 2^-64, T and f_c to 2^-58 absolutely, where the
-// terms of a molecule's sum are 2^-5 to 2^0; the FP64 expressions round each
-// term at 2^-53 of itself several times.  With a cutoff far beyond sigma
-// (e > 4) most terms are small: those with C y^3 < 2 then keep five more bits
-// (kFar).  Against quadruple precision, 59 random neighbours, rms errors of
-// force / energy / virial in eV, A: sigma 3.166, cutoff 6: 8e-17 / 8e-18 /
-// 1.1e-16 (FP64 expressions 1.8e-16 / 2.7e-17 / 3.8e-16).
+// Rounding: terms vary by 2^-3e (T) and 2^-4e (f) between the cutoff and the
+// closest pair, so each is formed from the reciprocal of the normalised x and
+// shifted to the sum's unit: T and f_c keep 2^-55 (at e = 7, 2^-53) or more of
+// the pair's own size, where the FP64 expressions round at 2^-53 several times.
+// Against 60 decimal digits, pairs from 0.85 of the cutoff on, sigma 3.166, rms
+// error of the force over the pair's own, at cutoffs 6, 12 and 20: 1.7e-16,
+// 1.8e-16, 1.8e-16 (its rounding to FP64 included); the FP64 expressions 3.9e-16,
+// 4.1e-16, 4.1e-16; every term cut at one place, Q58 or Q63, 2.8e-14, 2.0e-13,
+// 1.4e-11 (a pass of 512 molecules x 64 beads, 20 steps, took 1.56 ms so; 1.61 now).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -37,7 +40,6 @@ struct LjFix {
   uint64_t xmin;               // closer pairs in FP64, x Q62
   uint64_t C;                  // Q58
   float rpre2;                 // 1.008 rc^2 in units of 2^-18 A squared: the quick test
-  int far;                     // kFar
   double fs, us, ws, w3;       // force, energy (half), virial (half), diagonal virial of the sums
 };
 
@@ -48,7 +50,7 @@ inline LjFix lj_fix_setup(double eps, double sig, double rc, const double *box) 
   while (b > -10 && std::ldexp(1.0, b - 1) >= 1.01 * rc) --b;
   const double s2 = sig * sig * std::ldexp(1.0, -2 * b);
   int e = 0;
-  while (e < 8 && s2 * std::ldexp(1.0, e + 1) <= 3.17) ++e;
+  while (e < 7 && s2 * std::ldexp(1.0, e + 1) <= 3.17) ++e;
   const double ratio = s2 * std::ldexp(1.0, e);
   p.on = ratio <= 3.17 && std::ldexp(1.0, b) >= 1.01 * rc && rc > 0.01;
   for (int c = 0; c < 3; ++c) p.on = p.on && box[c] < 2048.0;
@@ -60,12 +62,10 @@ inline LjFix lj_fix_setup(double eps, double sig, double rc, const double *box) 
   p.xmin = (uint64_t)std::ldexp(1.0 + 1.0 / 1024, 62 - e);
   p.C = (uint64_t)std::ldexp(2.0 * c6, 58);
   p.rpre2 = (float)(1.008 * rc * rc * std::ldexp(1.0, 36));
-  p.far = e > 4;
-  const int q = p.far ? 63 : 58;   // fraction bits of the sums
-  p.fs = 24.0 * eps * c6 * std::ldexp(1.0, e - b - q);
-  p.w3 = 24.0 * eps * c6 * std::ldexp(1.0, e - q);
-  p.us = eps * c6 * std::ldexp(1.0, -q);
-  p.ws = 12.0 * eps * c6 * std::ldexp(1.0, -q);
+  p.fs = 24.0 * eps * c6 * std::ldexp(1.0, -b - 57 - 3 * e);
+  p.w3 = 24.0 * eps * c6 * std::ldexp(1.0, -57 - 3 * e);
+  p.us = eps * c6 * std::ldexp(1.0, -59 - 3 * e);
+  p.ws = 12.0 * eps * c6 * std::ldexp(1.0, -59 - 3 * e);
   return p;
 }
 
@@ -142,19 +142,28 @@ __host__ __device__ __forceinline__ int64_t fix_mic(int64_t d, int64_t LQ) {
 }
 
 struct LjSums {
-  __int128 f[3] = {0, 0, 0}, T = 0;   // Q58 (kFar: Q63)
-  __int128 y3 = 0;                    // Q64
-  __int128 w[3] = {0, 0, 0};          // f_c d_c (diagonal virial)
+  __int128 f[3] = {0, 0, 0};          // Q(57 + 4 e)
+  __int128 T = 0;                     // Q(59 + 3 e)
+  __int128 y3 = 0;                    // Q(58 + 3 e)
+  __int128 w[3] = {0, 0, 0};          // f_c d_c (diagonal virial), as f
 };
 
+// +-v 2^up, v < 2^63, up < 32
 __host__ __device__ __forceinline__ void add_signed(__int128 &s, uint64_t v, bool neg, int up) {
-  const __int128 t = (__int128)v << up;
-  s += neg ? -t : t;
+  const int64_t t = neg ? -(int64_t)v : (int64_t)v;
+#ifdef __CUDA_ARCH__   // three funnel shifts: a 128-bit shift by a variable is four times that
+  const uint32_t lo = (uint32_t)t, hi = (uint32_t)((uint64_t)t >> 32), sg = (uint32_t)((int)hi >> 31);
+  const uint64_t a = ((uint64_t)__funnelshift_l(lo, hi, up) << 32) | (lo << up);
+  const uint64_t b = ((uint64_t)sg << 32) | __funnelshift_l(hi, sg, up);
+  s += (__int128)(((unsigned __int128)b << 64) | a);
+#else
+  s += (__int128)t * ((__int128)1 << up);
+#endif
 }
 
 // One pair's terms; d = x_j - x_i minimum image, |d_c| < 2^b.  Returns false
 // for a pair closer than the fixed-point range.
-template <bool kDiag, bool kFar>
+template <bool kDiag>
 __host__ __device__ __forceinline__ bool lj_fix_pair(const LjFix &p, const int64_t (&d)[3], LjSums &s) {
   const int sh = 64 - kPosBits - p.b;
   uint64_t dn[3], r2 = 0;
@@ -165,44 +174,44 @@ __host__ __device__ __forceinline__ bool lj_fix_pair(const LjFix &p, const int64
   }
   if (r2 >= p.rc2) return true;
   if ((r2 >> 2) <= p.xmin) return false;
-  // y = 2^-e / x from the reciprocal of the normalised x; y < 1 above xmin
-  const int nx = PIMD_CLZ(r2), m = p.e - nx;   // m >= 1
-  const uint64_t w = lj_recip(r2 << nx);       // y = w 2^(2 - m)
-  const uint64_t y = m > 1 ? w >> (m - 2) : w << 1;                          // Q64
-  const uint64_t y3 = PIMD_MULHI(PIMD_MULHI(y, y), y);                       // Q64
+  // y = 2^-e / x = w 2^(2 - m), w the reciprocal of the normalised x; y < 1 above xmin
+  const int nx = PIMD_CLZ(r2), m3 = 3 * (p.e - nx);      // m >= 1
+  const uint64_t w = lj_recip(r2 << nx);                 // Q64, (1/4, 1/2]
+  const uint64_t w3 = PIMD_MULHI(PIMD_MULHI(w, w), w);   // (1/64, 1/8]
+  const uint64_t y3 = m3 > 6 ? w3 >> (m3 - 6) : w3 << (6 - m3);              // Q64
   const uint64_t Cy = PIMD_MULHI(p.C, y3), one = (uint64_t)1 << 58;          // Q58
   const bool neg = Cy < one;
-  uint64_t Pm = neg ? one - Cy : Cy - one;                                   // |C y^3 - 1|
-  int up = 0;
-  if (kFar) {
-    if (Pm >> 59)
-      up = 5;
-    else
-      Pm <<= 5;
-  }
-  const uint64_t T = PIMD_MULHI(y3, Pm), G = PIMD_MULHI(y, T);
-  add_signed(s.T, T, neg, up);
-  s.y3 += y3;
+  uint64_t Pm = neg ? one - Cy : Cy - one;                                   // |C y^3 - 1| Q58, below 64
+  const int k = Pm >> 59 ? PIMD_CLZ(Pm) : 5, up = 5 - k;
+  Pm <<= k;                                                                  // Q(58 + k)
+  const uint64_t T = PIMD_MULHI(w3 << 2, Pm), G = PIMD_MULHI(w, T);
+  add_signed(s.T, T, neg, 3 * nx + up);
+  add_signed(s.y3, w3, false, 3 * nx);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const uint64_t f = PIMD_MULHI(G, dn[c]);
-    add_signed(s.f[c], f, neg != (d[c] < 0), up);
-    if (kDiag) add_signed(s.w[c], PIMD_MULHI(f, dn[c]), neg, up);
+    add_signed(s.f[c], f, neg != (d[c] < 0), 4 * nx + up);
+    // x < 2^-nx: the shifted component is still below 1
+    if (kDiag) add_signed(s.w[c], PIMD_MULHI(f, dn[c] << (nx >> 1)), neg, 4 * nx + up - (nx >> 1));
   }
   return true;
 }
 
-// A sum as FP64.
+// A sum as FP64, correctly rounded: one conversion of its leading 64 bits.
 __host__ __device__ __forceinline__ double fix_sum(__int128 v) {
-  const int64_t lo = (int64_t)v;
-  if (v == (__int128)lo) return (double)lo;
-  return fma((double)(int64_t)(v >> 64), 18446744073709551616.0, (double)(uint64_t)v);
+  const int64_t hi = (int64_t)(v >> 64), lo = (int64_t)v;
+  if (hi == lo >> 63) return (double)lo;
+  const int n = PIMD_CLZ((uint64_t)(hi ^ (hi >> 63))) - 1;   // spare sign bits; hi is neither 0 nor -1 but for its sign
+  const unsigned __int128 u = (unsigned __int128)v << n;
+  const double d = (double)((int64_t)(u >> 64) | (int64_t)((uint64_t)u != 0));
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(__double2hiint(d) + ((64 - n) << 20), __double2loint(d));
+#else
+  return std::ldexp(d, 64 - n);
+#endif
 }
 
 // sum (T - y^3) in the units of T.
-template <bool kFar>
-__host__ __device__ __forceinline__ double fix_energy(const LjSums &s) {
-  return fix_sum(s.T) - fix_sum(s.y3) * (kFar ? 0.5 : 0.015625);
-}
+__host__ __device__ __forceinline__ double fix_energy(const LjSums &s) { return fix_sum(s.T - 2 * s.y3); }
 
 }  // namespace pimd
