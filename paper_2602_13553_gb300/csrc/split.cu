@@ -395,7 +395,8 @@ struct FloatPair {
 // more takes the bonds and the angle.  A pair vector is the minimum-image
 // difference of the wrapped FP32 centroids plus the difference of the FP32
 // deviations.  Candidates go two at a time on packed FP32 (each element rounds
-// as a scalar would), eight to a partial sum.
+// as a scalar would) and are summed one by one, in bucket and index order: the
+// sums of a warp depend on the interacting pairs alone, not on the list's age.
 //
 // What bounds it is the latency of the gathers: the rows of the next two
 // candidates are requested before the arithmetic of these.  No FP64 instruction
@@ -458,7 +459,6 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
     const float2 sig2 = make_float2(a.ff.sig2, a.ff.sig2);
     const float2 e4v = make_float2(e4, e4), ne4 = make_float2(-e4, -e4);
     const float2 e48 = make_float2(2.f * e24, 2.f * e24), ne24 = make_float2(-e24, -e24);
-    const float2 zero = make_float2(0.f, 0.f);
     struct Cand { float c[2][3], d[2][3]; };
     auto load = [&](int j0, int j1, Cand &v) {
 #pragma unroll
@@ -472,43 +472,35 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
     Cand cur, nxt;
     // a list's odd end pairs its last candidate with itself, masked
     if (q < q1) load(nl[q], nl[min(q + 1, q1 - 1)], cur);
-    float2 S[5] = {zero, zero, zero, zero, zero};   // F on this molecule (3), U, W
-    while (q < q1) {
-      float2 s[5] = {zero, zero, zero, zero, zero};
 #pragma unroll 1
-      for (int t = 0; t < 4 && q < q1; ++t, q += 2) {
-        if (q + 2 < q1) load(nl[q + 2], nl[min(q + 3, q1 - 1)], nxt);
-        float2 d[3];
+    for (; q < q1; q += 2) {
+      if (q + 2 < q1) load(nl[q + 2], nl[min(q + 3, q1 - 1)], nxt);
+      float2 d[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          float2 e = make_float2(cur.c[0][c] - co[c], cur.c[1][c] - co[c]);
-          e = __ffma2_rn(rint_mul2(e, make_float2(iL[c], iL[c])), make_float2(-L[c], -L[c]), e);
-          d[c] = __fadd2_rn(e, make_float2(cur.d[0][c] - dO[c], cur.d[1][c] - dO[c]));
-        }
-        const float2 r2 = __ffma2_rn(d[2], d[2], __ffma2_rn(d[1], d[1], __fmul2_rn(d[0], d[0])));
-        const bool i0 = r2.x < rc2, i1 = r2.y < rc2 && q + 1 < q1;
-        if (i0 || i1) {
-          // a candidate outside the cutoff gets 1 / r^2 = 0: it adds exact zeros
-          const float2 inv = make_float2(i0 ? __frcp_rn(r2.x) : 0.f, i1 ? __frcp_rn(r2.y) : 0.f);
-          const float2 s2 = __fmul2_rn(sig2, inv);
-          const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
-          s[3] = __ffma2_rn(s6, __ffma2_rn(e4v, s6, ne4), s[3]);
-          const float2 fr = __fmul2_rn(__fmul2_rn(__ffma2_rn(e48, s6, ne24), s6), inv);
-          const float2 nf = make_float2(-fr.x, -fr.y);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) s[c] = __ffma2_rn(nf, d[c], s[c]);
-          if (i0) s[4].x = fmaf(fr.x, r2.x, s[4].x);
-          if (i1) s[4].y = fmaf(fr.y, r2.y, s[4].y);
-        }
-        cur = nxt;
+      for (int c = 0; c < 3; ++c) {
+        float2 e = make_float2(cur.c[0][c] - co[c], cur.c[1][c] - co[c]);
+        e = __ffma2_rn(rint_mul2(e, make_float2(iL[c], iL[c])), make_float2(-L[c], -L[c]), e);
+        d[c] = __fadd2_rn(e, make_float2(cur.d[0][c] - dO[c], cur.d[1][c] - dO[c]));
       }
+      const float2 r2 = __ffma2_rn(d[2], d[2], __ffma2_rn(d[1], d[1], __fmul2_rn(d[0], d[0])));
+      const bool i0 = r2.x < rc2, i1 = r2.y < rc2 && q + 1 < q1;
+      if (i0 || i1) {
+        // a candidate outside the cutoff gets 1 / r^2 = 0: it adds exact zeros
+        const float2 inv = make_float2(i0 ? __frcp_rn(r2.x) : 0.f, i1 ? __frcp_rn(r2.y) : 0.f);
+        const float2 s2 = __fmul2_rn(sig2, inv);
+        const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
+        const float2 u = __ffma2_rn(e4v, s6, ne4);
+        const float2 fr = __fmul2_rn(__fmul2_rn(__ffma2_rn(e48, s6, ne24), s6), inv);
+        // one chain in list order: the zeros leave no trace of the list's other
+        // candidates, or of which two were taken together
+        lu = fmaf(s6.y, u.y, fmaf(s6.x, u.x, lu));
 #pragma unroll
-      for (int c = 0; c < 5; ++c) S[c] = __fadd2_rn(S[c], s[c]);
+        for (int c = 0; c < 3; ++c) F[c] = fmaf(-fr.y, d[c].y, fmaf(-fr.x, d[c].x, F[c]));
+        if (i0) lw = fmaf(fr.x, r2.x, lw);
+        if (i1) lw = fmaf(fr.y, r2.y, lw);
+      }
+      cur = nxt;
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) F[c] = S[c].x + S[c].y;
-    lu = S[3].x + S[3].y;
-    lw = S[4].x + S[4].y;
   }
   if (on && (!kSplit || role == split)) {
     float dv[2][3], r[2], ir[2];
