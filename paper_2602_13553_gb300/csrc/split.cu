@@ -376,14 +376,29 @@ __global__ void __launch_bounds__(256) k_force_harmonic_split(SplitForceArgs a) 
 
 __device__ __forceinline__ float micf(float d, float L, float invL) { return fmaf(-rint_mul(d, invL), L, d); }
 
-// Error-free sum of a few FP32 terms (Knuth's two-sum): the FP64 pipe would take
-// two slots a term.
+// FP32 sum with its rounding errors kept (Knuth's two-sum; intrinsics, so that no
+// product is contracted into one of its additions): the FP64 pipe would take two
+// slots a term.
 struct FloatPair {
   float h, l;
   __device__ __forceinline__ void add(float x) {
-    const float t = h + x, z = t - h;
-    l += (h - (t - z)) + (x - z);
+    const float t = __fadd_rn(h, x), z = __fadd_rn(t, -h);
+    l += __fadd_rn(__fadd_rn(h, -__fadd_rn(t, -z)), __fadd_rn(x, -z));
     h = t;
+  }
+  __device__ __forceinline__ void add(const FloatPair &o) {
+    add(o.h);
+    l += o.l;
+  }
+  // + a b, unrounded
+  __device__ __forceinline__ void fma(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    add(p);
+    l += fmaf(a, b, -p);
+  }
+  __device__ __forceinline__ void half() {
+    h *= 0.5f;
+    l *= 0.5f;
   }
   __device__ __forceinline__ double value() const { return (double)h + (double)l; }
 };
@@ -401,9 +416,10 @@ struct FloatPair {
 // What bounds it is the latency of the gathers: the rows of the next two
 // candidates are requested before the arithmetic of these.  No FP64 instruction
 // is left but the list build's and four at the end: constants come converted,
-// the list check compares in FP32, U and Tr Xi are joined as FP32 pairs (80 FP64
-// instructions a warp held 22 of 35.6 us at 512 molecules x 64 beads and 5 of
-// 13.4 at 216 x 20; now 15.5 and 8.1 us).
+// the list check compares in FP32, U and Tr Xi are sums of FP32 terms with their
+// rounding errors kept (plain FP32 chains were 3e-8 of the sum off and 1% of a pass
+// faster).  80 FP64 instructions a warp held 22 of 35.6 us at 512 molecules x 64
+// beads and 5 of 13.4 at 216 x 20; now 15.5 and 8.1 us.
 template <bool kSplit>
 __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitForceArgs a, int split) {
   extern __shared__ __align__(16) unsigned char fsm[];
@@ -440,7 +456,7 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
   float F[9];
 #pragma unroll
   for (int c = 0; c < 9; ++c) F[c] = 0.f;
-  float lu = 0.f, lw = 0.f;     // U and Tr Xi of the list (twice this molecule's)
+  FloatPair U{0.f, 0.f}, W{0.f, 0.f};   // U and Tr Xi of the list (twice this molecule's)
   float bu = 0.f, bw = 0.f, au = 0.f, aw = 0.f;   // of the bonds, of the angle
   float co[3] = {0.f, 0.f, 0.f}, dO[3] = {0.f, 0.f, 0.f};
   if (on) {
@@ -493,11 +509,12 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
         const float2 fr = __fmul2_rn(__fmul2_rn(__ffma2_rn(e48, s6, ne24), s6), inv);
         // one chain in list order: the zeros leave no trace of the list's other
         // candidates, or of which two were taken together
-        lu = fmaf(s6.y, u.y, fmaf(s6.x, u.x, lu));
+        U.fma(s6.x, u.x);
+        U.fma(s6.y, u.y);
+        W.fma(fr.x, i0 ? r2.x : 0.f);
+        W.fma(fr.y, i1 ? r2.y : 0.f);
 #pragma unroll
         for (int c = 0; c < 3; ++c) F[c] = fmaf(-fr.y, d[c].y, fmaf(-fr.x, d[c].x, F[c]));
-        if (i0) lw = fmaf(fr.x, r2.x, lw);
-        if (i1) lw = fmaf(fr.y, r2.y, lw);
       }
       cur = nxt;
     }
@@ -553,28 +570,31 @@ __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitF
     for (int c = 0; c < 3; ++c) F[c] += fO[c];
   }
   if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += a.inc;
-  FloatPair U{0.5f * lu, 0.f}, W{0.5f * lw, 0.f};
   if (kSplit) {
     // partial sums of the warps, joined in order by the last warp
-    float *sF = reinterpret_cast<float *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [split][5][32]
+    float *sF = reinterpret_cast<float *>(s_off + ((G * (NS + 1) + 3) & ~3));   // [split][7][32]
     if (role < split) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) sF[(role * 5 + c) * 32 + lane] = F[c];
-      sF[(role * 5 + 3) * 32 + lane] = lu;
-      sF[(role * 5 + 4) * 32 + lane] = lw;
+      for (int c = 0; c < 3; ++c) sF[(role * 7 + c) * 32 + lane] = F[c];
+      sF[(role * 7 + 3) * 32 + lane] = U.h;
+      sF[(role * 7 + 4) * 32 + lane] = U.l;
+      sF[(role * 7 + 5) * 32 + lane] = W.h;
+      sF[(role * 7 + 6) * 32 + lane] = W.l;
     }
     __syncthreads();
     if (role < split) return;
     float sum[3] = {0.f, 0.f, 0.f};
     for (int w = 0; w < split; ++w) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) sum[c] += sF[(w * 5 + c) * 32 + lane];
-      U.add(0.5f * sF[(w * 5 + 3) * 32 + lane]);
-      W.add(0.5f * sF[(w * 5 + 4) * 32 + lane]);
+      for (int c = 0; c < 3; ++c) sum[c] += sF[(w * 7 + c) * 32 + lane];
+      U.add(FloatPair{sF[(w * 7 + 3) * 32 + lane], sF[(w * 7 + 4) * 32 + lane]});
+      W.add(FloatPair{sF[(w * 7 + 5) * 32 + lane], sF[(w * 7 + 6) * 32 + lane]});
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) F[c] += sum[c];
   }
+  U.half();
+  W.half();
   U.add(bu);
   U.add(au);
   W.add(bw);
@@ -682,7 +702,7 @@ cudaError_t launch_force_split(const SplitForceArgs &a, bool water, cudaStream_t
       const int Bk = a.P < 32 ? a.P : 32, G = 32 / Bk, NS = kLJWarps * a.nb.groups;
       const size_t smem = (size_t)G * kMaxNeighbours * sizeof(int) +
                           (((size_t)G * (NS + 1) + 3) & ~(size_t)3) * sizeof(int) +
-                          (size_t)split * 32 * 5 * sizeof(float);
+                          (size_t)split * 32 * 7 * sizeof(float);
       k_force_water_split<true><<<units, 32 * (split + 1), smem, s>>>(a, split);
     }
   } else

@@ -55,3 +55,30 @@ def test_idle_candidates_change_nothing(pimd, nmol, P):
         out.append((xs[:, :3 * nmol], vs[:, :3 * nmol]))
         g.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+def test_energy_sums_do_not_depend_on_the_split(pimd):
+    """U and Tr Xi of one cluster of 64 molecules, its units' lists shared by seven
+    warps, by two and taken by one (idle molecules out of every reach bring the
+    number of units there; bonds and angles off): the FP32 terms are the same ones,
+    and sums that keep their rounding errors lose 2^-48 an addition, 190 additions
+    at most: 1e-12 of the terms' magnitudes, 1e-11 where they cancel by ten."""
+    P, L = 64, 12.42
+    x0, mass = inputs.water_lattice_box(64, L, P, 2, jitter=0.02)
+    x0 = x0 - x0[:, 0::3].mean(0).min(0)   # the cluster in a corner
+    big, a = 96.0, 8.0
+    g = np.stack(np.meshgrid(*[np.arange(2, 12) * a - 4.0] * 3, indexing="ij"), -1).reshape(-1, 3)
+    site = g[np.linalg.norm(np.maximum(g - L, 0.0), axis=1) > 7.9]
+    ff = (0.0,) + inputs.WATER_FF[1:2] + (0.0,) + inputs.WATER_FF[3:]
+    geo = x0[:1, 0:3] - x0[:1, 0:1]
+    out = []
+    for idle in (0, 236, 600):
+        x = np.concatenate([x0] + [np.repeat(geo + p, P, axis=0) for p in site[:idle]], axis=1)
+        sim = pimd.Simulation(x, np.tile(mass[:3], x.shape[1] // 3), v0=np.zeros_like(x), T=300.0, dt=1e-4,
+                              potential=1, ff=ff, box=(big,) * 3, seed=5, precision=pimd.PREC_SPLIT)
+        e = sim.estimators()
+        out.append((e["U_bead"], e["vir_sum"]))
+        sim.close()
+    for u, w in out[1:]:
+        assert np.abs(u - out[0][0]).max() < 1e-11 * np.abs(out[0][0]).max()
+        assert abs(w - out[0][1]) < 1e-11 * abs(out[0][1])
