@@ -1280,66 +1280,102 @@ __global__ void __launch_bounds__(128) k_bclose(const RepDesc *reps, const int2 
   }
 }
 
-// The closing kick of one warp item on tensor cores: F~ = M F as in the step,
-// then B(h/2) (and O(h/2)) on the velocities; lane (g, t) holds modes 16 mt + g
-// (+ 8) of atoms 2t, 2t + 1.
+// Mode k's terms of a row folded by parity (even modes k <= H = P / 2: terms j at
+// j; odd ones: terms j at P - j), and the sum over such a row x.
+template <int P>
+__device__ __forceinline__ void fold_row(const float *__restrict__ Mt, int k, float (&m)[P / 2], float &mH) {
+  constexpr int H = P / 2;
+  const bool even = k <= H;
+#pragma unroll
+  for (int b = 0; b < H / 4; ++b)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = even ? 4 * b + q : 4 * b + 4 - q;
+      m[4 * b + q] = !even && j == H ? 0.f : __ldg(Mt + j * P + k);
+    }
+  mH = even ? __ldg(Mt + H * P + k) : 0.f;
+}
+
+template <int P>
+__device__ __forceinline__ float fold_mode(const float *__restrict__ x, int k, const float (&m)[P / 2], float mH) {
+  constexpr int H = P / 2;
+  float qa = mH * x[H], qb = 0.f;
+#pragma unroll
+  for (int b = 0; b < H / 4; ++b) {
+    const float4 v = *reinterpret_cast<const float4 *>(x + (k <= H ? 4 * b : P - 4 - 4 * b));
+    qa = fmaf(m[4 * b], v.x, qa);
+    qb = fmaf(m[4 * b + 1], v.y, qb);
+    qa = fmaf(m[4 * b + 2], v.z, qa);
+    qb = fmaf(m[4 * b + 3], v.w, qb);
+  }
+  return qa + qb;
+}
+
+// The closing kick of one warp item, FP32: the staged forces are folded by the
+// parity of the modes (e_j = F_j + F_{P-j} kept at j, o_j = F_j - F_{P-j} at P - j),
+// lane (atom group, mode) forms F~ = M F with its row of M in registers, then
+// B(h/2) (and O(h/2)) on the velocities.  3xTF32 products on tensor cores, whose
+// accumulation truncates, were no faster (a pass of the 256-replica mix, 20 steps,
+// 6.55 ms; 6.53 so) and left an rms error of 1.7e-8 (16 beads) to 3.6e-8 (128) of
+// the centroid mode's kick; this form 2e-9 to 4e-9, the plain sum over a row 3e-9 to 6e-9.
 template <int P>
 __device__ __forceinline__ void bclose_warp(const RepDesc &R, int tile, float *__restrict__ sF, uint64_t step) {
-  constexpr int PS = P + 4, MT = (P + 15) / 16, CPR = P / 4;
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  constexpr int PS = P + 4, CPR = P / 4, H = P / 2;
+  constexpr int PL = P < 32 ? P : 32, NG = 32 / PL, NCH = (P + 31) / 32;
+  const int lane = threadIdx.x & 31, grp = lane / PL, kl = lane % PL;
   const int tile0 = tile * kWAtoms, na = min(kWAtoms, R.N - tile0);
   const size_t base = (size_t)tile0 * 3 * P;
   const float *__restrict__ gF = R.F + base;
   for (int q = lane; q < na * 3 * CPR; q += 32) {
     const int row = q / CPR, col = (q - row * CPR) * 4;
-    const int a = row / 3, c = row - 3 * a;
-    cp_async16(sF + (c * 8 + a) * PS + col, gF + (size_t)row * P + col);
+    cp_async16(sF + row * PS + col, gF + (size_t)row * P + col);
   }
   cp_async_commit();
-  for (int q = lane; q < (kWAtoms - na) * 3 * P; q += 32) {   // rows of missing atoms
-    const int r = q / P, j = q - r * P;
-    sF[((r % 3) * 8 + na + r / 3) * PS + j] = 0.f;
-  }
   cp_async_wait_all();
   __syncwarp();
-  float C[MT][3][4];
-  fwd_tile<P, MT>(R.mfa_hi, R.mfa_lo, sF, 0, C);
+  for (int q = lane; q < na * 3 * (H - 1); q += 32) {
+    const int row = q / (H - 1), j = 1 + q - row * (H - 1);
+    float *x = sF + row * PS;
+    const float u = x[j], w = x[P - j];
+    x[j] = u + w;
+    x[P - j] = u - w;
+  }
+  __syncwarp();
   const bool bath = R.integrator == 1 && R.thermo;
   const float half = 0.5f * (float)R.dt;
   float *__restrict__ vkg = R.vk + base;
 #pragma unroll
-  for (int mt = 0; mt < MT; ++mt)
+  for (int cc = 0; cc < NCH; ++cc) {
+    const int k = kl + 32 * cc;
+    float m[H], mH;
+    fold_row<P>(R.Mtf, k, m, mH);
+    const float c1 = __ldg(R.c1f + k), c2 = __ldg(R.c2f + k);
+    for (int a = grp; a < na; a += NG) {
+      const int i = tile0 + a;
+      float f[3], e[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = 16 * mt + g + 8 * h;
-      if (k >= P) continue;
+      for (int c = 0; c < 3; ++c) f[c] = fold_mode<P>(sF + (a * 3 + c) * PS, k, m, mH);
+      if (bath) gauss3f_b(R.seed, (uint32_t)i, (uint32_t)k, kStreamO2, step, e[0], e[1], e[2]);
+      if (k == 0) {
 #pragma unroll
-      for (int aa = 0; aa < 2; ++aa) {
-        const int a = 2 * t + aa, i = tile0 + a;
-        if (a >= na) continue;
-        float e[3] = {0.f, 0.f, 0.f};
-        if (bath) gauss3f_b(R.seed, (uint32_t)i, (uint32_t)k, kStreamO2, step, e[0], e[1], e[2]);
-        if (k == 0) {
+        for (int c = 0; c < 3; ++c) {
+          const size_t ic = (size_t)i * 3 + c;
+          double v = fma(0.5 * R.dt * __ldg(R.inv_mm + i), (double)f[c], R.v0[ic]);
+          if (bath) v = fma(R.c1_0, v, R.c2_0 * __ldg(R.sigv + i) * (double)e[c]);
+          R.v0[ic] = v;
+        }
+      } else {
+        const float kb = half * __ldg(R.inv_mmf + i), c2s = c2 * __ldg(R.sigvf + i);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const size_t ic = (size_t)i * 3 + c;
-            double v = fma(0.5 * R.dt * __ldg(R.inv_mm + i), (double)C[mt][c][2 * h + aa], R.v0[ic]);
-            if (bath) v = fma(R.c1_0, v, R.c2_0 * __ldg(R.sigv + i) * (double)e[c]);
-            R.v0[ic] = v;
-          }
-        } else {
-          const float kb = half * __ldg(R.inv_mmf + i);
-          const float c1 = __ldg(R.c1f + k), c2s = __ldg(R.c2f + k) * __ldg(R.sigvf + i);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            float *v = vkg + (a * 3 + c) * P + k;
-            float w = fmaf(kb, C[mt][c][2 * h + aa], *v);
-            if (bath) w = fmaf(c1, w, c2s * e[c]);
-            *v = w;
-          }
+        for (int c = 0; c < 3; ++c) {
+          float *v = vkg + (a * 3 + c) * P + k;
+          float w = fmaf(kb, f[c], *v);
+          if (bath) w = fmaf(c1, w, c2s * e[c]);
+          *v = w;
         }
       }
     }
+  }
   __syncwarp();   // the slot is free for the next item
 }
 
@@ -1878,32 +1914,13 @@ __device__ void best_warp(const RepDesc &R, int e, float *__restrict__ slot, dou
 #pragma unroll
     for (int cc = 0; cc < NCH; ++cc) {
       const int k = kl + 32 * cc;
-      const bool even = k <= H;
-      // even modes: terms j = 4 b + q at j, and j = H; odd ones: j = 4 b + 4 - q at P - j
-      float m[H];
-#pragma unroll
-      for (int b = 0; b < H / 4; ++b)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int jt = even ? 4 * b + q : 4 * b + 4 - q;
-          m[4 * b + q] = !even && jt == H ? 0.f : __ldg(R.Mtf + jt * P + k);
-        }
-      const float mH = even ? __ldg(R.Mtf + H * P + k) : 0.f;
+      float m[H], mH;
+      fold_row<P>(R.Mtf, k, m, mH);
       for (int a = grp; a < na; a += NG) {
         float q2 = 0.f, qc[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const float *x = sX + (c * 8 + a) * PS;
-          float qa = mH * x[H], qb = 0.f;
-#pragma unroll
-          for (int b = 0; b < H / 4; ++b) {
-            const float4 v = *reinterpret_cast<const float4 *>(x + (even ? 4 * b : P - 4 - 4 * b));
-            qa = fmaf(m[4 * b], v.x, qa);
-            qb = fmaf(m[4 * b + 1], v.y, qb);
-            qa = fmaf(m[4 * b + 2], v.z, qa);
-            qb = fmaf(m[4 * b + 3], v.w, qb);
-          }
-          qc[c] = qa + qb;
+          qc[c] = fold_mode<P>(sX + (c * 8 + a) * PS, k, m, mH);
           q2 = fmaf(qc[c], qc[c], q2);
         }
         const double md = __ldg(R.mass_mm + tile0 + a);
