@@ -400,7 +400,8 @@ pimd_status pimd_batch_get_state(pimd_batch *b, int32_t slot, double *x, double 
  * batch by timing candidates with CUDA events while the replicas step
  * (steps_per_trial steps per candidate; they count toward the replicas'
  * budgets; trajectories do not depend on the tile), and the blocks per SM of
- * the 64-bead warp-item step kernel.  tiles_out, if not NULL, receives
+ * the 64-bead warp-item step kernel, from one to its occupancy limit (one step,
+ * then two rounds over the candidates).  tiles_out, if not NULL, receives
  * PIMD_MAX_BEADS + 1 entries: [0] the 64-bead warp-item blocks per SM, [P]
  * the tile for bead count P (0 = unused; 8 for the warp-item counts). */
 pimd_status pimd_batch_autotune(pimd_batch *b, int32_t steps_per_trial, int32_t *tiles_out);

@@ -3362,25 +3362,24 @@ extern "C" pimd_status pimd_batch_autotune(pimd_batch *b, int32_t steps_per_tria
             cudaSuccess ||
         nbmax < 1)
       nbmax = 1;
-    // each candidate, the occupancy limit and the two below it: one untimed
-    // step (caches and clocks settle), then the faster of two timed trials; a
-    // smaller grid than the limit must win by more than 3% (the timings are a
-    // few milliseconds and noisy)
-    const int nbmin = std::max(1, nbmax - 2);
+    // every grid from one block an SM to the occupancy limit: an untimed step
+    // (caches and clocks settle), then two rounds over the candidates, the
+    // faster trial of each counting; a smaller grid than the limit must win by
+    // more than 3% (the timings are a few milliseconds and noisy).  Eight
+    // tunings of the 256-replica mix chose four blocks eight times.
+    if (launch_one_step(b, nullptr, nullptr) != cudaSuccess) return fail(PIMD_ECUDA, "autotune step failed");
+    b->launches += step_launches(b);
     std::vector<float> tms(nbmax + 1, 1e30f);
-    for (int nb = nbmax; nb >= nbmin && st == PIMD_OK; --nb) {
+    for (int t = 0; t < 2 * nbmax && st == PIMD_OK; ++t) {
+      const int nb = nbmax - t % nbmax;
       b->wblocks_sm = nb;
       b->grid_w = b->nsm * nb;
-      if (launch_one_step(b, nullptr, nullptr) != cudaSuccess) return fail(PIMD_ECUDA, "autotune step failed");
-      b->launches += step_launches(b);
-      for (int rep = 0; rep < 2 && st == PIMD_OK; ++rep) {
-        float ms = 0.f;
-        st = time_step(&ms);
-        if (st == PIMD_OK) tms[nb] = std::min(tms[nb], ms);
-      }
+      float ms = 0.f;
+      st = time_step(&ms);
+      if (st == PIMD_OK) tms[nb] = std::min(tms[nb], ms);
     }
     int best = nbmax;
-    for (int nb = nbmax - 1; nb >= nbmin; --nb)
+    for (int nb = nbmax - 1; nb >= 1; --nb)
       if (tms[nb] < 0.97f * tms[best]) best = nb;
     b->wblocks_sm = best;
     b->wtuned = best;
