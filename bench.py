@@ -17,7 +17,6 @@ host cores instead (rank 0 only).
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import math
 import os
@@ -169,6 +168,20 @@ def step_flops_per_bead_atom(P):
     return 9 * P + 78
 
 
+# 32 x 32 -> 64-bit integer multiply-adds of a GB300 a second (eight independent
+# chains a thread, four blocks of 256 threads an SM, measured): the rate that
+# the fixed-point transforms of the FP64 step are held against
+INT_MAD_RATE = 18.1e12
+
+
+def well_step_mads_per_bead_atom(P):
+    """Integer multiply-adds of the FP64 step kernel per bead-atom in a harmonic
+    well, where F~ = -k q~ leaves two transforms of 3 components: an output is a
+    sum over one half of its folded row in pairs of terms, three multiply-adds a
+    product (28-bit limbs).  Noise and scalings are not counted."""
+    return 2 * 3 * 3 * 2 * ((P // 2 + 2) // 2)
+
+
 def force_flops(x, L, rc, rlist):
     """Algorithmic FP64 flops of one water force launch (all beads) for the
     positions x [P][N][3]: 30 per O-O pair inside rc, each unordered pair
@@ -193,23 +206,6 @@ def force_flops(x, L, rc, rlist):
     return 30.0 * inside + 120.0 * nmol * P, 17.0 * cand * P
 
 
-def traffic_for(kernel):
-    """DRAM bytes per launch from the committed ncu summary, or None when the
-    kernel source changed since the counters were taken."""
-    path = os.path.join(ROOT, "profiles", "traffic.json")
-    if not os.path.exists(path):
-        return None
-    try:
-        t = json.load(open(path)).get(kernel)
-        src = os.path.join(ROOT, "paper_2602_13553_gb300", "csrc", t["source"])
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
-        if sha != t["source_sha256_16"]:
-            return None
-        return float(t["bytes_per_launch"])
-    except Exception:
-        return None
-
-
 def hbm_peak():
     """Measured copy bandwidth of this GPU pool (GB/s), else the fallback."""
     try:
@@ -221,15 +217,17 @@ def hbm_peak():
 SWEEP = ((1 << 20, 8), (1 << 18, 32), (1 << 17, 64), (1 << 16, 128))
 
 
-def sweep_bench(stream, fp64_peak, steps=4, warmup=2):
+def sweep_bench(stream, steps=4, warmup=2):
     """The oscillator throughput sweep: N independent 3D oscillators (m = 1.008
     amu, hbar omega = 0.1 eV, 300 K, dt = 0.25 fs, PILE_L) with N P = 2^23
     bead-atoms (201 MB of FP64 state, beyond the 129 MB L2) for P = 8, 32,
     64, 128, in FP64 and in split precision.  Per point: bead-atom-steps/s
     over `steps` calls of 10 MD steps (CUDA events on the library's stream)
     and the roofline of the step kernel, from its own CUDA-event time per
-    launch: FP64 against the FP64 pipe (step_flops_per_bead_atom: folded
-    transforms), split against HBM (60 B + 96 B / P per bead-atom)."""
+    launch: FP64 against the integer pipe, which holds its transforms
+    (well_step_mads_per_bead_atom), split against HBM (48 B + 96 B / P per
+    bead-atom: deviations and velocities read and written, no forces; the
+    centroids)."""
     import torch
     from paper_2602_13553_gb300 import binding, inputs
     hbar = 4.135667403e-3 / (2 * math.pi)
@@ -261,12 +259,12 @@ def sweep_bench(stream, fp64_peak, steps=4, warmup=2):
             pt = {"N": N, "P": P, "precision": name, "value": units * 10 * steps / (ms / 1e3),
                   "step_kernel_ms": step_ms}
             if prec == 0:
-                ach = step_flops_per_bead_atom(P) * units / (step_ms / 1e3) / 1e12
-                pt["roofline"] = {"bound": "alu", "achieved": ach, "peak": fp64_peak,
-                                  "unit": "TFLOP/s", "frac": ach / fp64_peak,
-                                  "peak_source": "measured FP64 FMA throughput"}
+                ach = well_step_mads_per_bead_atom(P) * units / (step_ms / 1e3) / 1e12
+                pt["roofline"] = {"bound": "alu", "achieved": ach, "peak": INT_MAD_RATE / 1e12,
+                                  "unit": "T 32-bit multiply-adds/s", "frac": ach / (INT_MAD_RATE / 1e12),
+                                  "peak_source": "measured 32 x 32 -> 64-bit multiply-add throughput"}
             else:
-                ach = (60.0 + 96.0 / P) * units / (step_ms / 1e3) / 1e9
+                ach = (48.0 + 96.0 / P) * units / (step_ms / 1e3) / 1e9
                 pt["roofline"] = {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",
                                   "frac": ach / hbm, "peak_source": hsrc}
             out.append(pt)
@@ -381,7 +379,6 @@ def batched_bench(stream, steps, warmup):
                      "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "peak_source": src, "algorithmic_bytes_per_launch": bytes_,
                      "avg_launch_ms": per_ms,
-                     "traffic": traffic_for("k_bstep_w" if dom == "step" else "k_bforce"),
                      "kernel_time_share": {k: round(v / tot, 4) for k, v in kt.items()}},
         "same_mix": {"plain_fp64_handles": same_mix_handles(reps, 0), "split_handles": same_mix_handles(reps, 1),
                      "unit": METRIC,
@@ -668,7 +665,6 @@ def run_ours(args):
                                                "md_step_latency_us": md_ms * 1e3}),
         "roofline": {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": fp64_peak,
                      "unit": "TFLOP/s", "frac": achieved / fp64_peak,
-                     "traffic": traffic_for(kname),
                      "peak_source": "measured: FP64 FMA throughput of this GPU (pimd_fp64_fma_rate), "
                                     "nominal %.2f" % (FP64_NOMINAL / 1e12),
                      "algorithmic_flops_per_launch": flops,
@@ -692,7 +688,7 @@ def run_ours(args):
     if world == 1 and not args.no_serve:
         line["serve"] = serve_bench(stream, args.serve_jobs, args.serve_step_scale)
     if world == 1 and not args.no_sweep:
-        line["sweep"] = sweep_bench(stream, fp64_peak)
+        line["sweep"] = sweep_bench(stream)
     if not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline()
         line["cpu_baseline"]["configs"] = oracle_configs()
