@@ -1315,9 +1315,11 @@ __device__ __forceinline__ float fold_mode(const float *__restrict__ x, int k, c
 // parity of the modes (e_j = F_j + F_{P-j} kept at j, o_j = F_j - F_{P-j} at P - j),
 // lane (atom group, mode) forms F~ = M F with its row of M in registers, then
 // B(h/2) (and O(h/2)) on the velocities.  3xTF32 products on tensor cores, whose
-// accumulation truncates, were no faster (a pass of the 256-replica mix, 20 steps,
-// 6.55 ms; 6.53 so) and left an rms error of 1.7e-8 (16 beads) to 3.6e-8 (128) of
-// the centroid mode's kick; this form 2e-9 to 4e-9, the plain sum over a row 3e-9 to 6e-9.
+// accumulation truncates, took 86 us on the 256-replica mix against 58 so, and
+// left an rms error of 1.7e-8 (16 beads) to 3.6e-8 (128) of the centroid mode's kick;
+// this form 2e-9 to 4e-9, the plain sum over a row 3e-9 to 6e-9.  The centroid mode's
+// FP64 comes after the others, a lane for each (atom, component): inside their loop,
+// an atom's three on one lane, it held the FP64 pipe for 86 of 116 us.
 template <int P>
 __device__ __forceinline__ void bclose_warp(const RepDesc &R, int tile, float *__restrict__ sF, uint64_t step) {
   constexpr int PS = P + 4, CPR = P / 4, H = P / 2;
@@ -1356,13 +1358,11 @@ __device__ __forceinline__ void bclose_warp(const RepDesc &R, int tile, float *_
 #pragma unroll
       for (int c = 0; c < 3; ++c) f[c] = fold_mode<P>(sF + (a * 3 + c) * PS, k, m, mH);
       if (bath) gauss3f_b(R.seed, (uint32_t)i, (uint32_t)k, kStreamO2, step, e[0], e[1], e[2]);
-      if (k == 0) {
+      if (k == 0) {   // for the centroid mode below: the rows' padding holds F~_0 and its deviate
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const size_t ic = (size_t)i * 3 + c;
-          double v = fma(0.5 * R.dt * __ldg(R.inv_mm + i), (double)f[c], R.v0[ic]);
-          if (bath) v = fma(R.c1_0, v, R.c2_0 * __ldg(R.sigv + i) * (double)e[c]);
-          R.v0[ic] = v;
+          sF[(a * 3 + c) * PS + P] = f[c];
+          sF[(a * 3 + c) * PS + P + 1] = e[c];
         }
       } else {
         const float kb = half * __ldg(R.inv_mmf + i), c2s = c2 * __ldg(R.sigvf + i);
@@ -1375,6 +1375,15 @@ __device__ __forceinline__ void bclose_warp(const RepDesc &R, int tile, float *_
         }
       }
     }
+  }
+  __syncwarp();
+  // centroid mode in FP64, one (atom, component) per lane
+  if (lane < 3 * na) {
+    const int i = tile0 + lane / 3;
+    const size_t ic = (size_t)tile0 * 3 + lane;
+    double v = fma(0.5 * R.dt * __ldg(R.inv_mm + i), (double)sF[lane * PS + P], R.v0[ic]);
+    if (bath) v = fma(R.c1_0, v, R.c2_0 * __ldg(R.sigv + i) * (double)sF[lane * PS + P + 1]);
+    R.v0[ic] = v;
   }
   __syncwarp();   // the slot is free for the next item
 }
