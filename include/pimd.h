@@ -280,7 +280,9 @@ pimd_status pimd_get_state(pimd_handle *h, double *x, double *v_nm, int64_t *ste
 /* Replace the state from host arrays (layouts as pimd_get_state; both x and
  * v_nm are required) and recompute the forces.  Together with
  * pimd_get_state this is checkpoint / resume: the noise is keyed on the step
- * counter, so a resumed run continues bit for bit. */
+ * counter, and in FP64 a resumed run continues bit for bit.  In split precision
+ * set_state makes the centroid the beads' mean and the deviations its FP32
+ * remainders, so a resumed run agrees to FP32 rounding of the deviations. */
 pimd_status pimd_set_state(pimd_handle *h, const double *x, const double *v_nm, int64_t step);
 
 /* The barostat state (App. E) for checkpoints: vW (1/ps) and box[3] (A).

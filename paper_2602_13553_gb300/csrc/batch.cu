@@ -1989,7 +1989,7 @@ __device__ void best_warp(const RepDesc &R, int e, float *__restrict__ slot, dou
 // and the bead mean of d in FP32 from the FP32 deviations).  One row of
 // est_columns(P) sums per e-block.  A thread-per-task form with every product
 // converted to FP64, and the rows of U and Tr Xi left to pass 2, took 694 +
-// 246 us on the 256-replica mix.
+// 246 us on the 256-replica mix; this one 229 + 28.
 __global__ void __launch_bounds__(128) k_best(const RepDesc *reps, const int2 *items, const int *count,
                                               int slot_floats) {
   extern __shared__ __align__(16) float wsm[];

@@ -2,7 +2,7 @@
 //
 // The FP64 pipe issues one warp instruction every 64 clocks per SM partition
 // (two FMAs a clock and SM, measured), the integer pipe a 32 x 32 -> 64
-// multiply-add every 2.4 (62 a clock and SM): a sum of products is therefore
+// multiply-add every 2.2 (58 a clock and SM): a sum of products is therefore
 // taken in integers, with more bits than FP64 keeps.
 //
 // A row x_0 .. x_{P-1} is scaled by the power of two above its largest element,

@@ -76,11 +76,12 @@ __global__ void __launch_bounds__(256) k_force_harmonic_f64(ForceArgs a) {
 //    list over `split` warps, which also take the step's list check, and gives
 //    its bonds and angle to one more that starts at once; the partial sums are
 //    joined as integers, a component to a warp, and converted once.
-// Measured, us a launch: 512 molecules x 64 beads 172 in FP64, now about 32 (FP64
-// instructions and integer issue 13.5 each of it).  With
-// seven list warps, FP64 partial sums and two bonded warps behind the list check
-// against now: 64 x 32 beads 11.1 / 10.4 (16.7 in FP64), 100 x 12 13.2 / 11.1,
-// 125 x 16 with the diagonal virial 16.1 / 13.5.
+// Measured, us a launch: 512 molecules x 64 beads 172 in FP64, now 39 (FP64
+// instructions 10, integer issue 16 of it); 64 x 32 16.7 and 9.8.  Seven list warps,
+// FP64 partial sums and two bonded warps behind the list check, against this form
+// (before a pair's terms were formed at its own scale, ljfix.cuh): 64 x 32 beads
+// 11.1 / 10.4, 100 x 12 13.2 / 11.1 (11.5 now), 125 x 16 with the diagonal virial
+// 16.1 / 13.5 (13.6 now).
 // A neighbour's bucket (j mod NS) decides its warp, so every sum depends only on
 // the set of interacting pairs: a rebuilt list cannot change a bit.
 // kDiag (anisotropic barostat) also sums the diagonal of the virial tensor,
@@ -177,9 +178,9 @@ __device__ __noinline__ void pair_f64(const ForceArgs &a, const double *L, const
 
 // kSplit: 0 one warp a unit, 1 up to 14 list warps, 2 four of them, with the
 // registers (96) that put four blocks on an SM: a pass of 512 molecules x 64
-// beads, 20 steps, 1.66 ms with 101 registers and three blocks, 1.56 so; five
-// blocks (72, spills) are faster only at 1024 units and more (68.7 against 69.5 us
-// a step there, 35.4 against 33.3 at 400)
+// beads, 20 steps, 1.66 ms with 101 registers and three blocks, 1.56 so (1.61 with
+// today's pair terms); five blocks (72, spills) are faster only at 1024 units and more
+// (68.7 against 69.5 us a step there, 35.4 against 33.3 at 400)
 template <bool kDiag, int kSplit>
 __global__ void __launch_bounds__(kSplit == 2 ? 160 : (kSplit ? 480 : 128), kSplit == 2 ? 4 : 1) k_force_water_f64(ForceArgs a, int split) {
   constexpr int NC = kDiag ? 14 : 11;   // F (9), U, Tr Xi, then Xi_xx, Xi_yy, Xi_zz
@@ -239,7 +240,9 @@ __global__ void __launch_bounds__(kSplit == 2 ? 160 : (kSplit ? 480 : 128), kSpl
       xi[c] = xp[(size_t)(3 * m + c) * P];
     }
     PairF64 far;
-    // fixed point holds edges below 8192 A (the barostat may change them)
+    // wrapped positions hold edges below 8192 A; half of that is used, with room
+    // for the wrap's rounding (a system set up with an edge of 2048 A or more is
+    // off from the start; the barostat may grow one past the line)
     const int top = __double2hiint(4096.0);
     const bool fixed =
         lj.on && __double2hiint(L[0]) < top && __double2hiint(L[1]) < top && __double2hiint(L[2]) < top;
@@ -424,12 +427,15 @@ int water_units(int nmol, int P) {
   return (nmol + G - 1) / G * ((P + Bk - 1) / Bk);
 }
 
-// Warps that share a unit's neighbour list (divisors of NS, a multiple of 14).
+// Warps that share a unit's neighbour list: each takes a range of consecutive
+// buckets, [role NS / split, (role + 1) NS / split), equal in size where split
+// divides NS (a multiple of 14) and one apart otherwise.
 // 1, a warp takes whole units and makes no reduction, from eight units an SM on:
-// us a step, split 1 against 4, 1024 units 69.8 against 65.4, 1400 units 87.3
-// against 91.1, 2048 equal.  Below, warps are short of work and the list's chain
-// is what counts: 4 against 7 at 432 units 33.8 against 41, at 160 24.5 against
-// 23.9; 7 against 14 at 125 units (a block has its SM to itself) 21.8 against 19.9.
+// us a step, split 1 against 4, 1024 units 68.1 against 66.4, 1200 73.2 against 73.8,
+// 1400 84.0 against 85.9, 2048 106 against 117.  Below, warps are short of work and
+// the list's chain is what counts: 4 against 7 at 432 units 33.1 against 39.2, at 160
+// 25.0 against 23.9; 7 against 14 at 125 units (a block has its SM to itself) 19.9
+// against 18.4.
 static int water_split(int nmol, int P) {
   const int n = water_units(nmol, P);
   return n >= 1216 ? 1 : (n >= 192 ? 4 : (n > 152 ? 7 : 14));

@@ -1,7 +1,7 @@
 // ljfix.cuh -- Lennard-Jones pairs in 64-bit fixed point (FP64 water force).
 //
-// An FP64 instruction costs a warp 64 clocks, a 64-bit high product 15.5 and
-// a 32-bit multiply-add 2.4, so the pairs of the O-O sum are evaluated in
+// An FP64 instruction costs a warp 64 clocks, a 64-bit high product 17 and
+// a 32-bit multiply-add 2.2, so the pairs of the O-O sum are evaluated in
 // integers.  Lengths are scaled by the power of two 2^b above the cutoff and
 // x = r^2 / 2^2b; y = 2^-e / x is in (0, 1] down to the distance 2^(b - e/2),
 // which lies between 0.56 and 0.79 sigma (farther out for sigma below a tenth of

@@ -419,7 +419,7 @@ struct FloatPair {
 // the list check compares in FP32, U and Tr Xi are sums of FP32 terms with their
 // rounding errors kept (plain FP32 chains were 3e-8 of the sum off and 1% of a pass
 // faster).  80 FP64 instructions a warp held 22 of 35.6 us at 512 molecules x 64
-// beads and 5 of 13.4 at 216 x 20; now 15.5 and 8.1 us.
+// beads and 5 of 13.4 at 216 x 20; now 15.0 and 7.8 us.
 template <bool kSplit>
 __global__ void __launch_bounds__(kSplit ? 256 : 128) k_force_water_split(SplitForceArgs a, int split) {
   extern __shared__ __align__(16) unsigned char fsm[];
@@ -676,11 +676,11 @@ int force_blocks(int n_groups, int P);
 int force_block_threads(int P);
 int water_units(int nmol, int P);
 
-// Warps that share a unit's neighbour list (divisors of NS, a multiple of 14);
-// 1: a warp takes whole units.  us a step, 1 against 2: 1024 units 39.2 against
-// 32.4, 1400 units 40.2 against 40.8, 2048 units 49.7 against 52.4; 2 against 7:
-// 600 units 29.7 against 30.2; 4 against 7: 432 units 26.0 against 25.6, 216
-// units 18.3 against 17.2 (14: 19.5).
+// Warps that share a unit's neighbour list (ranges of buckets, as in FP64);
+// 1: a warp takes whole units.  us a step, 1 against 2: 1024 units 32.1 against
+// 30.4, 1400 units 33.1 against 37.2, 2048 units 38.4 against 43.2; 2 against 7:
+// 600 units 27.6 against 28.4; 432 units 26.5 against 23.0; 4 against 7 at 432 units
+// 23.6 against 23.0.
 static int split_water_warps(int nmol, int P) {
   const int n = water_units(nmol, P);
   return n >= 1216 ? 1 : (n >= 512 ? 2 : 7);
