@@ -70,7 +70,7 @@ __device__ __forceinline__ double warp_max(double v) {
 //
 // Measured, us a launch, with FP64 transforms and noise and the forces read
 // against now: 65536 oscillators x 32 beads 1724 (and 61 of the force kernel) /
-// 262 (FP64 instructions 181, issue 185 of it), 512 molecules x 64 beads 121 / 28,
+// 259 (FP64 instructions 160, issue 186 of it), 512 molecules x 64 beads 121 / 28,
 // 64 x 32 14.4 / 7.6.
 template <int kPhase, bool kObabo, bool kHarm>
 __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {

@@ -13,7 +13,7 @@
 // single blocks with one thread per atom (strided reads, N P serial terms)
 // they were most of a step: the barostat 72 us a call (two a step) for 125
 // molecules x 16 beads, fixcom 50 us for 91 molecules x 17 beads and 192 us
-// for 100 molecules x 12 Cartesian beads; now 11.6, 10.1 and 9.5.  (The factor
+// for 100 molecules x 12 Cartesian beads; now 12.0, 10.1 and 9.5.  (The factor
 // (e^a - e^-a) / (2 v_W) from the series of sinh would need no division and no
 // cancellation, but leaves the published form by its 1e-11 at small a.)
 #include "common.cuh"
