@@ -367,6 +367,7 @@ static StepArgs step_args(pimd_handle *h) {
   a.step_off = 0;
   const bool water = h->potential == PIMD_POT_WATERLIKE;
   a.xi = water ? h->xi : nullptr;
+  a.pos = h->lj.pos;
   for (int d = 0; d < 3; ++d) {
     a.box[d] = h->box[d];
     a.invbox[d] = h->box[d] > 0 ? 1.0 / h->box[d] : 0.0;

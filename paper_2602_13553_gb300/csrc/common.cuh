@@ -186,6 +186,7 @@ struct StepArgs {
   const int64_t *step;         // device step counter (step index of this step = *step + step_off)
   int step_off;
   long long *xi;               // water: [nmol][3][P] wrapped fixed-point positions of the oxygens, or null
+  int pos;                     // their fraction bits (LjFix)
   double box[3], invbox[3];    // water
   const double *dbox;          // device box (barostat state at kBaroL), overriding box/invbox, or null
   // water-like systems: neighbour-list skin check of the oxygens (atoms 3m)

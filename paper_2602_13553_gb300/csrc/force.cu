@@ -236,14 +236,11 @@ __global__ void __launch_bounds__(kSplit == 2 ? 160 : (kSplit ? 480 : 128), kSpl
     const int64_t *__restrict__ xp = a.xi + k;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      LQ[c] = fix_pos(L[c]);
+      LQ[c] = fix_pos(L[c], lj.pos);
       xi[c] = xp[(size_t)(3 * m + c) * P];
     }
     PairF64 far;
-    // wrapped positions hold edges below 8192 A; half of that is used, with room
-    // for the wrap's rounding (a system set up with an edge of 2048 A or more is
-    // off from the start; the barostat may grow one past the line)
-    const int top = __double2hiint(4096.0);
+    const int top = __double2hiint(lj.edge);   // the barostat may change the box
     const bool fixed =
         lj.on && __double2hiint(L[0]) < top && __double2hiint(L[1]) < top && __double2hiint(L[2]) < top;
     auto pair = [&](const int64_t (&xj)[3], int j) {
@@ -500,7 +497,7 @@ __global__ void k_fix_positions(ForceArgs a, long long *xi) {
   double L[3], iL[3];
   list_box(a.nb, L, iL);
   const double x = a.x[(size_t)(9 * m + c) * a.P + k];
-  xi[t] = fix_wrap(x, (float)x, (float)iL[c], fix_pos(L[c]));
+  xi[t] = fix_wrap(x, a.lj.pos, (float)x, (float)iL[c], fix_pos(L[c], a.lj.pos));
 }
 
 cudaError_t launch_fix_positions(const ForceArgs &a, long long *xi, cudaStream_t s) {

@@ -31,15 +31,24 @@
 
 namespace pimd {
 
-constexpr int kPosBits = 50;   // positions and separations: Q50 angstrom
+// Positions and separations have `pos` fraction bits, in angstrom: 53 where every
+// edge is below 256 A, 50 below 2048 A.  Of the 2^(63 - pos) A that 64 bits hold a
+// quarter is used at set-up and half at run time (the barostat may grow a box; the
+// rest is room for the wrap's rounding).  A coordinate of less than 2^(52 - pos) A is
+// rounded where FP64 had it exactly: with 50 bits throughout, the force of a pair
+// 2.5 to 5.9 A apart in a box of 12.42 A was 5.4e-16 of itself off (rms, from FP64
+// positions around the origin), FP64 expressions 5.1e-16; with 53 bits 1.3e-16.
+constexpr int kPosFine = 53, kPosCoarse = 50;
 
 struct LjFix {
   int on;                      // 0: every pair in FP64
+  int pos;                     // fraction bits of positions and separations
   int b, e;
+  double edge;                 // edges from here on take the FP64 expressions
   uint64_t rc2;                // cutoff, x Q64
   uint64_t xmin;               // closer pairs in FP64, x Q62
   uint64_t C;                  // Q58
-  float rpre2;                 // 1.008 rc^2 in units of 2^-18 A squared: the quick test
+  float rpre2;                 // 1.008 rc^2 in units of 2^(32 - pos) A squared: the quick test
   double fs, us, ws, w3;       // force, energy (half), virial (half), diagonal virial of the sums
 };
 
@@ -53,7 +62,11 @@ inline LjFix lj_fix_setup(double eps, double sig, double rc, const double *box) 
   while (e < 7 && s2 * std::ldexp(1.0, e + 1) <= 3.17) ++e;
   const double ratio = s2 * std::ldexp(1.0, e);
   p.on = ratio <= 3.17 && std::ldexp(1.0, b) >= 1.01 * rc && rc > 0.01;
-  for (int c = 0; c < 3; ++c) p.on = p.on && box[c] < 2048.0;
+  p.pos = kPosFine;
+  for (int c = 0; c < 3; ++c)
+    if (!(box[c] < std::ldexp(1.0, 61 - kPosFine))) p.pos = kPosCoarse;
+  for (int c = 0; c < 3; ++c) p.on = p.on && box[c] < std::ldexp(1.0, 61 - p.pos);
+  p.edge = std::ldexp(1.0, 62 - p.pos);
   p.b = b;
   p.e = e;
   if (!p.on) return p;
@@ -61,7 +74,7 @@ inline LjFix lj_fix_setup(double eps, double sig, double rc, const double *box) 
   p.rc2 = (uint64_t)std::ldexp(rc * rc, 64 - 2 * b);
   p.xmin = (uint64_t)std::ldexp(1.0 + 1.0 / 1024, 62 - e);
   p.C = (uint64_t)std::ldexp(2.0 * c6, 58);
-  p.rpre2 = (float)(1.008 * rc * rc * std::ldexp(1.0, 36));
+  p.rpre2 = (float)(1.008 * rc * rc * std::ldexp(1.0, 2 * (p.pos - 32)));
   p.fs = 24.0 * eps * c6 * std::ldexp(1.0, -b - 57 - 3 * e);
   p.w3 = 24.0 * eps * c6 * std::ldexp(1.0, -57 - 3 * e);
   p.us = eps * c6 * std::ldexp(1.0, -59 - 3 * e);
@@ -108,16 +121,16 @@ __host__ __device__ __forceinline__ uint64_t lj_recip(uint64_t xn) {
   return (v1 << 22) + (uint64_t)(((int64_t)(int)(v1 >> 11) * (int)(e1 >> 32)) >> 37);         // Q62
 }
 
-// x 2^50 modulo 2^64, rounded (positions are kept wrapped into the box, so the
+// x 2^pos modulo 2^64, rounded (positions are kept wrapped into the box, so the
 // modulus never shows).
-__host__ __device__ __forceinline__ int64_t fix_pos(double x) {
+__host__ __device__ __forceinline__ int64_t fix_pos(double x, int pos) {
 #ifdef __CUDA_ARCH__
   const uint64_t bits = (uint64_t)__double_as_longlong(x);
 #else
   uint64_t bits;
   __builtin_memcpy(&bits, &x, 8);
 #endif
-  const int s = (int)((bits >> 52) & 0x7ff) - 1075 + kPosBits;
+  const int s = (int)((bits >> 52) & 0x7ff) - 1075 + pos;
   const uint64_t m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;
   uint64_t r;
   if (s >= 0)
@@ -129,8 +142,8 @@ __host__ __device__ __forceinline__ int64_t fix_pos(double x) {
 
 // Position wrapped into the box edge L (its fix_pos LQ): x - L floor(x / L),
 // up to one rounding of the quotient either side.
-__host__ __device__ __forceinline__ int64_t fix_wrap(double x, float xf, float invL, int64_t LQ) {
-  return fix_pos(x) - (int64_t)floorf(xf * invL) * LQ;
+__host__ __device__ __forceinline__ int64_t fix_wrap(double x, int pos, float xf, float invL, int64_t LQ) {
+  return fix_pos(x, pos) - (int64_t)floorf(xf * invL) * LQ;
 }
 
 // Minimum image of a difference of two wrapped positions.
@@ -165,7 +178,7 @@ __host__ __device__ __forceinline__ void add_signed(__int128 &s, uint64_t v, boo
 // for a pair closer than the fixed-point range.
 template <bool kDiag>
 __host__ __device__ __forceinline__ bool lj_fix_pair(const LjFix &p, const int64_t (&d)[3], LjSums &s) {
-  const int sh = 64 - kPosBits - p.b;
+  const int sh = 64 - p.pos - p.b;   // at least 2: 2^b < 2.02 rc, and rc is below half an edge
   uint64_t dn[3], r2 = 0;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {

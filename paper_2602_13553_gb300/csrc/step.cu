@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(384) k_step_f64(StepArgs a) {
     if (oxy) {
       const float sc = sh < -126 ? 0.f : (sh > 127 ? __int_as_float(0x7f800000) : __int_as_float((sh + 127) << 23));
       const double Lc = a.dbox ? a.dbox[c] : a.box[c], iLc = a.dbox ? a.dbox[3 + c] : a.invbox[c];
-      a.xi[((size_t)i + c) * P + k] = fix_wrap(xn, (float)Sj * sc, (float)iLc, fix_pos(Lc));   // row 3 (i / 3) + c
+      a.xi[((size_t)i + c) * P + k] = fix_wrap(xn, a.pos, (float)Sj * sc, (float)iLc, fix_pos(Lc, a.pos));   // row 3 (i / 3) + c
       dev = Eq > kFixMaxE ? __int_as_float(0x7f800000) : (float)(Sj - sC[row]) * sc;
       sD[c * AP + u] = dev;
     }
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(256) k_step_cart_f64(StepArgs a) {
     if (a.xi && i % 3 == 0) {
       const int c = r % 3;
       const double Lc = a.dbox ? a.dbox[c] : a.box[c], iLc = a.dbox ? a.dbox[3 + c] : a.invbox[c];
-      a.xi[((size_t)i + c) * P + k] = fix_wrap(x, (float)x, (float)iLc, fix_pos(Lc));   // row 3 (i / 3) + c
+      a.xi[((size_t)i + c) * P + k] = fix_wrap(x, a.pos, (float)x, (float)iLc, fix_pos(Lc, a.pos));   // row 3 (i / 3) + c
     }
     sN[task] = x;
   }
